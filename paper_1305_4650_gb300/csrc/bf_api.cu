@@ -11,6 +11,7 @@
 
 #include "../../include/bf.h"
 #include "bf_device.cuh"
+#include "bf_host.h"
 #include "bf_launch.h"
 #include "bf_mr.cuh"
 #include <algorithm>
@@ -39,6 +40,7 @@ struct bf_plan_s {
     void *w0 = nullptr, *w1 = nullptr;
     void *ctab = nullptr;      // target features at box centres, levels 0..ctab_levels
     int ctab_levels = -1;
+    int corner = 0;            // CORNER_* of the forward passes
     void *gstage = nullptr, *fstage = nullptr;
     size_t csize = 8;          // bytes per complex number
     int64_t ws_bytes = 0;
@@ -81,9 +83,10 @@ struct bf_batch_s {
 };
 
 namespace bfl {
-const PassFns *get_fns(int d, int q, int prec, int kind)
+const PassFns *get_fns(int d, int q, int prec, int kind, int nk)
 {
-#define BFL_PICK(dd, kn) (prec == 0 ? fns_d##dd##_f64_##kn(q) : prec == 1 ? fns_d##dd##_mix_##kn(q) : fns_d##dd##_sfu_##kn(q))
+#define BFL_PICK(dd, kn) \
+    (prec == 0 ? fns_d##dd##_f64_##kn(q, nk) : prec == 1 ? fns_d##dd##_mix_##kn(q, nk) : fns_d##dd##_sfu_##kn(q, nk))
     if (d == 2) {
         switch (kind) {
         case BF_PHASE_DOT: return BFL_PICK(2, dot);
@@ -154,7 +157,11 @@ void tfeat(int kind, double s, int k, double x, double f[3])
     f[0] = f[1] = f[2] = 0.0;
     switch (kind) {
     case BF_PHASE_DOT: f[0] = s * x; break;
-    case BF_PHASE_GENRADON: f[0] = s * x; f[1] = std::sin(2 * kPi * x); f[2] = std::cos(2 * kPi * x); break;
+    case BF_PHASE_GENRADON: {   // the factor makes the products of a_k carry |s|/3
+        const double c = std::sqrt(std::fabs(s) / 3.0);
+        f[0] = s * x; f[1] = c * std::sin(2 * kPi * x); f[2] = c * std::cos(2 * kPi * x);
+        break;
+    }
     case BF_PHASE_HYPRADON: f[0] = s * x; f[1] = x * x; break;
     default: f[0] = s * std::sin(2 * kPi * (x + (k + 1) / 7.0)); break;
     }
@@ -247,20 +254,13 @@ bf_status build_tables(bf_plan p)
     return BF_OK;
 }
 
-// shared memory of a pass: T tiles of 2^{dk} pairs, plus twice that as stage scratch
+// shared memory of a forward single-RHS pass
+size_t fwd_smem(const bf_plan_s *p, const Pass &ps, bool tab = false) { return p->fns->tile_smem(ps.row, ps.T, ps.k, tab); }
+
+// shared memory of an adjoint pass: T tiles of 2^{dk} pairs, plus twice that as stage scratch
 size_t pass_smem(const bf_plan_s *p, const Pass &ps)
 {
     return (size_t)3 * (size_t)ps.T * ((size_t)1 << (p->d * ps.k)) * (size_t)p->r * p->csize;
-}
-
-// plus, for a row pass, the cache of the parents' node features (T 2^{d(k-1)} boxes x r nodes);
-// for a column pass, the geometry of every output pair of a level (T 2^{dk} records of the
-// centre features and four ints, rounded to 16 bytes)
-size_t row_cache_smem(const bf_plan_s *p, const Pass &ps)
-{
-    if (!ps.row) return (size_t)ps.T * ((size_t)1 << (p->d * ps.k)) * (((size_t)p->fns->tsize + 16 + 15) / 16 * 16);
-    if (ps.k < 1) return 0;
-    return (size_t)ps.T * ((size_t)1 << (p->d * (ps.k - 1))) * (size_t)p->r * (size_t)p->fns->tsize;
 }
 
 // the adjoint row pass caches children's and parents' node features (T (2^{dk} + 2^{d(k-1)}) boxes x r);
@@ -280,7 +280,7 @@ size_t row_adj_cache_smem(const bf_plan_s *p, const Pass &ps)
 size_t mr_smem(const bf_plan_s *p, const Pass &ps, int nr, int rc)
 {
     const size_t npr = (size_t)ps.T << (p->d * ps.k);
-    return p->csize * (npr * (size_t)p->r * (size_t)(nr + 5) + (size_t)rc * (size_t)bfk::mr_s_stride(p->q, (int64_t)npr) +
+    return p->csize * (npr * (size_t)p->r * (size_t)(nr + 5) + (size_t)bfk::mr_s_size(p->q, (int64_t)npr, rc) +
                        npr * (size_t)bfk::mr_pc_extra(p->q));
 }
 
@@ -291,47 +291,23 @@ size_t mr_smem_table(const bf_plan_s *p, const Pass &ps, int nr, int rc)
     const size_t npr = (size_t)ps.T << (p->d * ps.k);
     const size_t blk = (size_t)(p->q > 5 ? p->q : 5) * (size_t)p->r * npr;
     return (size_t)bfk::TABCTL_BYTES + 2 * blk * p->csize +
-           p->csize * (npr * (size_t)p->r * (size_t)nr + (size_t)rc * (size_t)bfk::mr_s_stride(p->q, (int64_t)npr));
+           p->csize * (npr * (size_t)p->r * (size_t)nr + (size_t)bfk::mr_s_size(p->q, (int64_t)npr, rc));
 }
 
 // A CTA owns np pairs (2^{d kmax} of the instantiation, fewer for tiny problems):
 // T = np / 2^{dk} tiles of a k-level pass.
 Pass make_pass(const bf_plan_s *p, int64_t np_cta, int row, int l0, int k, int flags)
 {
-    const int64_t np = p->npts < np_cta ? p->npts : np_cta;
-    Pass ps{row, l0, k, flags, (int)(np >> (p->d * k))};
-    if (ps.T < 1) ps.T = 1;
-    return ps;
+    return Pass{row, l0, k, flags, bfl::tiles_of(p->npts, np_cta, p->d, k)};
 }
 
 // column passes of <= kmax levels (init first, switch last), then row passes (final last)
 // (rem_first: the short pass of each run of levels goes first instead of last)
-std::vector<Pass> schedule(const bf_plan_s *p, int kmax, int64_t np_cta, bool rem_first = false)
+std::vector<Pass> schedule(const bf_plan_s *p, int kmax, int64_t np_cta, bool rem_first = false, int corner = 0)
 {
     std::vector<Pass> out;
-    const int m = p->m, L = p->L;
-    auto chunk = [&](int left, int total) {
-        const int r = total % kmax;
-        if (rem_first && r && left == total) return r;
-        return left < kmax ? left : kmax;
-    };
-    if (m == 0) {
-        out.push_back(make_pass(p, np_cta, 0, 0, 0, bfk::F_INIT | bfk::F_SWITCH));
-    } else {
-        for (int l = 0; l < m;) {
-            const int k = chunk(m - l, m);
-            int fl = 0;
-            if (l == 0) fl |= bfk::F_INIT;
-            if (l + k == m) fl |= bfk::F_SWITCH;
-            out.push_back(make_pass(p, np_cta, 0, l, k, fl));
-            l += k;
-        }
-    }
-    for (int l = m; l < L;) {
-        const int k = chunk(L - l, L - m);
-        out.push_back(make_pass(p, np_cta, 1, l, k, (l + k == L) ? bfk::F_FINAL : 0));
-        l += k;
-    }
+    bfl::each_pass(p->L, p->m, kmax, rem_first, corner,
+                   [&](int row, int l0, int k, int flags) { out.push_back(make_pass(p, np_cta, row, l0, k, flags)); });
     return out;
 }
 
@@ -387,17 +363,16 @@ void fill_args(const bf_plan_s *p, bfk::KArgs<P> &a)
     const double s = p->prm.phase_scale;
     const double sgn = s > 0 ? 1.0 : (s < 0 ? -1.0 : 0.0);
     if constexpr (P::is_f64) {
-        a.sc.s3 = s / 3.0;
+        a.sc.c2 = 2.0 * std::fabs(s) / 3.0;
         a.sc.sgn = sgn;
     } else {
-        float hi, lo;
-        split(s / 3.0, hi, lo);
-        a.sc.s3hi = hi;
-        a.sc.s3lo = lo;
+        split(2.0 * std::fabs(s) / 3.0, a.sc.c2hi, a.sc.c2lo);
         a.sc.sgn = (float)sgn;
+        a.sc.mg = bfl::sqrt_grid(p->d, p->kind, &p->prm);
     }
     a.ctab = p->ctab;
     a.ctab_levels = p->ctab_levels;
+    a.corner = p->corner;
     a.L = p->L;
     a.kind = p->kind;
     a.npts = p->npts;
@@ -518,7 +493,7 @@ bf_status run_forward(bf_plan p, const void *g, void *f, int nrhs, cudaStream_t 
         a.wout = static_cast<typename P::C *>(buf[(i + 1) & 1]);
         a.ftab = tab ? p->ftab + p->ftab_off[i] : nullptr;
         a.ftab_cta = tab ? p->ftab_cta[i] : 0;
-        const size_t smem = pass_smem(p, ps) + row_cache_smem(p, ps);
+        const size_t smem = fwd_smem(p, ps, tab);
         const bfl::pass_fn fn = tab ? (ps.row ? p->fns->row_tab : p->fns->col_tab)[1] : (ps.row ? p->fns->row : p->fns->col);
         cudaError_t e = fn(&a, (unsigned)ctas, (unsigned)nrhs, smem, s);
         if (e != cudaSuccess) return cuda_fail(p, e);
@@ -551,38 +526,6 @@ bf_status run_adjoint(bf_plan p, const void *f, void *g, int nrhs, cudaStream_t 
         if (e != cudaSuccess) return cuda_fail(p, e);
     }
     return BF_OK;
-}
-
-// Upper bound of |Phi| over X x Y.  The mixed path rounds to integers by adding
-// 1.5 * 2^23, which is exact only below 2^22 cycles (kept under 2^21 here).
-double phase_bound(int d, int kind, const bf_params *p)
-{
-    double mx[3], my[3];
-    for (int k = 0; k < d; ++k) {
-        mx[k] = std::fmax(std::fabs(p->x_lo[k]), std::fabs(p->x_lo[k] + p->x_w[k]));
-        my[k] = std::fmax(std::fabs(p->y_lo[k]), std::fabs(p->y_lo[k] + p->y_w[k]));
-    }
-    double b = 0.0;
-    switch (kind) {
-    case BF_PHASE_DOT:
-        for (int k = 0; k < d; ++k) b += mx[k] * my[k];
-        break;
-    case BF_PHASE_GENRADON: {
-        double q2 = 0.0;
-        for (int k = 0; k < d; ++k) {
-            b += mx[k] * my[k];
-            q2 += my[k] * my[k];                      // a_k(x) <= 1
-        }
-        b += std::sqrt(q2);
-        break;
-    }
-    case BF_PHASE_HYPRADON:
-        b = mx[0] * std::sqrt(my[0] * my[0] + my[1] * my[1] * mx[1] * mx[1]);
-        break;
-    default:
-        for (int k = 0; k < d; ++k) b += 1.0 + my[k] * my[k] / (k + 2.0);
-    }
-    return std::fabs(p->phase_scale) * b;
 }
 
 // the multi-RHS schedule serves nrhs >= 2 where it is compiled (mixed precisions, d = 2)
@@ -770,6 +713,7 @@ bf_status run_points(bf_plan p, const void *g, void *f, int nrhs, cudaStream_t s
     if (e != cudaSuccess) return cuda_fail(p, e);
     bfk::KArgs<P> a;
     fill_args<P>(p, a);
+    a.corner = 0;   // the points are not the grid's
     const int n = (int)p->passes_pts.size();
     for (int i = 0; i < n; ++i) {
         const Pass &ps = p->passes_pts[i];
@@ -780,7 +724,7 @@ bf_status run_points(bf_plan p, const void *g, void *f, int nrhs, cudaStream_t s
         a.win = static_cast<const typename P::C *>(buf[i & 1]);
         a.wout = static_cast<typename P::C *>(buf[(i + 1) & 1]);
         const int64_t ctas = (p->npts >> (p->d * ps.k)) / ps.T;
-        const size_t smem = pass_smem(p, ps) + row_cache_smem(p, ps);
+        const size_t smem = fwd_smem(p, ps);
         e = (ps.row ? p->fns->row : p->fns->col)(&a, (unsigned)ctas, (unsigned)nrhs, smem, s);
         if (e != cudaSuccess) return cuda_fail(p, e);
     }
@@ -897,7 +841,7 @@ bf_status build_tile_table(bf_plan p)
         a.ftab = p->ftab + p->ftab_off[i];
         a.ftab_cta = p->ftab_cta[i];
         const int64_t ctas = (p->npts >> (p->d * ps.k)) / ps.T;
-        const size_t smem = pass_smem(p, ps) + row_cache_smem(p, ps);
+        const size_t smem = fwd_smem(p, ps);
         e = (ps.row ? p->fns->row_tab : p->fns->col_tab)[0](&a, (unsigned)ctas, 1u, smem, 0);
     }
     if (e == cudaSuccess) e = cudaEventRecord(e1);
@@ -953,7 +897,7 @@ void build_weight_maps(bf_plan p)
     p->tmaps = d;
 }
 
-bool supported_q(int d, int q) { return bfl::get_fns(d, q, 1, 0) != nullptr && bfl::get_fns(d, q, 0, 0) != nullptr; }
+bool supported_q(int d, int q) { return bfl::get_fns(d, q, 1, 0, 0) != nullptr && bfl::get_fns(d, q, 0, 0, 0) != nullptr; }
 
 }  // namespace
 
@@ -1151,7 +1095,7 @@ bf_status bf_plan_create(int d, int64_t N, int q, bf_phase_kind phase, const bf_
     if (phase == BF_PHASE_HYPRADON && d != 2) return BF_ERR_INVALID_ARG;
     if (prm->precision < BF_PREC_FP64 || prm->precision > BF_PREC_TF32X3) return BF_ERR_INVALID_ARG;
     if (!supported_q(d, q)) return BF_ERR_UNSUPPORTED;
-    if (prm->precision != BF_PREC_FP64 && phase_bound(d, (int)phase, prm) >= 2097152.0) return BF_ERR_UNSUPPORTED;
+    if (prm->precision != BF_PREC_FP64 && bfl::phase_bound(d, (int)phase, prm) >= 2097152.0) return BF_ERR_UNSUPPORTED;
     for (int k = 0; k < d; ++k) {
         if (!(prm->x_w[k] > 0.0) || !(prm->y_w[k] > 0.0)) return BF_ERR_INVALID_ARG;
         if (!std::isfinite(prm->x_lo[k]) || !std::isfinite(prm->y_lo[k]) || !std::isfinite(prm->x_w[k]) ||
@@ -1189,7 +1133,7 @@ bf_status bf_plan_create(int d, int64_t N, int q, bf_phase_kind phase, const bf_
     p->prm = *prm;
     p->csize = p->prec == BF_PREC_FP64 ? 16 : 8;
     // BF16X3 and TF32X3 evaluate their phases as BF_PREC_MIXED does and run the same kernels but the switch
-    p->fns = bfl::get_fns(d, q, tc_prec(p->prec) ? (int)BF_PREC_MIXED : (int)p->prec, (int)phase);
+    p->fns = bfl::get_fns(d, q, tc_prec(p->prec) ? (int)BF_PREC_MIXED : (int)p->prec, (int)phase, p->node_kind);
     if (!p->fns) {   // this combination was not compiled into the library
         delete p;
         return BF_ERR_UNSUPPORTED;
@@ -1208,7 +1152,8 @@ bf_status bf_plan_create(int d, int64_t N, int q, bf_phase_kind phase, const bf_
     const int kfit = p->fns->kmax;
     const int kreq = prm->fuse_levels > 0 ? prm->fuse_levels : kfit;
     p->kc = p->kr = kreq < kfit ? kreq : kfit;
-    p->passes = schedule(p, p->kc, p->fns->np, true);
+    p->corner = bfl::corner_of(d, q, p->m, prm, p->fns->lobatto, tc_prec(p->prec));
+    p->passes = schedule(p, p->kc, p->fns->np, true, p->corner);
     if (p->fns->col_mr[0]) {
         // 2 fused levels, as many pairs per CTA as one switch round covers (at least one tile);
         // scratch for enough right-hand sides to give every thread an item, fewer if the
@@ -1216,7 +1161,7 @@ bf_status bf_plan_create(int d, int64_t N, int q, bf_phase_kind phase, const bf_
         const int kmr = kreq < 2 ? kreq : 2;
         const int nr = p->max_nrhs < p->fns->mr_max ? p->max_nrhs : p->fns->mr_max;
         const int64_t ppr = p->fns->mr_nthreads / p->r;
-        p->passes_mr = schedule(p, kmr, ppr, true);
+        p->passes_mr = schedule(p, kmr, ppr, true, p->corner);
         tc_switch_split(p, p->passes_mr);
         int64_t npr = 0;
         for (const Pass &ps : p->passes_mr)
@@ -1453,7 +1398,7 @@ bf_status bf_plan_autotune(bf_plan p, int nrhs, int reps, void *stream, double *
                     for (int ri = 0; ri < 6 && st == BF_OK; ++ri) {
                         const int rc = rcs[ri];
                         if (rc > nr) continue;
-                        std::vector<Pass> cand = schedule(p, k, np, rem != 0);
+                        std::vector<Pass> cand = schedule(p, k, np, rem != 0, p->corner);
                         tc_switch_split(p, cand);
                         bool fits = true;
                         for (const Pass &ps : cand)
@@ -1479,10 +1424,10 @@ bf_status bf_plan_autotune(bf_plan p, int nrhs, int reps, void *stream, double *
         st = time_it(best);
         for (int k = 1; k <= p->fns->kmax && st == BF_OK; ++k)
             for (int rem = 0; rem < 2 && st == BF_OK; ++rem) {
-                std::vector<Pass> cand = schedule(p, k, p->fns->np, rem != 0);
+                std::vector<Pass> cand = schedule(p, k, p->fns->np, rem != 0, p->corner);
                 bool fits = true;
                 for (const Pass &ps : cand)
-                    if (pass_smem(p, ps) + row_cache_smem(p, ps) > 227 * 1024) fits = false;
+                    if (fwd_smem(p, ps) > 227 * 1024) fits = false;
                 if (!fits) continue;
                 p->passes = cand;
                 double ms = 0.0;

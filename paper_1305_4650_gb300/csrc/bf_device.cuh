@@ -103,14 +103,27 @@ __device__ __forceinline__ df df_mul_u(df x, df y)
     return {p, e};
 }
 
-// sqrt of a non-negative (possibly unnormalised) double-float, to about 2^-44
-// relative, returned unnormalised: one Newton step from the FP32 reciprocal root
-__device__ __forceinline__ df df_sqrt_u(df x)
+// reciprocal square root from the special-function unit (arguments are normal FP32 numbers
+// here, so the form without denormal handling)
+__device__ __forceinline__ float rsqrt_approx(float x)
 {
-    float r = rsqrtf(fmaxf(x.hi, 1e-30f));
-    float s = __fmul_rn(x.hi, r);
-    float res = __fadd_rn(__fmaf_rn(-s, s, x.hi), x.lo);
-    return {s, __fmul_rn(res, __fmul_rn(0.5f, r))};
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+
+// sg sqrt(h + l) minus its nearest integer, sg = +-1, for h + l > 0 given to about 2^-44
+// relative: one Newton step from the FP32 reciprocal root, added to the exact difference of
+// the FP32 root and its nearest integer, so only a number of at most 1/2 is rounded
+__device__ __forceinline__ float sqrt_frac(float h, float l, float sg)
+{
+    const float M = 12582912.0f;
+    const float q = __fadd_rn(h, l);
+    const float r = __fmul_rn(sg, rsqrt_approx(q));
+    const float s = __fmul_rn(q, r);
+    const float w = __fsub_rn(s, __fsub_rn(__fadd_rn(s, M), M));
+    const float res = __fadd_rn(__fmaf_rn(-s, s, h), l);
+    return __fmaf_rn(0.5f, __fmul_rn(res, r), w);
 }
 
 // x - nearest integer (|x| < 2^22), one float in about [-0.5, 0.5]
@@ -135,14 +148,14 @@ struct PF64 {
     using C = double2;
     struct TE { double2 a, b; };   // target feature table entry: f0, f1 | f2, pad
     struct SE { double2 a; };      // source feature table entry: f0, f1
-    struct Sc { double s3, sgn; }; // s/3 and sign(s)
+    struct Sc { double c2, sgn; }; // 2|s|/3 and sign(s)
     static constexpr bool is_f64 = true;
     static constexpr bool sfu = false;
 };
 
 struct MixTE { float4 a, b; };  // (f0.hi, f0.lo, f1.hi, f1.lo) | (f2.hi, f2.lo, -, -)
 struct MixSE { float4 a; };     // (f0.hi, f0.lo, f1.hi, f1.lo)
-struct MixSc { float s3hi, s3lo, sgn, pad; };
+struct MixSc { float c2hi, c2lo, sgn, mg; };   // 2|s|/3, sign(s), grid constant of the sqrt parts (Ph::quant)
 
 // complex64 weights, double-float phase; SFU = true takes sin/cos of the reduced phase
 // from the special-function unit (__sincosf) instead of the polynomial below
@@ -169,12 +182,33 @@ __device__ __forceinline__ void sincos2pi(double fr, double &s, double &c) { sin
 constexpr float SC_S0 = 6.28318500518798828f, SC_S1 = -41.3416290283203125f, SC_S2 = 81.5881271362304688f,
                 SC_S3 = -75.2400665283203125f;
 constexpr float SC_C1 = -19.7391681671142578f, SC_C2 = 64.9232254028320312f, SC_C3 = -83.665924072265625f;
+__device__ __forceinline__ void quad_sincos(float r, int q, float &s, float &c);
 __device__ __forceinline__ void sincos2pi(float f, float &s, float &c)
 {
     const float M = 12582912.0f;
     const float t = __fmaf_rn(4.0f, f, M);                 // j + 1.5 * 2^23
-    const int q = __float_as_int(t);                       // low two bits: j mod 4
-    const float r = __fmaf_rn(-0.25f, __fsub_rn(t, M), f);
+    quad_sincos(__fmaf_rn(-0.25f, __fsub_rn(t, M), f), __float_as_int(t), s, c);
+}
+
+// sin and cos of 2 pi f from the special-function unit after reduction to |f| <= 1/2
+// (CUDA documents 2^-21.41 absolute error for |x| <= pi)
+__device__ __forceinline__ void sincos2pi_sfu(float f, float &s, float &c)
+{
+    const float r = __fsub_rn(f, fround(f));
+    __sincosf(__fmul_rn(r, 6.28318530717958647692f), &s, &c);
+}
+
+// the sincos above for a phase a + b given as two numbers: r keeps the rounding error of a
+// number of at most 1/8, not of a + b; the low two bits of j hold the quadrant
+__device__ __forceinline__ void quad_reduce(float a, float b, float &r, int &j)
+{
+    const float M = 12582912.0f;
+    const float t = __fmaf_rn(4.0f, __fadd_rn(a, b), M);
+    j = __float_as_int(t);
+    r = __fadd_rn(__fmaf_rn(-0.25f, __fsub_rn(t, M), a), b);
+}
+__device__ __forceinline__ void quad_sincos(float r, int q, float &s, float &c)
+{
     const float u = __fmul_rn(r, r);
     float ps = __fmaf_rn(u, SC_S3, SC_S2);
     ps = __fmaf_rn(u, ps, SC_S1);
@@ -187,14 +221,6 @@ __device__ __forceinline__ void sincos2pi(float f, float &s, float &c)
     const float c1 = (q & 1) ? sn : cs;
     s = __int_as_float(__float_as_int(s1) ^ ((q & 2) << 30));
     c = __int_as_float(__float_as_int(c1) ^ (((q + 1) & 2) << 30));
-}
-
-// sin and cos of 2 pi f from the special-function unit after reduction to |f| <= 1/2
-// (CUDA documents 2^-21.41 absolute error for |x| <= pi)
-__device__ __forceinline__ void sincos2pi_sfu(float f, float &s, float &c)
-{
-    const float r = __fsub_rn(f, fround(f));
-    __sincosf(__fmul_rn(r, 6.28318530717958647692f), &s, &c);
 }
 
 __device__ __forceinline__ float2 cmul(float2 a, float2 b)
@@ -239,6 +265,7 @@ struct KArgs {
     typename P::Sc sc;
     int L, l0, k, flags, kind;
     int T;                            // tiles per CTA (T * 2^{dk} pairs)
+    int corner;                       // CORNER_* (bf_tile2.cuh): grid points on nodes, first / last levels shortened
     int nrhs;                         // right-hand sides of the launch (multi-RHS kernels)
     int rc;                           // right-hand sides per scratch chunk (multi-RHS kernels)
     const void *ctab;                 // target features at box centres, levels 0..ctab_levels (or null)
@@ -335,7 +362,7 @@ template <int Q> __device__ __forceinline__ int soff(int L, int l) { return ((2 
 //
 // Target features per dimension (built on the host, kind-specific):
 //   DOT        f0 = s x
-//   GENRADON   f0 = s x, f1 = sin 2pi x, f2 = cos 2pi x
+//   GENRADON   f0 = s x, f1 = c sin 2pi x, f2 = c cos 2pi x with c = sqrt(|s|/3)
 //   HYPRADON   f0 = s x, f1 = x^2
 //   SEPARABLE  f0 = s sin 2pi (x + (k+1)/7)
 // Source features per dimension:
@@ -351,24 +378,26 @@ struct Ph<PMIXT<F>, D, K> {
     static __device__ __forceinline__ df hi(const float4 &v) { return {v.x, v.y}; }
     static __device__ __forceinline__ df lo(const float4 &v) { return {v.z, v.w}; }
 
-    // target point from its per-dimension table entries; GENRADON forms A_k = (s a_k(x))^2
+    // target point from its per-dimension table entries.  GENRADON: A_k = (s a_k(x))^2, from
+    // features that carry the factor sqrt(|s|/3); HYPRADON: A_0 = (s x_0)^2, A_1 = (s x_0 x_1)^2
     static __device__ __forceinline__ T tgt(const KArgs<PMIXT<F>> &a, const MixTE *e)
     {
         T t;
 #pragma unroll
         for (int k = 0; k < D; ++k) { t.x[k] = hi(e[k].a); t.A[k] = lo(e[k].a); }
         if constexpr (K == KIND_GENRADON) {
-            const df s3 = {a.sc.s3hi, a.sc.s3lo};
 #pragma unroll
             for (int k = 0; k < D; ++k) {
                 df u;
                 if constexpr (D == 2) u = (k == 0) ? df_mul_u(lo(e[0].a), lo(e[1].a)) : df_mul_u(hi(e[0].b), hi(e[1].b));
                 else u = df_mul_u(lo(e[k].a), hi(e[(k + 1) % D].b));
-                df two = two_sum(2.0f, u.hi);
-                u = {two.hi, __fadd_rn(two.lo, u.lo)};
-                u = df_mul_u(u, s3);
-                t.A[k] = df_mul(u, u);
+                const df two = fast_two_sum(a.sc.c2hi, u.hi);   // |u| <= |s|/3 < 2|s|/3
+                u = {two.hi, __fadd_rn(two.lo, __fadd_rn(u.lo, a.sc.c2lo))};
+                t.A[k] = df_mul_u(u, u);
             }
+        } else if constexpr (K == KIND_HYPRADON) {
+            t.A[0] = df_mul_u(t.x[0], t.x[0]);
+            t.A[1] = df_mul_u(t.A[0], t.A[1]);
         }
         return t;
     }
@@ -379,84 +408,86 @@ struct Ph<PMIXT<F>, D, K> {
         s.y2[k] = lo(e.a);
     }
 
-    // Per-dimension split of Phi: part(t, y_k entry, k) is the contribution of source
-    // coordinate k; parts add (add), and fin() turns their sum into Phi minus an integer.
-    // Loops hoist the parts of the source coordinates that do not change.
-    struct Part { float f; df q; };
-    static __device__ __forceinline__ Part part(const T &t, const MixSE &e, int k)
+    // Per-dimension split of Phi: the part of source coordinate k; parts add componentwise
+    // (add), and fin() turns their sum into Phi minus an integer.  f: a linear phase mod 1.
+    // h + l: a term of the sum of squares under the root, h a multiple of a power of two G
+    // (quant) such that the sum of the parts' h, below 2^22 G, is exact: adding two terms takes
+    // two additions instead of an exact sum of double-floats.  Loops hoist the
+    // parts of the source coordinates that do not change.
+    static constexpr bool HAS_F = K != KIND_HYPRADON, HAS_Q = K == KIND_GENRADON || K == KIND_HYPRADON;
+    struct Part { float f, h, l; };
+    static constexpr int NCMP = (HAS_F ? 1 : 0) + (HAS_Q ? 2 : 0);
+    // fn(component, its index) for the components that this kind uses
+    template <class PT, class Fn>
+    static __device__ __forceinline__ void each(PT &p, Fn fn)
     {
-        Part p{0.0f, {0.0f, 0.0f}};
-        const df y = hi(e.a), y2 = lo(e.a);
-        if constexpr (K == KIND_DOT) {
-            p.f = df_mul_frac(t.x[k], y);
-        } else if constexpr (K == KIND_GENRADON) {
-            p.f = df_mul_frac(t.x[k], y);
-            p.q = df_mul_u(t.A[k], y2);
-        } else if constexpr (K == KIND_HYPRADON) {
-            p.q = (k == 0) ? y2 : df_mul_u(t.A[1], y2);
-        } else {
-            p.q = df_add(t.x[k], y);
+        if constexpr (HAS_F) fn(p.f, 0);
+        if constexpr (HAS_Q) {
+            fn(p.h, NCMP - 2);
+            fn(p.l, NCMP - 1);
         }
+    }
+    // h = p rounded to a multiple of G (sc.mg = 1.5 * 2^23 G, p < 2^22 G); the first part adds
+    // a tiny number that keeps the root's argument positive
+    static __device__ __forceinline__ void quant(const KArgs<PMIXT<F>> &a, const df &p, bool first, Part &o)
+    {
+        o.h = __fsub_rn(__fadd_rn(p.hi, a.sc.mg), a.sc.mg);
+        o.l = __fadd_rn(__fsub_rn(p.hi, o.h), p.lo);
+        o.l = __fadd_rn(o.l, first ? 1e-30f : 0.0f);
+    }
+    // the part of one source coordinate from the target's features x and A of that coordinate
+    static __device__ __forceinline__ Part part_of(const KArgs<PMIXT<F>> &a, const df &x, const df &A, const MixSE &e, bool first)
+    {
+        Part p{0.0f, 0.0f, 0.0f};
+        if constexpr (K == KIND_DOT || K == KIND_GENRADON) p.f = df_mul_frac(x, hi(e.a));
+        if constexpr (K == KIND_SEPARABLE) p.f = df_frac(df_add(x, hi(e.a)));
+        if constexpr (HAS_Q) quant(a, df_mul_u(A, lo(e.a)), first, p);
         return p;
+    }
+    static __device__ __forceinline__ Part part(const KArgs<PMIXT<F>> &a, const T &t, const MixSE &e, int k)
+    {
+        return part_of(a, t.x[k], t.A[k], e, k == 0);
     }
     static __device__ __forceinline__ Part add(const Part &u, const Part &v)
     {
-        df s;
-        if constexpr (K == KIND_GENRADON || K == KIND_HYPRADON) {
-            // both parts are sums of squares times non-negative factors: with the larger one
-            // first the fast two-sum is exact (the same s and error term as the two-sum)
-            s = fast_two_sum(fmaxf(u.q.hi, v.q.hi), fminf(u.q.hi, v.q.hi));
-        } else {
-            s = two_sum(u.q.hi, v.q.hi);
+        Part p{0.0f, 0.0f, 0.0f};
+        if constexpr (HAS_F) p.f = __fadd_rn(u.f, v.f);
+        if constexpr (HAS_Q) {
+            p.h = __fadd_rn(u.h, v.h);
+            p.l = __fadd_rn(u.l, v.l);
         }
-        return Part{u.f + v.f, {s.hi, __fadd_rn(__fadd_rn(u.q.lo, v.q.lo), s.lo)}};
+        return p;
     }
-    static __device__ __forceinline__ float fin(const KArgs<PMIXT<F>> &a, const T &t, const Part &p)
+    // sign of the root's term at a target
+    static __device__ __forceinline__ float sign(const KArgs<PMIXT<F>> &a, const T &t)
     {
-        if constexpr (K == KIND_DOT) {
-            return p.f;
-        } else if constexpr (K == KIND_GENRADON) {
-            return __fmaf_rn(a.sc.sgn, df_frac(df_sqrt_u(p.q)), p.f);
-        } else if constexpr (K == KIND_HYPRADON) {
-            return df_mul_frac(t.x[0], df_sqrt_u(p.q));
-        } else {
-            return df_frac(p.q);
-        }
+        if constexpr (K == KIND_HYPRADON)
+            return copysignf(1.0f, t.x[0].hi);
+        else
+            return a.sc.sgn;
+    }
+    // Phi minus an integer as two numbers a + b (quad_reduce)
+    static __device__ __forceinline__ void fin2(float sg, const Part &p, float &ra, float &rb)
+    {
+        ra = rb = 0.0f;
+        if constexpr (HAS_F) ra = p.f;
+        if constexpr (HAS_Q) (HAS_F ? rb : ra) = sqrt_frac(p.h, p.l, sg);
+    }
+    static __device__ __forceinline__ float fin(float sg, const Part &p)
+    {
+        float ra, rb;
+        fin2(sg, p, ra, rb);
+        return __fadd_rn(ra, rb);
     }
 
-    // Phi(x, y) minus an integer, |result| < 2 (the sincos reduces it further)
+    // Phi(x, y) minus an integer, |result| < 3 (the sincos reduces it further)
     static __device__ __forceinline__ float frac(const KArgs<PMIXT<F>> &a, const T &t, const S &s)
     {
-        if constexpr (K == KIND_DOT) {
-            float f = 0.0f;
+        Part p = part(a, t, MixSE{make_float4(s.y[0].hi, s.y[0].lo, s.y2[0].hi, s.y2[0].lo)}, 0);
 #pragma unroll
-            for (int k = 0; k < D; ++k) f += df_mul_frac(t.x[k], s.y[k]);
-            return f;
-        } else if constexpr (K == KIND_GENRADON) {
-            float f = 0.0f;
-#pragma unroll
-            for (int k = 0; k < D; ++k) f += df_mul_frac(t.x[k], s.y[k]);
-            // sum_k A_k y_k^2 from unnormalised products and one two-sum of the leading parts
-            df p0 = df_mul_u(t.A[0], s.y2[0]);
-            float lo = p0.lo, hi = p0.hi;
-#pragma unroll
-            for (int k = 1; k < D; ++k) {
-                df pk = df_mul_u(t.A[k], s.y2[k]);
-                df sk = fast_two_sum(fmaxf(hi, pk.hi), fminf(hi, pk.hi));   // both non-negative
-                hi = sk.hi;
-                lo = __fadd_rn(lo, __fadd_rn(pk.lo, sk.lo));
-            }
-            const float fr = df_frac(df_sqrt_u({hi, lo}));
-            return __fmaf_rn(a.sc.sgn, fr, f);
-        } else if constexpr (K == KIND_HYPRADON) {
-            df q = df_add(s.y2[0], df_mul(t.A[1], s.y2[1]));
-            return df_mul_frac(t.x[0], df_sqrt_u(q));
-        } else {
-            df acc = {0.0f, 0.0f};
-#pragma unroll
-            for (int k = 0; k < D; ++k) acc = df_add(acc, df_add(t.x[k], s.y[k]));
-            return df_frac(acc);
-        }
+        for (int k = 1; k < D; ++k)
+            p = add(p, part(a, t, MixSE{make_float4(s.y[k].hi, s.y[k].lo, s.y2[k].hi, s.y2[k].lo)}, k));
+        return fin(sign(a, t), p);
     }
 };
 
@@ -476,7 +507,7 @@ struct Ph<PF64, D, K> {
                 double u;
                 if constexpr (D == 2) u = (k == 0) ? e[0].a.y * e[1].a.y : e[0].b.x * e[1].b.x;
                 else u = e[k].a.y * e[(k + 1) % D].b.x;
-                u = (2.0 + u) * a.sc.s3;
+                u += a.sc.c2;
                 t.A[k] = u * u;
             }
         }
@@ -489,22 +520,41 @@ struct Ph<PF64, D, K> {
         s.y2[k] = e.a.y;
     }
 
+    static constexpr bool HAS_F = K != KIND_HYPRADON, HAS_Q = K == KIND_GENRADON || K == KIND_HYPRADON;
     struct Part { double f, q; };
-    static __device__ __forceinline__ Part part(const T &t, const PF64::SE &e, int k)
+    static constexpr int NCMP = (HAS_F ? 1 : 0) + (HAS_Q ? 1 : 0);
+    template <class PT, class Fn>
+    static __device__ __forceinline__ void each(PT &p, Fn fn)
+    {
+        if constexpr (HAS_F) fn(p.f, 0);
+        if constexpr (HAS_Q) fn(p.q, NCMP - 1);
+    }
+    // the part of one source coordinate from the target's features x and A of that coordinate
+    static __device__ __forceinline__ Part part_of(const KArgs<PF64> &, double x, double A, const PF64::SE &e, bool first)
     {
         const double y = e.a.x, y2 = e.a.y;
-        if constexpr (K == KIND_DOT) return Part{t.x[k] * y, 0.0};
-        else if constexpr (K == KIND_GENRADON) return Part{t.x[k] * y, t.A[k] * y2};
-        else if constexpr (K == KIND_HYPRADON) return Part{0.0, k == 0 ? y2 : t.A[1] * y2};
-        else return Part{t.x[k] + y, 0.0};
+        if constexpr (K == KIND_DOT) return Part{x * y, 0.0};
+        else if constexpr (K == KIND_GENRADON) return Part{x * y, A * y2};
+        else if constexpr (K == KIND_HYPRADON) return Part{0.0, first ? y2 : A * y2};
+        else return Part{x + y, 0.0};
+    }
+    static __device__ __forceinline__ Part part(const KArgs<PF64> &a, const T &t, const PF64::SE &e, int k)
+    {
+        return part_of(a, t.x[k], t.A[k], e, k == 0);
     }
     static __device__ __forceinline__ Part add(const Part &u, const Part &v) { return Part{u.f + v.f, u.q + v.q}; }
-    static __device__ __forceinline__ double fin(const KArgs<PF64> &a, const T &t, const Part &p)
+    // factor of the root's term at a target
+    static __device__ __forceinline__ double sign(const KArgs<PF64> &a, const T &t)
+    {
+        if constexpr (K == KIND_HYPRADON) return t.x[0];
+        else return a.sc.sgn;
+    }
+    static __device__ __forceinline__ double fin(double sg, const Part &p)
     {
         double v;
         if constexpr (K == KIND_DOT || K == KIND_SEPARABLE) v = p.f;
-        else if constexpr (K == KIND_GENRADON) v = p.f + a.sc.sgn * sqrt(p.q);
-        else v = t.x[0] * sqrt(p.q);
+        else if constexpr (K == KIND_GENRADON) v = p.f + sg * sqrt(p.q);
+        else v = sg * sqrt(p.q);
         return v - rint(v);
     }
 
@@ -552,11 +602,19 @@ template <class P, int D, int K>
 __device__ __forceinline__ typename P::C expphase_part(const KArgs<P> &a, const typename Ph<P, D, K>::T &t,
                                                        const typename Ph<P, D, K>::Part &pt)
 {
-    typename P::R fr = Ph<P, D, K>::fin(a, t, pt), sn, cs;
-    if constexpr (P::sfu)
-        sincos2pi_sfu(fr, sn, cs);
-    else
-        sincos2pi(fr, sn, cs);
+    using PH = Ph<P, D, K>;
+    typename P::R sn, cs;
+    if constexpr (P::is_f64) {
+        sincos2pi(PH::fin(PH::sign(a, t), pt), sn, cs);
+    } else if constexpr (P::sfu) {
+        sincos2pi_sfu(PH::fin(PH::sign(a, t), pt), sn, cs);
+    } else {
+        float ra, rb, r;
+        int j;
+        PH::fin2(PH::sign(a, t), pt, ra, rb);
+        quad_reduce(ra, rb, r, j);
+        quad_sincos(r, j, sn, cs);
+    }
     typename P::C e;
     e.x = cs;
     e.y = sn;
@@ -655,6 +713,9 @@ __global__ void k_center_table(const KArgs<P> a, typename Ph<P, D, K>::T *out, i
 
 constexpr int kmax_for(int D, int RR, int CS, int Q)
 {
+    // d = 2 in FP64: the FP64 pipe is saturated by a warp or two per scheduler, so small CTAs
+    // (16 pairs) cost nothing there and spread small problems over more SMs
+    if (D == 2 && CS == 16) return 2;
     int k = 1;
     while (k < (D == 2 ? 4 : 2) && 3 * (1 << (D * (k + 1))) * RR * CS <= 100 * 1024 && (1 << (D * (k + 1))) * Q <= 512) ++k;
     return k;
@@ -698,9 +759,9 @@ struct Tile {
     // coalesced access.  The table holds the reduced phase that the evaluating kernel feeds
     // to its sincos, so reading it gives the evaluating kernel's results exactly.
     struct FT {
-        float *p;   // the stage's block
+        R *p;       // the stage's block
         int n;      // items of the stage
-        __device__ __forceinline__ float *at(int j, int it) const { return p + (int64_t)j * n + it; }
+        __device__ __forceinline__ R *at(int j, int it) const { return p + (int64_t)j * n + it; }
     };
     // items of the stages that evaluate phases, and phases per item
     static __device__ __forceinline__ int n_col_a(const KArgs<P> &a) { return a.T * ((1 << (D * a.k)) >> D) * NC * 2 * Q; }
@@ -747,22 +808,49 @@ struct Tile {
         e.y = sn;
         return e;
     }
-    // one factor from its reduced phase (summed parts): evaluated, evaluated and recorded, or read
-    template <int PM>
-    static __device__ __forceinline__ C ph(const KArgs<P> &a, const typename PH::T &t, const typename PH::Part &pt, float *q)
+    // One factor from its summed parts: evaluated, evaluated and recorded, or read.  The table
+    // holds the operand of the sincos: the reduced phase (SFU sincos), or 2^-64 r of quad_reduce
+    // with the quadrant in bits 29 and 30, which a number below 2^-64 leaves clear.
+    static __device__ __forceinline__ float tab_pack(float r, int j)
     {
-        R fr;
-        if constexpr (PM == PM_TABLE) {
-            fr = __ldcs(q);
+        return __int_as_float(__float_as_int(__fmul_rn(r, 0x1p-64f)) | ((j & 3) << 29));
+    }
+    static __device__ __forceinline__ void tab_unpack(float v, float &r, int &j)
+    {
+        r = __fmul_rn(__int_as_float(__float_as_int(v) & ~0x60000000), 0x1p64f);
+        j = __float_as_int(v) >> 29;
+    }
+    template <int PM>
+    static __device__ __forceinline__ C ph(R sg, const typename PH::Part &pt, R *q)
+    {
+        if constexpr (P::is_f64 || P::sfu) {
+            R fr;
+            if constexpr (PM == PM_TABLE) {
+                fr = __ldcs(q);
+            } else {
+                fr = PH::fin(sg, pt);
+                if constexpr (PM == PM_BUILD) __stcs(q, fr);
+            }
+            return cis(fr);
         } else {
-            fr = PH::fin(a, t, pt);
-            if constexpr (PM == PM_BUILD) __stcs(q, fr);
+            float r;
+            int j;
+            if constexpr (PM == PM_TABLE) {
+                tab_unpack(__ldcs(q), r, j);
+            } else {
+                float ra, rb;
+                PH::fin2(sg, pt, ra, rb);
+                quad_reduce(ra, rb, r, j);
+                if constexpr (PM == PM_BUILD) __stcs(q, tab_pack(r, j));
+            }
+            C e;
+            quad_sincos(r, j, e.y, e.x);
+            return e;
         }
-        return cis(fr);
     }
     // the same from the whole source point
     template <int PM>
-    static __device__ __forceinline__ C phs(const KArgs<P> &a, const typename PH::T &t, const typename PH::S &sv, float *q)
+    static __device__ __forceinline__ C phs(const KArgs<P> &a, const typename PH::T &t, const typename PH::S &sv, R *q)
     {
         R fr;
         if constexpr (PM == PM_TABLE) {
@@ -774,30 +862,48 @@ struct Tile {
         return cis(fr);
     }
     // two factors in the lanes of a float2 (bf_pair.cuh); q1 null: lane 1 is not recorded or read
-    template <int PM, class T2, class Part2>
-    static __device__ __forceinline__ void ph2(const KArgs<P> &a, const T2 &t, const Part2 &pt, float *q0, float *q1,
-                                               float2 &e0, float2 &e1)
+    template <int PM, class V, class Part2>
+    static __device__ __forceinline__ void ph2(V sg, const Part2 &pt, R *q0, R *q1, C &e0, C &e1)
     {
-        float2 fr;
-        if constexpr (PM == PM_TABLE) {
-            fr.x = __ldcs(q0);
-            fr.y = q1 ? __ldcs(q1) : 0.0f;
-        } else {
-            fr = Ph2<P, D, K>::fin(a, t, pt);
-            if constexpr (PM == PM_BUILD) {
-                __stcs(q0, fr.x);
-                if (q1) __stcs(q1, fr.y);
+        V sn, cs;
+        if constexpr (P::is_f64) {
+            sincos2pi(PH::fin(sg.x, Ph2<P, D, K>::lane0(pt)), sn.x, cs.x);
+            sincos2pi(PH::fin(sg.y, Ph2<P, D, K>::lane1(pt)), sn.y, cs.y);
+        } else if constexpr (P::sfu) {
+            float2 fr;
+            if constexpr (PM == PM_TABLE) {
+                fr.x = __ldcs(q0);
+                fr.y = q1 ? __ldcs(q1) : 0.0f;
+            } else {
+                fr = Ph2<P, D, K>::fin(sg, pt);
+                if constexpr (PM == PM_BUILD) {
+                    __stcs(q0, fr.x);
+                    if (q1) __stcs(q1, fr.y);
+                }
             }
-        }
-        float2 sn, cs;
-        if constexpr (P::sfu) {
             sincos2pi_sfu(fr.x, sn.x, cs.x);
             sincos2pi_sfu(fr.y, sn.y, cs.y);
         } else {
-            sincos2pi2(fr, sn, cs);
+            float2 r;
+            int j0, j1;
+            if constexpr (PM == PM_TABLE) {
+                tab_unpack(__ldcs(q0), r.x, j0);
+                tab_unpack(q1 ? __ldcs(q1) : 0.0f, r.y, j1);
+            } else {
+                float2 ra, rb;
+                Ph2<P, D, K>::fin2(sg, pt, ra, rb);
+                quad_reduce2(ra, rb, r, j0, j1);
+                if constexpr (PM == PM_BUILD) {
+                    __stcs(q0, tab_pack(r.x, j0));
+                    if (q1) __stcs(q1, tab_pack(r.y, j1));
+                }
+            }
+            quad_sincos2(r, j0, j1, sn, cs);
         }
-        e0 = make_float2(cs.x, sn.x);
-        e1 = make_float2(cs.y, sn.y);
+        e0.x = cs.x;
+        e0.y = sn.x;
+        e1.x = cs.y;
+        e1.y = sn.y;
     }
 
     static __device__ __forceinline__ float2 cadd(float2 x, float2 y) { return make_float2(x.x + y.x, x.y + y.y); }
@@ -890,7 +996,7 @@ struct Tile {
 
     // ---- one column-form merge level (l -> l+1) on all tiles of the CTA
     template <int PM = PM_COMPUTE>
-    static __device__ void col_level(const KArgs<P> &a, C *Wt, C *S, Geo *G, int l, int i, float *&tb)
+    static __device__ void col_level(const KArgs<P> &a, C *Wt, C *S, Geo *G, int l, int i, R *&tb)
     {
         const int k = a.k, n = 1 << (D * k), nblk = n >> D;
         const int L = a.L;
@@ -943,53 +1049,17 @@ struct Tile {
                 for (int j = 0; j < D; ++j) cb[j] = 2 * cbq[j] + ((c >> j) & 1);
                 typename PH::S sp;
                 PH::src1(sp, D - 1, sget<P, Q>(a, D - 1, l, cb[D - 1], tq));
-                if constexpr (D == 2 && !P::is_f64) {
-                    // phases two at a time: lanes t'_0 and t'_0 + 1 (the last one alone for odd q)
-                    using PH2 = Ph2<P, D, K>;
-                    const int c0 = c & 1;
-                    const typename PH2::T tA2 = PH2::dup(tA);
-                    const typename P::SE e1 = sget<P, Q>(a, 1, l, cb[1], tq);
-                    const typename PH2::Part p1 = PH2::part(tA2, e1, e1, 1);
-#pragma unroll
-                    for (int t0p = 0; t0p + 1 < Q; t0p += 2) {
-                        float2 E0, E1;
-                        ph2<PM>(a, tA2,
-                                PH2::add(PH2::part(tA2, sget<P, Q>(a, 0, l, cb[0], t0p), sget<P, Q>(a, 0, l, cb[0], t0p + 1), 0), p1),
-                                fa.at(cl * Q + t0p, it), fa.at(cl * Q + t0p + 1, it), E0, E1);
-                        const C u0 = cmul(E0, win[t0p + Q * tq]), u1 = cmul(E1, win[t0p + 1 + Q * tq]);
-#pragma unroll
-                        for (int t0 = 0; t0 < Q; ++t0) {
-                            imac(acc[t0], a, c0, t0, t0p, u0);
-                            imac(acc[t0], a, c0, t0, t0p + 1, u1);
-                        }
-                    }
-                    if constexpr (Q & 1) {
-                        const typename PH::Part pt = PH::add(PH::part(tA, sget<P, Q>(a, 0, l, cb[0], Q - 1), 0), PH2::lane0(p1));
-                        const C u = cmul(ph<PM>(a, tA, pt, fa.at(cl * Q + Q - 1, it)), win[Q - 1 + Q * tq]);
-#pragma unroll
-                        for (int t0 = 0; t0 < Q; ++t0) imac(acc[t0], a, c0, t0, Q - 1, u);
-                    }
-                } else if constexpr (D == 2) {
-                    const int c0 = c & 1;
-                    const typename PH::Part p1 = PH::part(tA, sget<P, Q>(a, 1, l, cb[1], tq), 1);
-#pragma unroll
-                    for (int t0p = 0; t0p < Q; ++t0p) {
-                        const typename PH::Part pt = PH::add(PH::part(tA, sget<P, Q>(a, 0, l, cb[0], t0p), 0), p1);
-                        const C u = cmul(expphase_part<P, D, K>(a, tA, pt), win[t0p + Q * tq]);
-#pragma unroll
-                        for (int t0 = 0; t0 < Q; ++t0) imac(acc[t0], a, c0, t0, t0p, u);
-                    }
-                } else if constexpr (!P::is_f64) {
+                if constexpr (!P::is_f64) {
                     // d = 3: the parts of coordinates 2 and 1 hoisted, phases two at a time over t'_0
                     using PH2 = Ph2<P, D, K>;
                     const int c0 = c & 1, c1 = (c >> 1) & 1;
                     const typename PH2::T tA2 = PH2::dup(tA);
                     const typename P::SE e2 = sget<P, Q>(a, 2, l, cb[2], tq);
-                    const typename PH2::Part p2 = PH2::part(tA2, e2, e2, 2);
+                    const typename PH2::Part p2 = PH2::part(a, tA2, e2, e2, 2);
 #pragma unroll
                     for (int t1p = 0; t1p < Q; ++t1p) {
                         const typename P::SE e1 = sget<P, Q>(a, 1, l, cb[1], t1p);
-                        const typename PH2::Part p12 = PH2::add(PH2::part(tA2, e1, e1, 1), p2);
+                        const typename PH2::Part p12 = PH2::add(PH2::part(a, tA2, e1, e1, 1), p2);
                         const C *wrow = win + Q * t1p + Q * Q * tq;
                         C tmp[Q];
 #pragma unroll
@@ -997,8 +1067,8 @@ struct Tile {
 #pragma unroll
                         for (int t0p = 0; t0p + 1 < Q; t0p += 2) {
                             float2 E0, E1;
-                            ph2<PM>(a, tA2,
-                                    PH2::add(PH2::part(tA2, sget<P, Q>(a, 0, l, cb[0], t0p),
+                            ph2<PM>(PH2::sign(a, tA2),
+                                    PH2::add(PH2::part(a, tA2, sget<P, Q>(a, 0, l, cb[0], t0p),
                                                        sget<P, Q>(a, 0, l, cb[0], t0p + 1), 0), p12),
                                     fa.at((cl * Q + t1p) * Q + t0p, it), fa.at((cl * Q + t1p) * Q + t0p + 1, it), E0, E1);
                             const C u0 = cmul(E0, wrow[t0p]), u1 = cmul(E1, wrow[t0p + 1]);
@@ -1009,8 +1079,8 @@ struct Tile {
                             }
                         }
                         if constexpr (Q & 1) {
-                            const typename PH::Part pt = PH::add(PH::part(tA, sget<P, Q>(a, 0, l, cb[0], Q - 1), 0), PH2::lane0(p12));
-                            const C u = cmul(ph<PM>(a, tA, pt, fa.at((cl * Q + t1p) * Q + Q - 1, it)), wrow[Q - 1]);
+                            const typename PH::Part pt = PH::add(PH::part(a, tA, sget<P, Q>(a, 0, l, cb[0], Q - 1), 0), PH2::lane0(p12));
+                            const C u = cmul(ph<PM>(PH::sign(a, tA), pt, fa.at((cl * Q + t1p) * Q + Q - 1, it)), wrow[Q - 1]);
 #pragma unroll
                             for (int t0 = 0; t0 < Q; ++t0) imac(tmp[t0], a, c0, t0, Q - 1, u);
                         }
@@ -1078,8 +1148,8 @@ struct Tile {
 #pragma unroll
                 for (int j = 0; j < D - 1; ++j) { tk[j] = tt % Q; tt /= Q; }
             }
-            typename PH::Part pl = PH::part(tA, sget<P, Q>(a, 0, l + 1, cbq[0], tk[0]), 0);
-            if constexpr (D == 3) pl = PH::add(pl, PH::part(tA, sget<P, Q>(a, 1, l + 1, cbq[1], tk[1]), 1));
+            typename PH::Part pl = PH::part(a, tA, sget<P, Q>(a, 0, l + 1, cbq[0], tk[0]), 0);
+            if constexpr (D == 3) pl = PH::add(pl, PH::part(a, tA, sget<P, Q>(a, 1, l + 1, cbq[1], tk[1]), 1));
             C *wo = Wt + tau * n * RR + (base + (alpha << (D * i))) * RR + tl;
             if constexpr (!P::is_f64) {
                 // phases two at a time: lanes t_{d-1} and t_{d-1} + 1 (the last one alone for odd q)
@@ -1089,21 +1159,21 @@ struct Tile {
 #pragma unroll
                 for (int tq = 0; tq + 1 < Q; tq += 2) {
                     float2 E0, E1;
-                    ph2<PM>(a, tA2,
-                            PH2::add(PH2::part(tA2, sget<P, Q>(a, D - 1, l + 1, cbq[D - 1], tq),
+                    ph2<PM>(PH2::sign(a, tA2),
+                            PH2::add(PH2::part(a, tA2, sget<P, Q>(a, D - 1, l + 1, cbq[D - 1], tq),
                                                sget<P, Q>(a, D - 1, l + 1, cbq[D - 1], tq + 1), D - 1), pl2),
                             fb.at(tq, it), fb.at(tq + 1, it), E0, E1);
                     wo[tq * QD1] = cjmul(E0, acc[tq]);
                     wo[(tq + 1) * QD1] = cjmul(E1, acc[tq + 1]);
                 }
                 if constexpr (Q & 1) {
-                    const typename PH::Part pt = PH::add(PH::part(tA, sget<P, Q>(a, D - 1, l + 1, cbq[D - 1], Q - 1), D - 1), pl);
-                    wo[(Q - 1) * QD1] = cjmul(ph<PM>(a, tA, pt, fb.at(Q - 1, it)), acc[Q - 1]);
+                    const typename PH::Part pt = PH::add(PH::part(a, tA, sget<P, Q>(a, D - 1, l + 1, cbq[D - 1], Q - 1), D - 1), pl);
+                    wo[(Q - 1) * QD1] = cjmul(ph<PM>(PH::sign(a, tA), pt, fb.at(Q - 1, it)), acc[Q - 1]);
                 }
             } else {
 #pragma unroll
                 for (int tq = 0; tq < Q; ++tq) {
-                    const typename PH::Part pt = PH::add(PH::part(tA, sget<P, Q>(a, D - 1, l + 1, cbq[D - 1], tq), D - 1), pl);
+                    const typename PH::Part pt = PH::add(PH::part(a, tA, sget<P, Q>(a, D - 1, l + 1, cbq[D - 1], tq), D - 1), pl);
                     wo[tq * QD1] = cjmul(expphase_part<P, D, K>(a, tA, pt), acc[tq]);
                 }
             }
@@ -1115,7 +1185,7 @@ struct Tile {
     // accumulate over t for the q values of s_0.  Results go through S so no item reads a
     // slot that another item has already rewritten.
     template <int PM = PM_COMPUTE>
-    static __device__ void switch_tiles(const KArgs<P> &a, C *Wt, C *S, int l, float *&tb)
+    static __device__ void switch_tiles(const KArgs<P> &a, C *Wt, C *S, int l, R *&tb)
     {
         if constexpr (!P::is_f64 && K == KIND_GENRADON) {   // the phase whose pairs pay for their registers
             switch_tiles_pair<PM>(a, Wt, S, l, tb);
@@ -1159,8 +1229,8 @@ struct Tile {
                 typename PH::Part hp[Q];
 #pragma unroll
                 for (int s0 = 0; s0 < Q; ++s0) {
-                    hp[s0] = PH::part(tS[s0], sget<P, Q>(a, 1, l, cb[1], tk[1]), 1);
-                    if constexpr (D == 3) hp[s0] = PH::add(hp[s0], PH::part(tS[s0], sget<P, Q>(a, 2, l, cb[2], tk[2]), 2));
+                    hp[s0] = PH::part(a, tS[s0], sget<P, Q>(a, 1, l, cb[1], tk[1]), 1);
+                    if constexpr (D == 3) hp[s0] = PH::add(hp[s0], PH::part(a, tS[s0], sget<P, Q>(a, 2, l, cb[2], tk[2]), 2));
                 }
 #pragma unroll
                 for (int t0 = 0; t0 < Q; ++t0) {
@@ -1168,7 +1238,7 @@ struct Tile {
                     const C ut = u[t0 + Q * th];
 #pragma unroll
                     for (int s0 = 0; s0 < Q; ++s0)
-                        cmac(acc[s0], ph<PM>(a, tS[s0], PH::add(PH::part(tS[s0], e0, 0), hp[s0]), fs.at((th * Q + t0) * Q + s0, it)), ut);
+                        cmac(acc[s0], ph<PM>(PH::sign(a, tS[s0]), PH::add(PH::part(a, tS[s0], e0, 0), hp[s0]), fs.at((th * Q + t0) * Q + s0, it)), ut);
                 }
             }
             C *w = S + (tau * n + sl) * RR + sh * Q;
@@ -1184,7 +1254,7 @@ struct Tile {
     // targets s_0 = 2j and 2j + 1 share a pair; for odd q the last target takes two
     // consecutive t_0 in its lanes.  Each lane rounds exactly as the scalar code.
     template <int PM>
-    static __device__ void switch_tiles_pair(const KArgs<P> &a, C *Wt, C *S, int l, float *&tb)
+    static __device__ void switch_tiles_pair(const KArgs<P> &a, C *Wt, C *S, int l, R *&tb)
     {
         using PH2 = Ph2<P, D, K>;
         constexpr int NPR = Q / 2, ODD = Q & 1, NT2 = NPR + ODD;
@@ -1229,10 +1299,10 @@ struct Tile {
                 const typename P::SE e1 = sget<P, Q>(a, 1, l, cb[1], tk[1]);
 #pragma unroll
                 for (int j = 0; j < NT2; ++j) {
-                    hp[j] = PH2::part(tP[j], e1, e1, 1);
+                    hp[j] = PH2::part(a, tP[j], e1, e1, 1);
                     if constexpr (D == 3) {
                         const typename P::SE e2 = sget<P, Q>(a, 2, l, cb[2], tk[2]);
-                        hp[j] = PH2::add(hp[j], PH2::part(tP[j], e2, e2, 2));
+                        hp[j] = PH2::add(hp[j], PH2::part(a, tP[j], e2, e2, 2));
                     }
                 }
 #pragma unroll
@@ -1246,19 +1316,19 @@ struct Tile {
                     const int ja = (th * Q + t0) * Q, jb = ja + Q;
 #pragma unroll
                     for (int j = 0; j < NPR; ++j) {
-                        ph2<PM>(a, tP[j], PH2::add(PH2::part(tP[j], ea, ea, 0), hp[j]), fs.at(ja + 2 * j, it),
+                        ph2<PM>(PH2::sign(a, tP[j]), PH2::add(PH2::part(a, tP[j], ea, ea, 0), hp[j]), fs.at(ja + 2 * j, it),
                                 fs.at(ja + 2 * j + 1, it), E0, E1);
                         cmac(acc[2 * j], E0, ua);
                         cmac(acc[2 * j + 1], E1, ua);
                         if (two) {
-                            ph2<PM>(a, tP[j], PH2::add(PH2::part(tP[j], eb, eb, 0), hp[j]), fs.at(jb + 2 * j, it),
+                            ph2<PM>(PH2::sign(a, tP[j]), PH2::add(PH2::part(a, tP[j], eb, eb, 0), hp[j]), fs.at(jb + 2 * j, it),
                                     fs.at(jb + 2 * j + 1, it), E0, E1);
                             cmac(acc[2 * j], E0, ub);
                             cmac(acc[2 * j + 1], E1, ub);
                         }
                     }
                     if constexpr (ODD) {
-                        ph2<PM>(a, tP[NPR], PH2::add(PH2::part(tP[NPR], ea, eb, 0), hp[NPR]), fs.at(ja + Q - 1, it),
+                        ph2<PM>(PH2::sign(a, tP[NPR]), PH2::add(PH2::part(a, tP[NPR], ea, eb, 0), hp[NPR]), fs.at(ja + Q - 1, it),
                                 two ? fs.at(jb + Q - 1, it) : nullptr, E0, E1);
                         cmac(acc[Q - 1], E0, ua);
                         if (two) cmac(acc[Q - 1], E1, ub);
@@ -1320,7 +1390,7 @@ struct Tile {
                     const typename PH::T tS = tpoint<P, D, Q, K>(a, l, ca, sk);
 #pragma unroll
                     for (int u = 0; u < Q; ++u)
-                        e[u] = expphase_part<P, D, K>(a, tS, PH::part(tS, sget<P, Q>(a, dim, l, cb[dim], u), dim));
+                        e[u] = expphase_part<P, D, K>(a, tS, PH::part(a, tS, sget<P, Q>(a, dim, l, cb[dim], u), dim));
                 } else {
                     const typename P::SE ys = sget<P, Q>(a, dim, l, cb[dim], sd);
 #pragma unroll
@@ -1328,7 +1398,7 @@ struct Tile {
                         int sk[DMAX] = {Q, Q, Q};
                         sk[dim] = u;
                         const typename PH::T tS = tpoint<P, D, Q, K>(a, l, ca, sk);
-                        e[u] = expphase_part<P, D, K>(a, tS, PH::part(tS, ys, dim));
+                        e[u] = expphase_part<P, D, K>(a, tS, PH::part(a, tS, ys, dim));
                     }
                 }
                 const int base = (tau * n + sl) * RR + (D == 3 ? o1 * pw[oth[0]] : 0);
@@ -1364,7 +1434,7 @@ struct Tile {
     // ---- one row-form merge level (l -> l+1) on all tiles of the CTA.  TC caches the
     // target features of the parents' nodes (T * 2^{Di} boxes x q^d nodes) for stage A.
     template <int PM = PM_COMPUTE>
-    static __device__ void row_level(const KArgs<P> &a, C *Wt, C *S, typename PH::T *TC, int l, int i, float *&tb)
+    static __device__ void row_level(const KArgs<P> &a, C *Wt, C *S, typename PH::T *TC, int l, int i, R *&tb)
     {
         const int k = a.k, n = 1 << (D * k), nblk = n >> D;
         const int L = a.L;
@@ -1442,53 +1512,7 @@ struct Tile {
             C acc[QD1];
 #pragma unroll
             for (int j = 0; j < QD1; ++j) acc[j] = czero<C>();
-            if constexpr (D == 2) {
-                const int a1 = (alpha >> 1) & 1;
-                C v[NC][Q];
-                typename P::SE sc0[2], sc1[2];        // children's centres per dimension
-#pragma unroll
-                for (int h = 0; h < 2; ++h) {
-                    sc0[h] = sget<P, Q>(a, 0, l, 2 * cbq[0] + h, Q);
-                    sc1[h] = sget<P, Q>(a, 1, l, 2 * cbq[1] + h, Q);
-                }
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    const C *si = Sblk + c * QD1 * 2 * Q + a0 * Q + s0;   // [t1] stride 2Q
-#pragma unroll
-                    for (int s1 = 0; s1 < Q; ++s1) v[c][s1] = czero<C>();
-#pragma unroll
-                    for (int t1 = 0; t1 < Q; ++t1) {
-                        const C zz = si[t1 * 2 * Q];
-#pragma unroll
-                        for (int s1 = 0; s1 < Q; ++s1) cfma2(v[c][s1], a.M2[a1][t1][s1], zz);
-                    }
-                }
-#pragma unroll
-                for (int s1 = 0; s1 < Q; ++s1) {
-                    const int sk[DMAX] = {s0, s1, 0};
-                    const typename PH::T tS = tpoint<P, D, Q, K>(a, l + 1, ca, sk);
-                    if constexpr (!P::is_f64) {
-                        // phases two at a time: lanes c_0 = 0 and 1
-                        using PH2 = Ph2<P, D, K>;
-                        const typename PH2::T tS2 = PH2::dup(tS);
-                        const typename PH2::Part q0 = PH2::part(tS2, sc0[0], sc0[1], 0);
-#pragma unroll
-                        for (int c1 = 0; c1 < 2; ++c1) {
-                            float2 E0, E1;
-                            ph2<PM>(a, tS2, PH2::add(q0, PH2::part(tS2, sc1[c1], sc1[c1], 1)), fb.at(s1 * NC + 2 * c1, it),
-                                    fb.at(s1 * NC + 2 * c1 + 1, it), E0, E1);
-                            acc[s1] = cadd(acc[s1], cmul(E0, v[2 * c1][s1]));
-                            acc[s1] = cadd(acc[s1], cmul(E1, v[2 * c1 + 1][s1]));
-                        }
-                    } else {
-                        const typename PH::Part q0[2] = {PH::part(tS, sc0[0], 0), PH::part(tS, sc0[1], 0)};
-                        const typename PH::Part q1[2] = {PH::part(tS, sc1[0], 1), PH::part(tS, sc1[1], 1)};
-#pragma unroll
-                        for (int c = 0; c < NC; ++c)
-                            acc[s1] = cadd(acc[s1], cmul(expphase_part<P, D, K>(a, tS, PH::add(q0[c & 1], q1[c >> 1])), v[c][s1]));
-                    }
-                }
-            } else {
+            {
                 const int a1 = (alpha >> 1) & 1, a2 = (alpha >> 2) & 1;
 #pragma unroll 1
                 for (int c = 0; c < NC; ++c) {
@@ -1563,6 +1587,61 @@ struct Tile {
         }
     }
 
+    // ---- pass bodies (d = 3)
+    template <int PM>
+    static __device__ __forceinline__ void col_pass(const KArgs<P> &a, unsigned char *smem, R *tb)
+    {
+        if constexpr (PM == PM_TABLE) prefetch_l2(tb, level_floats(a, false));
+        C *Wt = reinterpret_cast<C *>(smem);
+        C *S = Wt + a.T * (1 << (D * a.k)) * RR;
+        Geo *G = reinterpret_cast<Geo *>(S + 2 * a.T * (1 << (D * a.k)) * RR);
+        const int rhs = blockIdx.y;
+        if (a.flags & F_INIT)
+            init(a, Wt, rhs);
+        else
+            load(a, Wt, rhs);
+        __syncthreads();
+        for (int i = 0; i < a.k; ++i) {
+            if constexpr (PM == PM_TABLE) {   // the next level's blocks (or the switch's) while this level runs
+                const int64_t lf = level_floats(a, false);
+                if (i + 1 < a.k)
+                    prefetch_l2(tb + lf, lf);
+                else if (a.flags & F_SWITCH)
+                    prefetch_l2(tb + lf, a.ftab_cta - (int64_t)a.k * lf);
+            }
+            col_level<PM>(a, Wt, S, G, a.l0 + i, i, tb);
+        }
+        if (a.flags & F_SWITCH) {
+            if constexpr (K == KIND_DOT || K == KIND_SEPARABLE)
+                switch_sep<false>(a, Wt, S, a.l0 + a.k);
+            else
+                switch_tiles<PM>(a, Wt, S, a.l0 + a.k, tb);
+        }
+        store(a, Wt, rhs);
+    }
+    template <int PM>
+    static __device__ __forceinline__ void row_pass(const KArgs<P> &a, unsigned char *smem, R *tb)
+    {
+        if constexpr (PM == PM_TABLE) prefetch_l2(tb, level_floats(a, true));
+        C *Wt = reinterpret_cast<C *>(smem);
+        C *S = Wt + a.T * (1 << (D * a.k)) * RR;
+        typename PH::T *TC = reinterpret_cast<typename PH::T *>(S + 2 * a.T * (1 << (D * a.k)) * RR);
+        const int rhs = blockIdx.y;
+        load(a, Wt, rhs);
+        __syncthreads();
+        for (int i = 0; i < a.k; ++i) {
+            if constexpr (PM == PM_TABLE) {   // the next level's blocks while this level runs
+                const int64_t lf = level_floats(a, true);
+                if (i + 1 < a.k) prefetch_l2(tb + lf, lf);
+            }
+            row_level<PM>(a, Wt, S, TC, a.l0 + i, i, tb);
+        }
+        if (a.flags & F_FINAL)
+            final_eval(a, Wt, rhs);
+        else
+            store(a, Wt, rhs);
+    }
+
     // =====================================================================
     // Adjoint passes: every step conjugate-transposed, levels in reverse.
     // On entry to a level the slot of output alpha of a merge block holds the
@@ -1595,8 +1674,8 @@ struct Tile {
 #pragma unroll
                 for (int j = 1; j < D; ++j) { tk[j] = tt % Q; tt /= Q; }
             }
-            typename PH::Part hp = PH::part(tA, sget<P, Q>(a, 1, l + 1, cbq[1], tk[1]), 1);
-            if constexpr (D == 3) hp = PH::add(hp, PH::part(tA, sget<P, Q>(a, 2, l + 1, cbq[2], tk[2]), 2));
+            typename PH::Part hp = PH::part(a, tA, sget<P, Q>(a, 1, l + 1, cbq[1], tk[1]), 1);
+            if constexpr (D == 3) hp = PH::add(hp, PH::part(a, tA, sget<P, Q>(a, 2, l + 1, cbq[2], tk[2]), 2));
             const C *wi = Wt + tau * n * RR + (base + (alpha << (D * i))) * RR + th * Q;
             C z[2][Q];
 #pragma unroll
@@ -1610,7 +1689,7 @@ struct Tile {
                 for (int t0 = 0; t0 + 1 < Q; t0 += 2) {
                     float2 E0, E1;
                     expphase_part2<P, D, K>(a, tA2,
-                                            PH2::add(PH2::part(tA2, sget<P, Q>(a, 0, l + 1, cbq[0], t0),
+                                            PH2::add(PH2::part(a, tA2, sget<P, Q>(a, 0, l + 1, cbq[0], t0),
                                                                sget<P, Q>(a, 0, l + 1, cbq[0], t0 + 1), 0), hp2),
                                             E0, E1);
                     const C u0 = cmul(E0, wi[t0]), u1 = cmul(E1, wi[t0 + 1]);
@@ -1623,7 +1702,7 @@ struct Tile {
                     }
                 }
                 if constexpr (Q & 1) {
-                    const C e = expphase_part<P, D, K>(a, tA, PH::add(PH::part(tA, sget<P, Q>(a, 0, l + 1, cbq[0], Q - 1), 0), hp));
+                    const C e = expphase_part<P, D, K>(a, tA, PH::add(PH::part(a, tA, sget<P, Q>(a, 0, l + 1, cbq[0], Q - 1), 0), hp));
                     const C u = cmul(e, wi[Q - 1]);
 #pragma unroll
                     for (int s0 = 0; s0 < Q; ++s0) {
@@ -1634,7 +1713,7 @@ struct Tile {
             } else {
 #pragma unroll
                 for (int t0 = 0; t0 < Q; ++t0) {
-                    const C e = expphase_part<P, D, K>(a, tA, PH::add(PH::part(tA, sget<P, Q>(a, 0, l + 1, cbq[0], t0), 0), hp));
+                    const C e = expphase_part<P, D, K>(a, tA, PH::add(PH::part(a, tA, sget<P, Q>(a, 0, l + 1, cbq[0], t0), 0), hp));
                     const C u = cmul(e, wi[t0]);
 #pragma unroll
                     for (int s0 = 0; s0 < Q; ++s0) {
@@ -1673,7 +1752,7 @@ struct Tile {
                 int ca[DMAX];
                 morton_decode<D>((Apg << D) + alpha, l + 1, ca);
                 const typename PH::T tA = tcenter<P, D, Q, K>(a, l + 1, (Apg << D) + alpha, ca);
-                const typename PH::Part p0 = PH::part(tA, e0, 0);
+                const typename PH::Part p0 = PH::part(a, tA, e0, 0);
                 const C *si = S + ((tau * nblk + beta) * NC + alpha) * QD1 * 2 * Q + c0 * Q + s0;   // [t_{>=1}] stride 2Q
                 if constexpr (D == 2) {
                     const int c1 = (c >> 1) & 1;
@@ -1695,20 +1774,20 @@ struct Tile {
                         for (int s1 = 0; s1 + 1 < Q; s1 += 2) {
                             float2 E0, E1;
                             expphase_part2<P, D, K>(a, tA2,
-                                                    PH2::add(p02, PH2::part(tA2, sget<P, Q>(a, 1, l, cb[1], s1),
+                                                    PH2::add(p02, PH2::part(a, tA2, sget<P, Q>(a, 1, l, cb[1], s1),
                                                                             sget<P, Q>(a, 1, l, cb[1], s1 + 1), 1)),
                                                     E0, E1);
                             acc[s1] = cadd(acc[s1], cjmul(E0, v[s1]));
                             acc[s1 + 1] = cadd(acc[s1 + 1], cjmul(E1, v[s1 + 1]));
                         }
                         if constexpr (Q & 1) {
-                            const C e = expphase_part<P, D, K>(a, tA, PH::add(p0, PH::part(tA, sget<P, Q>(a, 1, l, cb[1], Q - 1), 1)));
+                            const C e = expphase_part<P, D, K>(a, tA, PH::add(p0, PH::part(a, tA, sget<P, Q>(a, 1, l, cb[1], Q - 1), 1)));
                             acc[Q - 1] = cadd(acc[Q - 1], cjmul(e, v[Q - 1]));
                         }
                     } else {
 #pragma unroll
                         for (int s1 = 0; s1 < Q; ++s1) {
-                            const C e = expphase_part<P, D, K>(a, tA, PH::add(p0, PH::part(tA, sget<P, Q>(a, 1, l, cb[1], s1), 1)));
+                            const C e = expphase_part<P, D, K>(a, tA, PH::add(p0, PH::part(a, tA, sget<P, Q>(a, 1, l, cb[1], s1), 1)));
                             acc[s1] = cadd(acc[s1], cjmul(e, v[s1]));
                         }
                     }
@@ -1727,13 +1806,13 @@ struct Tile {
                         }
 #pragma unroll
                     for (int s2 = 0; s2 < Q; ++s2) {
-                        const typename PH::Part p2 = PH::add(p0, PH::part(tA, sget<P, Q>(a, 2, l, cb[2], s2), 2));
+                        const typename PH::Part p2 = PH::add(p0, PH::part(a, tA, sget<P, Q>(a, 2, l, cb[2], s2), 2));
 #pragma unroll
                         for (int s1 = 0; s1 < Q; ++s1) {
                             C v = czero<C>();
 #pragma unroll
                             for (int t1 = 0; t1 < Q; ++t1) cfma2(v, a.M2[c1][t1][s1], w[t1 * Q + s2]);
-                            const C e = expphase_part<P, D, K>(a, tA, PH::add(p2, PH::part(tA, sget<P, Q>(a, 1, l, cb[1], s1), 1)));
+                            const C e = expphase_part<P, D, K>(a, tA, PH::add(p2, PH::part(a, tA, sget<P, Q>(a, 1, l, cb[1], s1), 1)));
                             acc[s1 + Q * s2] = cadd(acc[s1 + Q * s2], cjmul(e, v));
                         }
                     }
@@ -1944,25 +2023,25 @@ struct Tile {
                 if constexpr (!P::is_f64) {
                     using PH2 = Ph2<P, D, K>;
                     const typename PH2::T tS2 = PH2::dup(tS);
-                    typename PH2::Part hp = PH2::part(tS2, eh[1], eh[1], 1);
-                    if constexpr (D == 3) hp = PH2::add(hp, PH2::part(tS2, eh[2], eh[2], 2));
+                    typename PH2::Part hp = PH2::part(a, tS2, eh[1], eh[1], 1);
+                    if constexpr (D == 3) hp = PH2::add(hp, PH2::part(a, tS2, eh[2], eh[2], 2));
 #pragma unroll
                     for (int t0 = 0; t0 + 1 < Q; t0 += 2) {
                         float2 E0, E1;
-                        expphase_part2<P, D, K>(a, tS2, PH2::add(PH2::part(tS2, e0[t0], e0[t0 + 1], 0), hp), E0, E1);
+                        expphase_part2<P, D, K>(a, tS2, PH2::add(PH2::part(a, tS2, e0[t0], e0[t0 + 1], 0), hp), E0, E1);
                         acc[t0] = cadd(acc[t0], cjmul(E0, vs));
                         acc[t0 + 1] = cadd(acc[t0 + 1], cjmul(E1, vs));
                     }
                     if constexpr (Q & 1)
                         acc[Q - 1] = cadd(acc[Q - 1], cjmul(expphase_part<P, D, K>(
-                                                                a, tS, PH::add(PH::part(tS, e0[Q - 1], 0), PH2::lane0(hp))),
+                                                                a, tS, PH::add(PH::part(a, tS, e0[Q - 1], 0), PH2::lane0(hp))),
                                                             vs));
                 } else {
-                    typename PH::Part hp = PH::part(tS, eh[1], 1);
-                    if constexpr (D == 3) hp = PH::add(hp, PH::part(tS, eh[2], 2));
+                    typename PH::Part hp = PH::part(a, tS, eh[1], 1);
+                    if constexpr (D == 3) hp = PH::add(hp, PH::part(a, tS, eh[2], 2));
 #pragma unroll
                     for (int t0 = 0; t0 < Q; ++t0)
-                        acc[t0] = cadd(acc[t0], cjmul(expphase_part<P, D, K>(a, tS, PH::add(PH::part(tS, e0[t0], 0), hp)), vs));
+                        acc[t0] = cadd(acc[t0], cjmul(expphase_part<P, D, K>(a, tS, PH::add(PH::part(a, tS, e0[t0], 0), hp)), vs));
                 }
             }
             C *w = S + (tau * n + sl) * RR + th * Q;
@@ -2113,93 +2192,59 @@ struct Tile {
     }
 };
 
+}  // namespace bfk
+
+#include "bf_tile2.cuh"   // forward passes at d = 2
+
+namespace bfk {
+
+// the tile code of a forward single-RHS pass
+template <int D, int Q, class P, int K, bool LB> struct TileOf { using type = Tile<D, Q, P, K>; };
+template <int Q, class P, int K, bool LB> struct TileOf<2, Q, P, K, LB> { using type = Tile2<Q, P, K, LB>; };
+
 // ------------------------------------------------------------------ kernels
 
 // init (l0 = 0) + k column merges + optional switch at level l0 + k
-// PM: phase factors evaluated, or (mixed precisions) recorded in or read from the pass's
-// reduced-phase table a.ftab (a.ftab_cta floats per CTA).  Reading the table, the d = 2
-// column pass fits one more CTA per SM (register budget cut accordingly): measured 7% faster
-// with the polynomial sincos, 19% with the SFU one; the row pass would spill.  At d = 3 the
-// shared memory holds two CTAs per SM either way.
-template <int D, int Q, class P, int K, int PM = PM_COMPUTE>
+// LB: Chebyshev-Lobatto nodes (d = 2, odd q; Tile2).  PM: phase factors evaluated, or (mixed
+// precisions) recorded in or read from the pass's table a.ftab (a.ftab_cta floats per CTA).
+// Reading the table, the d = 2 column pass fits one more CTA per SM (register budget cut
+// accordingly): measured 7% faster with the polynomial sincos, 19% with the SFU one; the row
+// pass would spill.  At d = 3 the shared memory holds two CTAs per SM either way.
+template <int D, int Q, class P, int K, bool LB, int PM = PM_COMPUTE>
 __global__ void __launch_bounds__(Cfg<D, Q, P>::NT, PM == PM_TABLE ? Cfg<D, Q, P>::MINB_TAB : Cfg<D, Q, P>::MINB_COL)
     k_col_pass(const KArgs<P> a)
 {
     static_assert(PM == PM_COMPUTE || !P::is_f64, "phase tables: mixed precisions");
     using C = typename P::C;
-    using TL = Tile<D, Q, P, K>;
+    using TL = typename TileOf<D, Q, P, K, LB>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *Wt = reinterpret_cast<C *>(smem_raw);
-    C *S = Wt + a.T * (1 << (D * a.k)) * TL::RR;
-    const int rhs = blockIdx.y;
-    float *tb = nullptr;
+    typename P::R *tb = nullptr;
     if constexpr (PM != PM_COMPUTE) {
         if (TL::table_floats(a, false) != a.ftab_cta) {   // the plan's layout disagrees: touch nothing
             if (threadIdx.x == 0 && a.err) atomicExch(a.err, 2);
             return;
         }
         tb = a.ftab + (int64_t)blockIdx.x * a.ftab_cta;
-        if constexpr (PM == PM_TABLE) TL::prefetch_l2(tb, TL::level_floats(a, false));
     }
-    if (a.flags & F_INIT)
-        TL::init(a, Wt, rhs);
-    else
-        TL::load(a, Wt, rhs);
-    __syncthreads();
-    typename TL::Geo *G = reinterpret_cast<typename TL::Geo *>(S + 2 * a.T * (1 << (D * a.k)) * TL::RR);
-    for (int i = 0; i < a.k; ++i) {
-        if constexpr (PM == PM_TABLE) {   // the next level's blocks (or the switch's) while this level runs
-            const int64_t lf = TL::level_floats(a, false);
-            if (i + 1 < a.k)
-                TL::prefetch_l2(tb + lf, lf);
-            else if (a.flags & F_SWITCH)
-                TL::prefetch_l2(tb + lf, a.ftab_cta - (int64_t)a.k * lf);
-        }
-        TL::template col_level<PM>(a, Wt, S, G, a.l0 + i, i, tb);
-    }
-    if (a.flags & F_SWITCH) {
-        if constexpr (K == KIND_DOT || K == KIND_SEPARABLE)
-            TL::template switch_sep<false>(a, Wt, S, a.l0 + a.k);
-        else
-            TL::template switch_tiles<PM>(a, Wt, S, a.l0 + a.k, tb);
-    }
-    TL::store(a, Wt, rhs);
+    TL::template col_pass<PM>(a, smem_raw, tb);
 }
 
 // k row merges + optional final evaluation (l0 + k = L)
-template <int D, int Q, class P, int K, int PM = PM_COMPUTE>
+template <int D, int Q, class P, int K, bool LB, int PM = PM_COMPUTE>
 __global__ void __launch_bounds__(Cfg<D, Q, P>::NT, Cfg<D, Q, P>::MINB) k_row_pass(const KArgs<P> a)
 {
     static_assert(PM == PM_COMPUTE || !P::is_f64, "phase tables: mixed precisions");
-    using C = typename P::C;
-    using TL = Tile<D, Q, P, K>;
+    using TL = typename TileOf<D, Q, P, K, LB>::type;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *Wt = reinterpret_cast<C *>(smem_raw);
-    C *S = Wt + a.T * (1 << (D * a.k)) * TL::RR;
-    const int rhs = blockIdx.y;
-    typename TL::PH::T *TC = reinterpret_cast<typename TL::PH::T *>(S + 2 * a.T * (1 << (D * a.k)) * TL::RR);
-    float *tb = nullptr;
+    typename P::R *tb = nullptr;
     if constexpr (PM != PM_COMPUTE) {
         if (TL::table_floats(a, true) != a.ftab_cta) {   // the plan's layout disagrees: touch nothing
             if (threadIdx.x == 0 && a.err) atomicExch(a.err, 2);
             return;
         }
         tb = a.ftab + (int64_t)blockIdx.x * a.ftab_cta;
-        if constexpr (PM == PM_TABLE) TL::prefetch_l2(tb, TL::level_floats(a, true));
     }
-    TL::load(a, Wt, rhs);
-    __syncthreads();
-    for (int i = 0; i < a.k; ++i) {
-        if constexpr (PM == PM_TABLE) {   // the next level's blocks while this level runs
-            const int64_t lf = TL::level_floats(a, true);
-            if (i + 1 < a.k) TL::prefetch_l2(tb + lf, lf);
-        }
-        TL::template row_level<PM>(a, Wt, S, TC, a.l0 + i, i, tb);
-    }
-    if (a.flags & F_FINAL)
-        TL::final_eval(a, Wt, rhs);
-    else
-        TL::store(a, Wt, rhs);
+    TL::template row_pass<PM>(a, smem_raw, tb);
 }
 
 // adjoint of a column pass: optional switch^H at level l0 + k, k column levels in

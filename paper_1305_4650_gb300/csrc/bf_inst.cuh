@@ -29,23 +29,23 @@ inline cudaError_t prepare(K kern, size_t smem, size_t *granted)
     return cudaSuccess;
 }
 
-template <int D, int Q, class P, int K, int PM = bfk::PM_COMPUTE>
+template <int D, int Q, class P, int K, bool LB, int PM = bfk::PM_COMPUTE>
 cudaError_t launch_col(const void *kargs, unsigned gx, unsigned gy, size_t smem, cudaStream_t s)
 {
     static size_t granted[64] = {0};
-    cudaError_t e = prepare(bfk::k_col_pass<D, Q, P, K, PM>, smem, granted);
+    cudaError_t e = prepare(bfk::k_col_pass<D, Q, P, K, LB, PM>, smem, granted);
     if (e != cudaSuccess) return e;
-    bfk::k_col_pass<D, Q, P, K, PM><<<dim3(gx, gy), bfk::Cfg<D, Q, P>::NT, smem, s>>>(*static_cast<const bfk::KArgs<P> *>(kargs));
+    bfk::k_col_pass<D, Q, P, K, LB, PM><<<dim3(gx, gy), bfk::Cfg<D, Q, P>::NT, smem, s>>>(*static_cast<const bfk::KArgs<P> *>(kargs));
     return cudaGetLastError();
 }
 
-template <int D, int Q, class P, int K, int PM = bfk::PM_COMPUTE>
+template <int D, int Q, class P, int K, bool LB, int PM = bfk::PM_COMPUTE>
 cudaError_t launch_row(const void *kargs, unsigned gx, unsigned gy, size_t smem, cudaStream_t s)
 {
     static size_t granted[64] = {0};
-    cudaError_t e = prepare(bfk::k_row_pass<D, Q, P, K, PM>, smem, granted);
+    cudaError_t e = prepare(bfk::k_row_pass<D, Q, P, K, LB, PM>, smem, granted);
     if (e != cudaSuccess) return e;
-    bfk::k_row_pass<D, Q, P, K, PM><<<dim3(gx, gy), bfk::Cfg<D, Q, P>::NT, smem, s>>>(*static_cast<const bfk::KArgs<P> *>(kargs));
+    bfk::k_row_pass<D, Q, P, K, LB, PM><<<dim3(gx, gy), bfk::Cfg<D, Q, P>::NT, smem, s>>>(*static_cast<const bfk::KArgs<P> *>(kargs));
     return cudaGetLastError();
 }
 
@@ -69,63 +69,63 @@ cudaError_t launch_row_adj(const void *kargs, unsigned gx, unsigned gy, size_t s
     return cudaGetLastError();
 }
 
-template <int Q, class P, int K, int PM>
+template <int Q, class P, int K, bool LB, int PM>
 cudaError_t launch_col_mr(const void *kargs, unsigned gx, unsigned gy, size_t smem, cudaStream_t s)
 {
     static size_t granted[64] = {0};
-    cudaError_t e = prepare(bfk::k_col_pass_mr<Q, P, K, PM>, smem, granted);
+    cudaError_t e = prepare(bfk::k_col_pass_mr<Q, P, K, LB, PM>, smem, granted);
     if (e != cudaSuccess) return e;
-    bfk::k_col_pass_mr<Q, P, K, PM><<<dim3(gx, gy), bfk::CfgMR<Q>::NT, smem, s>>>(*static_cast<const bfk::KArgs<P> *>(kargs));
+    bfk::k_col_pass_mr<Q, P, K, LB, PM><<<dim3(gx, gy), bfk::CfgMR<Q>::NT, smem, s>>>(*static_cast<const bfk::KArgs<P> *>(kargs));
     return cudaGetLastError();
 }
 
-template <int Q, class P, int K, int PM>
+template <int Q, class P, int K, bool LB, int PM>
 cudaError_t launch_row_mr(const void *kargs, unsigned gx, unsigned gy, size_t smem, cudaStream_t s)
 {
     static size_t granted[64] = {0};
-    cudaError_t e = prepare(bfk::k_row_pass_mr<Q, P, K, PM>, smem, granted);
+    cudaError_t e = prepare(bfk::k_row_pass_mr<Q, P, K, LB, PM>, smem, granted);
     if (e != cudaSuccess) return e;
-    bfk::k_row_pass_mr<Q, P, K, PM><<<dim3(gx, gy), bfk::CfgMR<Q>::NT, smem, s>>>(*static_cast<const bfk::KArgs<P> *>(kargs));
+    bfk::k_row_pass_mr<Q, P, K, LB, PM><<<dim3(gx, gy), bfk::CfgMR<Q>::NT, smem, s>>>(*static_cast<const bfk::KArgs<P> *>(kargs));
     return cudaGetLastError();
 }
 
 // CTAs per SM of the table-reading multi-RHS passes with `smem` bytes of shared memory
-template <int Q, class P, int K>
+template <int Q, class P, int K, bool LB>
 int mr_table_occupancy(int row, size_t smem)
 {
     static size_t granted_c[64] = {0}, granted_r[64] = {0};
     int n = 0;
     if (row) {
-        if (prepare(bfk::k_row_pass_mr<Q, P, K, bfk::PM_TABLE>, smem, granted_r) != cudaSuccess) return 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, bfk::k_row_pass_mr<Q, P, K, bfk::PM_TABLE>,
+        if (prepare(bfk::k_row_pass_mr<Q, P, K, LB, bfk::PM_TABLE>, smem, granted_r) != cudaSuccess) return 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, bfk::k_row_pass_mr<Q, P, K, LB, bfk::PM_TABLE>,
                                                           bfk::CfgMR<Q>::NT, smem) != cudaSuccess)
             return 0;
     } else {
-        if (prepare(bfk::k_col_pass_mr<Q, P, K, bfk::PM_TABLE>, smem, granted_c) != cudaSuccess) return 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, bfk::k_col_pass_mr<Q, P, K, bfk::PM_TABLE>,
+        if (prepare(bfk::k_col_pass_mr<Q, P, K, LB, bfk::PM_TABLE>, smem, granted_c) != cudaSuccess) return 0;
+        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, bfk::k_col_pass_mr<Q, P, K, LB, bfk::PM_TABLE>,
                                                           bfk::CfgMR<Q>::NT, smem) != cudaSuccess)
             return 0;
     }
     return n;
 }
 
-template <int Q, class P, int K>
+template <int Q, class P, int K, bool LB>
 cudaError_t launch_batch(const void *bargs, unsigned grid, size_t smem, cudaStream_t s)
 {
     static size_t granted[64] = {0};
-    cudaError_t e = prepare(bfk::k_batch_mr<Q, P, K>, smem, granted);
+    cudaError_t e = prepare(bfk::k_batch_mr<Q, P, K, LB>, smem, granted);
     if (e != cudaSuccess) return e;
-    bfk::k_batch_mr<Q, P, K><<<grid, bfk::CfgMR<Q>::NT, smem, s>>>(*static_cast<const bfk::BatchArgs<P> *>(bargs));
+    bfk::k_batch_mr<Q, P, K, LB><<<grid, bfk::CfgMR<Q>::NT, smem, s>>>(*static_cast<const bfk::BatchArgs<P> *>(bargs));
     return cudaGetLastError();
 }
 
-template <int Q, class P, int K>
+template <int Q, class P, int K, bool LB>
 int batch_ctas_per_sm(size_t smem)
 {
     static size_t granted[64] = {0};
-    if (prepare(bfk::k_batch_mr<Q, P, K>, smem, granted) != cudaSuccess) return 0;
+    if (prepare(bfk::k_batch_mr<Q, P, K, LB>, smem, granted) != cudaSuccess) return 0;
     int n = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, bfk::k_batch_mr<Q, P, K>, bfk::CfgMR<Q>::NT, smem) != cudaSuccess)
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, bfk::k_batch_mr<Q, P, K, LB>, bfk::CfgMR<Q>::NT, smem) != cudaSuccess)
         return 0;
     return n;
 }
@@ -213,8 +213,25 @@ cudaError_t launch_ctab(const void *kargs, void *out, int levels)
     return cudaGetLastError();
 }
 
+// W, twice that as stage scratch, and the caches of the pass: node features of the parents
+// (row) or the geometry of a level's output pairs (column); d = 2: Tile2
 template <int D, int Q, class P, int K>
-const PassFns *fns_for()
+size_t tile_smem(int row, int T, int k, int tab)
+{
+    const int np = T << (D * k);
+    if constexpr (D == 2) {
+        using T2 = bfk::Tile2<Q, P, K, false>;
+        return row ? T2::row_smem(np, T, k, tab != 0) : T2::col_smem(np, tab != 0);
+    } else {
+        using TL = bfk::Tile<D, Q, P, K>;
+        const size_t base = (size_t)3 * np * TL::RR * sizeof(typename P::C);
+        if (!row) return base + (size_t)np * sizeof(typename TL::Geo);
+        return base + (k > 0 ? ((size_t)T << (D * (k - 1))) * TL::RR * sizeof(typename TL::PH::T) : 0);
+    }
+}
+
+template <int D, int Q, class P, int K, bool LB>
+const PassFns *fns_set()
 {
     using CF = bfk::Cfg<D, Q, P>;
     if constexpr (D == 2 && !P::is_f64) {
@@ -223,19 +240,19 @@ const PassFns *fns_for()
         // tensor-core switch: q <= 5, polynomial sincos phases (the BF16x3 precision)
         constexpr bool TC = Q <= 5 && !P::sfu;
         constexpr int QT = TC ? Q : 2;
-        static const PassFns f = {launch_col<D, Q, P, K>, launch_row<D, Q, P, K>, launch_col_adj<D, Q, P, K>,
-                                  launch_row_adj<D, Q, P, K>, CF::KMAX, CF::NP, CF::NT,
-                                  {launch_col_mr<Q, P, K, bfk::PM_COMPUTE>, launch_col_mr<Q, P, K, bfk::PM_BUILD>,
-                                   launch_col_mr<Q, P, K, bfk::PM_TABLE>},
-                                  {launch_row_mr<Q, P, K, bfk::PM_COMPUTE>, launch_row_mr<Q, P, K, bfk::PM_BUILD>,
-                                   launch_row_mr<Q, P, K, bfk::PM_TABLE>},
+        static const PassFns f = {launch_col<D, Q, P, K, LB>, launch_row<D, Q, P, K, LB>, launch_col_adj<D, Q, P, K>,
+                                  launch_row_adj<D, Q, P, K>, CF::KMAX, CF::NP, CF::NT, LB ? 1 : 0, tile_smem<D, Q, P, K>,
+                                  {launch_col_mr<Q, P, K, LB, bfk::PM_COMPUTE>, launch_col_mr<Q, P, K, LB, bfk::PM_BUILD>,
+                                   launch_col_mr<Q, P, K, LB, bfk::PM_TABLE>},
+                                  {launch_row_mr<Q, P, K, LB, bfk::PM_COMPUTE>, launch_row_mr<Q, P, K, LB, bfk::PM_BUILD>,
+                                   launch_row_mr<Q, P, K, LB, bfk::PM_TABLE>},
                                   bfk::MRMAX, bfk::CfgMR<Q>::NT,
-                                  launch_batch<Q, P, K>, batch_ctas_per_sm<Q, P, K>, mr_table_occupancy<Q, P, K>,
+                                  launch_batch<Q, P, K, LB>, batch_ctas_per_sm<Q, P, K, LB>, mr_table_occupancy<Q, P, K, LB>,
                                   launch_ctab<D, Q, P, K>, (int)sizeof(typename bfk::Ph<P, D, K>::T),
-                                  {TAB ? launch_col<D, (TAB ? Q : 2), P, K, bfk::PM_BUILD> : nullptr,
-                                   TAB ? launch_col<D, (TAB ? Q : 2), P, K, bfk::PM_TABLE> : nullptr},
-                                  {TAB ? launch_row<D, (TAB ? Q : 2), P, K, bfk::PM_BUILD> : nullptr,
-                                   TAB ? launch_row<D, (TAB ? Q : 2), P, K, bfk::PM_TABLE> : nullptr},
+                                  {TAB ? launch_col<D, (TAB ? Q : 2), P, K, TAB && LB, bfk::PM_BUILD> : nullptr,
+                                   TAB ? launch_col<D, (TAB ? Q : 2), P, K, TAB && LB, bfk::PM_TABLE> : nullptr},
+                                  {TAB ? launch_row<D, (TAB ? Q : 2), P, K, TAB && LB, bfk::PM_BUILD> : nullptr,
+                                   TAB ? launch_row<D, (TAB ? Q : 2), P, K, TAB && LB, bfk::PM_TABLE> : nullptr},
                                   TC ? launch_switch_tc<QT, P, K, 0> : nullptr,
                                   TC ? switch_tc_ctas_per_sm<QT, P, K, 0> : nullptr, TC ? bfk::SwTC<QT, 0>::SMEM : 0,
                                   TC ? launch_col_tc<QT, P, K> : nullptr,
@@ -245,22 +262,32 @@ const PassFns *fns_for()
         return &f;
     } else if constexpr (!P::is_f64) {
         // d = 3: single-RHS passes with a reduced-phase table; no multi-RHS kernels
-        static const PassFns f = {launch_col<D, Q, P, K>, launch_row<D, Q, P, K>, launch_col_adj<D, Q, P, K>,
-                                  launch_row_adj<D, Q, P, K>, CF::KMAX, CF::NP, CF::NT, {nullptr, nullptr, nullptr},
+        static const PassFns f = {launch_col<D, Q, P, K, LB>, launch_row<D, Q, P, K, LB>, launch_col_adj<D, Q, P, K>,
+                                  launch_row_adj<D, Q, P, K>, CF::KMAX, CF::NP, CF::NT, LB ? 1 : 0, tile_smem<D, Q, P, K>, {nullptr, nullptr, nullptr},
                                   {nullptr, nullptr, nullptr}, 0, 0, nullptr, nullptr, nullptr,
                                   launch_ctab<D, Q, P, K>, (int)sizeof(typename bfk::Ph<P, D, K>::T),
-                                  {launch_col<D, Q, P, K, bfk::PM_BUILD>, launch_col<D, Q, P, K, bfk::PM_TABLE>},
-                                  {launch_row<D, Q, P, K, bfk::PM_BUILD>, launch_row<D, Q, P, K, bfk::PM_TABLE>},
+                                  {launch_col<D, Q, P, K, LB, bfk::PM_BUILD>, launch_col<D, Q, P, K, LB, bfk::PM_TABLE>},
+                                  {launch_row<D, Q, P, K, LB, bfk::PM_BUILD>, launch_row<D, Q, P, K, LB, bfk::PM_TABLE>},
                                   nullptr, nullptr, 0, nullptr, nullptr, 0};
         return &f;
     } else {
-        static const PassFns f = {launch_col<D, Q, P, K>, launch_row<D, Q, P, K>, launch_col_adj<D, Q, P, K>,
-                                  launch_row_adj<D, Q, P, K>, CF::KMAX, CF::NP, CF::NT, {nullptr, nullptr, nullptr},
+        static const PassFns f = {launch_col<D, Q, P, K, LB>, launch_row<D, Q, P, K, LB>, launch_col_adj<D, Q, P, K>,
+                                  launch_row_adj<D, Q, P, K>, CF::KMAX, CF::NP, CF::NT, LB ? 1 : 0, tile_smem<D, Q, P, K>, {nullptr, nullptr, nullptr},
                                   {nullptr, nullptr, nullptr}, 0, 0, nullptr, nullptr, nullptr,
                                   launch_ctab<D, Q, P, K>, (int)sizeof(typename bfk::Ph<P, D, K>::T),
                                   {nullptr, nullptr}, {nullptr, nullptr}, nullptr, nullptr, 0, nullptr, nullptr, 0};
         return &f;
     }
+}
+
+// kernels for node kind 0 (Lobatto) or 1: at d = 2 and odd q the Lobatto ones are their own
+template <int D, int Q, class P, int K>
+const PassFns *fns_for(int node_kind)
+{
+    if constexpr (D == 2 && (Q & 1)) {
+        if (node_kind == 0) return fns_set<D, Q, P, K, true>();
+    }
+    return fns_set<D, Q, P, K, false>();
 }
 
 }  // namespace bfl

@@ -3,15 +3,15 @@
 
 namespace bfl {
 
-const PassFns *fns_d2_mix_dot(int q)
+const PassFns *fns_d2_mix_dot(int q, int node_kind)
 {
     switch (q) {
-    case 2: return fns_for<2, 2, bfk::PMIX, bfk::KIND_DOT>();
-    case 3: return fns_for<2, 3, bfk::PMIX, bfk::KIND_DOT>();
-    case 4: return fns_for<2, 4, bfk::PMIX, bfk::KIND_DOT>();
-    case 5: return fns_for<2, 5, bfk::PMIX, bfk::KIND_DOT>();
-    case 6: return fns_for<2, 6, bfk::PMIX, bfk::KIND_DOT>();
-    case 8: return fns_for<2, 8, bfk::PMIX, bfk::KIND_DOT>();
+    case 2: return fns_for<2, 2, bfk::PMIX, bfk::KIND_DOT>(node_kind);
+    case 3: return fns_for<2, 3, bfk::PMIX, bfk::KIND_DOT>(node_kind);
+    case 4: return fns_for<2, 4, bfk::PMIX, bfk::KIND_DOT>(node_kind);
+    case 5: return fns_for<2, 5, bfk::PMIX, bfk::KIND_DOT>(node_kind);
+    case 6: return fns_for<2, 6, bfk::PMIX, bfk::KIND_DOT>(node_kind);
+    case 8: return fns_for<2, 8, bfk::PMIX, bfk::KIND_DOT>(node_kind);
     default: return nullptr;
     }
 }

@@ -3,15 +3,15 @@
 
 namespace bfl {
 
-const PassFns *fns_d2_sfu_separable(int q)
+const PassFns *fns_d2_sfu_separable(int q, int node_kind)
 {
     switch (q) {
-    case 2: return fns_for<2, 2, bfk::PMIXF, bfk::KIND_SEPARABLE>();
-    case 3: return fns_for<2, 3, bfk::PMIXF, bfk::KIND_SEPARABLE>();
-    case 4: return fns_for<2, 4, bfk::PMIXF, bfk::KIND_SEPARABLE>();
-    case 5: return fns_for<2, 5, bfk::PMIXF, bfk::KIND_SEPARABLE>();
-    case 6: return fns_for<2, 6, bfk::PMIXF, bfk::KIND_SEPARABLE>();
-    case 8: return fns_for<2, 8, bfk::PMIXF, bfk::KIND_SEPARABLE>();
+    case 2: return fns_for<2, 2, bfk::PMIXF, bfk::KIND_SEPARABLE>(node_kind);
+    case 3: return fns_for<2, 3, bfk::PMIXF, bfk::KIND_SEPARABLE>(node_kind);
+    case 4: return fns_for<2, 4, bfk::PMIXF, bfk::KIND_SEPARABLE>(node_kind);
+    case 5: return fns_for<2, 5, bfk::PMIXF, bfk::KIND_SEPARABLE>(node_kind);
+    case 6: return fns_for<2, 6, bfk::PMIXF, bfk::KIND_SEPARABLE>(node_kind);
+    case 8: return fns_for<2, 8, bfk::PMIXF, bfk::KIND_SEPARABLE>(node_kind);
     default: return nullptr;
     }
 }

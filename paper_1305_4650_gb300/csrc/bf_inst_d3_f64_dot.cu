@@ -3,12 +3,12 @@
 
 namespace bfl {
 
-const PassFns *fns_d3_f64_dot(int q)
+const PassFns *fns_d3_f64_dot(int q, int node_kind)
 {
     switch (q) {
-    case 2: return fns_for<3, 2, bfk::PF64, bfk::KIND_DOT>();
-    case 3: return fns_for<3, 3, bfk::PF64, bfk::KIND_DOT>();
-    case 4: return fns_for<3, 4, bfk::PF64, bfk::KIND_DOT>();
+    case 2: return fns_for<3, 2, bfk::PF64, bfk::KIND_DOT>(node_kind);
+    case 3: return fns_for<3, 3, bfk::PF64, bfk::KIND_DOT>(node_kind);
+    case 4: return fns_for<3, 4, bfk::PF64, bfk::KIND_DOT>(node_kind);
     default: return nullptr;
     }
 }

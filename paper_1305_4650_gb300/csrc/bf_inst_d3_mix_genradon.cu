@@ -3,12 +3,12 @@
 
 namespace bfl {
 
-const PassFns *fns_d3_mix_genradon(int q)
+const PassFns *fns_d3_mix_genradon(int q, int node_kind)
 {
     switch (q) {
-    case 2: return fns_for<3, 2, bfk::PMIX, bfk::KIND_GENRADON>();
-    case 3: return fns_for<3, 3, bfk::PMIX, bfk::KIND_GENRADON>();
-    case 4: return fns_for<3, 4, bfk::PMIX, bfk::KIND_GENRADON>();
+    case 2: return fns_for<3, 2, bfk::PMIX, bfk::KIND_GENRADON>(node_kind);
+    case 3: return fns_for<3, 3, bfk::PMIX, bfk::KIND_GENRADON>(node_kind);
+    case 4: return fns_for<3, 4, bfk::PMIX, bfk::KIND_GENRADON>(node_kind);
     default: return nullptr;
     }
 }

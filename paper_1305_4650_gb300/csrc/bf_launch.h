@@ -15,6 +15,9 @@ struct PassFns {
     int kmax;                    // most levels one pass fuses
     int np;                      // pairs per CTA (2^{d kmax})
     int nthreads;                // threads per CTA
+    int lobatto;                 // 1: the forward kernels use the Lobatto nodes (KArgs::corner may be set)
+    // shared memory (bytes) of a forward pass with T tiles of k levels per CTA; tab: reading a phase table
+    size_t (*tile_smem)(int row, int T, int k, int tab);
     // multi-RHS forward passes with a phase cache (null if absent), per phase mode:
     // [0] evaluate, [1] build the plan's phase table, [2] read the phase table
     pass_fn col_mr[3], row_mr[3];
@@ -46,12 +49,12 @@ struct PassFns {
     size_t switch_tc32_smem = 0;
 };
 
-// (d, q, precision, phase kind) -> kernels, or null if that combination is not compiled.
+// (d, q, precision, phase kind, node kind) -> kernels, or null if that combination is not compiled.
 // precision: 0 FP64, 1 mixed, 2 mixed with SFU sincos; kind: bf_phase_kind
-const PassFns *get_fns(int d, int q, int prec, int kind);
+const PassFns *get_fns(int d, int q, int prec, int kind, int node_kind);
 
 // one function per instantiation unit: bf_inst_d{d}_{f64|mix}_{kind}.cu
-#define BFL_DECLARE(d, pr, kn) const PassFns *fns_d##d##_##pr##_##kn(int q);
+#define BFL_DECLARE(d, pr, kn) const PassFns *fns_d##d##_##pr##_##kn(int q, int node_kind);
 BFL_DECLARE(2, f64, dot) BFL_DECLARE(2, f64, genradon) BFL_DECLARE(2, f64, hypradon) BFL_DECLARE(2, f64, separable)
 BFL_DECLARE(2, mix, dot) BFL_DECLARE(2, mix, genradon) BFL_DECLARE(2, mix, hypradon) BFL_DECLARE(2, mix, separable)
 BFL_DECLARE(3, f64, dot) BFL_DECLARE(3, f64, genradon) BFL_DECLARE(3, f64, separable)

@@ -126,19 +126,17 @@ __host__ __device__ constexpr int mr_pc_extra(int q)
 }
 // scratch entries per right-hand side (2 r per pair, plus the row scratch padding)
 __host__ __device__ constexpr int64_t mr_s_stride(int q, int64_t npr) { return 2 * npr * q * q + npr * q * mr_pad(q).rs; }
-
-// acc += M[h][t][u] v: two scalar FMAs, the coefficient an operand from the kernel
-// parameters (constant bank).  One packed FMA with the coefficient duplicated (KArgs::M2)
-// needs that pair loaded into registers first: measured 1% slower per apply at N = 512
-// with 16 right-hand sides (the same roundings either way; in the persistent batch kernel
-// the packed form also spilled)
-template <class MS, class C>
-__device__ __forceinline__ void mmac(C &acc, const MS &ms, int h, int t, int u, C v)
+// complex numbers of the scratch S: rc right-hand sides, and at least the parts of a level
+// (6 rows of up to three components of q, padded to even, and a sign per pair), which the
+// phase stage keeps there
+__host__ __device__ constexpr int64_t mr_s_size(int q, int64_t npr, int64_t rc)
 {
-    cfma(acc, ms.M[h][t][u], v);
+    const int64_t st = rc * mr_s_stride(q, npr), pt = (npr * (18 * ((q + 1) & ~1) + 1) + 1) / 2;
+    return ((st > pt ? st : pt) + 1) & ~(int64_t)1;
 }
 
-template <int Q, class P, int K>
+// LB: Lobatto nodes of odd q (unit columns of M, KArgs::corner; bf_tile2.cuh)
+template <int Q, class P, int K, bool LB>
 struct TileMR {
     static constexpr MRPad PAD = mr_pad(Q);
     static constexpr int D = 2, NC = 4, RR = Q * Q, NT = CfgMR<Q>::NT;
@@ -147,13 +145,8 @@ struct TileMR {
     using PH = Ph<P, 2, K>;
     using PH2 = Ph2<P, 2, K>;
     using TL = Tile<2, Q, P, K>;
-
-    // geometry of one output pair of a column level, computed once per level into the
-    // scratch S (idle during the phase stage) for the stage's phase items
-    struct __align__(16) GeoC {
-        typename PH::T tA;   // target features at the centre of the pair's target box (level l+1)
-        int cbq[2];          // coordinates of the parent source box (level l+1)
-    };
+    using T2 = Tile2<Q, P, K, LB>;
+    static constexpr int MID = T2::MID, END = T2::END;
 
     // geometry of one merge block of a row level (in S during the phase stage): the parent
     // target box (level l) and the parent source box (level l+1)
@@ -179,6 +172,10 @@ struct TileMR {
         Ap = tile >> sh;
         Bstar = tile & ((1u << sh) - 1u);
     }
+
+    // the pass's first step also does level 0, its last step level L - 1 (KArgs::corner)
+    static __device__ __forceinline__ bool skip_first(const KArgs<P> &a) { return LB && (a.corner & CORNER_SRC) && (a.flags & F_INIT); }
+    static __device__ __forceinline__ bool skip_last(const KArgs<P> &a) { return LB && (a.corner & CORNER_TGT) && (a.flags & F_FINAL); }
 
     static __device__ __forceinline__ int block_base(int beta, int i)
     {
@@ -207,13 +204,16 @@ struct TileMR {
             int64_t o = 0;
             auto add = [&](int64_t n) { c->off[nb++] = o; o += n; };
             if (!row) {
-                if (a.flags & F_INIT) add(RR * npr);
-                for (int i = 0; i < a.k; ++i) add(r5);
+                if (skip_first(a))
+                    o = RR * npr + r5;   // the blocks of the first step and of level 0 are not used
+                else if (a.flags & F_INIT)
+                    add(RR * npr);
+                for (int i = skip_first(a) ? 1 : 0; i < a.k; ++i) add(r5);
                 if (a.flags & F_SWITCH)
                     for (int th = 0; th < Q; ++th) add((int64_t)Q * RR * npr);
             } else {
-                for (int i = 0; i < a.k; ++i) add(r5);
-                if (a.flags & F_FINAL) add((RR + 1) * npr);
+                for (int i = 0; i < (skip_last(a) ? a.k - 1 : a.k); ++i) add(r5);
+                if ((a.flags & F_FINAL) && !skip_last(a)) add((RR + 1) * npr);
             }
             c->off[nb] = o;
             c->nblk = nb;
@@ -376,8 +376,50 @@ struct TileMR {
         if constexpr (PM == PM_TABLE) ts_release(ts);
     }
 
+    // ---- first step and first merge, last merge and last step with points at box corners
+    // (KArgs::corner; Tile2::init_corner, Tile2::final_corner)
+    static __device__ void init_corner(const KArgs<P> &a, const Ctx &x, C *W, const C *g)
+    {
+        const int k = a.k, n = 1 << (D * k), nblk = n >> D, L = a.L, WS = x.npr * RR;
+        if (a.k == 1) {   // no level of this pass follows: the switch may read every node
+            for (int j = threadIdx.x; j < x.nr * WS; j += NT) W[j] = czero<C>();
+            __syncthreads();
+        }
+        for (int it = threadIdx.x; it < x.nr * x.npr; it += NT) {
+            const int pr = it & (x.npr - 1), rb = it >> x.lgp;
+            const int c = pr & (NC - 1), b = (pr >> D) & (nblk - 1), tau = pr >> (D * k);
+            uint32_t Ap, Bstar;
+            tile_of(a, x, tau, Ap, Bstar);
+            int cb[DMAX];
+            morton_decode<D>((Bstar << (D * k)) + (pr & (n - 1)), L, cb);
+            const C v = g[(int64_t)(x.rhs0 + rb) * a.npts + ((int64_t)cb[0] << L) + cb[1]];
+            C *w = W + rb * WS + (tau * n + (b << D)) * RR + ((c & 1) ? MID : END) + ((c >> 1) ? MID : END) * Q;
+#pragma unroll
+            for (int al = 0; al < NC; ++al) w[al * RR] = v;
+        }
+        __syncthreads();
+    }
+    static __device__ void final_corner(const KArgs<P> &a, const Ctx &x, const C *W, C *f)
+    {
+        const int k = a.k, n = 1 << (D * k), nblk = n >> D, L = a.L, WS = x.npr * RR;
+        for (int it = threadIdx.x; it < x.nr * x.npr; it += NT) {
+            const int pr = it & (x.npr - 1), rb = it >> x.lgp;
+            const int al = pr & (NC - 1), ra = (pr >> D) & (nblk - 1), tau = pr >> (D * k);
+            uint32_t Ap, Bstar;
+            tile_of(a, x, tau, Ap, Bstar);
+            int ca[DMAX];
+            morton_decode<D>((((Ap << (D * (k - 1))) + digit_rev<D>(ra, k - 1)) << D) + al, L, ca);
+            const C *w = W + rb * WS + (tau * n + ra) * RR + ((al & 1) ? MID : END) + ((al >> 1) ? MID : END) * Q;
+            C acc = w[0];
+#pragma unroll
+            for (int c = 1; c < NC; ++c) acc = madd(acc, w[(c * nblk) * RR]);
+            f[(int64_t)(x.rhs0 + rb) * a.npts + ((int64_t)ca[0] << L) + ca[1]] = acc;
+        }
+    }
+
     // ---- one column-form merge level (l -> l+1); ms.M holds the child->parent matrices
-    template <int PM, class MS>
+    // SP: the inputs' nodes MID and END of both dimensions only (level 1 with KArgs::corner)
+    template <int PM, bool SP, class MS>
     static __device__ void col_level(const KArgs<P> &a, const MS &ms, const Ctx &x, C *W, C *S, C *PC, int l, int i,
                                      TS<C> &ts, uint64_t *wbar = nullptr, unsigned wpar = 0)
     {
@@ -387,9 +429,12 @@ struct TileMR {
         constexpr int PCA = 2 * RR + (PM == PM_COMPUTE ? PAD.ca : 0), PCB = RR + (PM == PM_COMPUTE ? PAD.cb : 0);
         C *PA = PC;                     // [pA][chi] blocks of PCA: [cl][tq][t0']  modulation of the inputs
         C *PB = PC + nout * 2 * PCA;    // [pA] blocks of PCB: [tq][tl]            demodulation of the output
-        GeoC *G = reinterpret_cast<GeoC *>(S);
-        for (int j = threadIdx.x; PM != PM_TABLE && j < nout; j += NT) {
-            const int alpha = j & (NC - 1), beta = (j >> D) & (nblk - 1), tau = j >> (D * k);
+        // the parts of every output pair's nodes, once per level, into S (idle during the phase
+        // stage): thread = (pair, coordinate, row of q parts), each with its own geometry
+        float *PT = reinterpret_cast<float *>(S), *SG = PT + nout * T2::PSTR;
+        for (int j = threadIdx.x; PM != PM_TABLE && j < nout * 6; j += NT) {
+            const int row = j % 3, dim = (j / 3) & 1, pA = j / 6;
+            const int alpha = pA & (NC - 1), beta = (pA >> D) & (nblk - 1), tau = pA >> (D * k);
             uint32_t Ap, Bstar, Apg, Bq;
             int base;
             tile_of(a, x, tau, Ap, Bstar);
@@ -398,40 +443,31 @@ struct TileMR {
             int ca[DMAX], cbq[DMAX];
             morton_decode<D>(Aa, l + 1, ca);
             morton_decode<D>(Bq, L - l - 1, cbq);
-            G[j].tA = tcenter<P, D, Q, K>(a, l + 1, Aa, ca);
-            G[j].cbq[0] = cbq[0];
-            G[j].cbq[1] = cbq[1];
+            const typename PH::T tA = tcenter<P, D, Q, K>(a, l + 1, Aa, ca);
+            const int cb = dim ? cbq[1] : cbq[0];
+            const typename P::SE *e = a.st[dim] + (row < 2 ? soff<Q>(L, l) + (2 * cb + row) * (Q + 2) : soff<Q>(L, l + 1) + cb * (Q + 2));
+            T2::part_row(a, dim ? tA.x[1] : tA.x[0], dim ? tA.A[1] : tA.A[0], dim == 0, e, PT + pA * T2::PSTR + (dim * 3 + row) * T2::PROW,
+                         SP && row < 2);
+            if (j % 6 == 0) SG[pA] = PH::sign(a, tA);
         }
         if constexpr (PM != PM_TABLE) __syncthreads();
-        for (int it = threadIdx.x; PM != PM_TABLE && it < nout * 4 * Q; it += NT) {
-            const int tq = it % Q, cl = (it / Q) & 1, chi = (it / (2 * Q)) & 1, pA = it / (4 * Q);
-            const typename PH::T tA = G[pA].tA;
-            const int cbq[2] = {G[pA].cbq[0], G[pA].cbq[1]};
-            const int c = cl | (chi << 1);
-            // phases two at a time: lanes t'_0 and t'_0 + 1 (the last one alone for odd q)
-            const typename PH2::T tA2 = PH2::dup(tA);
-            const typename P::SE e1 = sget<P, Q>(a, 1, l, 2 * cbq[1] + chi, tq);
-            const typename PH2::Part p1 = PH2::part(tA2, e1, e1, 1);
-            const int c0 = 2 * cbq[0] + (c & 1);
-            C *o = PA + (pA * 2 + chi) * PCA + cl * RR + tq * Q;
-#pragma unroll
-            for (int t0p = 0; t0p + 1 < Q; t0p += 2) {
-                const typename PH2::Part pt =
-                    PH2::add(PH2::part(tA2, sget<P, Q>(a, 0, l, c0, t0p), sget<P, Q>(a, 0, l, c0, t0p + 1), 0), p1);
-                expphase_part2<P, D, K>(a, tA2, pt, o[t0p], o[t0p + 1]);
+        // items (pair, g, t_1), q phases each: g < 4 modulations of child c_0 = g & 1, c_1 = g >> 1,
+        // g = 4 the demodulation
+        for (int it = threadIdx.x; PM != PM_TABLE && it < nout * 5 * Q; it += NT) {
+            const int tq = it % Q, g = (it / Q) % 5, pA = it / (5 * Q);
+            const float *pt = PT + pA * T2::PSTR;
+            const float *p0 = pt + (g < 4 ? g & 1 : 2) * T2::PROW;
+            const typename PH::Part p1 = T2::load1(pt + (3 + (g >> 1)) * T2::PROW + tq);
+            C *o = g < 4 ? PA + (pA * 2 + (g >> 1)) * PCA + (g & 1) * RR + tq * Q : PB + pA * PCB + tq * Q;
+            if (SP && g < 4) {
+                if (tq == MID || tq == END) {
+                    const auto sg = PH2::dup(K == KIND_HYPRADON ? SG[pA] : a.sc.sgn);
+                    TL::template ph2<PM_COMPUTE>(sg, PH2::add(T2::lanes(T2::load1(p0 + MID), T2::load1(p0 + END)), PH2::dup(p1)),
+                                                 nullptr, nullptr, o[MID], o[END]);
+                }
+                continue;
             }
-            if constexpr (Q & 1) {
-                const typename PH::Part pt = PH::add(PH::part(tA, sget<P, Q>(a, 0, l, c0, Q - 1), 0), PH2::lane0(p1));
-                o[Q - 1] = expphase_part<P, D, K>(a, tA, pt);
-            }
-        }
-        for (int it = threadIdx.x; PM != PM_TABLE && it < nout * RR; it += NT) {
-            const int tl = it % Q, tq = (it / Q) % Q, pA = it / RR;
-            const typename PH::T tA = G[pA].tA;
-            const int cbq[2] = {G[pA].cbq[0], G[pA].cbq[1]};
-            const typename PH::Part pl = PH::part(tA, sget<P, Q>(a, 0, l + 1, cbq[0], tl), 0);
-            const typename PH::Part pt = PH::add(PH::part(tA, sget<P, Q>(a, 1, l + 1, cbq[1], tq), 1), pl);
-            PB[pA * PCB + tq * Q + tl] = expphase_part<P, D, K>(a, tA, pt);
+            T2::phase_row(K == KIND_HYPRADON ? SG[pA] : a.sc.sgn, p0, p1, o);
         }
         __syncthreads();
         if (wbar) wait_input(a, wbar, wpar);   // the weights were copied in during the phase stage
@@ -443,8 +479,10 @@ struct TileMR {
         for (int r0 = 0; PM != PM_BUILD && r0 < x.nr; r0 += x.rc) {
             const int nrc = min(x.rc, x.nr - r0);
             // stage A: items (rb, pA, chi, tq): modulate the inputs, contract dimension 0
-            for (int it = threadIdx.x; it < nrc * nout * 2 * Q; it += NT) {
-                const int tq = it % Q, chi = (it / Q) & 1, pA = (it / (2 * Q)) & (nout - 1), rbl = (it / (2 * Q)) >> x.lgp;
+            constexpr int QA = SP ? 2 : Q;
+            for (int it = threadIdx.x; it < nrc * nout * 2 * QA; it += NT) {
+                const int tp = it % QA, chi = (it / QA) & 1, pA = (it / (2 * QA)) & (nout - 1), rbl = (it / (2 * QA)) >> x.lgp;
+                const int tq = SP ? (tp ? END : MID) : tp;
                 const int beta = (pA >> D) & (nblk - 1), tau = pA >> (D * k);
                 const int base = block_base(beta, i);
                 const C *Wr = W + (r0 + rbl) * WS + tau * n * RR;
@@ -458,9 +496,10 @@ struct TileMR {
                     const C *win = Wr + (base + (c << (D * i))) * RR + Q * tq;
 #pragma unroll
                     for (int t0p = 0; t0p < Q; ++t0p) {
+                        if (SP && t0p != MID && t0p != END) continue;
                         const C u = cmul(ph[cl * RR + t0p], win[t0p]);
 #pragma unroll
-                        for (int t0 = 0; t0 < Q; ++t0) mmac(acc[t0], ms, c & 1, t0, t0p, u);
+                        for (int t0 = 0; t0 < Q; ++t0) mmac<Q, LB>(acc[t0], ms, c & 1, t0, t0p, u);
                     }
                 }
                 C *so = S + rbl * SW + ((pA * 2 + chi) * Q + tq) * Q;
@@ -481,9 +520,10 @@ struct TileMR {
                     const C *si = S + rbl * SW + ((pA * 2 + chi) * Q) * Q + tl;
 #pragma unroll
                     for (int tqp = 0; tqp < Q; ++tqp) {
+                        if (SP && tqp != MID && tqp != END) continue;
                         const C v = si[tqp * Q];
 #pragma unroll
-                        for (int tq = 0; tq < Q; ++tq) mmac(acc[tq], ms, chi, tq, tqp, v);
+                        for (int tq = 0; tq < Q; ++tq) mmac<Q, LB>(acc[tq], ms, chi, tq, tqp, v);
                     }
                 }
                 C *wo = W + (r0 + rbl) * WS + tau * n * RR + (base + (alpha << (D * i))) * RR + tl;
@@ -533,16 +573,16 @@ struct TileMR {
                     if constexpr (PM != PM_TABLE) {
                         const typename PH2::T tS2 = PH2::dup(tS);
                         const typename P::SE e1 = sget<P, Q>(a, 1, l, cb[1], th);
-                        const typename PH2::Part hp = PH2::part(tS2, e1, e1, 1);
+                        const typename PH2::Part hp = PH2::part(a, tS2, e1, e1, 1);
 #pragma unroll
                         for (int t0 = 0; t0 + 1 < Q; t0 += 2)
                             expphase_part2<P, D, K>(
                                 a, tS2,
-                                PH2::add(PH2::part(tS2, sget<P, Q>(a, 0, l, cb[0], t0), sget<P, Q>(a, 0, l, cb[0], t0 + 1), 0), hp),
+                                PH2::add(PH2::part(a, tS2, sget<P, Q>(a, 0, l, cb[0], t0), sget<P, Q>(a, 0, l, cb[0], t0 + 1), 0), hp),
                                 ev[t0], ev[t0 + 1]);
                         if constexpr (Q & 1)
                             ev[Q - 1] = expphase_part<P, D, K>(
-                                a, tS, PH::add(PH::part(tS, sget<P, Q>(a, 0, l, cb[0], Q - 1), 0), PH2::lane0(hp)));
+                                a, tS, PH::add(PH::part(a, tS, sget<P, Q>(a, 0, l, cb[0], Q - 1), 0), PH2::lane0(hp)));
                     }
 #pragma unroll
                     for (int t0 = 0; t0 < Q; ++t0) {
@@ -578,8 +618,8 @@ struct TileMR {
         if constexpr (PM == PM_BUILD) ts.tb += (int64_t)x.npr * RR * RR;
     }
 
-    // ---- one row-form merge level (l -> l+1)
-    template <int PM, class MS>
+    // ---- one row-form merge level (l -> l+1); SP: the outputs' nodes MID and END only
+    template <int PM, bool SP, class MS>
     static __device__ void row_level(const KArgs<P> &a, const MS &ms, const Ctx &x, C *W, C *S, C *PC, int l, int i,
                                      TS<C> &ts, uint64_t *wbar = nullptr, unsigned wpar = 0)
     {
@@ -603,34 +643,27 @@ struct TileMR {
             GR[j] = GeoR{{ca[0], ca[1]}, {cbq[0], cbq[1]}};
         }
         if constexpr (PM != PM_TABLE) __syncthreads();
-        for (int it = threadIdx.x; PM != PM_TABLE && it < nout * RR; it += NT) {
-            const int t0 = it % Q, th = (it / Q) % Q, pin = it / RR;
-            const int c = pin & (NC - 1), b = pin >> D;
-            const int ca[DMAX] = {GR[b].ca[0], GR[b].ca[1], 0};
-            const int cb[DMAX] = {2 * GR[b].cbq[0] + (c & 1), 2 * GR[b].cbq[1] + ((c >> 1) & 1), 0};
-            const int ctr[DMAX] = {Q, Q, Q};
-            const int tk[DMAX] = {t0, th, 0};
-            PA[it] = expphase<P, D, K>(a, tpoint<P, D, Q, K>(a, l, ca, tk), spoint<P, D, Q, K>(a, l, cb, ctr));
-        }
-        for (int it = threadIdx.x; PM != PM_TABLE && it < nout * RR; it += NT) {
-            const int s0 = it % Q, s1 = (it / Q) % Q, pA = it / RR;
-            const int alpha = pA & (NC - 1), b = pA >> D;
-            // the child target box (level l+1) of the block's parent box
-            const int ca[DMAX] = {2 * GR[b].ca[0] + (alpha & 1), 2 * GR[b].ca[1] + ((alpha >> 1) & 1), 0};
-            const int cbq[DMAX] = {GR[b].cbq[0], GR[b].cbq[1], 0};
-            const int sk[DMAX] = {s0, s1, 0};
-            const typename PH::T tS = tpoint<P, D, Q, K>(a, l + 1, ca, sk);
-            // phases two at a time: lanes c_0 = 0 and 1
-            const typename PH2::T tS2 = PH2::dup(tS);
-            const typename PH2::Part q0 =
-                PH2::part(tS2, sget<P, Q>(a, 0, l, 2 * cbq[0], Q), sget<P, Q>(a, 0, l, 2 * cbq[0] + 1, Q), 0);
+        // items (pair, s), the four post-modulations at a child node, then (block, t), the four
+        // pre-modulations at a parent node
+        constexpr int RP = SP ? 4 : RR;   // output nodes
+        for (int it = threadIdx.x; PM != PM_TABLE && it < nout * RP + (nout >> D) * RR; it += NT) {
+            const bool post = it < nout * RP;
+            const int jt = post ? it : it - nout * RP, pj = post ? jt / RP : jt / RR;
+            const int t = SP && post ? ((jt & 1) ? END : MID) + ((jt & 2) ? END : MID) * Q : (post ? jt % RP : jt % RR);
+            const GeoR g = GR[post ? pj >> D : pj];
+            const int ca[DMAX] = {post ? 2 * g.ca[0] + (pj & 1) : g.ca[0], post ? 2 * g.ca[1] + ((pj >> 1) & 1) : g.ca[1], 0};
+            const int tk[DMAX] = {t % Q, t / Q, 0};
+            typename P::SE s0[2], s1[2];
 #pragma unroll
-            for (int c1 = 0; c1 < 2; ++c1) {
-                const typename P::SE e1 = sget<P, Q>(a, 1, l, 2 * cbq[1] + c1, Q);
-                expphase_part2<P, D, K>(a, tS2, PH2::add(q0, PH2::part(tS2, e1, e1, 1)),
-                                        PB[pA * PRB + ((2 * c1) * Q + s1) * Q + s0],
-                                        PB[pA * PRB + ((2 * c1 + 1) * Q + s1) * Q + s0]);
+            for (int h = 0; h < 2; ++h) {
+                s0[h] = sget<P, Q>(a, 0, l, 2 * g.cbq[0] + h, Q);
+                s1[h] = sget<P, Q>(a, 1, l, 2 * g.cbq[1] + h, Q);
             }
+            C E[NC];
+            T2::template four<PM_COMPUTE>(a, tpoint<P, D, Q, K>(a, post ? l + 1 : l, ca, tk), s0, s1, typename T2::FT{nullptr, 0}, 0, 0, E);
+            C *o = post ? PB + pj * PRB + t : PA + pj * NC * RR + t;
+#pragma unroll
+            for (int c = 0; c < NC; ++c) o[c * RR] = E[c];
         }
         __syncthreads();
         if (wbar) wait_input(a, wbar, wpar);   // the weights were copied in during the phase stage
@@ -659,45 +692,58 @@ struct TileMR {
                     const C u = cjmul(ph[t0], win[t0]);
 #pragma unroll
                     for (int s0 = 0; s0 < Q; ++s0) {
-                        mmac(z[0][s0], ms, 0, t0, s0, u);
-                        mmac(z[1][s0], ms, 1, t0, s0, u);
+                        if (SP && s0 != MID && s0 != END) continue;
+                        mmac<Q, LB>(z[0][s0], ms, 0, t0, s0, u);
+                        mmac<Q, LB>(z[1][s0], ms, 1, t0, s0, u);
                     }
                 }
                 C *so = S + rbl * SW + (pin * Q + th) * SU;
 #pragma unroll
                 for (int s0 = 0; s0 < Q; ++s0) {
+                    if (SP && s0 != MID && s0 != END) continue;
                     so[s0] = z[0][s0];
                     so[Q + s0] = z[1][s0];
                 }
             }
             __syncthreads();
-            // stage B: items (rb, pA, s0): contract dimension 1 per child, post-modulate, sum over c
-            for (int it = threadIdx.x; it < nrc * nout * Q; it += NT) {
-                const int s0 = it % Q, pA = (it / Q) & (nout - 1), rbl = (it / Q) >> x.lgp;
+            // stage B: items (rb, pA, s0): contract dimension 1 per child, post-modulate, sum over
+            // c.  M_1 is M_0 with both indices reversed: a child alpha_1 = 1 runs dimension 1
+            // backwards, so the coefficients are compile-time operands
+            constexpr int QB = SP ? 2 : Q;
+            for (int it = threadIdx.x; it < nrc * nout * QB; it += NT) {
+                const int sp = it % QB, s0 = SP ? (sp ? END : MID) : sp, pA = (it / QB) & (nout - 1), rbl = (it / QB) >> x.lgp;
                 const int alpha = pA & (NC - 1), beta = (pA >> D) & (nblk - 1), tau = pA >> (D * k);
                 const int base = block_base(beta, i);
-                const int a0 = alpha & 1, a1 = alpha >> 1;
-                const C *Sblk = S + rbl * SW + (pA - alpha) * Q * SU;
-                C v[NC][Q];
+                const int a0 = alpha & 1, a1 = alpha >> 1, rev = a1 ? -1 : 1;
+                const C *Sblk = S + rbl * SW + (pA - alpha) * Q * SU + a0 * Q + s0 + (a1 ? (Q - 1) * SU : 0);
+                C v[NC][QB];   // SP: nodes MID and END
 #pragma unroll
                 for (int c = 0; c < NC; ++c) {
-                    const C *si = Sblk + c * Q * SU + a0 * Q + s0;
+                    const C *si = Sblk + c * Q * SU;
+                    if constexpr (SP) {
+                        v[c][0] = czero<C>();
 #pragma unroll
-                    for (int s1 = 0; s1 < Q; ++s1) v[c][s1] = czero<C>();
+                        for (int t1 = 0; t1 < Q; ++t1) mmac<Q, LB>(v[c][0], ms, 0, t1, MID, si[t1 * rev * SU]);
+                        v[c][1] = si[(a1 ? MID : END) * rev * SU];
+                    } else {
 #pragma unroll
-                    for (int t1 = 0; t1 < Q; ++t1) {
-                        const C zz = si[t1 * SU];
+                        for (int s1 = 0; s1 < Q; ++s1) v[c][s1] = czero<C>();
 #pragma unroll
-                        for (int s1 = 0; s1 < Q; ++s1) mmac(v[c][s1], ms, a1, t1, s1, zz);
+                        for (int t1 = 0; t1 < Q; ++t1) {
+                            const C zz = si[t1 * rev * SU];
+#pragma unroll
+                            for (int s1 = 0; s1 < Q; ++s1) mmac<Q, LB>(v[c][s1], ms, 0, t1, s1, zz);
+                        }
                     }
                 }
                 C *wo = W + (r0 + rbl) * WS + tau * n * RR + (base + (alpha << (D * i))) * RR + s0;
                 const C *ph = PB + pA * PRB + s0;
 #pragma unroll
-                for (int s1 = 0; s1 < Q; ++s1) {
+                for (int j = 0; j < QB; ++j) {
+                    const int s1 = SP ? (j ? END : MID) : (a1 ? Q - 1 - j : j);
                     C acc = czero<C>();
 #pragma unroll
-                    for (int c = 0; c < NC; ++c) acc = TL::cadd(acc, cmul(ph[(c * Q + s1) * Q], v[c][s1]));
+                    for (int c = 0; c < NC; ++c) acc = TL::cadd(acc, cmul(ph[(c * Q + s1) * Q], v[c][j]));
                     wo[s1 * Q] = acc;
                 }
             }
@@ -764,7 +810,7 @@ struct TileMR {
     // shared memory of one CTA, bytes
     static __host__ __device__ size_t smem_bytes(int npr, int nr, int rc)
     {
-        return sizeof(C) * ((size_t)npr * RR * (size_t)(nr + 5) + (size_t)rc * (size_t)mr_s_stride(Q, npr) +
+        return sizeof(C) * ((size_t)npr * RR * (size_t)(nr + 5) + (size_t)mr_s_size(Q, npr, rc) +
                             (size_t)npr * mr_pc_extra(Q));
     }
 
@@ -786,19 +832,26 @@ struct TileMR {
 // constant bank; ts carries the phase table (PM_BUILD, PM_TABLE)
 // wbar (per-pass kernels): the input weights come by bulk copies that overlap the first
 // level's phase stage (wpar: the mbarrier phase of this tile group); null: plain loads first
-template <int Q, class P, int K, int PM, class MS>
-__device__ __forceinline__ bool col_pass_mr(const KArgs<P> &a, const MS &ms, const typename TileMR<Q, P, K>::Ctx &x,
+template <int Q, class P, int K, bool LB, int PM, class MS>
+__device__ __forceinline__ bool col_pass_mr(const KArgs<P> &a, const MS &ms, const typename TileMR<Q, P, K, LB>::Ctx &x,
                                             unsigned char *sm, const typename P::C *g, TS<typename P::C> &ts,
                                             uint64_t *wbar = nullptr, unsigned wpar = 0)
 {
     using C = typename P::C;
-    using TM = TileMR<Q, P, K>;
+    using TM = TileMR<Q, P, K, LB>;
     const int WS = x.npr * TM::RR;
     C *W = reinterpret_cast<C *>(sm);
     C *S = W + x.nr * WS;
-    C *PC = S + x.rc * mr_s_stride(Q, x.npr);
+    C *PC = S + mr_s_size(Q, x.npr, x.rc);
     const bool async = wbar && !(a.flags & F_INIT) && a.k > 0 && a.shard_mode != 2;
-    if (a.flags & F_INIT) {
+    // KArgs::corner: level 0 is done by the first step, level 1 has four non-zero nodes per input
+    const bool skip0 = TM::skip_first(a);
+    if (skip0) {
+        if constexpr (PM == PM_BUILD)
+            ts.tb += (int64_t)6 * TM::RR * x.npr;   // the blocks of the first step and of level 0 stay unused
+        else
+            TM::init_corner(a, x, W, g);
+    } else if (a.flags & F_INIT) {
         TM::template init<PM>(a, x, W, PC, g, ts);
     } else if (async) {
         TM::load_async(a, x, W, wbar);
@@ -806,34 +859,49 @@ __device__ __forceinline__ bool col_pass_mr(const KArgs<P> &a, const MS &ms, con
         TM::load(a, x, W);
         __syncthreads();
     }
-    for (int i = 0; i < a.k; ++i)
-        TM::template col_level<PM>(a, ms, x, W, S, PC, a.l0 + i, i, ts, async && i == 0 ? wbar : nullptr, wpar);
+    for (int i = skip0 ? 1 : 0; i < a.k; ++i) {
+        uint64_t *wb = async && i == 0 ? wbar : nullptr;
+        if (LB && (a.corner & CORNER_SRC) && a.l0 + i == 1)
+            TM::template col_level<PM, LB>(a, ms, x, W, S, PC, a.l0 + i, i, ts, wb, wpar);
+        else
+            TM::template col_level<PM, false>(a, ms, x, W, S, PC, a.l0 + i, i, ts, wb, wpar);
+    }
     if (a.flags & F_SWITCH) TM::template switch_tiles<PM>(a, x, W, a.l0 + a.k, ts);
     if (PM != PM_BUILD) TM::store(a, x, W);
     return async;
 }
 
-template <int Q, class P, int K, int PM, class MS>
-__device__ __forceinline__ bool row_pass_mr(const KArgs<P> &a, const MS &ms, const typename TileMR<Q, P, K>::Ctx &x,
+template <int Q, class P, int K, bool LB, int PM, class MS>
+__device__ __forceinline__ bool row_pass_mr(const KArgs<P> &a, const MS &ms, const typename TileMR<Q, P, K, LB>::Ctx &x,
                                             unsigned char *sm, typename P::C *f, TS<typename P::C> &ts,
                                             uint64_t *wbar = nullptr, unsigned wpar = 0)
 {
     using C = typename P::C;
-    using TM = TileMR<Q, P, K>;
+    using TM = TileMR<Q, P, K, LB>;
     const int WS = x.npr * TM::RR;
     C *W = reinterpret_cast<C *>(sm);
     C *S = W + x.nr * WS;
-    C *PC = S + x.rc * mr_s_stride(Q, x.npr);
-    const bool async = wbar && a.k > 0 && a.shard_mode != 2;
+    C *PC = S + mr_s_size(Q, x.npr, x.rc);
+    // KArgs::corner: the last step does the last level, and the level before it has four output nodes
+    const bool skip = TM::skip_last(a);
+    const int k1 = skip ? a.k - 1 : a.k;
+    const bool async = wbar && k1 > 0 && a.shard_mode != 2;
     if (async) {
         TM::load_async(a, x, W, wbar);
     } else if (PM != PM_BUILD) {
         TM::load(a, x, W);
         __syncthreads();
     }
-    for (int i = 0; i < a.k; ++i)
-        TM::template row_level<PM>(a, ms, x, W, S, PC, a.l0 + i, i, ts, async && i == 0 ? wbar : nullptr, wpar);
-    if (a.flags & F_FINAL)
+    for (int i = 0; i < k1; ++i) {
+        uint64_t *wb = async && i == 0 ? wbar : nullptr;
+        if (LB && (a.corner & CORNER_TGT) && a.l0 + i == a.L - 2)
+            TM::template row_level<PM, LB>(a, ms, x, W, S, PC, a.l0 + i, i, ts, wb, wpar);
+        else
+            TM::template row_level<PM, false>(a, ms, x, W, S, PC, a.l0 + i, i, ts, wb, wpar);
+    }
+    if (skip) {
+        if constexpr (PM != PM_BUILD) TM::final_corner(a, x, W, f);
+    } else if (a.flags & F_FINAL)
         TM::template final_eval<PM>(a, x, W, PC, f, ts);
     else if (PM != PM_BUILD)
         TM::store(a, x, W);
@@ -847,8 +915,8 @@ template <int Q>
 __host__ __device__ constexpr int tab_blk_factor() { return Q > 5 ? Q : 5; }
 
 // shared memory of a CTA: PM_TABLE puts the stream control and two block buffers first
-template <int Q, class P, int K, int PM>
-__device__ __forceinline__ unsigned char *mr_setup(const KArgs<P> &a, const typename TileMR<Q, P, K>::Ctx &x,
+template <int Q, class P, int K, bool LB, int PM>
+__device__ __forceinline__ unsigned char *mr_setup(const KArgs<P> &a, const typename TileMR<Q, P, K, LB>::Ctx &x,
                                                    unsigned char *smem, TS<typename P::C> &ts, bool row)
 {
     using C = typename P::C;
@@ -866,20 +934,20 @@ __device__ __forceinline__ unsigned char *mr_setup(const KArgs<P> &a, const type
     ts.ctl = reinterpret_cast<TabCtl *>(smem);
     ts.buf[0] = reinterpret_cast<C *>(smem + TABCTL_BYTES);
     ts.buf[1] = ts.buf[0] + blk;
-    TileMR<Q, P, K>::ts_setup(ts, a, x, row);
+    TileMR<Q, P, K, LB>::ts_setup(ts, a, x, row);
     return reinterpret_cast<unsigned char *>(ts.buf[1] + blk);
 }
 
 // Per-pass kernels.  A CTA runs tile groups blockIdx.x, blockIdx.x + gridDim.x, ... < a.ncta
 // (one with a full grid; PM_TABLE launches as many CTAs as fit and streams the table of
 // all its tile groups through one pipeline).
-template <int Q, class P, int K, int PM>
+template <int Q, class P, int K, bool LB, int PM>
 __global__ void __launch_bounds__(CfgMR<Q>::NT, CfgMR<Q>::MINB) k_col_pass_mr(const KArgs<P> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint64_t wbar;
     TS<typename P::C> ts;
-    unsigned char *work = mr_setup<Q, P, K, PM>(a, TileMR<Q, P, K>::ctx(a, blockIdx.x), smem_raw, ts, false);
+    unsigned char *work = mr_setup<Q, P, K, LB, PM>(a, TileMR<Q, P, K, LB>::ctx(a, blockIdx.x), smem_raw, ts, false);
     if (PM == PM_COMPUTE && threadIdx.x == 0) {
         mbar_init(&wbar, 1);
         mbar_init_fence();
@@ -888,19 +956,19 @@ __global__ void __launch_bounds__(CfgMR<Q>::NT, CfgMR<Q>::MINB) k_col_pass_mr(co
     unsigned it = 0;
     for (int c = blockIdx.x; c < a.ncta; c += gridDim.x, ++it) {
         if constexpr (PM == PM_BUILD) ts.tb = a.ptab + (int64_t)c * a.ptab_cta;
-        col_pass_mr<Q, P, K, PM>(a, a, TileMR<Q, P, K>::ctx(a, c), work, a.g, ts, PM == PM_COMPUTE ? &wbar : nullptr,
+        col_pass_mr<Q, P, K, LB, PM>(a, a, TileMR<Q, P, K, LB>::ctx(a, c), work, a.g, ts, PM == PM_COMPUTE ? &wbar : nullptr,
                                  it & 1u);
         __syncthreads();
     }
 }
 
-template <int Q, class P, int K, int PM>
+template <int Q, class P, int K, bool LB, int PM>
 __global__ void __launch_bounds__(CfgMR<Q>::NT, CfgMR<Q>::MINB) k_row_pass_mr(const KArgs<P> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint64_t wbar;
     TS<typename P::C> ts;
-    unsigned char *work = mr_setup<Q, P, K, PM>(a, TileMR<Q, P, K>::ctx(a, blockIdx.x), smem_raw, ts, true);
+    unsigned char *work = mr_setup<Q, P, K, LB, PM>(a, TileMR<Q, P, K, LB>::ctx(a, blockIdx.x), smem_raw, ts, true);
     if (PM == PM_COMPUTE && threadIdx.x == 0) {
         mbar_init(&wbar, 1);
         mbar_init_fence();
@@ -909,7 +977,7 @@ __global__ void __launch_bounds__(CfgMR<Q>::NT, CfgMR<Q>::MINB) k_row_pass_mr(co
     unsigned it = 0;
     for (int c = blockIdx.x; c < a.ncta; c += gridDim.x, ++it) {
         if constexpr (PM == PM_BUILD) ts.tb = a.ptab + (int64_t)c * a.ptab_cta;
-        row_pass_mr<Q, P, K, PM>(a, a, TileMR<Q, P, K>::ctx(a, c), work, a.f, ts, PM == PM_COMPUTE ? &wbar : nullptr,
+        row_pass_mr<Q, P, K, LB, PM>(a, a, TileMR<Q, P, K, LB>::ctx(a, c), work, a.f, ts, PM == PM_COMPUTE ? &wbar : nullptr,
                                  it & 1u);
         __syncthreads();
     }
@@ -983,10 +1051,10 @@ __device__ __forceinline__ int wait_count(const unsigned *ctr, unsigned target, 
     }
 }
 
-template <int Q, class P, int K>
+template <int Q, class P, int K, bool LB>
 __global__ void __launch_bounds__(CfgMR<Q>::NT, CfgMR<Q>::MINB) k_batch_mr(const BatchArgs<P> b)
 {
-    using TM = TileMR<Q, P, K>;
+    using TM = TileMR<Q, P, K, LB>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ int s_unit, s_job, s_skip;
     __shared__ uint64_t wbar;                                  // the units' input copies
@@ -1034,8 +1102,8 @@ __global__ void __launch_bounds__(CfgMR<Q>::NT, CfgMR<Q>::MINB) k_batch_mr(const
                 x.rc = a.rc;
                 x.lgp = __ffs(x.npr) - 1;
                 TS<typename P::C> ts{};
-                const bool used = jb.row ? row_pass_mr<Q, P, K, PM_COMPUTE>(a, b, x, smem_raw, b.f[jb.prob], ts, &wbar, wuse & 1u)
-                                         : col_pass_mr<Q, P, K, PM_COMPUTE>(a, b, x, smem_raw, b.g[jb.prob], ts, &wbar, wuse & 1u);
+                const bool used = jb.row ? row_pass_mr<Q, P, K, LB, PM_COMPUTE>(a, b, x, smem_raw, b.f[jb.prob], ts, &wbar, wuse & 1u)
+                                         : col_pass_mr<Q, P, K, LB, PM_COMPUTE>(a, b, x, smem_raw, b.g[jb.prob], ts, &wbar, wuse & 1u);
                 wuse += used ? 1u : 0u;
                 __syncthreads();
             }

@@ -13,6 +13,7 @@
 
 #include "../../include/bf.h"
 #include "bf_device.cuh"
+#include "bf_host.h"
 #include "bf_launch.h"
 
 // Every GPU that loads the library holds this array until the process exits.
@@ -72,7 +73,11 @@ __global__ void k_noalloc_tables(NaGeom g, int kdim, int L, int q, int kind, typ
         double f0 = 0.0, f1 = 0.0, f2 = 0.0;
         switch (kind) {
         case BF_PHASE_DOT: f0 = g.s * x; break;
-        case BF_PHASE_GENRADON: f0 = g.s * x; f1 = sin(2 * kPi * x); f2 = cos(2 * kPi * x); break;
+        case BF_PHASE_GENRADON: {
+            const double c = sqrt(fabs(g.s) / 3.0);
+            f0 = g.s * x; f1 = c * sin(2 * kPi * x); f2 = c * cos(2 * kPi * x);
+            break;
+        }
         case BF_PHASE_HYPRADON: f0 = g.s * x; f1 = x * x; break;
         default: f0 = g.s * sin(2 * kPi * (x + (kdim + 1) / 7.0)); break;
         }
@@ -167,12 +172,14 @@ bf_status run(int d, int L, int q, int kind, const bf_params *prm, const void *g
     const double sc = prm->phase_scale;
     const double sgn = sc > 0 ? 1.0 : (sc < 0 ? -1.0 : 0.0);
     if constexpr (P::is_f64) {
-        a.sc.s3 = sc / 3.0;
+        a.sc.c2 = 2.0 * std::fabs(sc) / 3.0;
         a.sc.sgn = sgn;
     } else {
-        a.sc.s3hi = (float)(sc / 3.0);
-        a.sc.s3lo = (float)(sc / 3.0 - (double)a.sc.s3hi);
+        const double c2 = 2.0 * std::fabs(sc) / 3.0;
+        a.sc.c2hi = (float)c2;
+        a.sc.c2lo = (float)(c2 - (double)a.sc.c2hi);
         a.sc.sgn = (float)sgn;
+        a.sc.mg = bfl::sqrt_grid(d, kind, prm);
     }
     a.ctab = nullptr;
     a.ctab_levels = -1;
@@ -183,37 +190,15 @@ bf_status run(int d, int L, int q, int kind, const bf_params *prm, const void *g
     a.g = static_cast<const typename P::C *>(g);
     a.f = static_cast<typename P::C *>(f);
 
-    // the default schedule of bf_plan_create: column passes of <= kmax levels (init first,
-    // switch last), then row passes (final last); in each run of levels the short pass
-    // (levels mod kmax) comes first
+    // the default schedule of bf_plan_create
     const int m = prm->switch_level < 0 ? L / 2 : prm->switch_level;
     const int kmax = prm->fuse_levels > 0 && prm->fuse_levels < fns->kmax ? prm->fuse_levels : fns->kmax;
     NaPass ps[kMaxPasses];
     int np = 0;
-    auto add = [&](int row, int l0, int k, int fl) {
-        const int64_t cta_pairs = npts < fns->np ? npts : fns->np;
-        int T = (int)(cta_pairs >> (d * k));
-        ps[np++] = NaPass{row, l0, k, fl, T < 1 ? 1 : T};
-    };
-    auto chunk = [&](int left, int total) {
-        const int rem = total % kmax;
-        if (rem && left == total) return rem;
-        return left < kmax ? left : kmax;
-    };
-    if (m == 0) {
-        add(0, 0, 0, bfk::F_INIT | bfk::F_SWITCH);
-    } else {
-        for (int l = 0; l < m;) {
-            const int k = chunk(m - l, m);
-            add(0, l, k, (l == 0 ? bfk::F_INIT : 0) | (l + k == m ? bfk::F_SWITCH : 0));
-            l += k;
-        }
-    }
-    for (int l = m; l < L;) {
-        const int k = chunk(L - l, L - m);
-        add(1, l, k, l + k == L ? bfk::F_FINAL : 0);
-        l += k;
-    }
+    a.corner = bfl::corner_of(d, q, m, prm, fns->lobatto, false);
+    bfl::each_pass(L, m, kmax, true, a.corner, [&](int row, int l0, int k, int fl) {
+        ps[np++] = NaPass{row, l0, k, fl, bfl::tiles_of(npts, fns->np, d, k)};
+    });
     void *buf[2] = {w0, w1};
     for (int i = 0; i < np; ++i) {
         a.l0 = ps[i].l0;
@@ -223,11 +208,7 @@ bf_status run(int d, int L, int q, int kind, const bf_params *prm, const void *g
         a.win = static_cast<const typename P::C *>(buf[i & 1]);
         a.wout = static_cast<typename P::C *>(buf[(i + 1) & 1]);
         const int64_t ctas = (npts >> (d * ps[i].k)) / ps[i].T;
-        size_t smem = (size_t)3 * ps[i].T * ((size_t)1 << (d * ps[i].k)) * r * sizeof(typename P::C);
-        if (ps[i].row && ps[i].k >= 1)   // cache of the parents' node features in the row kernels
-            smem += (size_t)ps[i].T * ((size_t)1 << (d * (ps[i].k - 1))) * r * (size_t)fns->tsize;
-        if (!ps[i].row)                  // geometry of a level's output pairs in the column kernels
-            smem += (size_t)ps[i].T * ((size_t)1 << (d * ps[i].k)) * (((size_t)fns->tsize + 16 + 15) / 16 * 16);
+        const size_t smem = fns->tile_smem(ps[i].row, ps[i].T, ps[i].k, 0);
         cudaError_t e = (ps[i].row ? fns->row : fns->col)(&a, (unsigned)ctas, (unsigned)nrhs, smem, s);
         if (e != cudaSuccess) return BF_ERR_CUDA;
     }
@@ -268,23 +249,9 @@ extern "C" bf_status bf_apply_noalloc(int d, int64_t N, int q, bf_phase_kind pha
     if (nrhs < 0 || nrhs > 65535) return BF_ERR_INVALID_ARG;
     const int prec = prm->precision;
     if (prec != BF_PREC_FP64) {   // |Phi| < 2^21 cycles for the mixed path's integer rounding
-        double b = 0.0, mx[3], my[3];
-        for (int k = 0; k < d; ++k) {
-            mx[k] = std::fmax(std::fabs(prm->x_lo[k]), std::fabs(prm->x_lo[k] + prm->x_w[k]));
-            my[k] = std::fmax(std::fabs(prm->y_lo[k]), std::fabs(prm->y_lo[k] + prm->y_w[k]));
-        }
-        if (phase == BF_PHASE_DOT || phase == BF_PHASE_GENRADON) {
-            double q2 = 0.0;
-            for (int k = 0; k < d; ++k) { b += mx[k] * my[k]; q2 += my[k] * my[k]; }
-            if (phase == BF_PHASE_GENRADON) b += std::sqrt(q2);
-        } else if (phase == BF_PHASE_HYPRADON) {
-            b = mx[0] * std::sqrt(my[0] * my[0] + my[1] * my[1] * mx[1] * mx[1]);
-        } else {
-            for (int k = 0; k < d; ++k) b += 1.0 + my[k] * my[k] / (k + 2.0);
-        }
-        if (std::fabs(prm->phase_scale) * b >= 2097152.0) return BF_ERR_UNSUPPORTED;
+        if (bfl::phase_bound(d, (int)phase, prm) >= 2097152.0) return BF_ERR_UNSUPPORTED;
     }
-    const bfl::PassFns *fns = bfl::get_fns(d, q, prec, (int)phase);
+    const bfl::PassFns *fns = bfl::get_fns(d, q, prec, (int)phase, prm->node_kind);
     if (!fns) return BF_ERR_UNSUPPORTED;
 
     // scratch needed: 2d tables of nent entries (32 B target, 16 B source) + 2 weight buffers

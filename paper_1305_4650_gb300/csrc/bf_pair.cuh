@@ -70,12 +70,16 @@ __device__ __forceinline__ float2 fround2(float2 x)
     return sub2(add2(x, M), M);
 }
 
-__device__ __forceinline__ df2 df_sqrt_u2(const df2 &x)
+// sqrt_frac of bf_device.cuh on both lanes
+__device__ __forceinline__ float2 sqrt_frac2(float2 h, float2 l, float2 sg)
 {
-    const float2 r = make_float2(rsqrtf(fmaxf(x.hi.x, 1e-30f)), rsqrtf(fmaxf(x.hi.y, 1e-30f)));
-    const float2 s = mul2(x.hi, r);
-    const float2 res = add2(fma2(neg2(s), s, x.hi), x.lo);
-    return {s, mul2(res, mul2(dup2(0.5f), r))};
+    const float2 M = dup2(12582912.0f);
+    const float2 q = add2(h, l);
+    const float2 r = mul2(sg, make_float2(rsqrt_approx(q.x), rsqrt_approx(q.y)));
+    const float2 s = mul2(q, r);
+    const float2 w = sub2(s, sub2(add2(s, M), M));
+    const float2 res = add2(fma2(neg2(s), s, h), l);
+    return fma2(dup2(0.5f), mul2(res, r), w);
 }
 
 __device__ __forceinline__ float2 df_frac2(const df2 &x) { return add2(sub2(x.hi, fround2(x.hi)), x.lo); }
@@ -88,12 +92,17 @@ __device__ __forceinline__ float2 df_mul_frac2(const df2 &x, const df2 &y)
     return fma2(x.hi, y.lo, fma2(x.lo, y.hi, f));
 }
 
-// the polynomial sincos of bf_device.cuh on both lanes
-__device__ __forceinline__ void sincos2pi2(float2 f, float2 &s, float2 &c)
+// quad_reduce and quad_sincos of bf_device.cuh on both lanes
+__device__ __forceinline__ void quad_reduce2(float2 a, float2 b, float2 &r, int &j0, int &j1)
 {
     const float2 M = dup2(12582912.0f);
-    const float2 t = fma2(dup2(4.0f), f, M);
-    const float2 r = fma2(dup2(-0.25f), sub2(t, M), f);
+    const float2 t = fma2(dup2(4.0f), add2(a, b), M);
+    j0 = __float_as_int(t.x);
+    j1 = __float_as_int(t.y);
+    r = add2(fma2(dup2(-0.25f), sub2(t, M), a), b);
+}
+__device__ __forceinline__ void quad_sincos2(float2 r, int q0, int q1, float2 &s, float2 &c)
+{
     const float2 u = mul2(r, r);
     float2 ps = fma2(u, dup2(SC_S3), dup2(SC_S2));
     ps = fma2(u, ps, dup2(SC_S1));
@@ -102,7 +111,6 @@ __device__ __forceinline__ void sincos2pi2(float2 f, float2 &s, float2 &c)
     float2 pc = fma2(u, dup2(SC_C3), dup2(SC_C2));
     pc = fma2(u, pc, dup2(SC_C1));
     const float2 cs = fma2(u, pc, dup2(1.0f));
-    const int q0 = __float_as_int(t.x), q1 = __float_as_int(t.y);
     const float s0 = (q0 & 1) ? cs.x : sn.x, c0 = (q0 & 1) ? sn.x : cs.x;
     const float s1 = (q1 & 1) ? cs.y : sn.y, c1 = (q1 & 1) ? sn.y : cs.y;
     s.x = __int_as_float(__float_as_int(s0) ^ ((q0 & 2) << 30));
@@ -117,19 +125,33 @@ template <class P, int D, int K> struct Ph2;
 template <bool F, int D, int K>
 struct Ph2<PMIXT<F>, D, K> {
     using PH = Ph<PMIXT<F>, D, K>;
+    using V = float2;   // two lanes
+    static __device__ __forceinline__ V dup(float a) { return dup2(a); }
     struct T { df2 x[D]; df2 A[D]; };
-    struct Part { float2 f; df2 q; };
+    struct Part { float2 f, h, l; };
 
     static __device__ __forceinline__ df2 pack(const df &a, const df &b) { return {make_float2(a.hi, b.hi), make_float2(a.lo, b.lo)}; }
 
     static __device__ __forceinline__ T dup(const typename PH::T &a) { return pair(a, a); }
     static __device__ __forceinline__ Part dup(const typename PH::Part &p)
     {
-        return Part{dup2(p.f), {dup2(p.q.hi), dup2(p.q.lo)}};
+        return Part{dup2(p.f), dup2(p.h), dup2(p.l)};
     }
     static __device__ __forceinline__ typename PH::Part lane0(const Part &p)
     {
-        return typename PH::Part{p.f.x, {p.q.hi.x, p.q.lo.x}};
+        return typename PH::Part{p.f.x, p.h.x, p.l.x};
+    }
+
+    // the target of lane 0
+    static __device__ __forceinline__ typename PH::T one(const T &t)
+    {
+        typename PH::T o;
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+            o.x[k] = {t.x[k].hi.x, t.x[k].lo.x};
+            o.A[k] = {t.A[k].hi.x, t.A[k].lo.x};
+        }
+        return o;
     }
 
     static __device__ __forceinline__ T pair(const typename PH::T &a, const typename PH::T &b)
@@ -144,44 +166,106 @@ struct Ph2<PMIXT<F>, D, K> {
     }
 
     // contribution of source coordinate k: entries e0 (lane 0) and e1 (lane 1)
-    static __device__ __forceinline__ Part part(const T &t, const MixSE &e0, const MixSE &e1, int k)
+    static __device__ __forceinline__ Part part(const KArgs<PMIXT<F>> &a, const T &t, const MixSE &e0, const MixSE &e1, int k)
     {
-        Part p{dup2(0.0f), {dup2(0.0f), dup2(0.0f)}};
+        return part_of(a, t.x[k], t.A[k], e0, e1, k == 0);
+    }
+    static __device__ __forceinline__ Part part_of(const KArgs<PMIXT<F>> &a, const df2 &x, const df2 &A, const MixSE &e0,
+                                                   const MixSE &e1, bool first)
+    {
+        Part p{dup2(0.0f), dup2(0.0f), dup2(0.0f)};
         const df2 y = {make_float2(e0.a.x, e1.a.x), make_float2(e0.a.y, e1.a.y)};
         const df2 y2 = {make_float2(e0.a.z, e1.a.z), make_float2(e0.a.w, e1.a.w)};
-        if constexpr (K == KIND_DOT) {
-            p.f = df_mul_frac2(t.x[k], y);
-        } else if constexpr (K == KIND_GENRADON) {
-            p.f = df_mul_frac2(t.x[k], y);
-            p.q = df_mul_u2(t.A[k], y2);
-        } else if constexpr (K == KIND_HYPRADON) {
-            p.q = (k == 0) ? y2 : df_mul_u2(t.A[1], y2);
-        } else {
-            p.q = df_add2(t.x[k], y);
+        if constexpr (K == KIND_DOT || K == KIND_GENRADON) p.f = df_mul_frac2(x, y);
+        if constexpr (K == KIND_SEPARABLE) p.f = df_frac2(df_add2(x, y));
+        if constexpr (PH::HAS_Q) {
+            const df2 v = df_mul_u2(A, y2);
+            p.h = sub2(add2(v.hi, dup2(a.sc.mg)), dup2(a.sc.mg));
+            p.l = add2(sub2(v.hi, p.h), v.lo);
+            p.l = add2(p.l, dup2(first ? 1e-30f : 0.0f));
         }
         return p;
     }
     static __device__ __forceinline__ Part add(const Part &u, const Part &v)
     {
-        df2 s;
-        if constexpr (K == KIND_GENRADON || K == KIND_HYPRADON)   // non-negative parts, larger first
-            s = fast_two_sum2(make_float2(fmaxf(u.q.hi.x, v.q.hi.x), fmaxf(u.q.hi.y, v.q.hi.y)),
-                              make_float2(fminf(u.q.hi.x, v.q.hi.x), fminf(u.q.hi.y, v.q.hi.y)));
-        else
-            s = two_sum2(u.q.hi, v.q.hi);
-        return Part{add2(u.f, v.f), {s.hi, add2(add2(u.q.lo, v.q.lo), s.lo)}};
-    }
-    static __device__ __forceinline__ float2 fin(const KArgs<PMIXT<F>> &a, const T &t, const Part &p)
-    {
-        if constexpr (K == KIND_DOT) {
-            return p.f;
-        } else if constexpr (K == KIND_GENRADON) {
-            return fma2(dup2(a.sc.sgn), df_frac2(df_sqrt_u2(p.q)), p.f);
-        } else if constexpr (K == KIND_HYPRADON) {
-            return df_mul_frac2(t.x[0], df_sqrt_u2(p.q));
-        } else {
-            return df_frac2(p.q);
+        Part p{dup2(0.0f), dup2(0.0f), dup2(0.0f)};
+        if constexpr (PH::HAS_F) p.f = add2(u.f, v.f);
+        if constexpr (PH::HAS_Q) {
+            p.h = add2(u.h, v.h);
+            p.l = add2(u.l, v.l);
         }
+        return p;
+    }
+    static __device__ __forceinline__ float2 sign(const KArgs<PMIXT<F>> &a, const T &t)
+    {
+        if constexpr (K == KIND_HYPRADON)
+            return make_float2(copysignf(1.0f, t.x[0].hi.x), copysignf(1.0f, t.x[0].hi.y));
+        else
+            return dup2(a.sc.sgn);
+    }
+    static __device__ __forceinline__ void fin2(float2 sg, const Part &p, float2 &ra, float2 &rb)
+    {
+        ra = rb = dup2(0.0f);
+        if constexpr (PH::HAS_F) ra = p.f;
+        if constexpr (PH::HAS_Q) (PH::HAS_F ? rb : ra) = sqrt_frac2(p.h, p.l, sg);
+    }
+    static __device__ __forceinline__ float2 fin(float2 sg, const Part &p)
+    {
+        float2 ra, rb;
+        fin2(sg, p, ra, rb);
+        return add2(ra, rb);
+    }
+};
+
+// FP64: the same interface on pairs of doubles (two scalar evaluations; nothing is paired in
+// the hardware), so that the d = 2 tile code serves both precisions
+template <int D, int K>
+struct Ph2<PF64, D, K> {
+    using PH = Ph<PF64, D, K>;
+    using V = double2;
+    struct T { V x[D]; V A[D]; };
+    struct Part { V f, q; };
+    static __device__ __forceinline__ V pack(double a, double b) { return make_double2(a, b); }
+    static __device__ __forceinline__ V dup(double a) { return make_double2(a, a); }
+    static __device__ __forceinline__ T dup(const typename PH::T &a)
+    {
+        T t;
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+            t.x[k] = dup(a.x[k]);
+            t.A[k] = dup(a.A[k]);
+        }
+        return t;
+    }
+    static __device__ __forceinline__ Part dup(const typename PH::Part &p) { return Part{dup(p.f), dup(p.q)}; }
+    static __device__ __forceinline__ typename PH::Part lane0(const Part &p) { return typename PH::Part{p.f.x, p.q.x}; }
+    static __device__ __forceinline__ typename PH::Part lane1(const Part &p) { return typename PH::Part{p.f.y, p.q.y}; }
+    static __device__ __forceinline__ typename PH::T one(const T &t)
+    {
+        typename PH::T o;
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+            o.x[k] = t.x[k].x;
+            o.A[k] = t.A[k].x;
+        }
+        return o;
+    }
+    static __device__ __forceinline__ Part part_of(const KArgs<PF64> &a, const V &x, const V &A, const PF64::SE &e0,
+                                                   const PF64::SE &e1, bool first)
+    {
+        const typename PH::Part p0 = PH::part_of(a, x.x, A.x, e0, first), p1 = PH::part_of(a, x.y, A.y, e1, first);
+        return Part{make_double2(p0.f, p1.f), make_double2(p0.q, p1.q)};
+    }
+    static __device__ __forceinline__ Part part(const KArgs<PF64> &a, const T &t, const PF64::SE &e0, const PF64::SE &e1, int k)
+    {
+        return part_of(a, t.x[k], t.A[k], e0, e1, k == 0);
+    }
+    static __device__ __forceinline__ Part add(const Part &u, const Part &v)
+    {
+        Part p{};
+        if constexpr (PH::HAS_F) p.f = make_double2(u.f.x + v.f.x, u.f.y + v.f.y);
+        if constexpr (PH::HAS_Q) p.q = make_double2(u.q.x + v.q.x, u.q.y + v.q.y);
+        return p;
     }
 };
 
@@ -190,13 +274,18 @@ template <class P, int D, int K>
 __device__ __forceinline__ void expphase_part2(const KArgs<P> &a, const typename Ph2<P, D, K>::T &t,
                                                const typename Ph2<P, D, K>::Part &pt, float2 &e0, float2 &e1)
 {
-    const float2 fr = Ph2<P, D, K>::fin(a, t, pt);
+    using PH2 = Ph2<P, D, K>;
     float2 s, c;
     if constexpr (P::sfu) {
+        const float2 fr = PH2::fin(PH2::sign(a, t), pt);
         sincos2pi_sfu(fr.x, s.x, c.x);
         sincos2pi_sfu(fr.y, s.y, c.y);
     } else {
-        sincos2pi2(fr, s, c);
+        float2 ra, rb, r;
+        int j0, j1;
+        PH2::fin2(PH2::sign(a, t), pt, ra, rb);
+        quad_reduce2(ra, rb, r, j0, j1);
+        quad_sincos2(r, j0, j1, s, c);
     }
     e0 = make_float2(c.x, s.x);
     e1 = make_float2(c.y, s.y);

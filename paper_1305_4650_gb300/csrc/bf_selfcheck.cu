@@ -164,21 +164,21 @@ __global__ void k_phase_rate(const bfk::KArgs<P> a, int L, int q, int iters, flo
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
             if constexpr (PAIRED) {
-                const typename PH2::Part hp = PH2::part(t2, s1[j], s1[j], 1);
+                const typename PH2::Part hp = PH2::part(a, t2, s1[j], s1[j], 1);
 #pragma unroll
                 for (int i = 0; i < 4; ++i) {
                     float2 e0, e1;
-                    bfk::expphase_part2<P, 2, K>(a, t2, PH2::add(PH2::part(t2, s0[i], s0[i], 0), hp), e0, e1);
+                    bfk::expphase_part2<P, 2, K>(a, t2, PH2::add(PH2::part(a, t2, s0[i], s0[i], 0), hp), e0, e1);
                     acc.x += e0.x + e1.x;
                     acc.y += e0.y + e1.y;
                 }
             } else {
 #pragma unroll
                 for (int u = 0; u < 2; ++u) {
-                    const typename PH::Part hp = PH::part(tg[u], s1[j], 1);
+                    const typename PH::Part hp = PH::part(a, tg[u], s1[j], 1);
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
-                        const float2 e = bfk::expphase_part<P, 2, K>(a, tg[u], PH::add(PH::part(tg[u], s0[i], 0), hp));
+                        const float2 e = bfk::expphase_part<P, 2, K>(a, tg[u], PH::add(PH::part(a, tg[u], s0[i], 0), hp));
                         acc.x += e.x;
                         acc.y += e.y;
                     }

@@ -277,14 +277,14 @@ __device__ __forceinline__ void switch_tc_body(const KArgs<P> &a)
             C ev[Q];
             const typename PH2::T tS2 = PH2::dup(tS);
             const typename P::SE e1 = sget<P, Q>(a, 1, l, cb[1], th);
-            const typename PH2::Part hp = PH2::part(tS2, e1, e1, 1);
+            const typename PH2::Part hp = PH2::part(a, tS2, e1, e1, 1);
 #pragma unroll
             for (int t0 = 0; t0 + 1 < Q; t0 += 2)
                 expphase_part2<P, D, K>(
-                    a, tS2, PH2::add(PH2::part(tS2, sget<P, Q>(a, 0, l, cb[0], t0), sget<P, Q>(a, 0, l, cb[0], t0 + 1), 0), hp),
+                    a, tS2, PH2::add(PH2::part(a, tS2, sget<P, Q>(a, 0, l, cb[0], t0), sget<P, Q>(a, 0, l, cb[0], t0 + 1), 0), hp),
                     ev[t0], ev[t0 + 1]);
             if constexpr (Q & 1)
-                ev[Q - 1] = expphase_part<P, D, K>(a, tS, PH::add(PH::part(tS, sget<P, Q>(a, 0, l, cb[0], Q - 1), 0),
+                ev[Q - 1] = expphase_part<P, D, K>(a, tS, PH::add(PH::part(a, tS, sget<P, Q>(a, 0, l, cb[0], Q - 1), 0),
                                                                  PH2::lane0(hp)));
             // row 2s takes (x, -y), row 2s + 1 takes (y, x) of every factor x + iy
             uint32_t h0[ST::NWS], l0[ST::NWS], h1[ST::NWS], l1[ST::NWS];
@@ -517,12 +517,12 @@ __global__ void __launch_bounds__(ColTC<Q>::NT) k_col_tc(const KArgs<P> a)
             const typename PH::T tA = tcenter<P, D, Q, K>(a, l + 1, Aa, ca);
             if (mod) {
                 const int c = rest / RR, tp = rest % RR;
-                const typename PH::Part pt = PH::add(PH::part(tA, sget<P, Q>(a, 0, l, 2 * cbq[0] + (c & 1), tp % Q), 0),
-                                                     PH::part(tA, sget<P, Q>(a, 1, l, 2 * cbq[1] + (c >> 1), tp / Q), 1));
+                const typename PH::Part pt = PH::add(PH::part(a, tA, sget<P, Q>(a, 0, l, 2 * cbq[0] + (c & 1), tp % Q), 0),
+                                                     PH::part(a, tA, sget<P, Q>(a, 1, l, 2 * cbq[1] + (c >> 1), tp / Q), 1));
                 PM[jt] = expphase_part<P, D, K>(a, tA, pt);
             } else {
-                const typename PH::Part pt = PH::add(PH::part(tA, sget<P, Q>(a, 0, l + 1, cbq[0], rest % Q), 0),
-                                                     PH::part(tA, sget<P, Q>(a, 1, l + 1, cbq[1], rest / Q), 1));
+                const typename PH::Part pt = PH::add(PH::part(a, tA, sget<P, Q>(a, 0, l + 1, cbq[0], rest % Q), 0),
+                                                     PH::part(a, tA, sget<P, Q>(a, 1, l + 1, cbq[1], rest / Q), 1));
                 PD[jt] = expphase_part<P, D, K>(a, tA, pt);
             }
         }
