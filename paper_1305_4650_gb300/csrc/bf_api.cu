@@ -62,7 +62,9 @@ struct bf_plan_s {
     std::vector<void *> pts_mem;
     std::vector<Pass> passes_pts;
     int mr_rc = 1;                 // right-hand sides per scratch chunk of the multi-RHS kernels
-    std::vector<Pass> passes_adj;  // schedule whose reverse is the adjoint (fits the row caches)
+    std::vector<Pass> passes_adj;  // schedule whose reverse is the single-RHS adjoint
+    std::vector<Pass> passes_mra;  // the same for the multi-RHS adjoint, for mra_nrhs right-hand sides
+    int mra_nrhs = 0, mra_rc = 0;
     const bfl::PassFns *fns = nullptr;
     int last_cuda = 0;
     cudaEvent_t busy_ev = nullptr;     // recorded after the last apply outside a stream capture
@@ -256,24 +258,6 @@ bf_status build_tables(bf_plan p)
 
 // shared memory of a forward single-RHS pass
 size_t fwd_smem(const bf_plan_s *p, const Pass &ps, bool tab = false) { return p->fns->tile_smem(ps.row, ps.T, ps.k, tab); }
-
-// shared memory of an adjoint pass: T tiles of 2^{dk} pairs, plus twice that as stage scratch
-size_t pass_smem(const bf_plan_s *p, const Pass &ps)
-{
-    return (size_t)3 * (size_t)ps.T * ((size_t)1 << (p->d * ps.k)) * (size_t)p->r * p->csize;
-}
-
-// the adjoint row pass caches children's and parents' node features (T (2^{dk} + 2^{d(k-1)}) boxes x r);
-// the adjoint column pass with the (unfactorised, d = 2) switch caches the features of every
-// (pair, node) of its tiles (T 2^{dk} pairs x r)
-size_t row_adj_cache_smem(const bf_plan_s *p, const Pass &ps)
-{
-    if (!ps.row && (ps.flags & bfk::F_SWITCH) && p->d == 2 && p->kind != BF_PHASE_DOT && p->kind != BF_PHASE_SEPARABLE)
-        return (size_t)ps.T * ((size_t)1 << (p->d * ps.k)) * (size_t)p->r * (size_t)p->fns->tsize;
-    if (!ps.row || ps.k < 1) return 0;
-    return (size_t)ps.T * (((size_t)1 << (p->d * ps.k)) + ((size_t)1 << (p->d * (ps.k - 1)))) * (size_t)p->r *
-           (size_t)p->fns->tsize;
-}
 
 // multi-RHS pass: nr right-hand sides of T 2^{dk} pairs, scratch for rc of them, a phase cache
 // of 5 r factors per pair, with the bank-conflict padding of bf_mr.cuh
@@ -521,17 +505,88 @@ bf_status run_adjoint(bf_plan p, const void *f, void *g, int nrhs, cudaStream_t 
         a.win = static_cast<const typename P::C *>(buf[(i + 1) & 1]);
         a.wout = static_cast<typename P::C *>(buf[i & 1]);
         const int64_t ctas = (p->npts >> (p->d * ps.k)) / ps.T;
-        const size_t smem = pass_smem(p, ps) + row_adj_cache_smem(p, ps);
+        const size_t smem = p->fns->adj_smem(ps.row, ps.T, ps.k);
         cudaError_t e = (ps.row ? p->fns->row_adj : p->fns->col_adj)(&a, (unsigned)ctas, (unsigned)nrhs, smem, s);
         if (e != cudaSuccess) return cuda_fail(p, e);
     }
     return BF_OK;
 }
 
-// the multi-RHS schedule serves nrhs >= 2 where it is compiled (mixed precisions, d = 2)
+// Multi-RHS adjoint (d = 2; FP64 for one right-hand side as well, where its pipe, not the
+// occupancy, is the bound): the transposed passes evaluate every phase factor once for up to mr_max
+// right-hand sides.  32 pairs per CTA (more items per stage) where two CTAs per SM still fit
+// and the grid keeps two CTAs per SM busy, else 16; the largest schedule that fits otherwise
+// (many nodes per box).
+bool schedule_adjoint_mr(bf_plan p, int nrhs)
+{
+    const int mx = p->fns->mr_max, nr = nrhs < mx ? nrhs : mx;
+    const int64_t ppr = p->fns->mr_nthreads / p->r;
+    auto fits = [&](const std::vector<Pass> &sc, int rc, size_t limit) {
+        for (const Pass &ps : sc)
+            if (mr_smem(p, ps, nr, rc) > limit) return false;
+        return true;
+    };
+    auto chunk = [&](int64_t np) {   // right-hand sides per scratch chunk: an item for every thread
+        const int64_t rc = p->fns->mr_nthreads / (np * p->q);
+        return (int)(rc < 1 ? 1 : (rc > nr ? nr : rc));
+    };
+    const int kmax = p->prm.fuse_levels == 1 ? 1 : 2;
+    std::vector<Pass> &sc = p->passes_mra;
+    int &rc = p->mra_rc;
+    rc = 0;
+    bool ok = false;
+    if (p->prec != BF_PREC_FP64 && p->npts >= 2 * ppr * 304) {
+        sc = schedule(p, kmax, 2 * ppr, true, p->corner);
+        rc = chunk(2 * ppr);
+        ok = fits(sc, rc, 112 * 1024);
+    }
+    for (int k = kmax; k >= 1 && !ok; --k)
+        for (int64_t np = ppr; np >= 4 && !ok; np /= 2) {
+            sc = schedule(p, k, np, true, p->corner);
+            for (rc = chunk(np); rc >= 1 && !ok; --rc) ok = fits(sc, rc, 227 * 1024);
+            ++rc;
+        }
+    return ok;
+}
+
+template <class P>
+bf_status run_adjoint_mr(bf_plan p, const void *f, void *g, int nrhs, cudaStream_t s)
+{
+    if (p->mra_nrhs != nrhs) {
+        p->mra_nrhs = 0;
+        if (!schedule_adjoint_mr(p, nrhs)) return BF_ERR_UNSUPPORTED;
+        p->mra_nrhs = nrhs;
+    }
+    const std::vector<Pass> &sc = p->passes_mra;
+    const int mx = p->fns->mr_max, nr = nrhs < mx ? nrhs : mx, rc = p->mra_rc;
+    bfk::KArgs<P> a;
+    fill_args<P>(p, a);
+    a.fadj = static_cast<const typename P::C *>(f);
+    a.gadj = static_cast<typename P::C *>(g);
+    a.nrhs = nrhs;
+    a.rc = rc;
+    void *buf[2] = {p->w0, p->w1};
+    for (int i = (int)sc.size() - 1; i >= 0; --i) {
+        const Pass &ps = sc[i];
+        a.l0 = ps.l0;
+        a.k = ps.k;
+        a.flags = ps.flags;
+        a.T = ps.T;
+        a.win = static_cast<const typename P::C *>(buf[(i + 1) & 1]);
+        a.wout = static_cast<typename P::C *>(buf[i & 1]);
+        const int64_t ctas = (p->npts >> (p->d * ps.k)) / ps.T;
+        a.ncta = (int)ctas;
+        cudaError_t e = (ps.row ? p->fns->row_mr_adj : p->fns->col_mr_adj)(&a, (unsigned)ctas, (unsigned)((nrhs + mx - 1) / mx),
+                                                                           mr_smem(p, ps, nr, rc), s);
+        if (e != cudaSuccess) return cuda_fail(p, e);
+    }
+    return BF_OK;
+}
+
+// the multi-RHS schedule serves nrhs >= 2 where it is compiled (d = 2)
 bool use_mr(const bf_plan_s *p, int nrhs)
 {
-    return (nrhs >= 2 || p->ptab) && p->prec != BF_PREC_FP64 && !p->passes_mr.empty() && !p->points;
+    return (nrhs >= 2 || p->ptab) && !p->passes_mr.empty() && !p->points;
 }
 
 // ------------------------------------------------------------ point sets
@@ -1177,16 +1232,16 @@ bf_status bf_plan_create(int d, int64_t N, int q, bf_phase_kind phase, const bf_
         }
         if (!fits) p->passes_mr.clear();
     }
-    // the adjoint's row passes also hold target-feature caches: fuse fewer levels, then put
-    // fewer tiles in a CTA, until every pass fits the shared memory of one CTA
-    {
+    // the single-RHS adjoint's row passes also hold products or feature caches: fuse fewer
+    // levels, then put fewer tiles in a CTA, until every pass fits the shared memory of one CTA
+    if (p->fns->col_adj) {
         bool fits = false;
         for (int ka = p->kc; ka >= 1 && !fits; --ka) {
             for (int64_t np = p->fns->np; np >= (1LL << (d * ka)) && !fits; np >>= d) {
-                p->passes_adj = schedule(p, ka, np);
+                p->passes_adj = schedule(p, ka, np, d == 2, p->corner);
                 fits = true;
                 for (const Pass &ps : p->passes_adj)
-                    if (pass_smem(p, ps) + row_adj_cache_smem(p, ps) > 227 * 1024) fits = false;
+                    if (p->fns->adj_smem(ps.row, ps.T, ps.k) > 227 * 1024) fits = false;
             }
         }
     }
@@ -1307,7 +1362,8 @@ bf_status bf_apply(bf_plan p, const void *g, void *f, int nrhs, void *stream)
         else st = run_points<bfk::PMIX>(p, g, f, nrhs, s);
     } else {
         const int n = (int)schedule_for(p, nrhs).size();
-        if (p->prec == BF_PREC_FP64) st = run_forward<bfk::PF64>(p, g, f, nrhs, s, 0, n);
+        if (p->prec == BF_PREC_FP64)
+            st = use_mr(p, nrhs) ? run_forward_mr<bfk::PF64>(p, g, f, nrhs, s, 0, n) : run_forward<bfk::PF64>(p, g, f, nrhs, s, 0, n);
         else if (use_mr(p, nrhs))
             st = p->prec == BF_PREC_MIXED_SFU ? run_forward_mr<bfk::PMIXF>(p, g, f, nrhs, s, 0, n)
                                               : run_forward_mr<bfk::PMIX>(p, g, f, nrhs, s, 0, n);
@@ -1341,7 +1397,9 @@ bf_status bf_apply_shard(bf_plan p, const void *g, void *f, int nrhs, int shard_
         sc.push_back(Pass{last.row, last.l0 + last.k - 1, 1, last.flags, (int)(npr >> p->d)});
     }
     const int n = (int)sc.size();
-    if (p->prec == BF_PREC_FP64) st = run_forward<bfk::PF64>(p, g, f, nrhs, s, 0, n, shard_g, shard_r, &sc);
+    if (p->prec == BF_PREC_FP64)
+        st = use_mr(p, nrhs) ? run_forward_mr<bfk::PF64>(p, g, f, nrhs, s, 0, n, shard_g, shard_r, &sc)
+                             : run_forward<bfk::PF64>(p, g, f, nrhs, s, 0, n, shard_g, shard_r, &sc);
     else if (use_mr(p, nrhs))
         st = p->prec == BF_PREC_MIXED_SFU ? run_forward_mr<bfk::PMIXF>(p, g, f, nrhs, s, 0, n, shard_g, shard_r, &sc)
                                           : run_forward_mr<bfk::PMIX>(p, g, f, nrhs, s, 0, n, shard_g, shard_r, &sc);
@@ -1469,7 +1527,8 @@ bf_status bf_apply_pass(bf_plan p, int i, const void *g, void *f, int nrhs, void
     bool capturing = false;
     bf_status st = stream_guard(p, s, &capturing);
     if (st != BF_OK) return st;
-    if (p->prec == BF_PREC_FP64) st = run_forward<bfk::PF64>(p, g, f, nrhs, s, i, i + 1);
+    if (p->prec == BF_PREC_FP64)
+        st = use_mr(p, nrhs) ? run_forward_mr<bfk::PF64>(p, g, f, nrhs, s, i, i + 1) : run_forward<bfk::PF64>(p, g, f, nrhs, s, i, i + 1);
     else if (use_mr(p, nrhs))
         st = p->prec == BF_PREC_MIXED_SFU ? run_forward_mr<bfk::PMIXF>(p, g, f, nrhs, s, i, i + 1)
                                           : run_forward_mr<bfk::PMIX>(p, g, f, nrhs, s, i, i + 1);
@@ -1506,7 +1565,11 @@ bf_status bf_apply_adjoint(bf_plan p, const void *f, void *g, int nrhs, void *st
     bool capturing = false;
     bf_status st = stream_guard(p, s, &capturing);
     if (st != BF_OK) return st;
-    if (p->prec == BF_PREC_FP64) st = run_adjoint<bfk::PF64>(p, f, g, nrhs, s);
+    if (p->d == 2 && (nrhs > 1 || p->prec == BF_PREC_FP64)) {
+        if (p->prec == BF_PREC_FP64) st = run_adjoint_mr<bfk::PF64>(p, f, g, nrhs, s);
+        else if (p->prec == BF_PREC_MIXED_SFU) st = run_adjoint_mr<bfk::PMIXF>(p, f, g, nrhs, s);
+        else st = run_adjoint_mr<bfk::PMIX>(p, f, g, nrhs, s);
+    } else if (p->prec == BF_PREC_FP64) st = run_adjoint<bfk::PF64>(p, f, g, nrhs, s);   // d = 3
     else if (p->prec == BF_PREC_MIXED_SFU) st = run_adjoint<bfk::PMIXF>(p, f, g, nrhs, s);
     else st = run_adjoint<bfk::PMIX>(p, f, g, nrhs, s);
     stream_mark(p, s, capturing);

@@ -200,12 +200,15 @@ __device__ __forceinline__ void sincos2pi_sfu(float f, float &s, float &c)
 
 // the sincos above for a phase a + b given as two numbers: r keeps the rounding error of a
 // number of at most 1/8, not of a + b; the low two bits of j hold the quadrant
+// (TWO = false: b is zero)
+template <bool TWO>
 __device__ __forceinline__ void quad_reduce(float a, float b, float &r, int &j)
 {
     const float M = 12582912.0f;
-    const float t = __fmaf_rn(4.0f, __fadd_rn(a, b), M);
+    const float t = __fmaf_rn(4.0f, TWO ? __fadd_rn(a, b) : a, M);
     j = __float_as_int(t);
-    r = __fadd_rn(__fmaf_rn(-0.25f, __fsub_rn(t, M), a), b);
+    r = __fmaf_rn(-0.25f, __fsub_rn(t, M), a);
+    if (TWO) r = __fadd_rn(r, b);
 }
 __device__ __forceinline__ void quad_sincos(float r, int q, float &s, float &c)
 {
@@ -413,9 +416,11 @@ struct Ph<PMIXT<F>, D, K> {
     // h + l: a term of the sum of squares under the root, h a multiple of a power of two G
     // (quant) such that the sum of the parts' h, below 2^22 G, is exact: adding two terms takes
     // two additions instead of an exact sum of double-floats.  Loops hoist the
-    // parts of the source coordinates that do not change.
+    // parts of the source coordinates that do not change.  g: at d = 2 the second linear part of
+    // a kind without a root, not added to the first (fin2), so that their sum is never rounded.
     static constexpr bool HAS_F = K != KIND_HYPRADON, HAS_Q = K == KIND_GENRADON || K == KIND_HYPRADON;
-    struct Part { float f, h, l; };
+    static constexpr bool PAIR_F = !HAS_Q && D == 2;
+    struct Part { float f, h, l, g; };
     static constexpr int NCMP = (HAS_F ? 1 : 0) + (HAS_Q ? 2 : 0);
     // fn(component, its index) for the components that this kind uses
     template <class PT, class Fn>
@@ -438,7 +443,7 @@ struct Ph<PMIXT<F>, D, K> {
     // the part of one source coordinate from the target's features x and A of that coordinate
     static __device__ __forceinline__ Part part_of(const KArgs<PMIXT<F>> &a, const df &x, const df &A, const MixSE &e, bool first)
     {
-        Part p{0.0f, 0.0f, 0.0f};
+        Part p{0.0f, 0.0f, 0.0f, 0.0f};
         if constexpr (K == KIND_DOT || K == KIND_GENRADON) p.f = df_mul_frac(x, hi(e.a));
         if constexpr (K == KIND_SEPARABLE) p.f = df_frac(df_add(x, hi(e.a)));
         if constexpr (HAS_Q) quant(a, df_mul_u(A, lo(e.a)), first, p);
@@ -450,8 +455,13 @@ struct Ph<PMIXT<F>, D, K> {
     }
     static __device__ __forceinline__ Part add(const Part &u, const Part &v)
     {
-        Part p{0.0f, 0.0f, 0.0f};
-        if constexpr (HAS_F) p.f = __fadd_rn(u.f, v.f);
+        Part p{0.0f, 0.0f, 0.0f, 0.0f};
+        if constexpr (PAIR_F) {
+            p.f = u.f;
+            p.g = v.f;
+        } else if constexpr (HAS_F) {
+            p.f = __fadd_rn(u.f, v.f);
+        }
         if constexpr (HAS_Q) {
             p.h = __fadd_rn(u.h, v.h);
             p.l = __fadd_rn(u.l, v.l);
@@ -466,11 +476,13 @@ struct Ph<PMIXT<F>, D, K> {
         else
             return a.sc.sgn;
     }
-    // Phi minus an integer as two numbers a + b (quad_reduce)
+    // Phi minus an integer as two numbers a + b (quad_reduce; TWO: b may be non-zero)
+    static constexpr bool TWO = PAIR_F || (HAS_F && HAS_Q);
     static __device__ __forceinline__ void fin2(float sg, const Part &p, float &ra, float &rb)
     {
         ra = rb = 0.0f;
         if constexpr (HAS_F) ra = p.f;
+        if constexpr (PAIR_F) rb = p.g;
         if constexpr (HAS_Q) (HAS_F ? rb : ra) = sqrt_frac(p.h, p.l, sg);
     }
     static __device__ __forceinline__ float fin(float sg, const Part &p)
@@ -612,7 +624,7 @@ __device__ __forceinline__ typename P::C expphase_part(const KArgs<P> &a, const 
         float ra, rb, r;
         int j;
         PH::fin2(PH::sign(a, t), pt, ra, rb);
-        quad_reduce(ra, rb, r, j);
+        quad_reduce<PH::TWO>(ra, rb, r, j);
         quad_sincos(r, j, sn, cs);
     }
     typename P::C e;
@@ -725,14 +737,18 @@ template <int D, int Q, class P>
 struct Cfg {
     static constexpr int RR = ipow(Q, D);
     static constexpr int KMAX = kmax_for(D, RR, (int)sizeof(typename P::C), Q);
-    static constexpr int NP = 1 << (D * KMAX);    // pairs per CTA
-    static constexpr int NT = NP * Q;             // threads per CTA
-    static constexpr int MINB = (640 / NT) < 1 ? 1 : ((640 / NT) > 8 ? 8 : 640 / NT);
-    // the mixed-precision column pass at d = 2, q = 5 runs 3 CTAs per SM (64 registers, some
-    // spills): measured 4.5% faster on its dominant pass and 9% on the init pass than 2 CTAs
-    static constexpr int MINB_COL = (D == 2 && Q == 5 && !P::is_f64) ? 3 : MINB;
+    static constexpr bool SMALL = P::is_f64 && D == 2;   // two tiles of 16 pairs: 32 q threads are whole warps
+    static constexpr int NP = SMALL ? 32 : 1 << (D * KMAX);   // pairs per CTA
+    static constexpr int NT = NP * Q;                         // threads per CTA
+    static constexpr int per_sm(int threads) { return threads / NT < 1 ? 1 : (threads / NT > 8 ? 8 : threads / NT); }
+    // CTAs per SM that the register budget is cut for.  The d = 2 mixed-precision column passes
+    // run 30 warps per SM (64 registers; 3 CTAs at q = 5), the row passes, whose stage B holds
+    // 4 q complex numbers, 30 warps for q <= 4 and 20 beyond; FP64 needs few warps.
+    static constexpr int MINB = SMALL ? 3 : per_sm(640);
+    static constexpr int MINB_COL = D == 2 && !P::is_f64 ? per_sm(960) : MINB;
+    static constexpr int MINB_ROW = D == 2 && !P::is_f64 && Q <= 4 ? per_sm(960) : MINB;
     // the column pass reading a phase table (d = 2: one more CTA per SM than evaluating)
-    static constexpr int MINB_TAB = D == 2 ? MINB + 1 : MINB;
+    static constexpr int MINB_TAB = D == 2 ? per_sm(640) + 1 : MINB;
 };
 
 template <int D, int Q, class P, int K>
@@ -840,7 +856,7 @@ struct Tile {
             } else {
                 float ra, rb;
                 PH::fin2(sg, pt, ra, rb);
-                quad_reduce(ra, rb, r, j);
+                quad_reduce<PH::TWO>(ra, rb, r, j);
                 if constexpr (PM == PM_BUILD) __stcs(q, tab_pack(r, j));
             }
             C e;
@@ -892,7 +908,7 @@ struct Tile {
             } else {
                 float2 ra, rb;
                 Ph2<P, D, K>::fin2(sg, pt, ra, rb);
-                quad_reduce2(ra, rb, r, j0, j1);
+                quad_reduce2<PH::TWO>(ra, rb, r, j0, j1);
                 if constexpr (PM == PM_BUILD) {
                     __stcs(q0, tab_pack(r.x, j0));
                     if (q1) __stcs(q1, tab_pack(r.y, j1));
@@ -1754,44 +1770,7 @@ struct Tile {
                 const typename PH::T tA = tcenter<P, D, Q, K>(a, l + 1, (Apg << D) + alpha, ca);
                 const typename PH::Part p0 = PH::part(a, tA, e0, 0);
                 const C *si = S + ((tau * nblk + beta) * NC + alpha) * QD1 * 2 * Q + c0 * Q + s0;   // [t_{>=1}] stride 2Q
-                if constexpr (D == 2) {
-                    const int c1 = (c >> 1) & 1;
-                    C v[Q];
-#pragma unroll
-                    for (int s1 = 0; s1 < Q; ++s1) v[s1] = czero<C>();
-#pragma unroll
-                    for (int t1 = 0; t1 < Q; ++t1) {
-                        const C zz = si[t1 * 2 * Q];
-#pragma unroll
-                        for (int s1 = 0; s1 < Q; ++s1) cfma2(v[s1], a.M2[c1][t1][s1], zz);
-                    }
-                    if constexpr (!P::is_f64) {
-                        // phases two at a time: lanes s_1 and s_1 + 1 (the last one alone for odd q)
-                        using PH2 = Ph2<P, D, K>;
-                        const typename PH2::T tA2 = PH2::dup(tA);
-                        const typename PH2::Part p02 = PH2::dup(p0);
-#pragma unroll
-                        for (int s1 = 0; s1 + 1 < Q; s1 += 2) {
-                            float2 E0, E1;
-                            expphase_part2<P, D, K>(a, tA2,
-                                                    PH2::add(p02, PH2::part(a, tA2, sget<P, Q>(a, 1, l, cb[1], s1),
-                                                                            sget<P, Q>(a, 1, l, cb[1], s1 + 1), 1)),
-                                                    E0, E1);
-                            acc[s1] = cadd(acc[s1], cjmul(E0, v[s1]));
-                            acc[s1 + 1] = cadd(acc[s1 + 1], cjmul(E1, v[s1 + 1]));
-                        }
-                        if constexpr (Q & 1) {
-                            const C e = expphase_part<P, D, K>(a, tA, PH::add(p0, PH::part(a, tA, sget<P, Q>(a, 1, l, cb[1], Q - 1), 1)));
-                            acc[Q - 1] = cadd(acc[Q - 1], cjmul(e, v[Q - 1]));
-                        }
-                    } else {
-#pragma unroll
-                        for (int s1 = 0; s1 < Q; ++s1) {
-                            const C e = expphase_part<P, D, K>(a, tA, PH::add(p0, PH::part(a, tA, sget<P, Q>(a, 1, l, cb[1], s1), 1)));
-                            acc[s1] = cadd(acc[s1], cjmul(e, v[s1]));
-                        }
-                    }
-                } else {
+                {
                     const int c1 = (c >> 1) & 1, c2 = (c >> 2) & 1;
                     C w[Q * Q];   // [t1][s2]
 #pragma unroll
@@ -1877,16 +1856,7 @@ struct Tile {
                 const int alpha = al | (ahi << (D - 1));
                 const typename PH::T *tn = TC + (tau * nb1 + (int)((digit_rev<D>(beta & (nb0 - 1), i) << D) + alpha)) * RR;
                 const C *wi = Wt + tau * n * RR + (base + (alpha << (D * i))) * RR;
-                if constexpr (D == 2) {
-                    const int a0 = alpha & 1;
-#pragma unroll
-                    for (int s0 = 0; s0 < Q; ++s0) {
-                        const C e = expphase<P, D, K>(a, tn[s0 + Q * sq], sc);
-                        const C u = cjmul(e, wi[s0 + Q * sq]);
-#pragma unroll
-                        for (int t0 = 0; t0 < Q; ++t0) cfma2(acc[t0], a.M2[a0][t0][s0], u);
-                    }
-                } else {
+                {
                     const int a0 = alpha & 1, a1 = (alpha >> 1) & 1;
 #pragma unroll 1
                     for (int s1 = 0; s1 < Q; ++s1) {
@@ -1958,26 +1928,12 @@ struct Tile {
     }
 
     // ---- adjoint of the switch at level l: u(t) = sum_s e^{-2pi i Phi(x_s^A, y_t^B)} v(s);
-    // items (tau, slot, t_{>=1}), the q values of t_0 accumulated together.  For d = 2 the
-    // target features of every (pair, s) are computed once into TC (the q^{d-1} items of a
-    // pair share them); the mixed precision evaluates the phases of t_0, t_0 + 1 in pairs.
-    static __device__ void switch_adj(const KArgs<P> &a, C *Wt, C *S, typename PH::T *TC, int l)
+    // items (tau, slot, t_{>=1}), the q values of t_0 accumulated together; the mixed precision
+    // evaluates the phases of t_0, t_0 + 1 in pairs.
+    static __device__ void switch_adj(const KArgs<P> &a, C *Wt, C *S, int l)
     {
         const int k = a.k, n = 1 << (D * k);
         const int L = a.L;
-        if constexpr (D == 2) {
-            for (int j = threadIdx.x; j < a.T * n * RR; j += blockDim.x) {
-                const int s = j % RR, pr = j / RR;
-                const int sl = pr & (n - 1), tau = pr >> (D * k);
-                uint32_t Ap, Bstar;
-                tile_of(a, tau, Ap, Bstar);
-                int ca[DMAX];
-                morton_decode<D>((Ap << (D * k)) + digit_rev<D>(sl, k), l, ca);
-                const int sk[DMAX] = {s % Q, s / Q, 0};
-                TC[j] = tpoint<P, D, Q, K>(a, l, ca, sk);
-            }
-            __syncthreads();
-        }
         for (int it = threadIdx.x; it < a.T * n * QD1; it += blockDim.x) {
             const int th = it % QD1;
             const int sl = (it / QD1) & (n - 1);
@@ -2002,23 +1958,12 @@ struct Tile {
 #pragma unroll
             for (int t0 = 0; t0 < Q; ++t0) acc[t0] = czero<C>();
             const C *v = Wt + (tau * n + sl) * RR;
-            const typename PH::T *tc = TC + (tau * n + sl) * RR;
-            // d = 2: q targets per iteration of the outer loop (more independent work per iteration)
-            constexpr int SI = D == 2 ? Q : 1;
 #pragma unroll 1
-            for (int s1 = 0; s1 < RR; s1 += SI)
+            for (int s = 0; s < RR; ++s) {
+                int sk[DMAX], ss = s;
 #pragma unroll
-            for (int s0 = 0; s0 < SI; ++s0) {
-                const int s = s1 + s0;
-                typename PH::T tS;
-                if constexpr (D == 2) {
-                    tS = tc[s];
-                } else {
-                    int sk[DMAX], ss = s;
-#pragma unroll
-                    for (int j = 0; j < D; ++j) { sk[j] = ss % Q; ss /= Q; }
-                    tS = tpoint<P, D, Q, K>(a, l, ca, sk);
-                }
+                for (int j = 0; j < D; ++j) { sk[j] = ss % Q; ss /= Q; }
+                const typename PH::T tS = tpoint<P, D, Q, K>(a, l, ca, sk);
                 const C vs = v[s];
                 if constexpr (!P::is_f64) {
                     using PH2 = Ph2<P, D, K>;
@@ -2138,6 +2083,41 @@ struct Tile {
         }
     }
 
+    // ---- adjoint pass bodies (d = 3)
+    static __device__ __forceinline__ void col_pass_adj(const KArgs<P> &a, unsigned char *smem)
+    {
+        C *Wt = reinterpret_cast<C *>(smem);
+        C *S = Wt + a.T * (1 << (D * a.k)) * RR;
+        const int rhs = blockIdx.y;
+        load_strided(a, Wt, rhs);
+        __syncthreads();
+        if (a.flags & F_SWITCH) {
+            if constexpr (K == KIND_DOT || K == KIND_SEPARABLE)
+                switch_sep<true>(a, Wt, S, a.l0 + a.k);
+            else
+                switch_adj(a, Wt, S, a.l0 + a.k);
+        }
+        for (int i = a.k - 1; i >= 0; --i) col_level_adj(a, Wt, S, a.l0 + i, i);
+        if (a.flags & F_INIT)
+            init_adj(a, Wt, rhs);
+        else
+            store_contig(a, Wt, rhs);
+    }
+    static __device__ __forceinline__ void row_pass_adj(const KArgs<P> &a, unsigned char *smem)
+    {
+        C *Wt = reinterpret_cast<C *>(smem);
+        C *S = Wt + a.T * (1 << (D * a.k)) * RR;
+        typename PH::T *TC = reinterpret_cast<typename PH::T *>(S + 2 * a.T * (1 << (D * a.k)) * RR);
+        const int rhs = blockIdx.y;
+        if (a.flags & F_FINAL)
+            final_adj(a, Wt, rhs);
+        else
+            load_strided(a, Wt, rhs);
+        __syncthreads();
+        for (int i = a.k - 1; i >= 0; --i) row_level_adj(a, Wt, S, TC, a.l0 + i, i);
+        store_contig(a, Wt, rhs);
+    }
+
     // ---- adjoint pass input: the forward pass's outputs (strided pairs) into digit-reversed slots
     static __device__ __forceinline__ void load_strided(const KArgs<P> &a, C *Wt, int rhs)
     {
@@ -2231,7 +2211,7 @@ __global__ void __launch_bounds__(Cfg<D, Q, P>::NT, PM == PM_TABLE ? Cfg<D, Q, P
 
 // k row merges + optional final evaluation (l0 + k = L)
 template <int D, int Q, class P, int K, bool LB, int PM = PM_COMPUTE>
-__global__ void __launch_bounds__(Cfg<D, Q, P>::NT, Cfg<D, Q, P>::MINB) k_row_pass(const KArgs<P> a)
+__global__ void __launch_bounds__(Cfg<D, Q, P>::NT, Cfg<D, Q, P>::MINB_ROW) k_row_pass(const KArgs<P> a)
 {
     static_assert(PM == PM_COMPUTE || !P::is_f64, "phase tables: mixed precisions");
     using TL = typename TileOf<D, Q, P, K, LB>::type;
@@ -2249,49 +2229,19 @@ __global__ void __launch_bounds__(Cfg<D, Q, P>::NT, Cfg<D, Q, P>::MINB) k_row_pa
 
 // adjoint of a column pass: optional switch^H at level l0 + k, k column levels in
 // reverse, optional init^H (writes the source values)
-template <int D, int Q, class P, int K>
+template <int D, int Q, class P, int K, bool LB>
 __global__ void __launch_bounds__(Cfg<D, Q, P>::NT, Cfg<D, Q, P>::MINB) k_col_pass_adj(const KArgs<P> a)
 {
-    using C = typename P::C;
-    using TL = Tile<D, Q, P, K>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *Wt = reinterpret_cast<C *>(smem_raw);
-    C *S = Wt + a.T * (1 << (D * a.k)) * TL::RR;
-    typename TL::PH::T *TC = reinterpret_cast<typename TL::PH::T *>(S + 2 * a.T * (1 << (D * a.k)) * TL::RR);
-    const int rhs = blockIdx.y;
-    TL::load_strided(a, Wt, rhs);
-    __syncthreads();
-    if (a.flags & F_SWITCH) {
-        if constexpr (K == KIND_DOT || K == KIND_SEPARABLE)
-            TL::template switch_sep<true>(a, Wt, S, a.l0 + a.k);
-        else
-            TL::switch_adj(a, Wt, S, TC, a.l0 + a.k);
-    }
-    for (int i = a.k - 1; i >= 0; --i) TL::col_level_adj(a, Wt, S, a.l0 + i, i);
-    if (a.flags & F_INIT)
-        TL::init_adj(a, Wt, rhs);
-    else
-        TL::store_contig(a, Wt, rhs);
+    TileOf<D, Q, P, K, LB>::type::col_pass_adj(a, smem_raw);
 }
 
 // adjoint of a row pass: optional final^H (reads the target values), k row levels in reverse
-template <int D, int Q, class P, int K>
+template <int D, int Q, class P, int K, bool LB>
 __global__ void __launch_bounds__(Cfg<D, Q, P>::NT, Cfg<D, Q, P>::MINB) k_row_pass_adj(const KArgs<P> a)
 {
-    using C = typename P::C;
-    using TL = Tile<D, Q, P, K>;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    C *Wt = reinterpret_cast<C *>(smem_raw);
-    C *S = Wt + a.T * (1 << (D * a.k)) * TL::RR;
-    const int rhs = blockIdx.y;
-    typename TL::PH::T *TC = reinterpret_cast<typename TL::PH::T *>(S + 2 * a.T * (1 << (D * a.k)) * TL::RR);
-    if (a.flags & F_FINAL)
-        TL::final_adj(a, Wt, rhs);
-    else
-        TL::load_strided(a, Wt, rhs);
-    __syncthreads();
-    for (int i = a.k - 1; i >= 0; --i) TL::row_level_adj(a, Wt, S, TC, a.l0 + i, i);
-    TL::store_contig(a, Wt, rhs);
+    TileOf<D, Q, P, K, LB>::type::row_pass_adj(a, smem_raw);
 }
 
 }  // namespace bfk

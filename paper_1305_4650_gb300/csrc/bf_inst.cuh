@@ -29,13 +29,23 @@ inline cudaError_t prepare(K kern, size_t smem, size_t *granted)
     return cudaSuccess;
 }
 
+// threads of a single-RHS pass: q per pair at d = 2 (at least four pairs), the compiled number at d = 3
+template <int D, int Q, class P>
+unsigned tile_threads(int T, int k)
+{
+    if constexpr (D == 3) return bfk::Cfg<D, Q, P>::NT;
+    const int np = T << (D * k);
+    return (unsigned)((np < 4 ? 4 : np) * Q);
+}
+
 template <int D, int Q, class P, int K, bool LB, int PM = bfk::PM_COMPUTE>
 cudaError_t launch_col(const void *kargs, unsigned gx, unsigned gy, size_t smem, cudaStream_t s)
 {
     static size_t granted[64] = {0};
     cudaError_t e = prepare(bfk::k_col_pass<D, Q, P, K, LB, PM>, smem, granted);
     if (e != cudaSuccess) return e;
-    bfk::k_col_pass<D, Q, P, K, LB, PM><<<dim3(gx, gy), bfk::Cfg<D, Q, P>::NT, smem, s>>>(*static_cast<const bfk::KArgs<P> *>(kargs));
+    const bfk::KArgs<P> &a = *static_cast<const bfk::KArgs<P> *>(kargs);
+    bfk::k_col_pass<D, Q, P, K, LB, PM><<<dim3(gx, gy), tile_threads<D, Q, P>(a.T, a.k), smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -45,27 +55,30 @@ cudaError_t launch_row(const void *kargs, unsigned gx, unsigned gy, size_t smem,
     static size_t granted[64] = {0};
     cudaError_t e = prepare(bfk::k_row_pass<D, Q, P, K, LB, PM>, smem, granted);
     if (e != cudaSuccess) return e;
-    bfk::k_row_pass<D, Q, P, K, LB, PM><<<dim3(gx, gy), bfk::Cfg<D, Q, P>::NT, smem, s>>>(*static_cast<const bfk::KArgs<P> *>(kargs));
+    const bfk::KArgs<P> &a = *static_cast<const bfk::KArgs<P> *>(kargs);
+    bfk::k_row_pass<D, Q, P, K, LB, PM><<<dim3(gx, gy), tile_threads<D, Q, P>(a.T, a.k), smem, s>>>(a);
     return cudaGetLastError();
 }
 
-template <int D, int Q, class P, int K>
+template <int D, int Q, class P, int K, bool LB>
 cudaError_t launch_col_adj(const void *kargs, unsigned gx, unsigned gy, size_t smem, cudaStream_t s)
 {
     static size_t granted[64] = {0};
-    cudaError_t e = prepare(bfk::k_col_pass_adj<D, Q, P, K>, smem, granted);
+    cudaError_t e = prepare(bfk::k_col_pass_adj<D, Q, P, K, LB>, smem, granted);
     if (e != cudaSuccess) return e;
-    bfk::k_col_pass_adj<D, Q, P, K><<<dim3(gx, gy), bfk::Cfg<D, Q, P>::NT, smem, s>>>(*static_cast<const bfk::KArgs<P> *>(kargs));
+    const bfk::KArgs<P> &a = *static_cast<const bfk::KArgs<P> *>(kargs);
+    bfk::k_col_pass_adj<D, Q, P, K, LB><<<dim3(gx, gy), tile_threads<D, Q, P>(a.T, a.k), smem, s>>>(a);
     return cudaGetLastError();
 }
 
-template <int D, int Q, class P, int K>
+template <int D, int Q, class P, int K, bool LB>
 cudaError_t launch_row_adj(const void *kargs, unsigned gx, unsigned gy, size_t smem, cudaStream_t s)
 {
     static size_t granted[64] = {0};
-    cudaError_t e = prepare(bfk::k_row_pass_adj<D, Q, P, K>, smem, granted);
+    cudaError_t e = prepare(bfk::k_row_pass_adj<D, Q, P, K, LB>, smem, granted);
     if (e != cudaSuccess) return e;
-    bfk::k_row_pass_adj<D, Q, P, K><<<dim3(gx, gy), bfk::Cfg<D, Q, P>::NT, smem, s>>>(*static_cast<const bfk::KArgs<P> *>(kargs));
+    const bfk::KArgs<P> &a = *static_cast<const bfk::KArgs<P> *>(kargs);
+    bfk::k_row_pass_adj<D, Q, P, K, LB><<<dim3(gx, gy), tile_threads<D, Q, P>(a.T, a.k), smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -86,6 +99,17 @@ cudaError_t launch_row_mr(const void *kargs, unsigned gx, unsigned gy, size_t sm
     cudaError_t e = prepare(bfk::k_row_pass_mr<Q, P, K, LB, PM>, smem, granted);
     if (e != cudaSuccess) return e;
     bfk::k_row_pass_mr<Q, P, K, LB, PM><<<dim3(gx, gy), bfk::CfgMR<Q>::NT, smem, s>>>(*static_cast<const bfk::KArgs<P> *>(kargs));
+    return cudaGetLastError();
+}
+
+template <int Q, class P, int K, bool LB, bool ROW>
+cudaError_t launch_mr_adj(const void *kargs, unsigned gx, unsigned gy, size_t smem, cudaStream_t s)
+{
+    static size_t granted[64] = {0};
+    auto kern = ROW ? bfk::k_row_pass_mr_adj<Q, P, K, LB> : bfk::k_col_pass_mr_adj<Q, P, K, LB>;
+    cudaError_t e = prepare(kern, smem, granted);
+    if (e != cudaSuccess) return e;
+    kern<<<dim3(gx, gy), bfk::CfgMR<Q>::NT, smem, s>>>(*static_cast<const bfk::KArgs<P> *>(kargs));
     return cudaGetLastError();
 }
 
@@ -230,6 +254,23 @@ size_t tile_smem(int row, int T, int k, int tab)
     }
 }
 
+// adjoint passes: W, stage scratch and, at d = 3, the features of the children's and the parents'
+// nodes of a row pass; d = 2: Tile2
+template <int D, int Q, class P, int K>
+size_t adj_smem(int row, int T, int k)
+{
+    const int np = T << (D * k);
+    if constexpr (D == 2) {
+        using T2 = bfk::Tile2<Q, P, K, false>;
+        return row ? T2::row_adj_smem(np, T, k) : T2::col_adj_smem(np);
+    } else {
+        using TL = bfk::Tile<D, Q, P, K>;
+        const size_t base = (size_t)3 * np * TL::RR * sizeof(typename P::C);
+        if (!row || k < 1) return base;
+        return base + (size_t)T * (((size_t)1 << (D * k)) + ((size_t)1 << (D * (k - 1)))) * TL::RR * sizeof(typename TL::PH::T);
+    }
+}
+
 template <int D, int Q, class P, int K, bool LB>
 const PassFns *fns_set()
 {
@@ -240,12 +281,13 @@ const PassFns *fns_set()
         // tensor-core switch: q <= 5, polynomial sincos phases (the BF16x3 precision)
         constexpr bool TC = Q <= 5 && !P::sfu;
         constexpr int QT = TC ? Q : 2;
-        static const PassFns f = {launch_col<D, Q, P, K, LB>, launch_row<D, Q, P, K, LB>, launch_col_adj<D, Q, P, K>,
-                                  launch_row_adj<D, Q, P, K>, CF::KMAX, CF::NP, CF::NT, LB ? 1 : 0, tile_smem<D, Q, P, K>,
+        static const PassFns f = {launch_col<D, Q, P, K, LB>, launch_row<D, Q, P, K, LB>, launch_col_adj<D, Q, P, K, LB>,
+                                  launch_row_adj<D, Q, P, K, LB>, CF::KMAX, CF::NP, CF::NT, LB ? 1 : 0, tile_smem<D, Q, P, K>, adj_smem<D, Q, P, K>,
                                   {launch_col_mr<Q, P, K, LB, bfk::PM_COMPUTE>, launch_col_mr<Q, P, K, LB, bfk::PM_BUILD>,
                                    launch_col_mr<Q, P, K, LB, bfk::PM_TABLE>},
                                   {launch_row_mr<Q, P, K, LB, bfk::PM_COMPUTE>, launch_row_mr<Q, P, K, LB, bfk::PM_BUILD>,
                                    launch_row_mr<Q, P, K, LB, bfk::PM_TABLE>},
+                                  launch_mr_adj<Q, P, K, LB, false>, launch_mr_adj<Q, P, K, LB, true>,
                                   bfk::MRMAX, bfk::CfgMR<Q>::NT,
                                   launch_batch<Q, P, K, LB>, batch_ctas_per_sm<Q, P, K, LB>, mr_table_occupancy<Q, P, K, LB>,
                                   launch_ctab<D, Q, P, K>, (int)sizeof(typename bfk::Ph<P, D, K>::T),
@@ -262,18 +304,29 @@ const PassFns *fns_set()
         return &f;
     } else if constexpr (!P::is_f64) {
         // d = 3: single-RHS passes with a reduced-phase table; no multi-RHS kernels
-        static const PassFns f = {launch_col<D, Q, P, K, LB>, launch_row<D, Q, P, K, LB>, launch_col_adj<D, Q, P, K>,
-                                  launch_row_adj<D, Q, P, K>, CF::KMAX, CF::NP, CF::NT, LB ? 1 : 0, tile_smem<D, Q, P, K>, {nullptr, nullptr, nullptr},
-                                  {nullptr, nullptr, nullptr}, 0, 0, nullptr, nullptr, nullptr,
+        static const PassFns f = {launch_col<D, Q, P, K, LB>, launch_row<D, Q, P, K, LB>, launch_col_adj<D, Q, P, K, LB>,
+                                  launch_row_adj<D, Q, P, K, LB>, CF::KMAX, CF::NP, CF::NT, LB ? 1 : 0, tile_smem<D, Q, P, K>, adj_smem<D, Q, P, K>, {nullptr, nullptr, nullptr},
+                                  {nullptr, nullptr, nullptr}, nullptr, nullptr, 0, 0, nullptr, nullptr, nullptr,
                                   launch_ctab<D, Q, P, K>, (int)sizeof(typename bfk::Ph<P, D, K>::T),
                                   {launch_col<D, Q, P, K, LB, bfk::PM_BUILD>, launch_col<D, Q, P, K, LB, bfk::PM_TABLE>},
                                   {launch_row<D, Q, P, K, LB, bfk::PM_BUILD>, launch_row<D, Q, P, K, LB, bfk::PM_TABLE>},
                                   nullptr, nullptr, 0, nullptr, nullptr, 0};
         return &f;
+    } else if constexpr (D == 2) {
+        // FP64: multi-RHS passes and adjoint as the mixed precisions, no phase tables or batches
+        static const PassFns f = {launch_col<D, Q, P, K, LB>, launch_row<D, Q, P, K, LB>, nullptr,
+                                  nullptr, CF::KMAX, CF::NP, CF::NT, LB ? 1 : 0, tile_smem<D, Q, P, K>, adj_smem<D, Q, P, K>,
+                                  {launch_col_mr<Q, P, K, LB, bfk::PM_COMPUTE>, nullptr, nullptr},
+                                  {launch_row_mr<Q, P, K, LB, bfk::PM_COMPUTE>, nullptr, nullptr},
+                                  launch_mr_adj<Q, P, K, LB, false>, launch_mr_adj<Q, P, K, LB, true>,
+                                  bfk::MRMAX, bfk::CfgMR<Q>::NT, nullptr, nullptr, nullptr,
+                                  launch_ctab<D, Q, P, K>, (int)sizeof(typename bfk::Ph<P, D, K>::T),
+                                  {nullptr, nullptr}, {nullptr, nullptr}, nullptr, nullptr, 0, nullptr, nullptr, 0};
+        return &f;
     } else {
-        static const PassFns f = {launch_col<D, Q, P, K, LB>, launch_row<D, Q, P, K, LB>, launch_col_adj<D, Q, P, K>,
-                                  launch_row_adj<D, Q, P, K>, CF::KMAX, CF::NP, CF::NT, LB ? 1 : 0, tile_smem<D, Q, P, K>, {nullptr, nullptr, nullptr},
-                                  {nullptr, nullptr, nullptr}, 0, 0, nullptr, nullptr, nullptr,
+        static const PassFns f = {launch_col<D, Q, P, K, LB>, launch_row<D, Q, P, K, LB>, launch_col_adj<D, Q, P, K, LB>,
+                                  launch_row_adj<D, Q, P, K, LB>, CF::KMAX, CF::NP, CF::NT, LB ? 1 : 0, tile_smem<D, Q, P, K>, adj_smem<D, Q, P, K>, {nullptr, nullptr, nullptr},
+                                  {nullptr, nullptr, nullptr}, nullptr, nullptr, 0, 0, nullptr, nullptr, nullptr,
                                   launch_ctab<D, Q, P, K>, (int)sizeof(typename bfk::Ph<P, D, K>::T),
                                   {nullptr, nullptr}, {nullptr, nullptr}, nullptr, nullptr, 0, nullptr, nullptr, 0};
         return &f;

@@ -11,16 +11,20 @@ typedef cudaError_t (*pass_fn)(const void *kargs, unsigned grid_x, unsigned grid
 
 struct PassFns {
     pass_fn col, row;            // forward: init/column/switch pass, row/final pass
-    pass_fn col_adj, row_adj;    // adjoint passes: transposes of col and row, levels reversed
+    // adjoint passes: transposes of col and row, levels reversed (d = 2: one right-hand side,
+    // mixed precisions)
+    pass_fn col_adj, row_adj;
     int kmax;                    // most levels one pass fuses
     int np;                      // pairs per CTA (2^{d kmax})
     int nthreads;                // threads per CTA
     int lobatto;                 // 1: the forward kernels use the Lobatto nodes (KArgs::corner may be set)
     // shared memory (bytes) of a forward pass with T tiles of k levels per CTA; tab: reading a phase table
     size_t (*tile_smem)(int row, int T, int k, int tab);
+    size_t (*adj_smem)(int row, int T, int k);   // of a single-RHS adjoint pass
     // multi-RHS forward passes with a phase cache (null if absent), per phase mode:
     // [0] evaluate, [1] build the plan's phase table, [2] read the phase table
     pass_fn col_mr[3], row_mr[3];
+    pass_fn col_mr_adj, row_mr_adj;   // multi-RHS adjoint passes (d = 2)
     int mr_max;                  // right-hand sides one multi-RHS CTA holds
     int mr_nthreads;             // threads per multi-RHS CTA
     // persistent batch kernel (bf_mr.cuh): bargs points to a bfk::BatchArgs<P>

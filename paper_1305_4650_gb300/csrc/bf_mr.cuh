@@ -104,7 +104,11 @@ struct CfgMR {
     static constexpr int RR = Q * Q;
     static constexpr int PPR = RR <= 32 ? 16 : (RR <= 64 ? 8 : 4);
     static constexpr int NT = PPR * RR;
-    static constexpr int MINB = RR <= 32 ? 2 : 1;   // CTAs per SM the register budget is cut for
+};
+// CTAs per SM the register budget is cut for (FP64: one, its pipe needs few warps)
+template <int Q, class P>
+struct MinbMR {
+    static constexpr int v = Q * Q <= 32 && !P::is_f64 ? 2 : 1;
 };
 
 // Padding (in complex numbers) of the shared-memory arrays read and written by the apply
@@ -209,7 +213,7 @@ struct TileMR {
                 else if (a.flags & F_INIT)
                     add(RR * npr);
                 for (int i = skip_first(a) ? 1 : 0; i < a.k; ++i) add(r5);
-                if (a.flags & F_SWITCH)
+                if ((a.flags & F_SWITCH) && K != KIND_DOT && K != KIND_SEPARABLE)
                     for (int th = 0; th < Q; ++th) add((int64_t)Q * RR * npr);
             } else {
                 for (int i = 0; i < (skip_last(a) ? a.k - 1 : a.k); ++i) add(r5);
@@ -314,15 +318,13 @@ struct TileMR {
     }
 
     // ---- init: PC[pair][t] = l_t(y) e^{-2pi i Phi(x0(X), y_t^B)} e^{2pi i Phi(x0(X), y)}, then W = PC g(y)
-    template <int PM>
-    static __device__ void init(const KArgs<P> &a, const Ctx &x, C *W, C *PC, const C *g, TS<C> &ts)
+    static __device__ void init_factors(const KArgs<P> &a, const Ctx &x, C *PC)
     {
         const int k = a.k, n = 1 << (D * k), L = a.L, WS = x.npr * RR;
         const int cX[DMAX] = {0, 0, 0};
         const int ctr[DMAX] = {Q, Q, Q};
         const typename PH::T tX = tpoint<P, D, Q, K>(a, 0, cX, ctr);
-        if constexpr (PM == PM_TABLE) PC = ts_acquire(ts);
-        for (int it = threadIdx.x; PM != PM_TABLE && it < WS; it += NT) {
+        for (int it = threadIdx.x; it < WS; it += NT) {
             const int t = it % RR, pr = it / RR;
             const int tk[DMAX] = {t % Q, t / Q, 0};
             const R lag = a.lsrc[tk[0]] * a.lsrc[tk[1]];
@@ -341,6 +343,13 @@ struct TileMR {
             }
             PC[it] = e;
         }
+    }
+    template <int PM>
+    static __device__ void init(const KArgs<P> &a, const Ctx &x, C *W, C *PC, const C *g, TS<C> &ts)
+    {
+        const int k = a.k, n = 1 << (D * k), L = a.L, WS = x.npr * RR;
+        if constexpr (PM == PM_TABLE) PC = ts_acquire(ts);
+        else init_factors(a, x, PC);
         __syncthreads();
         if constexpr (PM == PM_BUILD) {   // build: store the factors; no weights are touched
             tab_store(ts.tb, PC, WS);
@@ -417,22 +426,22 @@ struct TileMR {
         }
     }
 
-    // ---- one column-form merge level (l -> l+1); ms.M holds the child->parent matrices
-    // SP: the inputs' nodes MID and END of both dimensions only (level 1 with KArgs::corner)
-    template <int PM, bool SP, class MS>
-    static __device__ void col_level(const KArgs<P> &a, const MS &ms, const Ctx &x, C *W, C *S, C *PC, int l, int i,
-                                     TS<C> &ts, uint64_t *wbar = nullptr, unsigned wpar = 0)
+    // ---- the factors of a column level (l -> l+1), phase cache
+    //   PA [pair alpha][chi] blocks of PCA: [cl][t_1'][t_0']  e^{2 pi i Phi(x0(A_alpha), y_t'^{B_c})}, c = cl | chi << 1
+    //   PB [pair alpha] blocks of PCB: [t_1][t_0]             e^{2 pi i Phi(x0(A_alpha), y_t^{B'})}
+    // SP: the children's nodes MID and END of both dimensions only (level 1 with KArgs::corner)
+    template <int PM> static constexpr int PCA = 2 * RR + (PM == PM_COMPUTE ? PAD.ca : 0);
+    template <int PM> static constexpr int PCB = RR + (PM == PM_COMPUTE ? PAD.cb : 0);
+    template <int PM> static constexpr int PRB = 4 * RR + (PM == PM_COMPUTE ? PAD.rb : 0);
+    template <int PM, bool SP>
+    static __device__ void col_phases(const KArgs<P> &a, const Ctx &x, C *S, C *PC, int l, int i)
     {
-        const int k = a.k, n = 1 << (D * k), nblk = n >> D, L = a.L, WS = x.npr * RR, nout = x.npr;
-        if constexpr (PM == PM_TABLE) PC = ts_acquire(ts);
-        const int SW = (int)mr_s_stride(Q, x.npr);
-        constexpr int PCA = 2 * RR + (PM == PM_COMPUTE ? PAD.ca : 0), PCB = RR + (PM == PM_COMPUTE ? PAD.cb : 0);
-        C *PA = PC;                     // [pA][chi] blocks of PCA: [cl][tq][t0']  modulation of the inputs
-        C *PB = PC + nout * 2 * PCA;    // [pA] blocks of PCB: [tq][tl]            demodulation of the output
+        const int k = a.k, n = 1 << (D * k), nblk = n >> D, L = a.L, nout = x.npr;
+        C *PA = PC, *PB = PC + nout * 2 * PCA<PM>;
         // the parts of every output pair's nodes, once per level, into S (idle during the phase
         // stage): thread = (pair, coordinate, row of q parts), each with its own geometry
-        float *PT = reinterpret_cast<float *>(S), *SG = PT + nout * T2::PSTR;
-        for (int j = threadIdx.x; PM != PM_TABLE && j < nout * 6; j += NT) {
+        R *PT = reinterpret_cast<R *>(S), *SG = PT + nout * T2::PSTR;
+        for (int j = threadIdx.x; j < nout * 6; j += NT) {
             const int row = j % 3, dim = (j / 3) & 1, pA = j / 6;
             const int alpha = pA & (NC - 1), beta = (pA >> D) & (nblk - 1), tau = pA >> (D * k);
             uint32_t Ap, Bstar, Apg, Bq;
@@ -450,90 +459,246 @@ struct TileMR {
                          SP && row < 2);
             if (j % 6 == 0) SG[pA] = PH::sign(a, tA);
         }
-        if constexpr (PM != PM_TABLE) __syncthreads();
+        __syncthreads();
         // items (pair, g, t_1), q phases each: g < 4 modulations of child c_0 = g & 1, c_1 = g >> 1,
         // g = 4 the demodulation
-        for (int it = threadIdx.x; PM != PM_TABLE && it < nout * 5 * Q; it += NT) {
+        for (int it = threadIdx.x; it < nout * 5 * Q; it += NT) {
             const int tq = it % Q, g = (it / Q) % 5, pA = it / (5 * Q);
-            const float *pt = PT + pA * T2::PSTR;
-            const float *p0 = pt + (g < 4 ? g & 1 : 2) * T2::PROW;
+            const R *pt = PT + pA * T2::PSTR;
+            const R *p0 = pt + (g < 4 ? g & 1 : 2) * T2::PROW;
             const typename PH::Part p1 = T2::load1(pt + (3 + (g >> 1)) * T2::PROW + tq);
-            C *o = g < 4 ? PA + (pA * 2 + (g >> 1)) * PCA + (g & 1) * RR + tq * Q : PB + pA * PCB + tq * Q;
+            C *o = g < 4 ? PA + (pA * 2 + (g >> 1)) * PCA<PM> + (g & 1) * RR + tq * Q : PB + pA * PCB<PM> + tq * Q;
+            const R sg = K == KIND_HYPRADON ? SG[pA] : (R)a.sc.sgn;
             if (SP && g < 4) {
-                if (tq == MID || tq == END) {
-                    const auto sg = PH2::dup(K == KIND_HYPRADON ? SG[pA] : a.sc.sgn);
-                    TL::template ph2<PM_COMPUTE>(sg, PH2::add(T2::lanes(T2::load1(p0 + MID), T2::load1(p0 + END)), PH2::dup(p1)),
+                if (tq == MID || tq == END)
+                    TL::template ph2<PM_COMPUTE>(PH2::dup(sg), PH2::add(T2::lanes(T2::load1(p0 + MID), T2::load1(p0 + END)), PH2::dup(p1)),
                                                  nullptr, nullptr, o[MID], o[END]);
-                }
                 continue;
             }
-            T2::phase_row(K == KIND_HYPRADON ? SG[pA] : a.sc.sgn, p0, p1, o);
+            T2::phase_row(sg, p0, p1, o);
         }
+    }
+
+    // ---- the factors of a row level (l -> l+1), phase cache
+    //   PA [input pair c][t]                       e^{2 pi i Phi(x_t^{A_p}, y0(B_c))}
+    //   PB [output pair alpha] blocks of PRB: [c][s] e^{2 pi i Phi(x_s^{A_alpha}, y0(B_c))}
+    // SP: the child target boxes' nodes MID and END only
+    template <int PM, bool SP>
+    static __device__ void row_phases(const KArgs<P> &a, const Ctx &x, C *S, C *PC, int l, int i)
+    {
+        const int k = a.k, n = 1 << (D * k), nblk = n >> D, L = a.L, nout = x.npr;
+        C *PA = PC, *PB = PC + nout * RR;
+        // the blocks' geometry once per level, into S (idle during the phase stage)
+        GeoR *GR = reinterpret_cast<GeoR *>(S);
+        for (int j = threadIdx.x; j < (nout >> D); j += NT) {
+            const int beta = j & (nblk - 1), tau = j >> (D * (k - 1));
+            uint32_t Ap, Bstar, Apg, Bq;
+            int base;
+            tile_of(a, x, tau, Ap, Bstar);
+            TL::block_geo(Ap, Bstar, beta, i, k, Apg, Bq, base);
+            int ca[DMAX], cbq[DMAX];
+            morton_decode<D>(Apg, l, ca);
+            morton_decode<D>(Bq, L - l - 1, cbq);
+            GR[j] = GeoR{{ca[0], ca[1]}, {cbq[0], cbq[1]}};
+        }
+        __syncthreads();
+        // items (pair, s), the four factors at a child node, then (block, t), the four at a parent node
+        constexpr int RP = SP ? 4 : RR;   // child nodes
+        for (int it = threadIdx.x; it < nout * RP + (nout >> D) * RR; it += NT) {
+            const bool post = it < nout * RP;
+            const int jt = post ? it : it - nout * RP, pj = post ? jt / RP : jt / RR;
+            const int t = SP && post ? ((jt & 1) ? END : MID) + ((jt & 2) ? END : MID) * Q : (post ? jt % RP : jt % RR);
+            const GeoR g = GR[post ? pj >> D : pj];
+            const int ca[DMAX] = {post ? 2 * g.ca[0] + (pj & 1) : g.ca[0], post ? 2 * g.ca[1] + ((pj >> 1) & 1) : g.ca[1], 0};
+            const int tk[DMAX] = {t % Q, t / Q, 0};
+            typename P::SE s0[2], s1[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                s0[h] = sget<P, Q>(a, 0, l, 2 * g.cbq[0] + h, Q);
+                s1[h] = sget<P, Q>(a, 1, l, 2 * g.cbq[1] + h, Q);
+            }
+            C E[NC];
+            T2::template four<PM_COMPUTE>(a, tpoint<P, D, Q, K>(a, post ? l + 1 : l, ca, tk), s0, s1, typename T2::FT{nullptr, 0}, 0, 0, E);
+            C *o = post ? PB + pj * PRB<PM> + t : PA + pj * NC * RR + t;
+#pragma unroll
+            for (int c = 0; c < NC; ++c) o[c * RR] = E[c];
+        }
+    }
+
+    // ---- The two data flows of a level, in place on the tile, for nrc right-hand sides from r0.
+    // Factors come from pointer functions; CJ conjugates those of stage A, else those of stage B.
+    //
+    // spread (column level; adjoint of a row level): out_j(t) = fB(j, t) sum_c sum_u M_c[t][u]
+    // fA(j, c, u) in_c(u) for the four outputs j of a block, one dimension per stage.  SP: inputs
+    // at nodes MID and END only.
+    template <bool SP, bool CJ, class MS, class FA, class FB>
+    static __device__ __forceinline__ void spread(const MS &ms, const Ctx &x, int k, int i, C *W, C *S, int r0, int nrc, FA fA, FB fB)
+    {
+        const int n = 1 << (D * k), nblk = n >> D, WS = x.npr * RR, nout = x.npr, SW = (int)mr_s_stride(Q, x.npr);
+        constexpr int QA = SP ? 2 : Q;
+        // stage A: items (rb, j, c_1, u_1): modulate the inputs, contract dimension 0
+        for (int it = threadIdx.x; it < nrc * nout * 2 * QA; it += NT) {
+            const int tp = it % QA, chi = (it / QA) & 1, pj = (it / (2 * QA)) & (nout - 1), rbl = (it / (2 * QA)) >> x.lgp;
+            const int tq = SP ? (tp ? END : MID) : tp;
+            const int beta = (pj >> D) & (nblk - 1), tau = pj >> (D * k);
+            const C *Wr = W + (r0 + rbl) * WS + (tau * n + block_base(beta, i)) * RR + Q * tq;
+            C acc[Q];
+#pragma unroll
+            for (int j = 0; j < Q; ++j) acc[j] = czero<C>();
+#pragma unroll
+            for (int cl = 0; cl < 2; ++cl) {
+                const C *win = Wr + ((cl | (chi << 1)) << (D * i)) * RR, *ph = fA(pj, cl, chi) + tq * Q;
+#pragma unroll
+                for (int t0p = 0; t0p < Q; ++t0p) {
+                    if (SP && t0p != MID && t0p != END) continue;
+                    const C u = CJ ? cjmul(ph[t0p], win[t0p]) : cmul(ph[t0p], win[t0p]);
+#pragma unroll
+                    for (int t0 = 0; t0 < Q; ++t0) mmac<Q, LB>(acc[t0], ms, cl, t0, t0p, u);
+                }
+            }
+            C *so = S + rbl * SW + ((pj * 2 + chi) * Q + tq) * Q;
+#pragma unroll
+            for (int j = 0; j < Q; ++j) so[j] = acc[j];
+        }
+        __syncthreads();
+        // stage B: items (rb, j, t_0): contract dimension 1 and the child bit c_1
+        for (int it = threadIdx.x; it < nrc * nout * Q; it += NT) {
+            const int tl = it % Q, pj = (it / Q) & (nout - 1), rbl = (it / Q) >> x.lgp;
+            const int beta = (pj >> D) & (nblk - 1), tau = pj >> (D * k);
+            C acc[Q];
+#pragma unroll
+            for (int j = 0; j < Q; ++j) acc[j] = czero<C>();
+#pragma unroll
+            for (int chi = 0; chi < 2; ++chi) {
+                const C *si = S + rbl * SW + ((pj * 2 + chi) * Q) * Q + tl;
+#pragma unroll
+                for (int tqp = 0; tqp < Q; ++tqp) {
+                    if (SP && tqp != MID && tqp != END) continue;
+                    const C v = si[tqp * Q];
+#pragma unroll
+                    for (int tq = 0; tq < Q; ++tq) mmac<Q, LB>(acc[tq], ms, chi, tq, tqp, v);
+                }
+            }
+            C *wo = W + (r0 + rbl) * WS + (tau * n + block_base(beta, i) + ((pj & (NC - 1)) << (D * i))) * RR + tl;
+            const C *ph = fB(pj) + tl;
+#pragma unroll
+            for (int tq = 0; tq < Q; ++tq) wo[tq * Q] = CJ ? cmul(ph[tq * Q], acc[tq]) : cjmul(ph[tq * Q], acc[tq]);
+        }
+        __syncthreads();
+    }
+    // gather (row level; adjoint of a column level): out_j(s) = sum_c fB(j, c, s) sum_t M_j[t][s]
+    // fA(c, t) in_c(t).  SP: outputs at nodes MID and END only.
+    template <bool SP, bool CJ, class MS, class FA, class FB>
+    static __device__ __forceinline__ void gather(const MS &ms, const Ctx &x, int k, int i, C *W, C *S, int r0, int nrc, FA fA, FB fB)
+    {
+        const int n = 1 << (D * k), nblk = n >> D, WS = x.npr * RR, nout = x.npr, SW = (int)mr_s_stride(Q, x.npr);
+        constexpr int SU = 2 * Q + PAD.rs;
+        // stage A: items (rb, c, t_1): modulate input c, contract dimension 0 for both bits j_0
+        for (int it = threadIdx.x; it < nrc * nout * Q; it += NT) {
+            const int th = it % Q, pin = (it / Q) & (nout - 1), rbl = (it / Q) >> x.lgp;
+            const int c = pin & (NC - 1), beta = (pin >> D) & (nblk - 1), tau = pin >> (D * k);
+            const C *win = W + (r0 + rbl) * WS + (tau * n + block_base(beta, i) + (c << (D * i))) * RR + th * Q;
+            const C *ph = fA(pin) + th * Q;
+            C z[2][Q];
+#pragma unroll
+            for (int s0 = 0; s0 < Q; ++s0) z[0][s0] = z[1][s0] = czero<C>();
+#pragma unroll
+            for (int t0 = 0; t0 < Q; ++t0) {
+                const C u = CJ ? cjmul(ph[t0], win[t0]) : cmul(ph[t0], win[t0]);
+#pragma unroll
+                for (int s0 = 0; s0 < Q; ++s0) {
+                    if (SP && s0 != MID && s0 != END) continue;
+                    mmac<Q, LB>(z[0][s0], ms, 0, t0, s0, u);
+                    mmac<Q, LB>(z[1][s0], ms, 1, t0, s0, u);
+                }
+            }
+            C *so = S + rbl * SW + (pin * Q + th) * SU;
+#pragma unroll
+            for (int s0 = 0; s0 < Q; ++s0) {
+                if (SP && s0 != MID && s0 != END) continue;
+                so[s0] = z[0][s0];
+                so[Q + s0] = z[1][s0];
+            }
+        }
+        __syncthreads();
+        // stage B: items (rb, j, s_0): contract dimension 1 per input, modulate, sum over c.  M_1
+        // is M_0 with both indices reversed: j_1 = 1 runs dimension 1 backwards, so the
+        // coefficients are compile-time operands
+        constexpr int QB = SP ? 2 : Q;
+        for (int it = threadIdx.x; it < nrc * nout * QB; it += NT) {
+            const int sp = it % QB, s0 = SP ? (sp ? END : MID) : sp, pj = (it / QB) & (nout - 1), rbl = (it / QB) >> x.lgp;
+            const int al = pj & (NC - 1), beta = (pj >> D) & (nblk - 1), tau = pj >> (D * k);
+            const int a0 = al & 1, a1 = al >> 1, rev = a1 ? -1 : 1;
+            const C *Sblk = S + rbl * SW + (pj - al) * Q * SU + a0 * Q + s0 + (a1 ? (Q - 1) * SU : 0);
+            C v[NC][QB];   // SP: nodes MID and END
+#pragma unroll
+            for (int c = 0; c < NC; ++c) {
+                const C *si = Sblk + c * Q * SU;
+                if constexpr (SP) {
+                    v[c][0] = czero<C>();
+#pragma unroll
+                    for (int t1 = 0; t1 < Q; ++t1) mmac<Q, LB>(v[c][0], ms, 0, t1, MID, si[t1 * rev * SU]);
+                    v[c][1] = si[(a1 ? MID : END) * rev * SU];
+                } else {
+#pragma unroll
+                    for (int s1 = 0; s1 < Q; ++s1) v[c][s1] = czero<C>();
+#pragma unroll
+                    for (int t1 = 0; t1 < Q; ++t1) {
+                        const C zz = si[t1 * rev * SU];
+#pragma unroll
+                        for (int s1 = 0; s1 < Q; ++s1) mmac<Q, LB>(v[c][s1], ms, 0, t1, s1, zz);
+                    }
+                }
+            }
+            C *wo = W + (r0 + rbl) * WS + (tau * n + block_base(beta, i) + (al << (D * i))) * RR + s0;
+#pragma unroll
+            for (int j = 0; j < QB; ++j) {
+                const int s1 = SP ? (j ? END : MID) : (a1 ? Q - 1 - j : j);
+                C acc = czero<C>();
+#pragma unroll
+                for (int c = 0; c < NC; ++c) {
+                    const C e = fB(pj, c)[s1 * Q + s0];
+                    acc = TL::cadd(acc, CJ ? cmul(e, v[c][j]) : cjmul(e, v[c][j]));
+                }
+                wo[s1 * Q] = acc;
+            }
+        }
+        __syncthreads();
+    }
+
+    // ---- one column-form merge level (l -> l+1); ms.M holds the child->parent matrices
+    template <int PM, bool SP, class MS>
+    static __device__ void col_level(const KArgs<P> &a, const MS &ms, const Ctx &x, C *W, C *S, C *PC, int l, int i,
+                                     TS<C> &ts, uint64_t *wbar = nullptr, unsigned wpar = 0)
+    {
+        const int nout = x.npr;
+        if constexpr (PM == PM_TABLE) PC = ts_acquire(ts);
+        else col_phases<PM, SP>(a, x, S, PC, l, i);
         __syncthreads();
         if (wbar) wait_input(a, wbar, wpar);   // the weights were copied in during the phase stage
         if constexpr (PM == PM_BUILD) {   // build: store the factors; no weights are touched
             tab_store(ts.tb, PC, 5 * RR * nout);
             ts.tb += 5 * RR * nout;
             __syncthreads();
-        }
-        for (int r0 = 0; PM != PM_BUILD && r0 < x.nr; r0 += x.rc) {
-            const int nrc = min(x.rc, x.nr - r0);
-            // stage A: items (rb, pA, chi, tq): modulate the inputs, contract dimension 0
-            constexpr int QA = SP ? 2 : Q;
-            for (int it = threadIdx.x; it < nrc * nout * 2 * QA; it += NT) {
-                const int tp = it % QA, chi = (it / QA) & 1, pA = (it / (2 * QA)) & (nout - 1), rbl = (it / (2 * QA)) >> x.lgp;
-                const int tq = SP ? (tp ? END : MID) : tp;
-                const int beta = (pA >> D) & (nblk - 1), tau = pA >> (D * k);
-                const int base = block_base(beta, i);
-                const C *Wr = W + (r0 + rbl) * WS + tau * n * RR;
-                const C *ph = PA + (pA * 2 + chi) * PCA + tq * Q;
-                C acc[Q];
-#pragma unroll
-                for (int j = 0; j < Q; ++j) acc[j] = czero<C>();
-#pragma unroll
-                for (int cl = 0; cl < 2; ++cl) {
-                    const int c = cl | (chi << 1);
-                    const C *win = Wr + (base + (c << (D * i))) * RR + Q * tq;
-#pragma unroll
-                    for (int t0p = 0; t0p < Q; ++t0p) {
-                        if (SP && t0p != MID && t0p != END) continue;
-                        const C u = cmul(ph[cl * RR + t0p], win[t0p]);
-#pragma unroll
-                        for (int t0 = 0; t0 < Q; ++t0) mmac<Q, LB>(acc[t0], ms, c & 1, t0, t0p, u);
-                    }
-                }
-                C *so = S + rbl * SW + ((pA * 2 + chi) * Q + tq) * Q;
-#pragma unroll
-                for (int j = 0; j < Q; ++j) so[j] = acc[j];
-            }
-            __syncthreads();
-            // stage B: items (rb, pA, tl): contract dimension 1 and the child bit, demodulate
-            for (int it = threadIdx.x; it < nrc * nout * Q; it += NT) {
-                const int tl = it % Q, pA = (it / Q) & (nout - 1), rbl = (it / Q) >> x.lgp;
-                const int alpha = pA & (NC - 1), beta = (pA >> D) & (nblk - 1), tau = pA >> (D * k);
-                const int base = block_base(beta, i);
-                C acc[Q];
-#pragma unroll
-                for (int j = 0; j < Q; ++j) acc[j] = czero<C>();
-#pragma unroll
-                for (int chi = 0; chi < 2; ++chi) {
-                    const C *si = S + rbl * SW + ((pA * 2 + chi) * Q) * Q + tl;
-#pragma unroll
-                    for (int tqp = 0; tqp < Q; ++tqp) {
-                        if (SP && tqp != MID && tqp != END) continue;
-                        const C v = si[tqp * Q];
-#pragma unroll
-                        for (int tq = 0; tq < Q; ++tq) mmac<Q, LB>(acc[tq], ms, chi, tq, tqp, v);
-                    }
-                }
-                C *wo = W + (r0 + rbl) * WS + tau * n * RR + (base + (alpha << (D * i))) * RR + tl;
-                const C *ph = PB + pA * PCB + tl;
-#pragma unroll
-                for (int tq = 0; tq < Q; ++tq) wo[tq * Q] = cjmul(ph[tq * Q], acc[tq]);
-            }
-            __syncthreads();
+        } else {
+            const C *PA = PC, *PB = PC + nout * 2 * PCA<PM>;
+            for (int r0 = 0; r0 < x.nr; r0 += x.rc)
+                spread<SP, false>(ms, x, a.k, i, W, S, r0, min(x.rc, x.nr - r0),
+                                  [&](int pj, int cl, int chi) { return PA + (pj * 2 + chi) * PCA<PM> + cl * RR; },
+                                  [&](int pj) { return PB + pj * PCB<PM>; });
         }
         if constexpr (PM == PM_TABLE) ts_release(ts);
+    }
+    // its conjugate transpose (level l+1 -> l)
+    template <bool SP>
+    static __device__ void col_level_adj(const KArgs<P> &a, const Ctx &x, C *W, C *S, C *PC, int l, int i)
+    {
+        col_phases<PM_COMPUTE, SP>(a, x, S, PC, l, i);
+        __syncthreads();
+        const C *PA = PC, *PB = PC + x.npr * 2 * PCA<PM_COMPUTE>;
+        for (int r0 = 0; r0 < x.nr; r0 += x.rc)
+            gather<SP, false>(a, x, a.k, i, W, S, r0, min(x.rc, x.nr - r0), [&](int pj) { return PB + pj * PCB<PM_COMPUTE>; },
+                              [&](int pj, int al) { return PA + (((pj & ~3) + al) * 2 + ((pj >> 1) & 1)) * PCA<PM_COMPUTE> + (pj & 1) * RR; });
     }
 
     // ---- switch at level l: one thread per (pair, s), one accumulator per right-hand side;
@@ -572,17 +737,18 @@ struct TileMR {
                     C ev[Q];   // the factors of this digit t_1: two at a time (lanes t_0, t_0 + 1)
                     if constexpr (PM != PM_TABLE) {
                         const typename PH2::T tS2 = PH2::dup(tS);
-                        const typename P::SE e1 = sget<P, Q>(a, 1, l, cb[1], th);
-                        const typename PH2::Part hp = PH2::part(a, tS2, e1, e1, 1);
+                        const R sg = PH::sign(a, tS);
+                        const typename PH::Part h1 = PH::part(a, tS, sget<P, Q>(a, 1, l, cb[1], th), 1);
+                        const typename PH2::Part hp = PH2::dup(h1);
 #pragma unroll
                         for (int t0 = 0; t0 + 1 < Q; t0 += 2)
-                            expphase_part2<P, D, K>(
-                                a, tS2,
+                            TL::template ph2<PM_COMPUTE>(
+                                PH2::dup(sg),
                                 PH2::add(PH2::part(a, tS2, sget<P, Q>(a, 0, l, cb[0], t0), sget<P, Q>(a, 0, l, cb[0], t0 + 1), 0), hp),
-                                ev[t0], ev[t0 + 1]);
+                                nullptr, nullptr, ev[t0], ev[t0 + 1]);
                         if constexpr (Q & 1)
-                            ev[Q - 1] = expphase_part<P, D, K>(
-                                a, tS, PH::add(PH::part(a, tS, sget<P, Q>(a, 0, l, cb[0], Q - 1), 0), PH2::lane0(hp)));
+                            ev[Q - 1] = TL::template ph<PM_COMPUTE>(
+                                sg, PH::add(PH::part(a, tS, sget<P, Q>(a, 0, l, cb[0], Q - 1), 0), h1), nullptr);
                     }
 #pragma unroll
                     for (int t0 = 0; t0 < Q; ++t0) {
@@ -618,150 +784,171 @@ struct TileMR {
         if constexpr (PM == PM_BUILD) ts.tb += (int64_t)x.npr * RR * RR;
     }
 
+    // ---- conjugate transpose of the switch: u(t) = sum_s e^{-2 pi i Phi(x_s^A, y_t^B)} v(s); one
+    // thread per (pair, t), one accumulator per right-hand side.  The sum runs over the digit
+    // s_1: the parts of its q targets x_s (q per coordinate and target) go to PC first, the
+    // targets in lane order, so a phase costs the addition of two of them.
+    static __device__ void switch_adj(const KArgs<P> &a, const Ctx &x, C *W, C *PC, int l)
+    {
+        constexpr int QE = T2::QE, NCMP = T2::NCMP, PSW = 2 * Q * NCMP * QE;   // [coordinate][t][component][s_0]
+        const int k = a.k, n = 1 << (D * k), L = a.L, WS = x.npr * RR;
+        R *PT = reinterpret_cast<R *>(PC), *SG = PT + x.npr * PSW;
+        for (int p0 = 0; p0 < x.npr; p0 += CfgMR<Q>::PPR) {
+            const int pl = p0 + (int)threadIdx.x / RR, t = (int)threadIdx.x % RR;
+            const bool act = (int)threadIdx.x < CfgMR<Q>::PPR * RR && pl < x.npr;
+            C acc[MRMAX];
+#pragma unroll
+            for (int rb = 0; rb < MRMAX; ++rb) acc[rb] = czero<C>();
+#pragma unroll 1
+            for (int s1 = 0; s1 < Q; ++s1) {
+                __syncthreads();   // the previous digit's (or round's) parts have been used
+                for (int it = threadIdx.x; it < CfgMR<Q>::PPR * 2 * Q; it += NT) {
+                    const int s0 = it % Q, dim = (it / Q) & 1, pr = p0 + it / (2 * Q);
+                    if (pr >= x.npr) break;
+                    uint32_t Ap, Bstar;
+                    tile_of(a, x, pr >> (D * k), Ap, Bstar);
+                    int ca[DMAX], cb[DMAX];
+                    morton_decode<D>((Ap << (D * k)) + digit_rev<D>(pr & (n - 1), k), l, ca);
+                    morton_decode<D>(Bstar, L - l, cb);
+                    const int sk[DMAX] = {s0, s1, 0};
+                    const typename PH::T tS = tpoint<P, D, Q, K>(a, l, ca, sk);
+                    const auto xf = dim ? tS.x[1] : tS.x[0];
+                    const auto Af = dim ? tS.A[1] : tS.A[0];
+                    const typename P::SE *e = a.st[dim] + soff<Q>(L, l) + (dim ? cb[1] : cb[0]) * (Q + 2);
+                    R *o = PT + pr * PSW + dim * Q * NCMP * QE + s0;
+#pragma unroll
+                    for (int tt = 0; tt < Q; ++tt) T2::store1(o + tt * NCMP * QE, PH::part_of(a, xf, Af, e[tt], dim == 0));
+                    if (dim == 0) SG[pr * Q + s0] = PH::sign(a, tS);
+                }
+                __syncthreads();
+                if (act) {
+                    const R *q0 = PT + pl * PSW + (t % Q) * NCMP * QE, *q1 = PT + pl * PSW + (Q + t / Q) * NCMP * QE;
+                    const C *v = W + pl * RR + s1 * Q;
+                    auto put = [&](const C &e, int s0) {
+#pragma unroll
+                        for (int rb = 0; rb < MRMAX; ++rb)
+                            if (rb < x.nr) acc[rb] = TL::cadd(acc[rb], cjmul(e, v[rb * WS + s0]));
+                    };
+#pragma unroll
+                    for (int s0 = 0; s0 + 1 < Q; s0 += 2) {
+                        typename PH2::V sg = PH2::dup((R)a.sc.sgn);
+                        if constexpr (K == KIND_HYPRADON) {
+                            sg.x = SG[pl * Q + s0];
+                            sg.y = SG[pl * Q + s0 + 1];
+                        }
+                        C E0, E1;
+                        TL::template ph2<PM_COMPUTE>(sg, PH2::add(T2::load2(q0 + s0), T2::load2(q1 + s0)), nullptr, nullptr, E0, E1);
+                        put(E0, s0);
+                        put(E1, s0 + 1);
+                    }
+                    if constexpr (Q & 1) {
+                        const R sg = K == KIND_HYPRADON ? SG[pl * Q + Q - 1] : (R)a.sc.sgn;
+                        put(TL::template ph<PM_COMPUTE>(sg, PH::add(T2::load1(q0 + Q - 1), T2::load1(q1 + Q - 1)), nullptr), Q - 1);
+                    }
+                }
+            }
+            __syncthreads();
+            if (act) {
+#pragma unroll
+                for (int rb = 0; rb < MRMAX; ++rb)
+                    if (rb < x.nr) W[rb * WS + pl * RR + t] = acc[rb];
+            }
+        }
+        __syncthreads();
+    }
+
+    // ---- switch of a phase that is a sum over dimensions (Tile::switch_sep): the factors of both
+    // dimensions (q x q per pair each; mr_s_size holds them for any rc) go to the scratch S, then
+    // one sweep per dimension, in place.  ADJ: the conjugate transpose.
+    template <bool ADJ>
+    static __device__ void switch_sep(const KArgs<P> &a, const Ctx &x, C *W, C *S, int l)
+    {
+        const int k = a.k, n = 1 << (D * k), L = a.L, WS = x.npr * RR;
+        for (int it = threadIdx.x; it < x.npr * 2 * RR; it += NT) {   // [pair][dim][s][t]
+            const int t = it % Q, sd = (it / Q) % Q, dim = (it / RR) & 1, pr = it / (2 * RR);
+            uint32_t Ap, Bstar;
+            tile_of(a, x, pr >> (D * k), Ap, Bstar);
+            int ca[DMAX], cb[DMAX];
+            morton_decode<D>((Ap << (D * k)) + digit_rev<D>(pr & (n - 1), k), l, ca);
+            morton_decode<D>(Bstar, L - l, cb);
+            const int sk[DMAX] = {dim ? Q : sd, dim ? sd : Q, 0};
+            const typename PH::T tS = tpoint<P, D, Q, K>(a, l, ca, sk);
+            S[it] = TL::template ph<PM_COMPUTE>(
+                PH::sign(a, tS),
+                PH::part_of(a, dim ? tS.x[1] : tS.x[0], dim ? tS.A[1] : tS.A[0], sget<P, Q>(a, dim, l, dim ? cb[1] : cb[0], t), dim == 0),
+                nullptr);
+        }
+        __syncthreads();
+#pragma unroll
+        for (int dim = 0; dim < 2; ++dim) {
+            for (int it = threadIdx.x; it < x.nr * x.npr * Q; it += NT) {   // one line of q values
+                const int o = it % Q, pr = (it / Q) & (x.npr - 1), rb = (it / Q) >> x.lgp;
+                C *w = W + rb * WS + pr * RR + (dim ? o : o * Q);
+                const C *e = S + (pr * 2 + dim) * RR;
+                const int st = dim ? Q : 1;
+                C v[Q];
+#pragma unroll
+                for (int u = 0; u < Q; ++u) v[u] = w[u * st];
+#pragma unroll
+                for (int s = 0; s < Q; ++s) {
+                    C acc = czero<C>();
+#pragma unroll
+                    for (int u = 0; u < Q; ++u) {
+                        if constexpr (ADJ)
+                            acc = TL::cadd(acc, cjmul(e[u * Q + s], v[u]));
+                        else
+                            cmac(acc, e[s * Q + u], v[u]);
+                    }
+                    w[s * st] = acc;
+                }
+            }
+            __syncthreads();
+        }
+    }
+
     // ---- one row-form merge level (l -> l+1); SP: the outputs' nodes MID and END only
     template <int PM, bool SP, class MS>
     static __device__ void row_level(const KArgs<P> &a, const MS &ms, const Ctx &x, C *W, C *S, C *PC, int l, int i,
                                      TS<C> &ts, uint64_t *wbar = nullptr, unsigned wpar = 0)
     {
-        const int k = a.k, n = 1 << (D * k), nblk = n >> D, L = a.L, WS = x.npr * RR, nout = x.npr;
+        const int nout = x.npr;
         if constexpr (PM == PM_TABLE) PC = ts_acquire(ts);
-        const int SW = (int)mr_s_stride(Q, x.npr);
-        constexpr int PRB = 4 * RR + (PM == PM_COMPUTE ? PAD.rb : 0), SU = 2 * Q + PAD.rs;
-        C *PA = PC;              // [pin][th][t0]                       pre-modulation at the parent's nodes
-        C *PB = PC + nout * RR;  // [pA] blocks of PRB: [c][s1][s0]     post-modulation at the child's nodes
-        // the blocks' geometry once per level, into S (idle during the phase stage)
-        GeoR *GR = reinterpret_cast<GeoR *>(S);
-        for (int j = threadIdx.x; PM != PM_TABLE && j < (nout >> D); j += NT) {
-            const int beta = j & (nblk - 1), tau = j >> (D * (k - 1));
-            uint32_t Ap, Bstar, Apg, Bq;
-            int base;
-            tile_of(a, x, tau, Ap, Bstar);
-            TL::block_geo(Ap, Bstar, beta, i, k, Apg, Bq, base);
-            int ca[DMAX], cbq[DMAX];
-            morton_decode<D>(Apg, l, ca);
-            morton_decode<D>(Bq, L - l - 1, cbq);
-            GR[j] = GeoR{{ca[0], ca[1]}, {cbq[0], cbq[1]}};
-        }
-        if constexpr (PM != PM_TABLE) __syncthreads();
-        // items (pair, s), the four post-modulations at a child node, then (block, t), the four
-        // pre-modulations at a parent node
-        constexpr int RP = SP ? 4 : RR;   // output nodes
-        for (int it = threadIdx.x; PM != PM_TABLE && it < nout * RP + (nout >> D) * RR; it += NT) {
-            const bool post = it < nout * RP;
-            const int jt = post ? it : it - nout * RP, pj = post ? jt / RP : jt / RR;
-            const int t = SP && post ? ((jt & 1) ? END : MID) + ((jt & 2) ? END : MID) * Q : (post ? jt % RP : jt % RR);
-            const GeoR g = GR[post ? pj >> D : pj];
-            const int ca[DMAX] = {post ? 2 * g.ca[0] + (pj & 1) : g.ca[0], post ? 2 * g.ca[1] + ((pj >> 1) & 1) : g.ca[1], 0};
-            const int tk[DMAX] = {t % Q, t / Q, 0};
-            typename P::SE s0[2], s1[2];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                s0[h] = sget<P, Q>(a, 0, l, 2 * g.cbq[0] + h, Q);
-                s1[h] = sget<P, Q>(a, 1, l, 2 * g.cbq[1] + h, Q);
-            }
-            C E[NC];
-            T2::template four<PM_COMPUTE>(a, tpoint<P, D, Q, K>(a, post ? l + 1 : l, ca, tk), s0, s1, typename T2::FT{nullptr, 0}, 0, 0, E);
-            C *o = post ? PB + pj * PRB + t : PA + pj * NC * RR + t;
-#pragma unroll
-            for (int c = 0; c < NC; ++c) o[c * RR] = E[c];
-        }
+        else row_phases<PM, SP>(a, x, S, PC, l, i);
         __syncthreads();
         if (wbar) wait_input(a, wbar, wpar);   // the weights were copied in during the phase stage
         if constexpr (PM == PM_BUILD) {   // build: store the factors; no weights are touched
             tab_store(ts.tb, PC, 5 * RR * nout);
             ts.tb += 5 * RR * nout;
             __syncthreads();
-        }
-        for (int r0 = 0; PM != PM_BUILD && r0 < x.nr; r0 += x.rc) {
-            const int nrc = min(x.rc, x.nr - r0);
-            // stage A: items (rb, pin, th): pre-modulate input c, contract dimension 0 for both alpha_0
-            for (int it = threadIdx.x; it < nrc * nout * Q; it += NT) {
-                const int th = it % Q, pin = (it / Q) & (nout - 1), rbl = (it / Q) >> x.lgp;
-                const int c = pin & (NC - 1), beta = (pin >> D) & (nblk - 1), tau = pin >> (D * k);
-                const int base = block_base(beta, i);
-                const C *win = W + (r0 + rbl) * WS + tau * n * RR + (base + (c << (D * i))) * RR + th * Q;
-                const C *ph = PA + (pin * Q + th) * Q;
-                C z[2][Q];
-#pragma unroll
-                for (int s0 = 0; s0 < Q; ++s0) {
-                    z[0][s0] = czero<C>();
-                    z[1][s0] = czero<C>();
-                }
-#pragma unroll
-                for (int t0 = 0; t0 < Q; ++t0) {
-                    const C u = cjmul(ph[t0], win[t0]);
-#pragma unroll
-                    for (int s0 = 0; s0 < Q; ++s0) {
-                        if (SP && s0 != MID && s0 != END) continue;
-                        mmac<Q, LB>(z[0][s0], ms, 0, t0, s0, u);
-                        mmac<Q, LB>(z[1][s0], ms, 1, t0, s0, u);
-                    }
-                }
-                C *so = S + rbl * SW + (pin * Q + th) * SU;
-#pragma unroll
-                for (int s0 = 0; s0 < Q; ++s0) {
-                    if (SP && s0 != MID && s0 != END) continue;
-                    so[s0] = z[0][s0];
-                    so[Q + s0] = z[1][s0];
-                }
-            }
-            __syncthreads();
-            // stage B: items (rb, pA, s0): contract dimension 1 per child, post-modulate, sum over
-            // c.  M_1 is M_0 with both indices reversed: a child alpha_1 = 1 runs dimension 1
-            // backwards, so the coefficients are compile-time operands
-            constexpr int QB = SP ? 2 : Q;
-            for (int it = threadIdx.x; it < nrc * nout * QB; it += NT) {
-                const int sp = it % QB, s0 = SP ? (sp ? END : MID) : sp, pA = (it / QB) & (nout - 1), rbl = (it / QB) >> x.lgp;
-                const int alpha = pA & (NC - 1), beta = (pA >> D) & (nblk - 1), tau = pA >> (D * k);
-                const int base = block_base(beta, i);
-                const int a0 = alpha & 1, a1 = alpha >> 1, rev = a1 ? -1 : 1;
-                const C *Sblk = S + rbl * SW + (pA - alpha) * Q * SU + a0 * Q + s0 + (a1 ? (Q - 1) * SU : 0);
-                C v[NC][QB];   // SP: nodes MID and END
-#pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    const C *si = Sblk + c * Q * SU;
-                    if constexpr (SP) {
-                        v[c][0] = czero<C>();
-#pragma unroll
-                        for (int t1 = 0; t1 < Q; ++t1) mmac<Q, LB>(v[c][0], ms, 0, t1, MID, si[t1 * rev * SU]);
-                        v[c][1] = si[(a1 ? MID : END) * rev * SU];
-                    } else {
-#pragma unroll
-                        for (int s1 = 0; s1 < Q; ++s1) v[c][s1] = czero<C>();
-#pragma unroll
-                        for (int t1 = 0; t1 < Q; ++t1) {
-                            const C zz = si[t1 * rev * SU];
-#pragma unroll
-                            for (int s1 = 0; s1 < Q; ++s1) mmac<Q, LB>(v[c][s1], ms, 0, t1, s1, zz);
-                        }
-                    }
-                }
-                C *wo = W + (r0 + rbl) * WS + tau * n * RR + (base + (alpha << (D * i))) * RR + s0;
-                const C *ph = PB + pA * PRB + s0;
-#pragma unroll
-                for (int j = 0; j < QB; ++j) {
-                    const int s1 = SP ? (j ? END : MID) : (a1 ? Q - 1 - j : j);
-                    C acc = czero<C>();
-#pragma unroll
-                    for (int c = 0; c < NC; ++c) acc = TL::cadd(acc, cmul(ph[(c * Q + s1) * Q], v[c][j]));
-                    wo[s1 * Q] = acc;
-                }
-            }
-            __syncthreads();
+        } else {
+            const C *PA = PC, *PB = PC + nout * RR;
+            for (int r0 = 0; r0 < x.nr; r0 += x.rc)
+                gather<SP, true>(ms, x, a.k, i, W, S, r0, min(x.rc, x.nr - r0), [&](int pj) { return PA + pj * RR; },
+                                 [&](int pj, int c) { return PB + pj * PRB<PM> + c * RR; });
         }
         if constexpr (PM == PM_TABLE) ts_release(ts);
     }
+    // its conjugate transpose (level l+1 -> l); SP: inputs at nodes MID and END only
+    template <bool SP>
+    static __device__ void row_level_adj(const KArgs<P> &a, const Ctx &x, C *W, C *S, C *PC, int l, int i)
+    {
+        row_phases<PM_COMPUTE, SP>(a, x, S, PC, l, i);
+        __syncthreads();
+        const C *PA = PC, *PB = PC + x.npr * RR;
+        for (int r0 = 0; r0 < x.nr; r0 += x.rc)
+            spread<SP, true>(a, x, a.k, i, W, S, r0, min(x.rc, x.nr - r0),
+                             [&](int pj, int cl, int chi) { return PB + ((pj & ~3) + (cl | (chi << 1))) * PRB<PM_COMPUTE> + (pj & 3) * RR; },
+                             [&](int pj) { return PA + pj * RR; });
+    }
 
     // ---- final evaluation: PC[pair][t] = l_t(x) conj(e^{2pi i Phi(x_t, y0(Y))}), PC[pair][r] = e^{2pi i Phi(x, y0(Y))}
-    template <int PM>
-    static __device__ void final_eval(const KArgs<P> &a, const Ctx &x, const C *W, C *PC, C *f, TS<C> &ts)
+    static __device__ void final_factors(const KArgs<P> &a, const Ctx &x, C *PC)
     {
-        const int k = a.k, n = 1 << (D * k), L = a.L, WS = x.npr * RR;
+        const int k = a.k, n = 1 << (D * k), L = a.L;
         const int cY[DMAX] = {0, 0, 0};
         const int ctr[DMAX] = {Q, Q, Q};
         const typename PH::S sY = spoint<P, D, Q, K>(a, L, cY, ctr);
-        if constexpr (PM == PM_TABLE) PC = ts_acquire(ts);
-        for (int it = threadIdx.x; PM != PM_TABLE && it < x.npr * (RR + 1); it += NT) {
+        for (int it = threadIdx.x; it < x.npr * (RR + 1); it += NT) {
             const int t = it % (RR + 1), pl = it / (RR + 1);
             C e = czero<C>();
             const R lag = t < RR ? a.ltgt[t % Q] * a.ltgt[t / Q] : R(1);
@@ -781,6 +968,13 @@ struct TileMR {
             }
             PC[it] = e;
         }
+    }
+    template <int PM>
+    static __device__ void final_eval(const KArgs<P> &a, const Ctx &x, const C *W, C *PC, C *f, TS<C> &ts)
+    {
+        const int k = a.k, n = 1 << (D * k), L = a.L, WS = x.npr * RR;
+        if constexpr (PM == PM_TABLE) PC = ts_acquire(ts);
+        else final_factors(a, x, PC);
         __syncthreads();
         if constexpr (PM == PM_BUILD) {   // build: store the factors; no weights are touched
             tab_store(ts.tb, PC, x.npr * (RR + 1));
@@ -805,6 +999,102 @@ struct TileMR {
             __syncthreads();
             ts_release(ts);
         }
+    }
+
+    // ---- adjoint pass input: the forward pass's outputs (strided pairs) into digit-reversed
+    // slots; output: natural order, contiguous
+    static __device__ void load_strided(const KArgs<P> &a, const Ctx &x, C *W)
+    {
+        __shared__ int64_t poff[64];
+        const int k = a.k, n = 1 << (D * k), WS = x.npr * RR;
+        const int64_t Sstar = 1LL << (D * (a.L - a.l0 - k));
+        for (int pl = threadIdx.x; pl < x.npr; pl += NT) {
+            uint32_t Ap, Bstar;
+            tile_of(a, x, pl >> (D * k), Ap, Bstar);
+            poff[pl] = ((((int64_t)Ap << (D * k)) + digit_rev<D>(pl & (n - 1), k)) * Sstar + Bstar) * RR;
+        }
+        __syncthreads();
+        for (int j = threadIdx.x; j < x.nr * WS; j += NT) {
+            const int rb = (j / RR) >> x.lgp, e = j - rb * WS;
+            const int pl = e / RR, t = e - pl * RR;
+            W[j] = __ldcg(a.win + (int64_t)(x.rhs0 + rb) * a.wstride + poff[pl] + t);
+        }
+    }
+    static __device__ void store_contig(const KArgs<P> &a, const Ctx &x, const C *W)
+    {
+        const int WS = x.npr * RR;
+        const int64_t off = (int64_t)x.tile0 * ((int64_t)RR << (D * a.k));
+        for (int j = threadIdx.x; j < x.nr * WS; j += NT) {
+            const int rb = (j / RR) >> x.lgp, e = j - rb * WS;
+            a.wout[(int64_t)(x.rhs0 + rb) * a.wstride + off + e] = W[j];
+        }
+    }
+    // ---- init^H: g(y) = sum_t conj(PC[pair][t]) w(t), PC as in init (slots in natural order)
+    static __device__ void init_adj(const KArgs<P> &a, const Ctx &x, const C *W, C *PC)
+    {
+        const int k = a.k, n = 1 << (D * k), nblk = n >> D, L = a.L, WS = x.npr * RR;
+        const bool corner = skip_first(a);
+        if (!corner) {
+            init_factors(a, x, PC);
+            __syncthreads();
+        }
+        for (int it = threadIdx.x; it < x.nr * x.npr; it += NT) {
+            const int pr = it & (x.npr - 1), rb = it >> x.lgp;
+            uint32_t Ap, Bstar;
+            tile_of(a, x, pr >> (D * k), Ap, Bstar);
+            int cb[DMAX];
+            morton_decode<D>((Bstar << (D * k)) + (pr & (n - 1)), L, cb);
+            C acc = czero<C>();
+            if (corner) {   // the four outputs of the block (level 1) at the leaf's node
+                const int c = pr & (NC - 1), b = (pr >> D) & (nblk - 1), tau = pr >> (D * k);
+                const C *w = W + rb * WS + (tau * n + (b << D)) * RR + ((c & 1) ? MID : END) + ((c >> 1) ? MID : END) * Q;
+#pragma unroll
+                for (int al = 0; al < NC; ++al) acc = madd(acc, w[al * RR]);
+            } else {
+                const C *w = W + rb * WS + pr * RR;
+                for (int t = 0; t < RR; ++t)
+                    if (a.lsrc[t % Q] * a.lsrc[t / Q] != R(0)) acc = TL::cadd(acc, cjmul(PC[pr * RR + t], w[t]));
+            }
+            a.gadj[(int64_t)(x.rhs0 + rb) * a.npts + ((int64_t)cb[0] << L) + cb[1]] = acc;
+        }
+    }
+    // ---- final^H: w(t) = conj(PC[pair][t] PC[pair][r]) f(x), PC as in final_eval (slots in
+    // digit-reversed order at level L; with a corner, level L - 1, the four inputs of a block)
+    static __device__ void final_adj(const KArgs<P> &a, const Ctx &x, C *W, C *PC)
+    {
+        const int k = a.k, n = 1 << (D * k), nblk = n >> D, L = a.L, WS = x.npr * RR;
+        const bool corner = skip_last(a);
+        if (corner ? a.k == 1 : true)   // nodes beyond the four are read by no level of this pass
+            for (int j = threadIdx.x; j < x.nr * WS; j += NT) W[j] = czero<C>();
+        if (!corner) final_factors(a, x, PC);
+        __syncthreads();
+        if (corner) {
+            for (int it = threadIdx.x; it < x.nr * x.npr; it += NT) {
+                const int pr = it & (x.npr - 1), rb = it >> x.lgp;
+                const int al = pr & (NC - 1), ra = (pr >> D) & (nblk - 1), tau = pr >> (D * k);
+                uint32_t Ap, Bstar;
+                tile_of(a, x, tau, Ap, Bstar);
+                int ca[DMAX];
+                morton_decode<D>((((Ap << (D * (k - 1))) + digit_rev<D>(ra, k - 1)) << D) + al, L, ca);
+                const C v = a.fadj[(int64_t)(x.rhs0 + rb) * a.npts + ((int64_t)ca[0] << L) + ca[1]];
+                C *w = W + rb * WS + (tau * n + ra) * RR + ((al & 1) ? MID : END) + ((al >> 1) ? MID : END) * Q;
+#pragma unroll
+                for (int c = 0; c < NC; ++c) w[(c * nblk) * RR] = v;
+            }
+        } else {
+            for (int it = threadIdx.x; it < x.nr * x.npr; it += NT) {
+                const int pl = it & (x.npr - 1), rb = it >> x.lgp;
+                uint32_t Ap, Bstar;
+                tile_of(a, x, pl >> (D * k), Ap, Bstar);
+                int ca[DMAX];
+                morton_decode<D>((Ap << (D * k)) + digit_rev<D>(pl & (n - 1), k), L, ca);
+                const C *pc = PC + pl * (RR + 1);
+                const C v = cjmul(pc[RR], a.fadj[(int64_t)(x.rhs0 + rb) * a.npts + ((int64_t)ca[0] << L) + ca[1]]);
+                for (int t = 0; t < RR; ++t)
+                    if (a.ltgt[t % Q] * a.ltgt[t / Q] != R(0)) W[rb * WS + pl * RR + t] = cjmul(pc[t], v);
+            }
+        }
+        __syncthreads();
     }
 
     // shared memory of one CTA, bytes
@@ -866,7 +1156,13 @@ __device__ __forceinline__ bool col_pass_mr(const KArgs<P> &a, const MS &ms, con
         else
             TM::template col_level<PM, false>(a, ms, x, W, S, PC, a.l0 + i, i, ts, wb, wpar);
     }
-    if (a.flags & F_SWITCH) TM::template switch_tiles<PM>(a, x, W, a.l0 + a.k, ts);
+    if (a.flags & F_SWITCH) {
+        if constexpr (K == KIND_DOT || K == KIND_SEPARABLE) {   // evaluated, not tabled
+            if constexpr (PM != PM_BUILD) TM::template switch_sep<false>(a, x, W, S, a.l0 + a.k);
+        } else {
+            TM::template switch_tiles<PM>(a, x, W, a.l0 + a.k, ts);
+        }
+    }
     if (PM != PM_BUILD) TM::store(a, x, W);
     return async;
 }
@@ -942,7 +1238,7 @@ __device__ __forceinline__ unsigned char *mr_setup(const KArgs<P> &a, const type
 // (one with a full grid; PM_TABLE launches as many CTAs as fit and streams the table of
 // all its tile groups through one pipeline).
 template <int Q, class P, int K, bool LB, int PM>
-__global__ void __launch_bounds__(CfgMR<Q>::NT, CfgMR<Q>::MINB) k_col_pass_mr(const KArgs<P> a)
+__global__ void __launch_bounds__(CfgMR<Q>::NT, MinbMR<Q, P>::v) k_col_pass_mr(const KArgs<P> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint64_t wbar;
@@ -963,7 +1259,7 @@ __global__ void __launch_bounds__(CfgMR<Q>::NT, CfgMR<Q>::MINB) k_col_pass_mr(co
 }
 
 template <int Q, class P, int K, bool LB, int PM>
-__global__ void __launch_bounds__(CfgMR<Q>::NT, CfgMR<Q>::MINB) k_row_pass_mr(const KArgs<P> a)
+__global__ void __launch_bounds__(CfgMR<Q>::NT, MinbMR<Q, P>::v) k_row_pass_mr(const KArgs<P> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ uint64_t wbar;
@@ -981,6 +1277,58 @@ __global__ void __launch_bounds__(CfgMR<Q>::NT, CfgMR<Q>::MINB) k_row_pass_mr(co
                                  it & 1u);
         __syncthreads();
     }
+}
+
+// Adjoint passes: the tiles of a forward pass, its steps conjugate-transposed in reverse order,
+// for up to MRMAX right-hand sides per CTA.
+template <int Q, class P, int K, bool LB>
+__global__ void __launch_bounds__(CfgMR<Q>::NT, MinbMR<Q, P>::v) k_col_pass_mr_adj(const KArgs<P> a)
+{
+    using C = typename P::C;
+    using TM = TileMR<Q, P, K, LB>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const typename TM::Ctx x = TM::ctx(a, blockIdx.x);
+    C *W = reinterpret_cast<C *>(smem_raw), *S = W + x.nr * x.npr * TM::RR, *PC = S + mr_s_size(Q, x.npr, x.rc);
+    TM::load_strided(a, x, W);
+    __syncthreads();
+    if (a.flags & F_SWITCH) {
+        if constexpr (K == KIND_DOT || K == KIND_SEPARABLE)
+            TM::template switch_sep<true>(a, x, W, S, a.l0 + a.k);
+        else
+            TM::switch_adj(a, x, W, PC, a.l0 + a.k);
+    }
+    for (int i = a.k - 1; i >= (TM::skip_first(a) ? 1 : 0); --i) {
+        if (LB && (a.corner & CORNER_SRC) && a.l0 + i == 1)
+            TM::template col_level_adj<LB>(a, x, W, S, PC, a.l0 + i, i);
+        else
+            TM::template col_level_adj<false>(a, x, W, S, PC, a.l0 + i, i);
+    }
+    if (a.flags & F_INIT)
+        TM::init_adj(a, x, W, PC);
+    else
+        TM::store_contig(a, x, W);
+}
+
+template <int Q, class P, int K, bool LB>
+__global__ void __launch_bounds__(CfgMR<Q>::NT, MinbMR<Q, P>::v) k_row_pass_mr_adj(const KArgs<P> a)
+{
+    using C = typename P::C;
+    using TM = TileMR<Q, P, K, LB>;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    const typename TM::Ctx x = TM::ctx(a, blockIdx.x);
+    C *W = reinterpret_cast<C *>(smem_raw), *S = W + x.nr * x.npr * TM::RR, *PC = S + mr_s_size(Q, x.npr, x.rc);
+    if (a.flags & F_FINAL)
+        TM::final_adj(a, x, W, PC);
+    else
+        TM::load_strided(a, x, W);
+    __syncthreads();
+    for (int i = (TM::skip_last(a) ? a.k - 1 : a.k) - 1; i >= 0; --i) {
+        if (LB && (a.corner & CORNER_TGT) && a.l0 + i == a.L - 2)
+            TM::template row_level_adj<LB>(a, x, W, S, PC, a.l0 + i, i);
+        else
+            TM::template row_level_adj<false>(a, x, W, S, PC, a.l0 + i, i);
+    }
+    TM::store_contig(a, x, W);
 }
 
 // ====================================================================== persistent batch
@@ -1052,7 +1400,7 @@ __device__ __forceinline__ int wait_count(const unsigned *ctr, unsigned target, 
 }
 
 template <int Q, class P, int K, bool LB>
-__global__ void __launch_bounds__(CfgMR<Q>::NT, CfgMR<Q>::MINB) k_batch_mr(const BatchArgs<P> b)
+__global__ void __launch_bounds__(CfgMR<Q>::NT, MinbMR<Q, P>::v) k_batch_mr(const BatchArgs<P> b)
 {
     using TM = TileMR<Q, P, K, LB>;
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -93,13 +93,15 @@ __device__ __forceinline__ float2 df_mul_frac2(const df2 &x, const df2 &y)
 }
 
 // quad_reduce and quad_sincos of bf_device.cuh on both lanes
+template <bool TWO>
 __device__ __forceinline__ void quad_reduce2(float2 a, float2 b, float2 &r, int &j0, int &j1)
 {
     const float2 M = dup2(12582912.0f);
-    const float2 t = fma2(dup2(4.0f), add2(a, b), M);
+    const float2 t = fma2(dup2(4.0f), TWO ? add2(a, b) : a, M);
     j0 = __float_as_int(t.x);
     j1 = __float_as_int(t.y);
-    r = add2(fma2(dup2(-0.25f), sub2(t, M), a), b);
+    r = fma2(dup2(-0.25f), sub2(t, M), a);
+    if (TWO) r = add2(r, b);
 }
 __device__ __forceinline__ void quad_sincos2(float2 r, int q0, int q1, float2 &s, float2 &c)
 {
@@ -128,18 +130,18 @@ struct Ph2<PMIXT<F>, D, K> {
     using V = float2;   // two lanes
     static __device__ __forceinline__ V dup(float a) { return dup2(a); }
     struct T { df2 x[D]; df2 A[D]; };
-    struct Part { float2 f, h, l; };
+    struct Part { float2 f, h, l, g; };
 
     static __device__ __forceinline__ df2 pack(const df &a, const df &b) { return {make_float2(a.hi, b.hi), make_float2(a.lo, b.lo)}; }
 
     static __device__ __forceinline__ T dup(const typename PH::T &a) { return pair(a, a); }
     static __device__ __forceinline__ Part dup(const typename PH::Part &p)
     {
-        return Part{dup2(p.f), dup2(p.h), dup2(p.l)};
+        return Part{dup2(p.f), dup2(p.h), dup2(p.l), dup2(p.g)};
     }
     static __device__ __forceinline__ typename PH::Part lane0(const Part &p)
     {
-        return typename PH::Part{p.f.x, p.h.x, p.l.x};
+        return typename PH::Part{p.f.x, p.h.x, p.l.x, p.g.x};
     }
 
     // the target of lane 0
@@ -173,7 +175,7 @@ struct Ph2<PMIXT<F>, D, K> {
     static __device__ __forceinline__ Part part_of(const KArgs<PMIXT<F>> &a, const df2 &x, const df2 &A, const MixSE &e0,
                                                    const MixSE &e1, bool first)
     {
-        Part p{dup2(0.0f), dup2(0.0f), dup2(0.0f)};
+        Part p{dup2(0.0f), dup2(0.0f), dup2(0.0f), dup2(0.0f)};
         const df2 y = {make_float2(e0.a.x, e1.a.x), make_float2(e0.a.y, e1.a.y)};
         const df2 y2 = {make_float2(e0.a.z, e1.a.z), make_float2(e0.a.w, e1.a.w)};
         if constexpr (K == KIND_DOT || K == KIND_GENRADON) p.f = df_mul_frac2(x, y);
@@ -188,8 +190,13 @@ struct Ph2<PMIXT<F>, D, K> {
     }
     static __device__ __forceinline__ Part add(const Part &u, const Part &v)
     {
-        Part p{dup2(0.0f), dup2(0.0f), dup2(0.0f)};
-        if constexpr (PH::HAS_F) p.f = add2(u.f, v.f);
+        Part p{dup2(0.0f), dup2(0.0f), dup2(0.0f), dup2(0.0f)};
+        if constexpr (PH::PAIR_F) {
+            p.f = u.f;
+            p.g = v.f;
+        } else if constexpr (PH::HAS_F) {
+            p.f = add2(u.f, v.f);
+        }
         if constexpr (PH::HAS_Q) {
             p.h = add2(u.h, v.h);
             p.l = add2(u.l, v.l);
@@ -207,6 +214,7 @@ struct Ph2<PMIXT<F>, D, K> {
     {
         ra = rb = dup2(0.0f);
         if constexpr (PH::HAS_F) ra = p.f;
+        if constexpr (PH::PAIR_F) rb = p.g;
         if constexpr (PH::HAS_Q) (PH::HAS_F ? rb : ra) = sqrt_frac2(p.h, p.l, sg);
     }
     static __device__ __forceinline__ float2 fin(float2 sg, const Part &p)
@@ -284,7 +292,7 @@ __device__ __forceinline__ void expphase_part2(const KArgs<P> &a, const typename
         float2 ra, rb, r;
         int j0, j1;
         PH2::fin2(PH2::sign(a, t), pt, ra, rb);
-        quad_reduce2(ra, rb, r, j0, j1);
+        quad_reduce2<PH2::PH::TWO>(ra, rb, r, j0, j1);
         quad_sincos2(r, j0, j1, s, c);
     }
     e0 = make_float2(c.x, s.x);

@@ -172,11 +172,16 @@ struct Tile2 {
         }
     }
     // the q parts of one row: target features x and A of the row's coordinate, source entries
-    // e[0..q); sp: the two nodes MID and END only
-    template <class XF>
+    // e[0..q); sp: the two nodes MID and END only; REV: in reverse order
+    template <bool REV = false, class XF>
     static __device__ __forceinline__ void part_row(const KArgs<P> &a, const XF &x, const XF &A, bool first, const typename P::SE *e,
                                                     R *o, bool sp = false)
     {
+        if constexpr (REV) {
+#pragma unroll
+            for (int j = 0; j < Q; ++j) store1(o + Q - 1 - j, PH::part_of(a, x, A, e[j], first));
+            return;
+        }
         if constexpr (LB) {
             if (sp) {
                 store1(o + MID, PH::part_of(a, x, A, e[MID], first));
@@ -477,8 +482,9 @@ struct Tile2 {
         TL::template ph2<PM>(sg, PH2::add(P0, P1), ft.at(j0, it), ft.at(j0 + 3, it), E[0], E[3]);
         TL::template ph2<PM>(sg, PH2::add(P0, swap(P1)), ft.at(j0 + 2, it), ft.at(j0 + 1, it), E[2], E[1]);
     }
-    // pre-modulation, in place: items (block, t), the block's four inputs at node t of the parent box
-    template <int PM>
+    // pre-modulation, in place: items (block, t), the block's four inputs at node t of the parent
+    // box (conjugate factors; ADJ: the factors themselves)
+    template <int PM, bool ADJ = false>
     static __device__ __forceinline__ void row_p(const KArgs<P> &a, C *Wt, const GeoR *G, const typename PH::T *TC, int l, int i,
                                                  const FT &fa)
     {
@@ -501,7 +507,7 @@ struct Tile2 {
 #pragma unroll
             for (int c = 0; c < NC; ++c) {
                 C &x = w[(c << (D * i)) * RR];
-                x = cjmul(E[c], x);
+                x = ADJ ? cmul(E[c], x) : cjmul(E[c], x);
             }
         }
     }
@@ -603,6 +609,386 @@ struct Tile2 {
                 wo[s1 * Q] = acc;
             }
         }
+    }
+
+    // ====================================================================
+    // Conjugate transposes for one right-hand side (mixed precisions): the same parts and
+    // factors, the levels in reverse.  On entry to a level the slot of output alpha of a merge
+    // block holds the level-(l+1) weights, on exit the slot of input c the level-l weights.
+
+    // column level, stage A: items (pair alpha, t_1): re-modulate out_alpha at the nodes of B',
+    // contract dimension 0 into both children c_0 -> S[pair][t_1][c_0][t'_0]; SP: nodes MID and
+    // END of the children only
+    template <bool SP>
+    static __device__ __forceinline__ void col_adj_a(const KArgs<P> &a, const C *Wt, C *S, const Geo *G, const R *PT, int i)
+    {
+        const int th = threadIdx.x % Q;
+        for (int j = threadIdx.x / Q; j < npr(a); j += blockDim.x / Q) {
+            const C *w = Wt + (G[j].base + ((j & (NC - 1)) << (D * i))) * RR + th * Q;
+            const R *pt = PT + j * PSTR;
+            C E[Q], z[2][Q];
+            phase_row(sgn(a, G[j]), pt + 2 * PROW, load1(pt + 5 * PROW + th), E);
+#pragma unroll
+            for (int s0 = 0; s0 < Q; ++s0) z[0][s0] = z[1][s0] = czero<C>();
+#pragma unroll
+            for (int t0 = 0; t0 < Q; ++t0) {
+                const C u = cmul(E[t0], w[t0]);
+#pragma unroll
+                for (int s0 = 0; s0 < Q; ++s0) {
+                    if (SP && s0 != MID && s0 != END) continue;
+                    imac(z[0][s0], a, 0, t0, s0, u);
+                    imac(z[1][s0], a, 1, t0, s0, u);
+                }
+            }
+            C *so = S + (j * Q + th) * 2 * Q;
+#pragma unroll
+            for (int s0 = 0; s0 < Q; ++s0) {
+                if (SP && s0 != MID && s0 != END) continue;
+                so[s0] = z[0][s0];
+                so[Q + s0] = z[1][s0];
+            }
+        }
+    }
+    // stage B: items (input pair c, t'_0): contract dimension 1 per output alpha, conjugate
+    // modulation at the nodes of B_c, sum over alpha.  The rows of parts of children c_1 = 1 are
+    // stored in reverse order (parts_in_adj), as dimension 1 runs backwards there (row_b).
+    template <bool SP>
+    static __device__ __forceinline__ void col_adj_b(const KArgs<P> &a, C *Wt, const C *S, const Geo *G, const R *PT, int i)
+    {
+        constexpr int QB = SP ? 2 : Q;
+        const int sp = threadIdx.x % QB, s0 = SP ? (sp ? END : MID) : sp;
+        if (threadIdx.x / QB >= blockDim.x / QB) return;   // threads beyond a whole number of pairs
+        for (int j = threadIdx.x / QB; j < npr(a); j += blockDim.x / QB) {
+            const int c0 = j & 1, c1 = (j >> 1) & 1, b0 = j & ~(NC - 1);
+            C acc[QB];
+#pragma unroll
+            for (int e = 0; e < QB; ++e) acc[e] = czero<C>();
+#pragma unroll 1
+            for (int al = 0; al < NC; ++al) {
+                const C *sc = S + (b0 + al) * Q * 2 * Q + c0 * Q + s0 + (c1 ? (Q - 1) * 2 * Q : 0);
+                const int ts = c1 ? -2 * Q : 2 * Q;
+                const R *pt = PT + (b0 + al) * PSTR;
+                const R sg = sgn(a, G[b0 + al]);
+                const Part P0 = load1(pt + c0 * PROW + s0);
+                const R *p1 = pt + (3 + c1) * PROW;
+                if constexpr (SP) {   // dimension-1 nodes MID and END: positions MID and (reversed) 0 or END
+                    C v0 = czero<C>(), E0, E1;
+#pragma unroll
+                    for (int t1 = 0; t1 < Q; ++t1) imac(v0, a, 0, t1, MID, sc[t1 * ts]);
+                    const C v1 = sc[(c1 ? MID : END) * ts];
+                    TL::template ph2<PM_COMPUTE>(PH2::dup(sg), PH2::add(lanes(load1(p1 + MID), load1(p1 + (c1 ? 0 : END))), PH2::dup(P0)),
+                                                 nullptr, nullptr, E0, E1);
+                    acc[0] = madd(acc[0], cjmul(E0, v0));
+                    acc[1] = madd(acc[1], cjmul(E1, v1));
+                } else {
+                    C v[Q], E[Q];
+#pragma unroll
+                    for (int e = 0; e < Q; ++e) v[e] = czero<C>();
+#pragma unroll
+                    for (int t1 = 0; t1 < Q; ++t1) {
+                        const C zz = sc[t1 * ts];
+#pragma unroll
+                        for (int e = 0; e < Q; ++e) imac(v[e], a, 0, t1, e, zz);
+                    }
+                    phase_row(sg, p1, P0, E);
+#pragma unroll
+                    for (int e = 0; e < Q; ++e) acc[e] = madd(acc[e], cjmul(E[e], v[e]));
+                }
+            }
+            C *wo = Wt + (G[j].base + ((j & (NC - 1)) << (D * i))) * RR + s0;
+#pragma unroll
+            for (int e = 0; e < QB; ++e) wo[(SP ? (e ? END : MID) : (c1 ? Q - 1 - e : e)) * Q] = acc[e];
+        }
+    }
+    static __device__ __forceinline__ void parts_in_adj(const KArgs<P> &a, const Geo *G, R *PT, int l)
+    {
+        for (int it = threadIdx.x; it < npr(a) * 4; it += blockDim.x) {
+            const int c = it & 1, dim = (it >> 1) & 1, j = it >> 2;
+            const typename P::SE *e = a.st[dim] + soff<Q>(a.L, l) + (2 * G[j].cb[dim] + c) * (Q + 2);
+            R *o = PT + j * PSTR + (dim * 3 + c) * PROW;
+            if (dim && c)
+                part_row<true>(a, G[j].tA.x[1], G[j].tA.A[1], false, e, o);
+            else
+                part_row(a, G[j].tA.x[dim], G[j].tA.A[dim], dim == 0, e, o);
+        }
+    }
+    // switch: u(t) = sum_s e^{-2 pi i Phi(x_s, y_t)} v(s); items (pair, t), q per thread.  As in
+    // TileMR::switch_adj the sum runs over s_1, whose parts go to shared memory first (in the
+    // space behind W, idle here).
+    static constexpr int PSW = 2 * Q * NCMP * QE;   // [coordinate][t][component][s_0]
+    static __device__ __forceinline__ void sw_adj(const KArgs<P> &a, C *Wt, R *PS, int l)
+    {
+        const int k = a.k, n = 1 << (D * k), np = npr(a);
+        R *SG = PS + np * PSW;
+        C acc[Q];
+#pragma unroll
+        for (int j = 0; j < Q; ++j) acc[j] = czero<C>();
+#pragma unroll 1
+        for (int s1 = 0; s1 < Q; ++s1) {
+            if (s1) __syncthreads();   // the previous digit's parts have been used
+            for (int it = threadIdx.x; it < np * 2 * Q; it += blockDim.x) {
+                const int s0 = it % Q, dim = (it / Q) & 1, pr = it / (2 * Q);
+                uint32_t Ap, Bstar;
+                TL::tile_of(a, pr >> (D * k), Ap, Bstar);
+                int ca[DMAX], cb[DMAX];
+                morton_decode<D>((Ap << (D * k)) + digit_rev<D>(pr & (n - 1), k), l, ca);
+                morton_decode<D>(Bstar, a.L - l, cb);
+                const int sk[DMAX] = {s0, s1, 0};
+                const typename PH::T tS = tpoint<P, D, Q, K>(a, l, ca, sk);
+                const auto xf = dim ? tS.x[1] : tS.x[0];
+                const auto Af = dim ? tS.A[1] : tS.A[0];
+                const typename P::SE *e = a.st[dim] + soff<Q>(a.L, l) + (dim ? cb[1] : cb[0]) * (Q + 2);
+                R *o = PS + pr * PSW + dim * Q * NCMP * QE + s0;
+#pragma unroll
+                for (int tt = 0; tt < Q; ++tt) store1(o + tt * NCMP * QE, PH::part_of(a, xf, Af, e[tt], dim == 0));
+                if (dim == 0) SG[pr * Q + s0] = PH::sign(a, tS);
+            }
+            __syncthreads();
+#pragma unroll
+            for (int j = 0; j < Q; ++j) {
+                const int it = threadIdx.x + j * blockDim.x;
+                if (it >= np * RR) continue;
+                const int t = it % RR, pl = it / RR;
+                const R *q0 = PS + pl * PSW + (t % Q) * NCMP * QE, *q1 = PS + pl * PSW + (Q + t / Q) * NCMP * QE;
+                const C *v = Wt + pl * RR + s1 * Q;
+#pragma unroll
+                for (int s0 = 0; s0 + 1 < Q; s0 += 2) {
+                    V sg = PH2::dup((R)a.sc.sgn);
+                    if constexpr (K == KIND_HYPRADON) {
+                        sg.x = SG[pl * Q + s0];
+                        sg.y = SG[pl * Q + s0 + 1];
+                    }
+                    C E0, E1;
+                    TL::template ph2<PM_COMPUTE>(sg, PH2::add(load2(q0 + s0), load2(q1 + s0)), nullptr, nullptr, E0, E1);
+                    acc[j] = madd(acc[j], cjmul(E0, v[s0]));
+                    acc[j] = madd(acc[j], cjmul(E1, v[s0 + 1]));
+                }
+                if constexpr (Q & 1) {
+                    const R sg = K == KIND_HYPRADON ? SG[pl * Q + Q - 1] : (R)a.sc.sgn;
+                    acc[j] = madd(acc[j], cjmul(TL::template ph<PM_COMPUTE>(sg, PH::add(load1(q0 + Q - 1), load1(q1 + Q - 1)), nullptr),
+                                                v[Q - 1]));
+                }
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int j = 0; j < Q; ++j) {
+            const int it = threadIdx.x + j * blockDim.x;
+            if (it < np * RR) Wt[it] = acc[j];
+        }
+        __syncthreads();
+    }
+
+    // row level, stage E: items (pair alpha, s): the products of out_alpha(s) with the conjugate
+    // factors of the four inputs c -> X[block][c][alpha][s]; SP: nodes MID and END only
+    template <bool SP>
+    static __device__ __forceinline__ void row_adj_e(const KArgs<P> &a, const C *Wt, C *X, const GeoR *G, const typename PH::T *TC, int l,
+                                                     int i)
+    {
+        constexpr int RS = SP ? 4 : RR;
+        for (int it = threadIdx.x; it < npr(a) * RS; it += blockDim.x) {
+            const int e = it % RS, j = it / RS, al = j & (NC - 1), b = j >> D;
+            const int t = SP ? ((e & 1) ? END : MID) + ((e & 2) ? END : MID) * Q : e;
+            const GeoR g = G[b];
+            typename PH::T tS;
+            if (TC) {
+                tS = TC[(g.tcp * NC + al) * RR + t];
+            } else {
+                const int ca[DMAX] = {2 * g.ca[0] + (al & 1), 2 * g.ca[1] + (al >> 1), 0}, sk[DMAX] = {t % Q, t / Q, 0};
+                tS = tpoint<P, D, Q, K>(a, l + 1, ca, sk);
+            }
+            typename P::SE s0[2], s1[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                s0[h] = sget<P, Q>(a, 0, l, 2 * g.cb[0] + h, Q);
+                s1[h] = sget<P, Q>(a, 1, l, 2 * g.cb[1] + h, Q);
+            }
+            C E[NC];
+            four<PM_COMPUTE>(a, tS, s0, s1, FT{nullptr, 0}, 0, 0, E);
+            const C w = Wt[(g.base + (al << (D * i))) * RR + t];
+            C *o = X + (b * NC * NC + al) * RR + t;
+#pragma unroll
+            for (int c = 0; c < NC; ++c) o[c * NC * RR] = cjmul(E[c], w);
+        }
+    }
+    // stage A: items (input pair c, alpha_1, s_1): contract dimension 0 and alpha_0
+    template <bool SP>
+    static __device__ __forceinline__ void row_adj_a(const KArgs<P> &a, const C *X, C *S)
+    {
+        constexpr int QA = SP ? 2 : Q;
+        const int tp = threadIdx.x % QA, hh = threadIdx.x / QA, ahi = hh & 1, sq = SP ? (tp ? END : MID) : tp;
+        const int step = blockDim.x / (2 * QA);
+        if (hh >> 1 >= step) return;   // threads beyond a whole number of pairs
+        for (int j = hh >> 1; j < npr(a); j += step) {
+            C acc[Q];
+#pragma unroll
+            for (int t = 0; t < Q; ++t) acc[t] = czero<C>();
+#pragma unroll
+            for (int al = 0; al < 2; ++al) {
+                const C *xi = X + (j * NC + (al | (ahi << 1))) * RR + sq * Q;
+#pragma unroll
+                for (int s0 = 0; s0 < Q; ++s0) {
+                    if (SP && s0 != MID && s0 != END) continue;
+                    const C u = xi[s0];
+#pragma unroll
+                    for (int t0 = 0; t0 < Q; ++t0) imac(acc[t0], a, al, t0, s0, u);
+                }
+            }
+            C *so = S + ((j * 2 + ahi) * Q + sq) * Q;
+#pragma unroll
+            for (int t = 0; t < Q; ++t) so[t] = acc[t];
+        }
+    }
+    // stage B: items (input pair c, t_0): contract dimension 1 and alpha_1
+    template <bool SP>
+    static __device__ __forceinline__ void row_adj_b(const KArgs<P> &a, C *Wt, const C *S, const GeoR *G, int i)
+    {
+        const int tl = threadIdx.x % Q;
+        for (int j = threadIdx.x / Q; j < npr(a); j += blockDim.x / Q) {
+            C acc[Q];
+#pragma unroll
+            for (int t = 0; t < Q; ++t) acc[t] = czero<C>();
+#pragma unroll
+            for (int ahi = 0; ahi < 2; ++ahi)
+#pragma unroll
+                for (int sq = 0; sq < Q; ++sq) {
+                    if (SP && sq != MID && sq != END) continue;
+                    const C v = S[((j * 2 + ahi) * Q + sq) * Q + tl];
+#pragma unroll
+                    for (int tq = 0; tq < Q; ++tq) imac(acc[tq], a, ahi, tq, sq, v);
+                }
+            C *wo = Wt + (G[j >> D].base + ((j & (NC - 1)) << (D * i))) * RR + tl;
+#pragma unroll
+            for (int tq = 0; tq < Q; ++tq) wo[tq * Q] = acc[tq];
+        }
+    }
+
+    static __host__ __device__ size_t col_adj_smem(int np) { return col_smem(np, false); }
+    static __host__ __device__ size_t row_adj_smem(int np, int T, int k)
+    {
+        const size_t boxes = (size_t)T * ((((size_t)1 << (D * k)) - 1) / 3);   // levels 0 .. k-1 of the tiles
+        return (size_t)np * (3 + NC) * RR * sizeof(C) + (size_t)k * (size_t)(np >> D) * sizeof(GeoR) + boxes * RR * sizeof(typename PH::T);
+    }
+
+    static __device__ __forceinline__ void col_pass_adj(const KArgs<P> &a, unsigned char *smem)
+    {
+        const int np = npr(a), rhs = blockIdx.y;
+        C *Wt = reinterpret_cast<C *>(smem), *S = Wt + np * RR;
+        Geo *G = reinterpret_cast<Geo *>(S + 2 * np * RR);
+        R *PT = reinterpret_cast<R *>(reinterpret_cast<int4 *>(G + 2 * np) + np);
+        const bool skip0 = LB && (a.corner & CORNER_SRC) && (a.flags & F_INIT), sp1 = LB && (a.corner & CORNER_SRC);
+        const int i0 = skip0 ? 1 : 0;
+        TL::load_strided(a, Wt, rhs);
+        __syncthreads();
+        if (a.flags & F_SWITCH) {
+            if constexpr (K == KIND_DOT || K == KIND_SEPARABLE)
+                TL::template switch_sep<true>(a, Wt, S, a.l0 + a.k);
+            else
+                sw_adj(a, Wt, reinterpret_cast<R *>(S), a.l0 + a.k);
+        }
+        if (a.k > i0) {
+            geo_col(a, G + ((a.k - 1) & 1) * np, a.l0 + a.k - 1, a.k - 1);
+            __syncthreads();
+            parts_out(a, G + ((a.k - 1) & 1) * np, PT, a.l0 + a.k - 1);
+            __syncthreads();
+        }
+        for (int i = a.k - 1; i >= i0; --i) {
+            const int l = a.l0 + i;
+            const bool sp = sp1 && l == 1;
+            Geo *Gi = G + (i & 1) * np, *Gn = G + (~i & 1) * np;
+            if (LB && sp)
+                col_adj_a<LB>(a, Wt, S, Gi, PT, i);
+            else
+                col_adj_a<false>(a, Wt, S, Gi, PT, i);
+            parts_in_adj(a, Gi, PT, l);
+            if (i > i0) geo_col(a, Gn, l - 1, i - 1);
+            __syncthreads();
+            if (LB && sp)
+                col_adj_b<LB>(a, Wt, S, Gi, PT, i);
+            else
+                col_adj_b<false>(a, Wt, S, Gi, PT, i);
+            if (i > i0) parts_out(a, Gn, PT, l - 1);
+            __syncthreads();
+        }
+        if (skip0) {   // g of a leaf: the four outputs of its block (level 1) at the leaf's node
+            const int k = a.k, n = 1 << (D * k), nblk = n >> D, L = a.L;
+            for (int it = threadIdx.x; it < np; it += blockDim.x) {
+                const int c = it & (NC - 1), b = (it >> D) & (nblk - 1), tau = it >> (D * k);
+                uint32_t Ap, Bstar;
+                TL::tile_of(a, tau, Ap, Bstar);
+                int cb[DMAX];
+                morton_decode<D>((Bstar << (D * k)) + (it & (n - 1)), L, cb);
+                const C *w = Wt + (tau * n + (b << D)) * RR + ((c & 1) ? MID : END) + ((c >> 1) ? MID : END) * Q;
+                C acc = w[0];
+#pragma unroll
+                for (int al = 1; al < NC; ++al) acc = madd(acc, w[al * RR]);
+                a.gadj[(int64_t)rhs * a.npts + ((int64_t)cb[0] << L) + cb[1]] = acc;
+            }
+        } else if (a.flags & F_INIT) {
+            TL::init_adj(a, Wt, rhs);
+        } else {
+            TL::store_contig(a, Wt, rhs);
+        }
+    }
+
+    static __device__ __forceinline__ void row_pass_adj(const KArgs<P> &a, unsigned char *smem)
+    {
+        const int np = npr(a), rhs = blockIdx.y, nb = np >> D;
+        C *Wt = reinterpret_cast<C *>(smem), *S = Wt + np * RR, *X = S + 2 * np * RR;
+        GeoR *G = reinterpret_cast<GeoR *>(X + NC * np * RR);
+        typename PH::T *TC = reinterpret_cast<typename PH::T *>(G + a.k * nb);
+        auto tc = [&](int i) { return TC + a.T * (((1 << (D * i)) - 1) / 3) * RR; };   // nodes of level l0 + i
+        const bool skip = LB && (a.corner & CORNER_TGT) && (a.flags & F_FINAL);
+        const int lsp = LB && (a.corner & CORNER_TGT) ? a.L - 2 : -1;
+        const int k1 = skip ? a.k - 1 : a.k;
+        if (skip) {
+            const int k = a.k, n = 1 << (D * k), nblk = n >> D, L = a.L;
+            if (k == 1) {   // no level of this pass follows: the switch may read every node
+                for (int j = threadIdx.x; j < np * RR; j += blockDim.x) Wt[j] = czero<C>();
+                __syncthreads();
+            }
+            for (int it = threadIdx.x; it < np; it += blockDim.x) {
+                const int al = it & (NC - 1), ra = (it >> D) & (nblk - 1), tau = it >> (D * k);
+                uint32_t Ap, Bstar;
+                TL::tile_of(a, tau, Ap, Bstar);
+                int ca[DMAX];
+                morton_decode<D>((((Ap << (D * (k - 1))) + digit_rev<D>(ra, k - 1)) << D) + al, L, ca);
+                const C v = a.fadj[(int64_t)rhs * a.npts + ((int64_t)ca[0] << L) + ca[1]];
+                C *w = Wt + (tau * n + ra) * RR + ((al & 1) ? MID : END) + ((al >> 1) ? MID : END) * Q;
+#pragma unroll
+                for (int c = 0; c < NC; ++c) w[(c * nblk) * RR] = v;
+            }
+        } else if (a.flags & F_FINAL) {
+            TL::final_adj(a, Wt, rhs);
+        } else {
+            TL::load_strided(a, Wt, rhs);
+        }
+        for (int i = 0; i < k1; ++i) {
+            geo_row(a, G + i * nb, a.l0 + i, i);
+            node_cache(a, tc(i), a.l0 + i, i);
+        }
+        __syncthreads();
+        for (int i = k1 - 1; i >= 0; --i) {
+            const int l = a.l0 + i;
+            const GeoR *Gi = G + i * nb;
+            if (LB && l == lsp) {
+                row_adj_e<LB>(a, Wt, X, Gi, nullptr, l, i);
+                __syncthreads();
+                row_adj_a<LB>(a, X, S);
+                __syncthreads();
+                row_adj_b<LB>(a, Wt, S, Gi, i);
+            } else {
+                row_adj_e<false>(a, Wt, X, Gi, i + 1 < k1 ? tc(i + 1) : nullptr, l, i);
+                __syncthreads();
+                row_adj_a<false>(a, X, S);
+                __syncthreads();
+                row_adj_b<false>(a, Wt, S, Gi, i);
+            }
+            __syncthreads();
+            row_p<PM_COMPUTE, true>(a, Wt, Gi, tc(i), l, i, FT{nullptr, 0});
+            __syncthreads();
+        }
+        TL::store_contig(a, Wt, rhs);
     }
 
     // ---- shared memory of a CTA (bytes): W, twice that as stage scratch, then for a column
