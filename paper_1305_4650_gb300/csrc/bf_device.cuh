@@ -649,6 +649,22 @@ __device__ __forceinline__ void cmac(double2 &acc, double2 e, double2 u)
     acc.y = fma(e.y, u.x, acc.y);
 }
 
+// acc += conj(e) * u
+__device__ __forceinline__ void cjmac(float2 &acc, float2 e, float2 u)
+{
+    acc.x = __fmaf_rn(e.x, u.x, acc.x);
+    acc.x = __fmaf_rn(e.y, u.y, acc.x);
+    acc.y = __fmaf_rn(e.x, u.y, acc.y);
+    acc.y = __fmaf_rn(-e.y, u.x, acc.y);
+}
+__device__ __forceinline__ void cjmac(double2 &acc, double2 e, double2 u)
+{
+    acc.x = fma(e.x, u.x, acc.x);
+    acc.x = fma(e.y, u.y, acc.x);
+    acc.y = fma(e.x, u.y, acc.y);
+    acc.y = fma(-e.y, u.x, acc.y);
+}
+
 }  // namespace bfk
 
 #include "bf_pair.cuh"   // the same phase arithmetic on the two lanes of a float2

@@ -113,9 +113,8 @@ struct MinbMR {
 
 // Padding (in complex numbers) of the shared-memory arrays read and written by the apply
 // stages, so that the 64-bit accesses of a warp fall in distinct banks (32 banks of 4
-// bytes).  Chosen for q = 5 by counting the wavefronts of every access pattern of the
-// stages for 16 and 32 pairs per CTA and 1 or 2 fused levels (46% more wavefronts than the
-// minimum before, 3% after); the phase-table layout stays compact.
+// bytes), chosen for q = 5 by counting the wavefronts of every access pattern of the stages
+// (TileMR::spread, gather); the phase-table layout stays compact.
 struct MRPad {
     int ca;   // column modulation: per (pair, chi) block of 2 r factors
     int cb;   // column demodulation: per pair (r factors)
@@ -128,8 +127,13 @@ __host__ __device__ constexpr int mr_pc_extra(int q)
 {
     return 2 * mr_pad(q).ca + mr_pad(q).cb > mr_pad(q).rb ? 2 * mr_pad(q).ca + mr_pad(q).cb : mr_pad(q).rb;
 }
-// scratch entries per right-hand side (2 r per pair, plus the row scratch padding)
-__host__ __device__ constexpr int64_t mr_s_stride(int q, int64_t npr) { return 2 * npr * q * q + npr * q * mr_pad(q).rs; }
+// scratch entries per right-hand side (2 r per pair, plus the padding: of the units of gather,
+// or one entry per half of spread)
+__host__ __device__ constexpr int64_t mr_s_stride(int q, int64_t npr)
+{
+    const int64_t pad = npr * q * mr_pad(q).rs;
+    return 2 * npr * q * q + (pad > 2 ? pad : 2);
+}
 // complex numbers of the scratch S: rc right-hand sides, and at least the parts of a level
 // (6 rows of up to three components of q, padded to even, and a sign per pair), which the
 // phase stage keeps there
@@ -427,12 +431,17 @@ struct TileMR {
     }
 
     // ---- the factors of a column level (l -> l+1), phase cache
-    //   PA [pair alpha][chi] blocks of PCA: [cl][t_1'][t_0']  e^{2 pi i Phi(x0(A_alpha), y_t'^{B_c})}, c = cl | chi << 1
+    //   PA [alpha_0][pair alpha / 2][chi] blocks of PCA: [cl][t_1'][t_0']  e^{2 pi i Phi(x0(A_alpha), y_t'^{B_c})}, c = cl | chi << 1
     //   PB [pair alpha] blocks of PCB: [t_1][t_0]             e^{2 pi i Phi(x0(A_alpha), y_t^{B'})}
     // SP: the children's nodes MID and END of both dimensions only (level 1 with KArgs::corner)
     template <int PM> static constexpr int PCA = 2 * RR + (PM == PM_COMPUTE ? PAD.ca : 0);
     template <int PM> static constexpr int PCB = RR + (PM == PM_COMPUTE ? PAD.cb : 0);
     template <int PM> static constexpr int PRB = 4 * RR + (PM == PM_COMPUTE ? PAD.rb : 0);
+    template <int PM>
+    static __device__ __forceinline__ int pa_at(int npr, int pj, int chi)
+    {
+        return (pj & 1) * npr * PCA<PM> + ((pj >> 1) * 2 + chi) * PCA<PM>;
+    }
     template <int PM, bool SP>
     static __device__ void col_phases(const KArgs<P> &a, const Ctx &x, C *S, C *PC, int l, int i)
     {
@@ -467,7 +476,7 @@ struct TileMR {
             const R *pt = PT + pA * T2::PSTR;
             const R *p0 = pt + (g < 4 ? g & 1 : 2) * T2::PROW;
             const typename PH::Part p1 = T2::load1(pt + (3 + (g >> 1)) * T2::PROW + tq);
-            C *o = g < 4 ? PA + (pA * 2 + (g >> 1)) * PCA<PM> + (g & 1) * RR + tq * Q : PB + pA * PCB<PM> + tq * Q;
+            C *o = g < 4 ? PA + pa_at<PM>(nout, pA, g >> 1) + (g & 1) * RR + tq * Q : PB + pA * PCB<PM> + tq * Q;
             const R sg = K == KIND_HYPRADON ? SG[pA] : (R)a.sc.sgn;
             if (SP && g < 4) {
                 if (tq == MID || tq == END)
@@ -525,146 +534,209 @@ struct TileMR {
         }
     }
 
-    // ---- The two data flows of a level, in place on the tile, for nrc right-hand sides from r0.
+    // ---- The two data flows of a level, in place on the tile, in chunks of rc right-hand sides.
     // Factors come from pointer functions; CJ conjugates those of stage A, else those of stage B.
+    // An item's digits other than its right-hand side depend on the thread only: every stage
+    // has per <= NT items per right-hand side, NT / per of them run side by side, and the item
+    // decoding and the pointers are computed once per level instead of once per item.
+    //
+    // Lanes run over the pairs first: with q = 5 and the paddings of mr_pad every access of spread
+    // then takes the fewest wavefronts its bytes allow, those of gather 1.4 times that at most
+    // (counted over the access patterns for 16 pairs; lanes over nodes first took 2.2 and 1.7
+    // times, and shared-memory wavefronts are what these stages are bound by).
     //
     // spread (column level; adjoint of a row level): out_j(t) = fB(j, t) sum_c sum_u M_c[t][u]
-    // fA(j, c, u) in_c(u) for the four outputs j of a block, one dimension per stage.  SP: inputs
-    // at nodes MID and END only.
+    // fA(j, c, u) in_c(u) for the four outputs j of a block, one dimension per stage.  A stage-A
+    // item serves the two outputs j_0 = 0, 1 (SA: distance of their factors), which share the
+    // inputs it reads.  SP: inputs at nodes MID and END only.
     template <bool SP, bool CJ, class MS, class FA, class FB>
-    static __device__ __forceinline__ void spread(const MS &ms, const Ctx &x, int k, int i, C *W, C *S, int r0, int nrc, FA fA, FB fB)
+    static __device__ __forceinline__ void spread(const MS &ms, const Ctx &x, int k, int i, C *W, C *S, int SA, FA fA, FB fB)
     {
-        const int n = 1 << (D * k), nblk = n >> D, WS = x.npr * RR, nout = x.npr, SW = (int)mr_s_stride(Q, x.npr);
+        const int n = 1 << (D * k), nblk = n >> D, WS = x.npr * RR, SW = (int)mr_s_stride(Q, x.npr);
         constexpr int QA = SP ? 2 : Q;
-        // stage A: items (rb, j, c_1, u_1): modulate the inputs, contract dimension 0
-        for (int it = threadIdx.x; it < nrc * nout * 2 * QA; it += NT) {
-            const int tp = it % QA, chi = (it / QA) & 1, pj = (it / (2 * QA)) & (nout - 1), rbl = (it / (2 * QA)) >> x.lgp;
-            const int tq = SP ? (tp ? END : MID) : tp;
-            const int beta = (pj >> D) & (nblk - 1), tau = pj >> (D * k);
-            const C *Wr = W + (r0 + rbl) * WS + (tau * n + block_base(beta, i)) * RR + Q * tq;
-            C acc[Q];
-#pragma unroll
-            for (int j = 0; j < Q; ++j) acc[j] = czero<C>();
-#pragma unroll
-            for (int cl = 0; cl < 2; ++cl) {
-                const C *win = Wr + ((cl | (chi << 1)) << (D * i)) * RR, *ph = fA(pj, cl, chi) + tq * Q;
-#pragma unroll
-                for (int t0p = 0; t0p < Q; ++t0p) {
-                    if (SP && t0p != MID && t0p != END) continue;
-                    const C u = CJ ? cjmul(ph[t0p], win[t0p]) : cmul(ph[t0p], win[t0p]);
-#pragma unroll
-                    for (int t0 = 0; t0 < Q; ++t0) mmac<Q, LB>(acc[t0], ms, cl, t0, t0p, u);
-                }
-            }
-            C *so = S + rbl * SW + ((pj * 2 + chi) * Q + tq) * Q;
-#pragma unroll
-            for (int j = 0; j < Q; ++j) so[j] = acc[j];
-        }
-        __syncthreads();
+        // stage A: items (rb, block and j_1, c_1, u_1): modulate the inputs, contract dimension 0
+        const int perA = x.npr * QA, rA = NT / perA, a0 = (int)threadIdx.x % perA, rbA = (int)threadIdx.x / perA;
+        const int tp = a0 >> x.lgp, chi = (a0 >> (x.lgp - 1)) & 1, pa = (a0 << 1) & (x.npr - 1), tq = SP ? (tp ? END : MID) : tp;
+        const int SH = x.npr * RR + 1;   // scratch of the outputs with j_0 = 1
+        const C *winA = W + (((pa >> (D * k)) << (D * k)) + block_base((pa >> D) & (nblk - 1), i) + (chi << (D * i + 1))) * RR + Q * tq;
+        const C *phA = fA(pa, chi) + tq * Q;
+        C *soA = S + ((pa + chi) * Q + tq) * Q;
         // stage B: items (rb, j, t_0): contract dimension 1 and the child bit c_1
-        for (int it = threadIdx.x; it < nrc * nout * Q; it += NT) {
-            const int tl = it % Q, pj = (it / Q) & (nout - 1), rbl = (it / Q) >> x.lgp;
-            const int beta = (pj >> D) & (nblk - 1), tau = pj >> (D * k);
-            C acc[Q];
+        const int perB = x.npr * Q, rB = NT / perB, b0 = (int)threadIdx.x % perB, rbB = (int)threadIdx.x / perB;
+        const int tl = b0 >> x.lgp, pj = b0 & (x.npr - 1);
+        const C *siB = S + (pj & 1) * SH + (pj >> 1) * 2 * RR + tl;
+        C *woB = W + (((pj >> (D * k)) << (D * k)) + block_base((pj >> D) & (nblk - 1), i) + ((pj & (NC - 1)) << (D * i))) * RR + tl;
+        const C *phB = fB(pj) + tl;
+        for (int r0 = 0; r0 < x.nr; r0 += x.rc) {
+            const int nrc = min(x.rc, x.nr - r0);
+            if (rbA < rA)
+                for (int rb = rbA; rb < nrc; rb += rA) {
+                    const C *w = winA + (r0 + rb) * WS;
+                    C acc[2][Q];
 #pragma unroll
-            for (int j = 0; j < Q; ++j) acc[j] = czero<C>();
+                    for (int j = 0; j < Q; ++j) acc[0][j] = acc[1][j] = czero<C>();
 #pragma unroll
-            for (int chi = 0; chi < 2; ++chi) {
-                const C *si = S + rbl * SW + ((pj * 2 + chi) * Q) * Q + tl;
+                    for (int cl = 0; cl < 2; ++cl)
 #pragma unroll
-                for (int tqp = 0; tqp < Q; ++tqp) {
-                    if (SP && tqp != MID && tqp != END) continue;
-                    const C v = si[tqp * Q];
+                        for (int t0p = 0; t0p < Q; ++t0p) {
+                            if (SP && t0p != MID && t0p != END) continue;
+                            const C v = w[(cl << (D * i)) * RR + t0p];
 #pragma unroll
-                    for (int tq = 0; tq < Q; ++tq) mmac<Q, LB>(acc[tq], ms, chi, tq, tqp, v);
+                            for (int j = 0; j < 2; ++j) {
+                                const C e = phA[j * SA + fA.child(cl) + t0p];
+                                const C u = CJ ? cjmul(e, v) : cmul(e, v);
+#pragma unroll
+                                for (int t0 = 0; t0 < Q; ++t0) mmac<Q, LB>(acc[j][t0], ms, cl, t0, t0p, u);
+                            }
+                        }
+                    C *so = soA + rb * SW;
+#pragma unroll
+                    for (int j = 0; j < 2; ++j)
+#pragma unroll
+                        for (int t0 = 0; t0 < Q; ++t0) so[j * SH + t0] = acc[j][t0];
                 }
-            }
-            C *wo = W + (r0 + rbl) * WS + (tau * n + block_base(beta, i) + ((pj & (NC - 1)) << (D * i))) * RR + tl;
-            const C *ph = fB(pj) + tl;
+            __syncthreads();
+            if (rbB < rB)
+                for (int rb = rbB; rb < nrc; rb += rB) {
+                    const C *si = siB + rb * SW;
+                    C acc[Q];
 #pragma unroll
-            for (int tq = 0; tq < Q; ++tq) wo[tq * Q] = CJ ? cmul(ph[tq * Q], acc[tq]) : cjmul(ph[tq * Q], acc[tq]);
+                    for (int j = 0; j < Q; ++j) acc[j] = czero<C>();
+#pragma unroll
+                    for (int ch = 0; ch < 2; ++ch)
+#pragma unroll
+                        for (int tqp = 0; tqp < Q; ++tqp) {
+                            if (SP && tqp != MID && tqp != END) continue;
+                            const C v = si[(ch * Q + tqp) * Q];
+#pragma unroll
+                            for (int t1 = 0; t1 < Q; ++t1) mmac<Q, LB>(acc[t1], ms, ch, t1, tqp, v);
+                        }
+                    C *wo = woB + (r0 + rb) * WS;
+#pragma unroll
+                    for (int t1 = 0; t1 < Q; ++t1) wo[t1 * Q] = CJ ? cmul(phB[t1 * Q], acc[t1]) : cjmul(phB[t1 * Q], acc[t1]);
+                }
+            __syncthreads();
         }
-        __syncthreads();
     }
     // gather (row level; adjoint of a column level): out_j(s) = sum_c fB(j, c, s) sum_t M_j[t][s]
-    // fA(c, t) in_c(t).  SP: outputs at nodes MID and END only.
+    // fA(c, t) in_c(t); fB.at(c): distance of the factors of input c.  SP: outputs at nodes MID and
+    // END only.
     template <bool SP, bool CJ, class MS, class FA, class FB>
-    static __device__ __forceinline__ void gather(const MS &ms, const Ctx &x, int k, int i, C *W, C *S, int r0, int nrc, FA fA, FB fB)
+    static __device__ __forceinline__ void gather(const MS &ms, const Ctx &x, int k, int i, C *W, C *S, FA fA, FB fB)
     {
-        const int n = 1 << (D * k), nblk = n >> D, WS = x.npr * RR, nout = x.npr, SW = (int)mr_s_stride(Q, x.npr);
-        constexpr int SU = 2 * Q + PAD.rs;
+        const int n = 1 << (D * k), nblk = n >> D, WS = x.npr * RR, SW = (int)mr_s_stride(Q, x.npr);
+        constexpr int SU = 2 * Q + PAD.rs, QB = SP ? 2 : Q;
         // stage A: items (rb, c, t_1): modulate input c, contract dimension 0 for both bits j_0
-        for (int it = threadIdx.x; it < nrc * nout * Q; it += NT) {
-            const int th = it % Q, pin = (it / Q) & (nout - 1), rbl = (it / Q) >> x.lgp;
-            const int c = pin & (NC - 1), beta = (pin >> D) & (nblk - 1), tau = pin >> (D * k);
-            const C *win = W + (r0 + rbl) * WS + (tau * n + block_base(beta, i) + (c << (D * i))) * RR + th * Q;
-            const C *ph = fA(pin) + th * Q;
-            C z[2][Q];
-#pragma unroll
-            for (int s0 = 0; s0 < Q; ++s0) z[0][s0] = z[1][s0] = czero<C>();
-#pragma unroll
-            for (int t0 = 0; t0 < Q; ++t0) {
-                const C u = CJ ? cjmul(ph[t0], win[t0]) : cmul(ph[t0], win[t0]);
-#pragma unroll
-                for (int s0 = 0; s0 < Q; ++s0) {
-                    if (SP && s0 != MID && s0 != END) continue;
-                    mmac<Q, LB>(z[0][s0], ms, 0, t0, s0, u);
-                    mmac<Q, LB>(z[1][s0], ms, 1, t0, s0, u);
-                }
-            }
-            C *so = S + rbl * SW + (pin * Q + th) * SU;
-#pragma unroll
-            for (int s0 = 0; s0 < Q; ++s0) {
-                if (SP && s0 != MID && s0 != END) continue;
-                so[s0] = z[0][s0];
-                so[Q + s0] = z[1][s0];
-            }
-        }
-        __syncthreads();
+        const int perA = x.npr * Q, rA = NT / perA, a0 = (int)threadIdx.x % perA, rbA = (int)threadIdx.x / perA;
+        const int th = a0 >> x.lgp, pin = a0 & (x.npr - 1);
+        const C *winA = W + (((pin >> (D * k)) << (D * k)) + block_base((pin >> D) & (nblk - 1), i) + ((pin & (NC - 1)) << (D * i))) * RR + th * Q;
+        const C *phA = fA(pin) + th * Q;
+        C *soA = S + (pin * Q + th) * SU;
         // stage B: items (rb, j, s_0): contract dimension 1 per input, modulate, sum over c.  M_1
         // is M_0 with both indices reversed: j_1 = 1 runs dimension 1 backwards, so the
         // coefficients are compile-time operands
-        constexpr int QB = SP ? 2 : Q;
-        for (int it = threadIdx.x; it < nrc * nout * QB; it += NT) {
-            const int sp = it % QB, s0 = SP ? (sp ? END : MID) : sp, pj = (it / QB) & (nout - 1), rbl = (it / QB) >> x.lgp;
-            const int al = pj & (NC - 1), beta = (pj >> D) & (nblk - 1), tau = pj >> (D * k);
-            const int a0 = al & 1, a1 = al >> 1, rev = a1 ? -1 : 1;
-            const C *Sblk = S + rbl * SW + (pj - al) * Q * SU + a0 * Q + s0 + (a1 ? (Q - 1) * SU : 0);
-            C v[NC][QB];   // SP: nodes MID and END
+        const int perB = x.npr * QB, rB = NT / perB, b0 = (int)threadIdx.x % perB, rbB = (int)threadIdx.x / perB;
+        const int sp = b0 >> x.lgp, s0 = SP ? (sp ? END : MID) : sp, pj = b0 & (x.npr - 1), al = pj & (NC - 1), j0 = al & 1, j1 = al >> 1;
+        const int rev = j1 ? -SU : SU, wst = j1 ? -Q : Q, first = j1 && !SP ? Q - 1 : 0;
+        const C *siB = S + (pj - al) * Q * SU + j0 * Q + s0 + (j1 ? (Q - 1) * SU : 0);
+        C *woB = W + (((pj >> (D * k)) << (D * k)) + block_base((pj >> D) & (nblk - 1), i) + (al << (D * i))) * RR + s0 + first * Q;
+        const C *phB = fB(pj) + s0 + first * Q;
+        for (int r0 = 0; r0 < x.nr; r0 += x.rc) {
+            const int nrc = min(x.rc, x.nr - r0);
+            if (rbA < rA)
+                for (int rb = rbA; rb < nrc; rb += rA) {
+                    const C *w = winA + (r0 + rb) * WS;
+                    C z[2][Q];
 #pragma unroll
-            for (int c = 0; c < NC; ++c) {
-                const C *si = Sblk + c * Q * SU;
-                if constexpr (SP) {
-                    v[c][0] = czero<C>();
+                    for (int e = 0; e < Q; ++e) z[0][e] = z[1][e] = czero<C>();
 #pragma unroll
-                    for (int t1 = 0; t1 < Q; ++t1) mmac<Q, LB>(v[c][0], ms, 0, t1, MID, si[t1 * rev * SU]);
-                    v[c][1] = si[(a1 ? MID : END) * rev * SU];
-                } else {
+                    for (int t0 = 0; t0 < Q; ++t0) {
+                        const C u = CJ ? cjmul(phA[t0], w[t0]) : cmul(phA[t0], w[t0]);
 #pragma unroll
-                    for (int s1 = 0; s1 < Q; ++s1) v[c][s1] = czero<C>();
+                        for (int e = 0; e < Q; ++e) {
+                            if (SP && e != MID && e != END) continue;
+                            mmac<Q, LB>(z[0][e], ms, 0, t0, e, u);
+                            mmac<Q, LB>(z[1][e], ms, 1, t0, e, u);
+                        }
+                    }
+                    C *so = soA + rb * SW;
 #pragma unroll
-                    for (int t1 = 0; t1 < Q; ++t1) {
-                        const C zz = si[t1 * rev * SU];
-#pragma unroll
-                        for (int s1 = 0; s1 < Q; ++s1) mmac<Q, LB>(v[c][s1], ms, 0, t1, s1, zz);
+                    for (int e = 0; e < Q; ++e) {
+                        if (SP && e != MID && e != END) continue;
+                        so[e] = z[0][e];
+                        so[Q + e] = z[1][e];
                     }
                 }
-            }
-            C *wo = W + (r0 + rbl) * WS + (tau * n + block_base(beta, i) + (al << (D * i))) * RR + s0;
+            __syncthreads();
+            if (rbB < rB)
+                for (int rb = rbB; rb < nrc; rb += rB) {
+                    C acc[QB];   // SP: nodes MID and END
 #pragma unroll
-            for (int j = 0; j < QB; ++j) {
-                const int s1 = SP ? (j ? END : MID) : (a1 ? Q - 1 - j : j);
-                C acc = czero<C>();
+                    for (int c = 0; c < NC; ++c) {
+                        const C *si = siB + rb * SW + c * Q * SU;
+                        const C *ph = phB + fB.at(c);
+                        if constexpr (SP) {
+                            C v = czero<C>();
 #pragma unroll
-                for (int c = 0; c < NC; ++c) {
-                    const C e = fB(pj, c)[s1 * Q + s0];
-                    acc = TL::cadd(acc, CJ ? cmul(e, v[c][j]) : cjmul(e, v[c][j]));
+                            for (int t1 = 0; t1 < Q; ++t1) mmac<Q, LB>(v, ms, 0, t1, MID, si[t1 * rev]);
+                            const C e0 = ph[MID * Q], e1 = ph[END * Q], v1 = si[(j1 ? MID : END) * rev];
+                            const C u0 = CJ ? cmul(e0, v) : cjmul(e0, v), u1 = CJ ? cmul(e1, v1) : cjmul(e1, v1);
+                            acc[0] = c ? madd(acc[0], u0) : u0;
+                            acc[1] = c ? madd(acc[1], u1) : u1;
+                        } else {
+                            C v[Q];
+#pragma unroll
+                            for (int e = 0; e < Q; ++e) v[e] = czero<C>();
+#pragma unroll
+                            for (int t1 = 0; t1 < Q; ++t1) {
+                                const C zz = si[t1 * rev];
+#pragma unroll
+                                for (int e = 0; e < Q; ++e) mmac<Q, LB>(v[e], ms, 0, t1, e, zz);
+                            }
+#pragma unroll
+                            for (int e = 0; e < Q; ++e) {
+                                const C f = ph[e * wst], u = CJ ? cmul(f, v[e]) : cjmul(f, v[e]);
+                                acc[e] = c ? madd(acc[e], u) : u;
+                            }
+                        }
+                    }
+                    C *wo = woB + (r0 + rb) * WS;
+#pragma unroll
+                    for (int e = 0; e < QB; ++e) wo[SP ? (e ? END : MID) * Q : e * wst] = acc[e];
                 }
-                wo[s1 * Q] = acc;
-            }
+            __syncthreads();
         }
-        __syncthreads();
     }
+    // factors of a column level for spread and for gather (its adjoint), of a row level for
+    // gather and for spread (its adjoint)
+    template <int PM> struct ColFA {
+        const C *p;
+        int npr;
+        __device__ __forceinline__ const C *operator()(int pj, int chi) const { return p + pa_at<PM>(npr, pj, chi); }
+        static __device__ __forceinline__ constexpr int child(int cl) { return cl * RR; }
+    };
+    struct ColAdjFB {
+        const C *p;
+        int npr;
+        __device__ __forceinline__ const C *operator()(int pj) const
+        {
+            return p + pa_at<PM_COMPUTE>(npr, pj & ~3, (pj >> 1) & 1) + (pj & 1) * RR;
+        }
+        __device__ __forceinline__ int at(int al) const { return (al & 1) * npr * PCA<PM_COMPUTE> + (al >> 1) * 2 * PCA<PM_COMPUTE>; }
+    };
+    template <int PM> struct RowFB {
+        const C *p;
+        __device__ __forceinline__ const C *operator()(int pj) const { return p + pj * PRB<PM>; }
+        static __device__ __forceinline__ constexpr int at(int c) { return c * RR; }
+    };
+    struct RowAdjFA {
+        const C *p;
+        __device__ __forceinline__ const C *operator()(int pj, int chi) const
+        {
+            return p + ((pj & ~3) + 2 * chi) * PRB<PM_COMPUTE> + (pj & 3) * RR;
+        }
+        static __device__ __forceinline__ constexpr int child(int cl) { return cl * PRB<PM_COMPUTE>; }
+    };
 
     // ---- one column-form merge level (l -> l+1); ms.M holds the child->parent matrices
     template <int PM, bool SP, class MS>
@@ -682,10 +754,7 @@ struct TileMR {
             __syncthreads();
         } else {
             const C *PA = PC, *PB = PC + nout * 2 * PCA<PM>;
-            for (int r0 = 0; r0 < x.nr; r0 += x.rc)
-                spread<SP, false>(ms, x, a.k, i, W, S, r0, min(x.rc, x.nr - r0),
-                                  [&](int pj, int cl, int chi) { return PA + (pj * 2 + chi) * PCA<PM> + cl * RR; },
-                                  [&](int pj) { return PB + pj * PCB<PM>; });
+            spread<SP, false>(ms, x, a.k, i, W, S, nout * PCA<PM>, ColFA<PM>{PA, nout}, [&](int pj) { return PB + pj * PCB<PM>; });
         }
         if constexpr (PM == PM_TABLE) ts_release(ts);
     }
@@ -696,9 +765,24 @@ struct TileMR {
         col_phases<PM_COMPUTE, SP>(a, x, S, PC, l, i);
         __syncthreads();
         const C *PA = PC, *PB = PC + x.npr * 2 * PCA<PM_COMPUTE>;
-        for (int r0 = 0; r0 < x.nr; r0 += x.rc)
-            gather<SP, false>(a, x, a.k, i, W, S, r0, min(x.rc, x.nr - r0), [&](int pj) { return PB + pj * PCB<PM_COMPUTE>; },
-                              [&](int pj, int al) { return PA + (((pj & ~3) + al) * 2 + ((pj >> 1) & 1)) * PCA<PM_COMPUTE> + (pj & 1) * RR; });
+        gather<SP, false>(a, x, a.k, i, W, S, [&](int pj) { return PB + pj * PCB<PM_COMPUTE>; }, ColAdjFB{PA, x.npr});
+    }
+
+    // fn(rb) for the CTA's right-hand sides, rb a compile-time index of accumulators; a full CTA
+    // runs without the checks
+    template <class Fn>
+    static __device__ __forceinline__ void each_rhs(const Ctx &x, Fn fn)
+    {
+        if (x.nr == MRMAX) {
+#pragma unroll
+            for (int rb = 0; rb < MRMAX; ++rb) fn(rb);
+        } else {
+#pragma unroll
+            for (int rb = 0; rb < MRMAX; ++rb) {
+                if (rb >= x.nr) break;
+                fn(rb);
+            }
+        }
     }
 
     // ---- switch at level l: one thread per (pair, s), one accumulator per right-hand side;
@@ -750,20 +834,18 @@ struct TileMR {
                             ev[Q - 1] = TL::template ph<PM_COMPUTE>(
                                 sg, PH::add(PH::part(a, tS, sget<P, Q>(a, 0, l, cb[0], Q - 1), 0), h1), nullptr);
                     }
+                    if constexpr (PM == PM_TABLE)
 #pragma unroll
-                    for (int t0 = 0; t0 < Q; ++t0) {
-                        C e;
-                        if constexpr (PM == PM_TABLE)
-                            e = chunk[(pl * Q + t0) * RR + s];
-                        else
-                            e = ev[t0];
-                        if constexpr (PM == PM_BUILD) {
-                            __stcs(ts.tb + ((int64_t)th * x.npr * Q + pl * Q + t0) * RR + s, e);
-                        } else {
+                        for (int t0 = 0; t0 < Q; ++t0) ev[t0] = chunk[(pl * Q + t0) * RR + s];
+                    if constexpr (PM == PM_BUILD) {
 #pragma unroll
-                            for (int rb = 0; rb < MRMAX; ++rb)
-                                if (rb < x.nr) cmac(acc[rb], e, u[rb * WS + t0 + Q * th]);
-                        }
+                        for (int t0 = 0; t0 < Q; ++t0) __stcs(ts.tb + ((int64_t)th * x.npr * Q + pl * Q + t0) * RR + s, ev[t0]);
+                    } else {
+                        each_rhs(x, [&](int rb) {   // the q weights of a digit t_1 are adjacent: one pointer per right-hand side
+                            const C *v = u + rb * WS + Q * th;
+#pragma unroll
+                            for (int t0 = 0; t0 < Q; ++t0) cmac(acc[rb], ev[t0], v[t0]);
+                        });
                     }
                 }
                 if constexpr (PM == PM_TABLE) {
@@ -824,11 +906,7 @@ struct TileMR {
                 if (act) {
                     const R *q0 = PT + pl * PSW + (t % Q) * NCMP * QE, *q1 = PT + pl * PSW + (Q + t / Q) * NCMP * QE;
                     const C *v = W + pl * RR + s1 * Q;
-                    auto put = [&](const C &e, int s0) {
-#pragma unroll
-                        for (int rb = 0; rb < MRMAX; ++rb)
-                            if (rb < x.nr) acc[rb] = TL::cadd(acc[rb], cjmul(e, v[rb * WS + s0]));
-                    };
+                    C ev[Q];
 #pragma unroll
                     for (int s0 = 0; s0 + 1 < Q; s0 += 2) {
                         typename PH2::V sg = PH2::dup((R)a.sc.sgn);
@@ -836,15 +914,17 @@ struct TileMR {
                             sg.x = SG[pl * Q + s0];
                             sg.y = SG[pl * Q + s0 + 1];
                         }
-                        C E0, E1;
-                        TL::template ph2<PM_COMPUTE>(sg, PH2::add(T2::load2(q0 + s0), T2::load2(q1 + s0)), nullptr, nullptr, E0, E1);
-                        put(E0, s0);
-                        put(E1, s0 + 1);
+                        TL::template ph2<PM_COMPUTE>(sg, PH2::add(T2::load2(q0 + s0), T2::load2(q1 + s0)), nullptr, nullptr, ev[s0], ev[s0 + 1]);
                     }
                     if constexpr (Q & 1) {
                         const R sg = K == KIND_HYPRADON ? SG[pl * Q + Q - 1] : (R)a.sc.sgn;
-                        put(TL::template ph<PM_COMPUTE>(sg, PH::add(T2::load1(q0 + Q - 1), T2::load1(q1 + Q - 1)), nullptr), Q - 1);
+                        ev[Q - 1] = TL::template ph<PM_COMPUTE>(sg, PH::add(T2::load1(q0 + Q - 1), T2::load1(q1 + Q - 1)), nullptr);
                     }
+                    each_rhs(x, [&](int rb) {
+                        const C *w = v + rb * WS;
+#pragma unroll
+                        for (int s0 = 0; s0 < Q; ++s0) cjmac(acc[rb], ev[s0], w[s0]);
+                    });
                 }
             }
             __syncthreads();
@@ -922,9 +1002,7 @@ struct TileMR {
             __syncthreads();
         } else {
             const C *PA = PC, *PB = PC + nout * RR;
-            for (int r0 = 0; r0 < x.nr; r0 += x.rc)
-                gather<SP, true>(ms, x, a.k, i, W, S, r0, min(x.rc, x.nr - r0), [&](int pj) { return PA + pj * RR; },
-                                 [&](int pj, int c) { return PB + pj * PRB<PM> + c * RR; });
+            gather<SP, true>(ms, x, a.k, i, W, S, [&](int pj) { return PA + pj * RR; }, RowFB<PM>{PB});
         }
         if constexpr (PM == PM_TABLE) ts_release(ts);
     }
@@ -935,10 +1013,7 @@ struct TileMR {
         row_phases<PM_COMPUTE, SP>(a, x, S, PC, l, i);
         __syncthreads();
         const C *PA = PC, *PB = PC + x.npr * RR;
-        for (int r0 = 0; r0 < x.nr; r0 += x.rc)
-            spread<SP, true>(a, x, a.k, i, W, S, r0, min(x.rc, x.nr - r0),
-                             [&](int pj, int cl, int chi) { return PB + ((pj & ~3) + (cl | (chi << 1))) * PRB<PM_COMPUTE> + (pj & 3) * RR; },
-                             [&](int pj) { return PA + pj * RR; });
+        spread<SP, true>(a, x, a.k, i, W, S, RR, RowAdjFA{PB}, [&](int pj) { return PA + pj * RR; });
     }
 
     // ---- final evaluation: PC[pair][t] = l_t(x) conj(e^{2pi i Phi(x_t, y0(Y))}), PC[pair][r] = e^{2pi i Phi(x, y0(Y))}
