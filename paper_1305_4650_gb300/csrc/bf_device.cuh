@@ -35,6 +35,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include "bf_sctab.h"
+
 namespace bfk {
 
 constexpr int QMAX = 8;
@@ -172,7 +174,37 @@ struct PMIXT {
 using PMIX = PMIXT<false>;
 using PMIXF = PMIXT<true>;
 
-__device__ __forceinline__ void sincos2pi(double fr, double &s, double &c) { sincospi(2.0 * fr, &s, &c); }
+// sin and cos of 2 pi v in FP64, v not reduced: v = k/512 + r with |r| <= 1/1024, cos and sin of
+// 2 pi k/512 from a table (8 KB, read through L1) and of 2 pi r from two short polynomials
+// (Taylor, the cosine's last term economised on the interval; truncation below 1e-17), joined
+// by the angle addition: 13 FP64 operations where sincospi of a separately reduced argument
+// takes about 25.  FP64 operations are what every FP64 pass is bound by (1.7 FMAs per clock and
+// SM); the table's loads and the integer work run beside them.
+__device__ __forceinline__ void sincos2pi(double v, double &s, double &c)
+{
+    if ((__double2hiint(v) & 0x7fffffff) >= 0x42700000) v -= rint(v);   // |v| >= 2^40: reduce first
+    const double M = 6755399441055744.0;                                // 1.5 * 2^52
+    const double t = fma(v, 512.0, M);
+    const double2 e = __ldg(reinterpret_cast<const double2 *>(&g_cos_sin.v[__double2loint(t) & (SCT_N - 1)]));
+    const double r = fma(t - M, -1.0 / 512.0, v);
+    const double u = r * r;
+    const double sn = r * fma(u, fma(u, 81.60524927607506, -41.34170224039976), 6.283185307179586);
+    const double cm = u * fma(u, 64.93931761831979, -19.739208802178716);   // cos(2 pi r) - 1
+    c = fma(e.x, cm, fma(-e.y, sn, e.x));
+    s = fma(e.y, cm, fma(e.x, sn, e.y));
+}
+
+// square root of q > 0 in FP64 to about an ulp: two Newton steps from the special-function unit's
+// reciprocal root (5 FP64 operations; q >= 1e-300, no special values)
+__device__ __forceinline__ double sqrt_newton(double q)
+{
+    double r;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(q));
+    const double h = __hiloint2double(__double2hiint(r) - 0x00100000, __double2loint(r));   // r / 2
+    double s = q * r;
+    s = fma(fma(-s, s, q), h, s);
+    return fma(fma(-s, s, q), h, s);
+}
 // sin and cos of 2 pi f for |f| < 2^20: quadrant reduction f = j/4 + r with |r| <= 1/8,
 // then sin(2 pi r) = r S(r^2) (degree 7) and cos(2 pi r) = C(r^2) (degree 6) with 2 pi
 // folded into the coefficients, which are minimax fits of the absolute error on
@@ -546,8 +578,9 @@ struct Ph<PF64, D, K> {
     {
         const double y = e.a.x, y2 = e.a.y;
         if constexpr (K == KIND_DOT) return Part{x * y, 0.0};
-        else if constexpr (K == KIND_GENRADON) return Part{x * y, A * y2};
-        else if constexpr (K == KIND_HYPRADON) return Part{0.0, first ? y2 : A * y2};
+        // (the first part of a root adds a tiny number that keeps its argument positive)
+        else if constexpr (K == KIND_GENRADON) return Part{x * y, first ? fma(A, y2, 1e-300) : A * y2};
+        else if constexpr (K == KIND_HYPRADON) return Part{0.0, first ? y2 + 1e-300 : A * y2};
         else return Part{x + y, 0.0};
     }
     static __device__ __forceinline__ Part part(const KArgs<PF64> &a, const T &t, const PF64::SE &e, int k)
@@ -561,13 +594,12 @@ struct Ph<PF64, D, K> {
         if constexpr (K == KIND_HYPRADON) return t.x[0];
         else return a.sc.sgn;
     }
+    // Phi (the sincos reduces it)
     static __device__ __forceinline__ double fin(double sg, const Part &p)
     {
-        double v;
-        if constexpr (K == KIND_DOT || K == KIND_SEPARABLE) v = p.f;
-        else if constexpr (K == KIND_GENRADON) v = p.f + sg * sqrt(p.q);
-        else v = sg * sqrt(p.q);
-        return v - rint(v);
+        if constexpr (K == KIND_DOT || K == KIND_SEPARABLE) return p.f;
+        else if constexpr (K == KIND_GENRADON) return fma(sg, sqrt_newton(p.q), p.f);
+        else return sg * sqrt_newton(p.q);
     }
 
     static __device__ __forceinline__ double frac(const KArgs<PF64> &a, const T &t, const S &s)
@@ -583,14 +615,14 @@ struct Ph<PF64, D, K> {
                 p += t.x[k] * s.y[k];
                 q += t.A[k] * s.y2[k];
             }
-            p += a.sc.sgn * sqrt(q);
+            p = fma(a.sc.sgn, sqrt_newton(q + 1e-300), p);
         } else if constexpr (K == KIND_HYPRADON) {
-            p = t.x[0] * sqrt(s.y2[0] + t.A[1] * s.y2[1]);
+            p = t.x[0] * sqrt_newton(fma(t.A[1], s.y2[1], s.y2[0] + 1e-300));
         } else {
 #pragma unroll
             for (int k = 0; k < D; ++k) p += t.x[k] + s.y[k];
         }
-        return p - rint(p);
+        return p;   // the sincos reduces it
     }
 };
 
