@@ -830,10 +830,10 @@ struct Tile {
     // items of the stages that evaluate phases, and phases per item
     static __device__ __forceinline__ int n_col_a(const KArgs<P> &a) { return a.T * ((1 << (D * a.k)) >> D) * NC * 2 * Q; }
     static __device__ __forceinline__ int n_col_b(const KArgs<P> &a) { return a.T * ((1 << (D * a.k)) >> D) * NC * QD1; }
-    static __device__ __forceinline__ int n_switch(const KArgs<P> &a) { return a.T * (1 << (D * a.k)) * QD1; }
-    static __device__ __forceinline__ int n_row_a(const KArgs<P> &a) { return a.T * ((1 << (D * a.k)) >> D) * NC * QD1; }
+    static __device__ __forceinline__ int n_switch(const KArgs<P> &a) { return a.T * (1 << (D * a.k)) * RR; }
+    static __device__ __forceinline__ int n_row_a(const KArgs<P> &a) { return a.T * ((1 << (D * a.k)) >> D) * RR; }
     static __device__ __forceinline__ int n_row_b(const KArgs<P> &a) { return a.T * ((1 << (D * a.k)) >> D) * NC * Q; }
-    static constexpr int PH_COL_A = (NC / 2) * QD1, PH_COL_B = Q, PH_SWITCH = Q * RR, PH_ROW_A = Q, PH_ROW_B = NC * QD1;
+    static constexpr int PH_COL_A = (NC / 2) * QD1, PH_COL_B = Q, PH_SWITCH = RR, PH_ROW_A = NC, PH_ROW_B = NC * QD1;
     // floats of the table one CTA of this pass reads (the phases of the switch of the
     // factorised kinds are evaluated, not tabled)
     static __device__ __forceinline__ int64_t table_floats(const KArgs<P> &a, bool row)
@@ -911,19 +911,6 @@ struct Tile {
             quad_sincos(r, j, e.y, e.x);
             return e;
         }
-    }
-    // the same from the whole source point
-    template <int PM>
-    static __device__ __forceinline__ C phs(const KArgs<P> &a, const typename PH::T &t, const typename PH::S &sv, R *q)
-    {
-        R fr;
-        if constexpr (PM == PM_TABLE) {
-            fr = __ldcs(q);
-        } else {
-            fr = PH::frac(a, t, sv);
-            if constexpr (PM == PM_BUILD) __stcs(q, fr);
-        }
-        return cis(fr);
     }
     // two factors in the lanes of a float2 (bf_pair.cuh); q1 null: lane 1 is not recorded or read
     template <int PM, class V, class Part2>
@@ -1114,12 +1101,17 @@ struct Tile {
                 typename PH::S sp;
                 PH::src1(sp, D - 1, sget<P, Q>(a, D - 1, l, cb[D - 1], tq));
                 if constexpr (!P::is_f64) {
-                    // d = 3: the parts of coordinates 2 and 1 hoisted, phases two at a time over t'_0
+                    // d = 3: the parts of all coordinates hoisted, phases two at a time over t'_0
                     using PH2 = Ph2<P, D, K>;
                     const int c0 = c & 1, c1 = (c >> 1) & 1;
                     const typename PH2::T tA2 = PH2::dup(tA);
                     const typename P::SE e2 = sget<P, Q>(a, 2, l, cb[2], tq);
                     const typename PH2::Part p2 = PH2::part(a, tA2, e2, e2, 2);
+                    typename PH2::Part P0[(Q + 1) / 2];   // lanes t'_0, t'_0 + 1 (the last one alone for odd q)
+#pragma unroll
+                    for (int t0p = 0; t0p < Q; t0p += 2)
+                        P0[t0p / 2] = PH2::part(a, tA2, sget<P, Q>(a, 0, l, cb[0], t0p),
+                                                sget<P, Q>(a, 0, l, cb[0], t0p + 1 < Q ? t0p + 1 : t0p), 0);
 #pragma unroll
                     for (int t1p = 0; t1p < Q; ++t1p) {
                         const typename P::SE e1 = sget<P, Q>(a, 1, l, cb[1], t1p);
@@ -1132,9 +1124,7 @@ struct Tile {
                         for (int t0p = 0; t0p + 1 < Q; t0p += 2) {
                             float2 E0, E1;
                             ph2<PM>(PH2::sign(a, tA2),
-                                    PH2::add(PH2::part(a, tA2, sget<P, Q>(a, 0, l, cb[0], t0p),
-                                                       sget<P, Q>(a, 0, l, cb[0], t0p + 1), 0), p12),
-                                    fa.at((cl * Q + t1p) * Q + t0p, it), fa.at((cl * Q + t1p) * Q + t0p + 1, it), E0, E1);
+                                    PH2::add(P0[t0p / 2], p12), fa.at((cl * Q + t1p) * Q + t0p, it), fa.at((cl * Q + t1p) * Q + t0p + 1, it), E0, E1);
                             const C u0 = cmul(E0, wrow[t0p]), u1 = cmul(E1, wrow[t0p + 1]);
 #pragma unroll
                             for (int t0 = 0; t0 < Q; ++t0) {
@@ -1143,7 +1133,7 @@ struct Tile {
                             }
                         }
                         if constexpr (Q & 1) {
-                            const typename PH::Part pt = PH::add(PH::part(a, tA, sget<P, Q>(a, 0, l, cb[0], Q - 1), 0), PH2::lane0(p12));
+                            const typename PH::Part pt = PH::add(PH2::lane0(P0[Q / 2]), PH2::lane0(p12));
                             const C u = cmul(ph<PM>(PH::sign(a, tA), pt, fa.at((cl * Q + t1p) * Q + Q - 1, it)), wrow[Q - 1]);
 #pragma unroll
                             for (int t0 = 0; t0 < Q; ++t0) imac(tmp[t0], a, c0, t0, Q - 1, u);
@@ -1245,163 +1235,65 @@ struct Tile {
         __syncthreads();
     }
 
-    // ---- switch at level l on every pair (slots in digit-reversed order); items (tau, slot, s_{>=1})
-    // accumulate over t for the q values of s_0.  Results go through S so no item reads a
-    // slot that another item has already rewritten.
+    // ---- switch at level l on every pair (slots in digit-reversed order); items (pair, s), the
+    // r sources in pairs of lanes (t_0, t_0 + 1).  The parts of coordinates 0 and 1 stay in
+    // registers.  Results go through S so no item reads a slot that another item has already
+    // rewritten.
     template <int PM = PM_COMPUTE>
     static __device__ void switch_tiles(const KArgs<P> &a, C *Wt, C *S, int l, R *&tb)
     {
-        if constexpr (!P::is_f64 && K == KIND_GENRADON) {   // the phase whose pairs pay for their registers
-            switch_tiles_pair<PM>(a, Wt, S, l, tb);
-            return;
-        }
-        const FT fs{tb, n_switch(a)};   // phase (th q + t_0) q + s_0 of an item
-        if constexpr (PM != PM_COMPUTE) tb += (int64_t)fs.n * PH_SWITCH;
-        const int k = a.k, n = 1 << (D * k);
-        const int L = a.L;
-        for (int it = threadIdx.x; it < a.T * n * QD1; it += blockDim.x) {
-            const int sh = it % QD1;
-            const int sl = (it / QD1) & (n - 1);
-            const int tau = (it / QD1) >> (D * k);
-            uint32_t Ap, Bstar;
-            tile_of(a, tau, Ap, Bstar);
-            const uint32_t A = (Ap << (D * k)) + digit_rev<D>(sl, k);
-            int ca[DMAX], cb[DMAX];
-            morton_decode<D>(A, l, ca);
-            morton_decode<D>(Bstar, L - l, cb);
-            typename PH::T tS[Q];
-            C acc[Q];
-            int sk[DMAX];
-            {
-                int tt = sh;
-#pragma unroll
-                for (int j = 1; j < D; ++j) { sk[j] = tt % Q; tt /= Q; }
-            }
-#pragma unroll
-            for (int s0 = 0; s0 < Q; ++s0) {
-                sk[0] = s0;
-                tS[s0] = tpoint<P, D, Q, K>(a, l, ca, sk);
-                acc[s0] = czero<C>();
-            }
-            const C *u = Wt + (tau * n + sl) * RR;
-            // t = t_0 + q t_{>=1}: the parts of coordinates >= 1 are fixed over the t_0 loop
-#pragma unroll 1
-            for (int th = 0; th < QD1; ++th) {
-                int tk[DMAX], tt = th;
-#pragma unroll
-                for (int j = 1; j < D; ++j) { tk[j] = tt % Q; tt /= Q; }
-                typename PH::Part hp[Q];
-#pragma unroll
-                for (int s0 = 0; s0 < Q; ++s0) {
-                    hp[s0] = PH::part(a, tS[s0], sget<P, Q>(a, 1, l, cb[1], tk[1]), 1);
-                    if constexpr (D == 3) hp[s0] = PH::add(hp[s0], PH::part(a, tS[s0], sget<P, Q>(a, 2, l, cb[2], tk[2]), 2));
-                }
-#pragma unroll
-                for (int t0 = 0; t0 < Q; ++t0) {
-                    const typename P::SE e0 = sget<P, Q>(a, 0, l, cb[0], t0);
-                    const C ut = u[t0 + Q * th];
-#pragma unroll
-                    for (int s0 = 0; s0 < Q; ++s0)
-                        cmac(acc[s0], ph<PM>(PH::sign(a, tS[s0]), PH::add(PH::part(a, tS[s0], e0, 0), hp[s0]), fs.at((th * Q + t0) * Q + s0, it)), ut);
-                }
-            }
-            C *w = S + (tau * n + sl) * RR + sh * Q;
-#pragma unroll
-            for (int s0 = 0; s0 < Q; ++s0) w[s0] = acc[s0];
-        }
-        __syncthreads();
-        for (int j = threadIdx.x; j < a.T * n * RR; j += blockDim.x) Wt[j] = S[j];
-        __syncthreads();
-    }
-
-    // ---- the same switch with the phases evaluated two at a time (lanes of a float2):
-    // targets s_0 = 2j and 2j + 1 share a pair; for odd q the last target takes two
-    // consecutive t_0 in its lanes.  Each lane rounds exactly as the scalar code.
-    template <int PM>
-    static __device__ void switch_tiles_pair(const KArgs<P> &a, C *Wt, C *S, int l, R *&tb)
-    {
         using PH2 = Ph2<P, D, K>;
-        constexpr int NPR = Q / 2, ODD = Q & 1, NT2 = NPR + ODD;
-        const FT fs{tb, n_switch(a)};   // phase (th q + t_0) q + s_0 of an item
+        const FT fs{tb, n_switch(a)};   // phase t of an item
         if constexpr (PM != PM_COMPUTE) tb += (int64_t)fs.n * PH_SWITCH;
         const int k = a.k, n = 1 << (D * k);
         const int L = a.L;
-        for (int it = threadIdx.x; it < a.T * n * QD1; it += blockDim.x) {
-            const int sh = it % QD1;
-            const int sl = (it / QD1) & (n - 1);
-            const int tau = (it / QD1) >> (D * k);
-            uint32_t Ap, Bstar;
-            tile_of(a, tau, Ap, Bstar);
-            const uint32_t A = (Ap << (D * k)) + digit_rev<D>(sl, k);
-            int ca[DMAX], cb[DMAX];
-            morton_decode<D>(A, l, ca);
-            morton_decode<D>(Bstar, L - l, cb);
-            typename PH2::T tP[NT2];
-            C acc[Q];
-            int sk[DMAX];
-            {
-                int tt = sh;
+        for (int it = threadIdx.x; it < a.T * n * RR; it += blockDim.x) {
+            const int s = it % RR, pr = it / RR;
+            typename PH2::T t2{};
+            typename PH2::V sg{};
+            typename PH2::Part P0[(Q + 1) / 2];
+            typename PH::Part P1[Q];
+            int cb2 = 0;
+            if constexpr (PM != PM_TABLE) {
+                uint32_t Ap, Bstar;
+                tile_of(a, pr >> (D * k), Ap, Bstar);
+                int ca[DMAX], cb[DMAX], sk[DMAX], ss = s;
+                morton_decode<D>((Ap << (D * k)) + digit_rev<D>(pr & (n - 1), k), l, ca);
+                morton_decode<D>(Bstar, L - l, cb);
 #pragma unroll
-                for (int j = 1; j < D; ++j) { sk[j] = tt % Q; tt /= Q; }
+                for (int j = 0; j < D; ++j) { sk[j] = ss % Q; ss /= Q; }
+                const typename PH::T t = tpoint<P, D, Q, K>(a, l, ca, sk);
+                t2 = PH2::dup(t);
+                sg = PH2::dup(PH::sign(a, t));
+                cb2 = cb[2];
+#pragma unroll
+                for (int t0 = 0; t0 < Q; t0 += 2)
+                    P0[t0 / 2] = PH2::part(a, t2, sget<P, Q>(a, 0, l, cb[0], t0), sget<P, Q>(a, 0, l, cb[0], t0 + 1 < Q ? t0 + 1 : t0), 0);
+#pragma unroll
+                for (int t1 = 0; t1 < Q; ++t1) P1[t1] = PH::part(a, t, sget<P, Q>(a, 1, l, cb[1], t1), 1);
             }
-#pragma unroll
-            for (int j = 0; j < NT2; ++j) {
-                sk[0] = 2 * j;
-                const typename PH::T t0 = tpoint<P, D, Q, K>(a, l, ca, sk);
-                sk[0] = (2 * j + 1 < Q) ? 2 * j + 1 : 2 * j;
-                tP[j] = PH2::pair(t0, tpoint<P, D, Q, K>(a, l, ca, sk));
-            }
-#pragma unroll
-            for (int s0 = 0; s0 < Q; ++s0) acc[s0] = czero<C>();
-            const C *u = Wt + (tau * n + sl) * RR;
+            C acc = czero<C>();
+            const C *u = Wt + pr * RR;
 #pragma unroll 1
-            for (int th = 0; th < QD1; ++th) {
-                int tk[DMAX], tt = th;
+            for (int td = 0; td < Q; ++td) {
+                typename PH::Part p2{};
+                if constexpr (PM != PM_TABLE) p2 = PH::part(a, PH2::one(t2), sget<P, Q>(a, 2, l, cb2, td), 2);
 #pragma unroll
-                for (int j = 1; j < D; ++j) { tk[j] = tt % Q; tt /= Q; }
-                typename PH2::Part hp[NT2];
-                const typename P::SE e1 = sget<P, Q>(a, 1, l, cb[1], tk[1]);
+                for (int t1 = 0; t1 < Q; ++t1) {
+                    const typename PH::Part p12 = PH::add(P1[t1], p2);
+                    const int tt = (td * Q + t1) * Q;
 #pragma unroll
-                for (int j = 0; j < NT2; ++j) {
-                    hp[j] = PH2::part(a, tP[j], e1, e1, 1);
-                    if constexpr (D == 3) {
-                        const typename P::SE e2 = sget<P, Q>(a, 2, l, cb[2], tk[2]);
-                        hp[j] = PH2::add(hp[j], PH2::part(a, tP[j], e2, e2, 2));
+                    for (int t0 = 0; t0 + 1 < Q; t0 += 2) {
+                        C E0, E1;
+                        ph2<PM>(sg, PH2::add(P0[t0 / 2], PH2::dup(p12)), fs.at(tt + t0, it), fs.at(tt + t0 + 1, it), E0, E1);
+                        cmac(acc, E0, u[tt + t0]);
+                        cmac(acc, E1, u[tt + t0 + 1]);
                     }
-                }
-#pragma unroll
-                for (int t0 = 0; t0 < Q; t0 += 2) {
-                    const bool two = t0 + 1 < Q;
-                    const typename P::SE ea = sget<P, Q>(a, 0, l, cb[0], t0);
-                    const typename P::SE eb = two ? sget<P, Q>(a, 0, l, cb[0], t0 + 1) : ea;
-                    const C ua = u[t0 + Q * th];
-                    const C ub = two ? u[t0 + 1 + Q * th] : czero<C>();
-                    float2 E0, E1;
-                    const int ja = (th * Q + t0) * Q, jb = ja + Q;
-#pragma unroll
-                    for (int j = 0; j < NPR; ++j) {
-                        ph2<PM>(PH2::sign(a, tP[j]), PH2::add(PH2::part(a, tP[j], ea, ea, 0), hp[j]), fs.at(ja + 2 * j, it),
-                                fs.at(ja + 2 * j + 1, it), E0, E1);
-                        cmac(acc[2 * j], E0, ua);
-                        cmac(acc[2 * j + 1], E1, ua);
-                        if (two) {
-                            ph2<PM>(PH2::sign(a, tP[j]), PH2::add(PH2::part(a, tP[j], eb, eb, 0), hp[j]), fs.at(jb + 2 * j, it),
-                                    fs.at(jb + 2 * j + 1, it), E0, E1);
-                            cmac(acc[2 * j], E0, ub);
-                            cmac(acc[2 * j + 1], E1, ub);
-                        }
-                    }
-                    if constexpr (ODD) {
-                        ph2<PM>(PH2::sign(a, tP[NPR]), PH2::add(PH2::part(a, tP[NPR], ea, eb, 0), hp[NPR]), fs.at(ja + Q - 1, it),
-                                two ? fs.at(jb + Q - 1, it) : nullptr, E0, E1);
-                        cmac(acc[Q - 1], E0, ua);
-                        if (two) cmac(acc[Q - 1], E1, ub);
-                    }
+                    if constexpr (Q & 1)
+                        cmac(acc, ph<PM>(sg.x, PH::add(PH2::lane0(P0[Q / 2]), p12), fs.at(tt + Q - 1, it)), u[tt + Q - 1]);
                 }
             }
-            C *w = S + (tau * n + sl) * RR + sh * Q;
-#pragma unroll
-            for (int s0 = 0; s0 < Q; ++s0) w[s0] = acc[s0];
+            S[it] = acc;
         }
         __syncthreads();
         for (int j = threadIdx.x; j < a.T * n * RR; j += blockDim.x) Wt[j] = S[j];
@@ -1495,56 +1387,80 @@ struct Tile {
         }
     }
 
-    // ---- one row-form merge level (l -> l+1) on all tiles of the CTA.  TC caches the
-    // target features of the parents' nodes (T * 2^{Di} boxes x q^d nodes) for stage A.
-    template <int PM = PM_COMPUTE>
-    static __device__ void row_level(const KArgs<P> &a, C *Wt, C *S, typename PH::T *TC, int l, int i, R *&tb)
+    // the factors e^{2 pi i Phi(x, y0(B_c))} of the four inputs c = c_0 + 2 c_1 (+ 4 c_2 in P2) at
+    // one target node from the parts of coordinates 0 and 1 (lanes c_0 and c_1) and of coordinate 2
+    template <int PM, class Part2, class Part1, class V>
+    static __device__ __forceinline__ void four(V sg, const Part2 &P0, const Part2 &P1, const Part1 &p2, const FT &ft, int j0, int it, C *E)
     {
+        using PH2 = Ph2<P, D, K>;
+        const Part2 q = PH2::dup(p2);
+        ph2<PM>(sg, PH2::add(PH2::add(P0, P1), q), ft.at(j0, it), ft.at(j0 + 3, it), E[0], E[3]);
+        ph2<PM>(sg, PH2::add(PH2::add(P0, PH2::swap(P1)), q), ft.at(j0 + 2, it), ft.at(j0 + 1, it), E[2], E[1]);
+    }
+
+    // ---- one row-form merge level (l -> l+1) on all tiles of the CTA
+    template <int PM = PM_COMPUTE>
+    static __device__ void row_level(const KArgs<P> &a, C *Wt, C *S, int l, int i, R *&tb)
+    {
+        using PH2 = Ph2<P, D, K>;
         const int k = a.k, n = 1 << (D * k), nblk = n >> D;
         const int L = a.L;
-        const int nbox = 1 << (D * i);
         FT fa{tb, n_row_a(a)}, fb{tb, n_row_b(a)};
         if constexpr (PM != PM_COMPUTE) {
             fb.p = tb + (int64_t)fa.n * PH_ROW_A;
             tb = fb.p + (int64_t)fb.n * PH_ROW_B;
         }
-        for (int j = threadIdx.x; PM != PM_TABLE && j < a.T * nbox * RR; j += blockDim.x) {
-            const int t = j % RR, aloc = (j / RR) & (nbox - 1), tau = (j / RR) >> (D * i);
-            uint32_t Ap, Bstar;
+        // pre-modulation, in place: items (tau, block, t), the block's eight inputs at node t of the
+        // parent target box: one target point and two parts per coordinate for eight phases
+        for (int it = threadIdx.x; it < a.T * nblk * RR; it += blockDim.x) {
+            const int t = it % RR, beta = (it / RR) & (nblk - 1), tau = (it / RR) >> (D * (k - 1));
+            uint32_t Ap, Bstar, Apg, Bq;
+            int base;
             tile_of(a, tau, Ap, Bstar);
-            int ca[DMAX], tk[DMAX], tt = t;
-            morton_decode<D>((Ap << (D * i)) + aloc, l, ca);
+            block_geo(Ap, Bstar, beta, i, k, Apg, Bq, base);
+            typename PH2::Part P0{}, P1{}, P2{};
+            typename PH2::V sg{};
+            if constexpr (PM != PM_TABLE) {
+                int ca[DMAX], cb[DMAX], tk[DMAX], tt = t;
+                morton_decode<D>(Apg, l, ca);
+                morton_decode<D>(Bq, L - l - 1, cb);
 #pragma unroll
-            for (int jj = 0; jj < D; ++jj) { tk[jj] = tt % Q; tt /= Q; }
-            TC[j] = tpoint<P, D, Q, K>(a, l, ca, tk);
+                for (int j = 0; j < D; ++j) { tk[j] = tt % Q; tt /= Q; }
+                const typename PH::T tn = tpoint<P, D, Q, K>(a, l, ca, tk);
+                const typename PH2::T t2 = PH2::dup(tn);
+                sg = PH2::dup(PH::sign(a, tn));
+                P0 = PH2::part(a, t2, sget<P, Q>(a, 0, l, 2 * cb[0], Q), sget<P, Q>(a, 0, l, 2 * cb[0] + 1, Q), 0);
+                P1 = PH2::part(a, t2, sget<P, Q>(a, 1, l, 2 * cb[1], Q), sget<P, Q>(a, 1, l, 2 * cb[1] + 1, Q), 1);
+                P2 = PH2::part(a, t2, sget<P, Q>(a, 2, l, 2 * cb[2], Q), sget<P, Q>(a, 2, l, 2 * cb[2] + 1, Q), 2);
+            }
+            C *w = Wt + (tau * n + base) * RR + t;
+#pragma unroll
+            for (int c2 = 0; c2 < 2; ++c2) {
+                C E[4];
+                four<PM>(sg, P0, P1, c2 ? PH2::lane1(P2) : PH2::lane0(P2), fa, c2 * 4, it, E);
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    C &v = w[((c | (c2 << 2)) << (D * i)) * RR];
+                    v = cjmul(E[c], v);
+                }
+            }
         }
         __syncthreads();
-        // stage A: items (tau, block, c, t_{>=1}): pre-modulate input c at the nodes of the
-        // parent target box and contract dim 0 for both children alpha_0
+        // stage A: items (tau, block, c, t_{>=1}): contract dim 0 for both children alpha_0
         //   -> S[tau][block][c][t_{>=1}][alpha_0][s_0]
         for (int it = threadIdx.x; it < a.T * nblk * NC * QD1; it += blockDim.x) {
             const int th = it % QD1;
             const int c = (it / QD1) % NC;
             const int beta = (it / (QD1 * NC)) & (nblk - 1);
             const int tau = (it / (QD1 * NC)) >> (D * (k - 1));
-            uint32_t Ap, Bstar, Apg, Bq;
-            int base;
-            tile_of(a, tau, Ap, Bstar);
-            block_geo(Ap, Bstar, beta, i, k, Apg, Bq, base);
-            int cbq[DMAX], cb[DMAX];
-            morton_decode<D>(Bq, L - l - 1, cbq);
-#pragma unroll
-            for (int j = 0; j < D; ++j) cb[j] = 2 * cbq[j] + ((c >> j) & 1);
-            const int ctr[DMAX] = {Q, Q, Q};
-            const typename PH::S sc = spoint<P, D, Q, K>(a, l, cb, ctr);
-            const typename PH::T *tn = TC + (tau * nbox + (int)digit_rev<D>(beta & (nbox - 1), i)) * RR + th * Q;
+            const int base = ((beta >> (D * i)) << (D * (i + 1))) + (beta & ((1 << (D * i)) - 1));
             const C *win = Wt + tau * n * RR + (base + (c << (D * i))) * RR + th * Q;
             C z[2][Q];
 #pragma unroll
             for (int s0 = 0; s0 < Q; ++s0) { z[0][s0] = czero<C>(); z[1][s0] = czero<C>(); }
 #pragma unroll
             for (int t0 = 0; t0 < Q; ++t0) {
-                const C u = cjmul(phs<PM>(a, tn[t0], sc, fa.at(t0, it)), win[t0]);
+                const C u = win[t0];
 #pragma unroll
                 for (int s0 = 0; s0 < Q; ++s0) {
                     imac(z[0][s0], a, 0, t0, s0, u);
@@ -1556,8 +1472,10 @@ struct Tile {
             for (int s0 = 0; s0 < Q; ++s0) { so[s0] = z[0][s0]; so[Q + s0] = z[1][s0]; }
         }
         __syncthreads();
-        // stage B: items (tau, block, alpha, s_0): contract dims >= 1 per child c,
-        // post-modulate at the child's nodes, sum over c
+        // stage B: items (tau, block, alpha, s_0): for each half c_2 of the inputs and each s_2 of
+        // the child's nodes contract dim 2, then for each s_1 contract dim 1 and add the four
+        // post-modulated inputs (one target point and its parts for four phases).  The second
+        // half adds to the item's own outputs of the first.
         for (int it = threadIdx.x; it < a.T * nblk * NC * Q; it += blockDim.x) {
             const int s0 = it % Q;
             const int alpha = (it / Q) % NC;
@@ -1571,47 +1489,67 @@ struct Tile {
             int ca[DMAX], cbq[DMAX];
             morton_decode<D>(Aa, l + 1, ca);
             morton_decode<D>(Bq, L - l - 1, cbq);
-            const int a0 = alpha & 1;
-            const C *Sblk = S + ((tau * nblk + beta) * NC) * QD1 * 2 * Q;
-            C acc[QD1];
+            const int a0 = alpha & 1, a1 = (alpha >> 1) & 1, a2 = (alpha >> 2) & 1;
+            const C *Sblk = S + ((tau * nblk + beta) * NC) * QD1 * 2 * Q + a0 * Q + s0;   // [c][t1 + Q t2] stride 2Q
+            C *wo = Wt + tau * n * RR + (base + (alpha << (D * i))) * RR + s0;
+            typename P::SE e0[2], e1[2];
+            if constexpr (PM != PM_TABLE) {
 #pragma unroll
-            for (int j = 0; j < QD1; ++j) acc[j] = czero<C>();
-            {
-                const int a1 = (alpha >> 1) & 1, a2 = (alpha >> 2) & 1;
-#pragma unroll 1
-                for (int c = 0; c < NC; ++c) {
-                    int cb[DMAX], ctr[DMAX] = {Q, Q, Q};
-#pragma unroll
-                    for (int j = 0; j < D; ++j) cb[j] = 2 * cbq[j] + ((c >> j) & 1);
-                    const typename PH::S sc = spoint<P, D, Q, K>(a, l, cb, ctr);
-                    const C *si = Sblk + c * QD1 * 2 * Q + a0 * Q + s0;   // [t1 + Q t2] stride 2Q
-                    C w[Q * Q];   // [t1][s2]
-#pragma unroll
-                    for (int j = 0; j < Q * Q; ++j) w[j] = czero<C>();
-#pragma unroll
-                    for (int t2 = 0; t2 < Q; ++t2)
-#pragma unroll
-                        for (int t1 = 0; t1 < Q; ++t1) {
-                            const C zz = si[(t1 + Q * t2) * 2 * Q];
-#pragma unroll
-                            for (int s2 = 0; s2 < Q; ++s2) cfma2(w[t1 * Q + s2], a.M2[a2][t2][s2], zz);
-                        }
-#pragma unroll
-                    for (int s2 = 0; s2 < Q; ++s2)
-#pragma unroll
-                        for (int s1 = 0; s1 < Q; ++s1) {
-                            C v = czero<C>();
-#pragma unroll
-                            for (int t1 = 0; t1 < Q; ++t1) cfma2(v, a.M2[a1][t1][s1], w[t1 * Q + s2]);
-                            const int sk[DMAX] = {s0, s1, s2};
-                            const typename PH::T tS = tpoint<P, D, Q, K>(a, l + 1, ca, sk);
-                            acc[s1 + Q * s2] = cadd(acc[s1 + Q * s2], cmul(phs<PM>(a, tS, sc, fb.at((s1 + Q * s2) * NC + c, it)), v));
-                        }
+                for (int h = 0; h < 2; ++h) {
+                    e0[h] = sget<P, Q>(a, 0, l, 2 * cbq[0] + h, Q);
+                    e1[h] = sget<P, Q>(a, 1, l, 2 * cbq[1] + h, Q);
                 }
             }
-            C *wo = Wt + tau * n * RR + (base + (alpha << (D * i))) * RR + s0;
+#pragma unroll 1
+            for (int h = 0; h < 2 * Q; ++h) {
+                const int c2 = h / Q, s2 = h % Q;
+                typename P::SE e2;
+                if constexpr (PM != PM_TABLE) e2 = sget<P, Q>(a, 2, l, 2 * cbq[2] + c2, Q);
+                C w[4][Q];   // [c_0 + 2 c_1][t_1]
 #pragma unroll
-            for (int sh = 0; sh < QD1; ++sh) wo[sh * Q] = acc[sh];
+                for (int c = 0; c < 4; ++c)
+#pragma unroll
+                    for (int t1 = 0; t1 < Q; ++t1) w[c][t1] = czero<C>();
+#pragma unroll
+                for (int t2 = 0; t2 < Q; ++t2) {
+                    const R m = a.M[a2][t2][s2];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c)
+#pragma unroll
+                        for (int t1 = 0; t1 < Q; ++t1) cfma(w[c][t1], m, Sblk[((c | (c2 << 2)) * QD1 + t1 + Q * t2) * 2 * Q]);
+                }
+#pragma unroll
+                for (int s1 = 0; s1 < Q; ++s1) {
+                    C v[4];
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) v[c] = czero<C>();
+#pragma unroll
+                    for (int t1 = 0; t1 < Q; ++t1) {
+                        const R m = a.M[a1][t1][s1];
+#pragma unroll
+                        for (int c = 0; c < 4; ++c) cfma(v[c], m, w[c][t1]);
+                    }
+                    typename PH2::Part P0{}, P1{};
+                    typename PH::Part p2{};
+                    typename PH2::V sg{};
+                    if constexpr (PM != PM_TABLE) {
+                        const int sk[DMAX] = {s0, s1, s2};
+                        const typename PH::T tS = tpoint<P, D, Q, K>(a, l + 1, ca, sk);
+                        const typename PH2::T t2 = PH2::dup(tS);
+                        sg = PH2::dup(PH::sign(a, tS));
+                        P0 = PH2::part(a, t2, e0[0], e0[1], 0);
+                        P1 = PH2::part(a, t2, e1[0], e1[1], 1);
+                        p2 = PH::part(a, tS, e2, 2);
+                    }
+                    C E[4];
+                    four<PM>(sg, P0, P1, p2, fb, (s1 + Q * s2) * NC + c2 * 4, it, E);
+                    C &o = wo[(s1 + Q * s2) * Q];
+                    C acc = c2 ? o : czero<C>();
+#pragma unroll
+                    for (int c = 0; c < 4; ++c) cmac(acc, E[c], v[c]);
+                    o = acc;
+                }
+            }
         }
         __syncthreads();
     }
@@ -1689,7 +1627,6 @@ struct Tile {
         if constexpr (PM == PM_TABLE) prefetch_l2(tb, level_floats(a, true));
         C *Wt = reinterpret_cast<C *>(smem);
         C *S = Wt + a.T * (1 << (D * a.k)) * RR;
-        typename PH::T *TC = reinterpret_cast<typename PH::T *>(S + 2 * a.T * (1 << (D * a.k)) * RR);
         const int rhs = blockIdx.y;
         load(a, Wt, rhs);
         __syncthreads();
@@ -1698,7 +1635,7 @@ struct Tile {
                 const int64_t lf = level_floats(a, true);
                 if (i + 1 < a.k) prefetch_l2(tb + lf, lf);
             }
-            row_level<PM>(a, Wt, S, TC, a.l0 + i, i, tb);
+            row_level<PM>(a, Wt, S, a.l0 + i, i, tb);
         }
         if (a.flags & F_FINAL)
             final_eval(a, Wt, rhs);

@@ -237,8 +237,8 @@ cudaError_t launch_ctab(const void *kargs, void *out, int levels)
     return cudaGetLastError();
 }
 
-// W, twice that as stage scratch, and the caches of the pass: node features of the parents
-// (row) or the geometry of a level's output pairs (column); d = 2: Tile2
+// W, twice that as stage scratch and, in a column pass, the geometry of a level's output pairs;
+// d = 2: Tile2
 template <int D, int Q, class P, int K>
 size_t tile_smem(int row, int T, int k, int tab)
 {
@@ -249,8 +249,7 @@ size_t tile_smem(int row, int T, int k, int tab)
     } else {
         using TL = bfk::Tile<D, Q, P, K>;
         const size_t base = (size_t)3 * np * TL::RR * sizeof(typename P::C);
-        if (!row) return base + (size_t)np * sizeof(typename TL::Geo);
-        return base + (k > 0 ? ((size_t)T << (D * (k - 1))) * TL::RR * sizeof(typename TL::PH::T) : 0);
+        return row ? base : base + (size_t)np * sizeof(typename TL::Geo);
     }
 }
 

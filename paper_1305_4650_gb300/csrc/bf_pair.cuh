@@ -156,6 +156,15 @@ struct Ph2<PMIXT<F>, D, K> {
         return o;
     }
 
+    static __device__ __forceinline__ typename PH::Part lane1(const Part &p)
+    {
+        return typename PH::Part{p.f.y, p.h.y, p.l.y, p.g.y};
+    }
+    static __device__ __forceinline__ Part swap(const Part &p)
+    {
+        return Part{make_float2(p.f.y, p.f.x), make_float2(p.h.y, p.h.x), make_float2(p.l.y, p.l.x), make_float2(p.g.y, p.g.x)};
+    }
+
     static __device__ __forceinline__ T pair(const typename PH::T &a, const typename PH::T &b)
     {
         T t;
@@ -248,6 +257,7 @@ struct Ph2<PF64, D, K> {
     static __device__ __forceinline__ Part dup(const typename PH::Part &p) { return Part{dup(p.f), dup(p.q)}; }
     static __device__ __forceinline__ typename PH::Part lane0(const Part &p) { return typename PH::Part{p.f.x, p.q.x}; }
     static __device__ __forceinline__ typename PH::Part lane1(const Part &p) { return typename PH::Part{p.f.y, p.q.y}; }
+    static __device__ __forceinline__ Part swap(const Part &p) { return Part{make_double2(p.f.y, p.f.x), make_double2(p.q.y, p.q.x)}; }
     static __device__ __forceinline__ typename PH::T one(const T &t)
     {
         typename PH::T o;
