@@ -44,6 +44,10 @@ constexpr int DMAX = 3;
 
 enum { KIND_DOT = 0, KIND_GENRADON = 1, KIND_HYPRADON = 2, KIND_SEPARABLE = 3 };
 enum { F_INIT = 1, F_SWITCH = 2, F_FINAL = 4 };
+// KArgs::corner: grid points at the lower corners of their boxes, which are nodes of the boxes
+// (Lobatto).  SRC, TGT: the shortened levels of Tile2 and TileMR (d = 2, odd q); LEAF_*: the
+// sources' (targets') first (last) level has one node per input (output) pair (d = 3)
+enum { CORNER_SRC = 1, CORNER_TGT = 2, LEAF_SRC = 4, LEAF_TGT = 8 };
 
 // Where a kernel's phase factors come from: evaluated (PM_COMPUTE), evaluated and recorded
 // in the plan's phase table (PM_BUILD, at plan creation), or read from it (PM_TABLE)
@@ -300,7 +304,7 @@ struct KArgs {
     typename P::Sc sc;
     int L, l0, k, flags, kind;
     int T;                            // tiles per CTA (T * 2^{dk} pairs)
-    int corner;                       // CORNER_* (bf_tile2.cuh): grid points on nodes, first / last levels shortened
+    int corner;                       // CORNER_*, LEAF_*: grid points on nodes, end levels shortened
     int nrhs;                         // right-hand sides of the launch (multi-RHS kernels)
     int rc;                           // right-hand sides per scratch chunk (multi-RHS kernels)
     const void *ctab;                 // target features at box centres, levels 0..ctab_levels (or null)
@@ -974,6 +978,19 @@ struct Tile {
     {
         const int k = a.k, n = 1 << (D * k);
         const int L = a.L;
+        if (D == 3 && (a.corner & LEAF_SRC)) {   // the point is the last node: the factors cancel, level 0 reads no other node
+            for (int pr = threadIdx.x; pr < a.T * n; pr += blockDim.x) {
+                uint32_t Ap, Bstar;
+                tile_of(a, pr >> (D * k), Ap, Bstar);
+                int cb[DMAX];
+                morton_decode<D>((Bstar << (D * k)) + (pr & (n - 1)), L, cb);
+                int64_t flat = 0;
+#pragma unroll
+                for (int j = 0; j < D; ++j) flat = (flat << L) + cb[j];
+                Wt[pr * RR + RR - 1] = a.g[(int64_t)rhs * a.npts + flat];
+            }
+            return;
+        }
         const int cX[DMAX] = {0, 0, 0};
         const int ctr[DMAX] = {Q, Q, Q};
         const typename PH::T tX = tpoint<P, D, Q, K>(a, 0, cX, ctr);   // centre of X
@@ -1074,8 +1091,41 @@ struct Tile {
             if constexpr (PM != PM_TABLE) g.tA = tcenter<P, D, Q, K>(a, l + 1, Aa, ca);
         }
         __syncthreads();
+        const bool leaf = (a.corner & LEAF_SRC) && l == 0;   // inputs at their last node only
+        constexpr int END = Q - 1;
+        if (leaf) {
+            for (int jt = threadIdx.x; jt < a.T * nblk * NC * 2; jt += blockDim.x) {
+                const int chi = jt & 1, alpha = (jt >> 1) % NC, bt = (jt >> 1) / NC;
+                const Geo &g = G[bt * NC + alpha];
+                const C *Wtau = Wt + (bt >> (D * (k - 1))) * n * RR;
+                const int it = (bt * NC + alpha) * 2 * Q + chi * Q + END;
+                C acc[QD1];
+#pragma unroll
+                for (int j = 0; j < QD1; ++j) acc[j] = czero<C>();
+#pragma unroll
+                for (int cl = 0; cl < (NC >> 1); ++cl) {
+                    typename PH::Part pt{};
+                    if constexpr (PM != PM_TABLE) {
+                        pt = PH::part(a, g.tA, sget<P, Q>(a, 0, l, 2 * g.cbq[0] + (cl & 1), END), 0);
+                        pt = PH::add(pt, PH::part(a, g.tA, sget<P, Q>(a, 1, l, 2 * g.cbq[1] + (cl >> 1), END), 1));
+                        pt = PH::add(pt, PH::part(a, g.tA, sget<P, Q>(a, 2, l, 2 * g.cbq[2] + chi, END), 2));
+                    }
+                    const C e = ph<PM>(PH::sign(a, g.tA), pt, fa.at((cl * Q + END) * Q + END, it));
+                    const C u = cmul(e, Wtau[(g.base + ((cl | (chi << (D - 1))) << (D * i))) * RR + RR - 1]);
+#pragma unroll
+                    for (int t1 = 0; t1 < Q; ++t1) {
+                        const R m1 = a.M[cl >> 1][t1][END];
+#pragma unroll
+                        for (int t0 = 0; t0 < Q; ++t0) cfma(acc[t0 + Q * t1], m1 * a.M[cl & 1][t0][END], u);
+                    }
+                }
+                C *so = S + it * QD1;
+#pragma unroll
+                for (int j = 0; j < QD1; ++j) so[j] = acc[j];
+            }
+        }
         // stage A: items (tau, block, alpha, c_{D-1}, t'_{D-1}): modulate and contract dims 0..D-2
-        for (int it = threadIdx.x; it < a.T * nblk * NC * 2 * Q; it += blockDim.x) {
+        for (int it = threadIdx.x; !leaf && it < a.T * nblk * NC * 2 * Q; it += blockDim.x) {
             const int tq = it % Q;
             const int chi = (it / Q) & 1;
             const int alpha = (it / (2 * Q)) % NC;
@@ -1191,6 +1241,7 @@ struct Tile {
                 const C *si = S + ((((tau * nblk + beta) * NC + alpha) * 2 + chi) * Q) * QD1 + tl;
 #pragma unroll
                 for (int tqp = 0; tqp < Q; ++tqp) {
+                    if (leaf && tqp != END) continue;
                     const C v = si[tqp * QD1];
 #pragma unroll
                     for (int tq = 0; tq < Q; ++tq) imac(acc[tq], a, chi, tq, tqp, v);
@@ -1446,6 +1497,67 @@ struct Tile {
             }
         }
         __syncthreads();
+        if ((a.corner & LEAF_TGT) && l == L - 1) {   // outputs at their last node only
+            constexpr int END = Q - 1;
+            for (int it = threadIdx.x; it < a.T * nblk * NC * QD1; it += blockDim.x) {   // contract dim 0
+                const int th = it % QD1, c = (it / QD1) % NC, beta = (it / (QD1 * NC)) & (nblk - 1);
+                const int tau = (it / (QD1 * NC)) >> (D * (k - 1));
+                const int base = ((beta >> (D * i)) << (D * (i + 1))) + (beta & ((1 << (D * i)) - 1));
+                const C *win = Wt + tau * n * RR + (base + (c << (D * i))) * RR + th * Q;
+                C z[2] = {czero<C>(), czero<C>()};
+#pragma unroll
+                for (int t0 = 0; t0 < Q; ++t0) {
+                    cfma(z[0], a.M[0][t0][END], win[t0]);
+                    cfma(z[1], a.M[1][t0][END], win[t0]);
+                }
+                S[it * 2] = z[0];
+                S[it * 2 + 1] = z[1];
+            }
+            __syncthreads();
+            // items (tau, block, alpha, c): contract dims 1 and 2, post-modulate; sum over c below
+            C *X = S + a.T * n * RR;
+            for (int it = threadIdx.x; it < a.T * nblk * NC * NC; it += blockDim.x) {
+                const int c = it % NC, alpha = (it / NC) % NC, bt = it / (NC * NC);
+                const int beta = bt & (nblk - 1), tau = bt >> (D * (k - 1));
+                const C *si = S + (bt * NC + c) * QD1 * 2 + (alpha & 1);
+                C v = czero<C>();
+#pragma unroll
+                for (int t2 = 0; t2 < Q; ++t2) {
+                    C x = czero<C>();
+#pragma unroll
+                    for (int t1 = 0; t1 < Q; ++t1) cfma(x, a.M[(alpha >> 1) & 1][t1][END], si[(t1 + Q * t2) * 2]);
+                    cfma(v, a.M[alpha >> 2][t2][END], x);
+                }
+                typename PH::Part pt{};
+                R sg{};
+                if constexpr (PM != PM_TABLE) {
+                    uint32_t Ap, Bstar, Apg, Bq;
+                    int base, ca[DMAX], cb[DMAX];
+                    tile_of(a, tau, Ap, Bstar);
+                    block_geo(Ap, Bstar, beta, i, k, Apg, Bq, base);
+                    morton_decode<D>((Apg << D) + alpha, l + 1, ca);
+                    morton_decode<D>(Bq, L - l - 1, cb);
+                    const int sk[DMAX] = {END, END, END};
+                    const typename PH::T tS = tpoint<P, D, Q, K>(a, l + 1, ca, sk);
+                    sg = PH::sign(a, tS);
+                    pt = PH::part(a, tS, sget<P, Q>(a, 0, l, 2 * cb[0] + (c & 1), Q), 0);
+                    pt = PH::add(pt, PH::part(a, tS, sget<P, Q>(a, 1, l, 2 * cb[1] + ((c >> 1) & 1), Q), 1));
+                    pt = PH::add(pt, PH::part(a, tS, sget<P, Q>(a, 2, l, 2 * cb[2] + (c >> 2), Q), 2));
+                }
+                X[it] = cmul(ph<PM>(sg, pt, fb.at((END + Q * END) * NC + c, (bt * NC + alpha) * Q + END)), v);
+            }
+            __syncthreads();
+            for (int it = threadIdx.x; it < a.T * nblk * NC; it += blockDim.x) {
+                const int alpha = it % NC, bt = it / NC, beta = bt & (nblk - 1), tau = bt >> (D * (k - 1));
+                const int base = ((beta >> (D * i)) << (D * (i + 1))) + (beta & ((1 << (D * i)) - 1));
+                C acc = X[it * NC];
+#pragma unroll
+                for (int c = 1; c < NC; ++c) acc = cadd(acc, X[it * NC + c]);
+                Wt[(tau * n + base + (alpha << (D * i))) * RR + RR - 1] = acc;
+            }
+            __syncthreads();
+            return;
+        }
         // stage A: items (tau, block, c, t_{>=1}): contract dim 0 for both children alpha_0
         //   -> S[tau][block][c][t_{>=1}][alpha_0][s_0]
         for (int it = threadIdx.x; it < a.T * nblk * NC * QD1; it += blockDim.x) {
@@ -1570,6 +1682,13 @@ struct Tile {
             int ca[DMAX];
             morton_decode<D>(A, L, ca);
             const C *w = Wt + it * RR;
+            int64_t flat = 0;
+#pragma unroll
+            for (int j = 0; j < D; ++j) flat = (flat << L) + ca[j];
+            if (D == 3 && (a.corner & LEAF_TGT)) {   // the point is the last node: the factors cancel
+                a.f[(int64_t)rhs * a.npts + flat] = w[RR - 1];
+                continue;
+            }
             C acc = czero<C>();
             for (int t = 0; t < RR; ++t) {
                 R lag = R(1);
@@ -1582,9 +1701,6 @@ struct Tile {
             }
             const int pslot[DMAX] = {Q + 1, Q + 1, Q + 1};
             const C e = expphase<P, D, K>(a, tpoint<P, D, Q, K>(a, L, ca, pslot), sY);
-            int64_t flat = 0;
-#pragma unroll
-            for (int j = 0; j < D; ++j) flat = (flat << L) + ca[j];
             a.f[(int64_t)rhs * a.npts + flat] = cmul(e, acc);
         }
     }

@@ -60,11 +60,13 @@ inline int tiles_of(int64_t npts, int64_t np_cta, int d, int k)
     return T < 1 ? 1 : T;
 }
 
-// CORNER_* bits of a plan (bf_tile2.cuh): Lobatto kernels and grid points at the lower corners
-// of their boxes.  The first level must be a column level.  tc_levels runs every column level
-// in a pass of its own kind, with the general first step.
+// KArgs::corner of a plan: Lobatto nodes and grid points at the lower corners of their boxes.
+// The first level must be a column level.  tc_levels runs every column level in a pass of its
+// own kind, with the general first step.
 inline int corner_of(int d, int q, int m, const bf_params *p, int lobatto, bool tc)
 {
+    if (d == 3 && p->node_kind == 0)
+        return (p->src_off == 0.0 && m >= 1 ? bfk::LEAF_SRC : 0) | (p->tgt_off == 0.0 ? bfk::LEAF_TGT : 0);
     if (!lobatto || d != 2 || !(q & 1)) return 0;
     const bool src = p->src_off == 0.0 && m >= 1 && !(tc && p->tc_levels);
     return (src ? bfk::CORNER_SRC : 0) | (p->tgt_off == 0.0 ? bfk::CORNER_TGT : 0);

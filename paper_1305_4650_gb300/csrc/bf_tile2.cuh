@@ -30,8 +30,6 @@
 
 namespace bfk {
 
-enum { CORNER_SRC = 1, CORNER_TGT = 2 };   // KArgs::corner
-
 // parent node that child node u of half h coincides with, or -1 (Lobatto nodes, odd q, in
 // descending order: node 0 at +1/2, q - 1 at -1/2)
 template <int Q, bool LB>
