@@ -9,7 +9,8 @@
 namespace bfl {
 
 // Raise the kernel's dynamic shared-memory limit to what this launch needs,
-// checked against the device's opt-in maximum.  `granted` is owned by the one
+// checked against the device's opt-in maximum.  A kernel's static shared memory (under 8 KB)
+// counts against the 48 KB that need no raising.  `granted` is owned by the one
 // kernel instantiation that calls this (per device).
 template <class K>
 inline cudaError_t prepare(K kern, size_t smem, size_t *granted)
@@ -18,7 +19,7 @@ inline cudaError_t prepare(K kern, size_t smem, size_t *granted)
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (smem <= 48 * 1024 || smem <= granted[dev]) return cudaSuccess;
+    if (smem <= 40 * 1024 || smem <= granted[dev]) return cudaSuccess;
     int optin = 0;
     e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
     if (e != cudaSuccess) return e;
