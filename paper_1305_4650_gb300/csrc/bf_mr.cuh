@@ -113,15 +113,25 @@ struct MinbMR {
 
 // Padding (in complex numbers) of the shared-memory arrays read and written by the apply
 // stages, so that the 64-bit accesses of a warp fall in distinct banks (32 banks of 4
-// bytes), chosen for q = 5 by counting the wavefronts of every access pattern of the stages
-// (TileMR::spread, gather); the phase-table layout stays compact.
+// bytes), chosen per q by counting the wavefronts of every access pattern of the stages
+// (TileMR::spread, gather) for 16 pairs; the phase-table layout stays compact.  Wavefronts
+// without and with them: q = 3 1242 and 720, q = 4 5120 and 3264, q = 6 6360 and 4956,
+// q = 7 7770 and 4032, q = 8 33792 and 20736.
 struct MRPad {
     int ca;   // column modulation: per (pair, chi) block of 2 r factors
     int cb;   // column demodulation: per pair (r factors)
     int rb;   // row post-modulation: per pair (4 r factors)
     int rs;   // row scratch: per (pair, t_1) unit of 2 q partial sums
 };
-__host__ __device__ constexpr MRPad mr_pad(int q) { return q == 5 ? MRPad{7, 12, 1, 1} : MRPad{0, 0, 0, 0}; }
+__host__ __device__ constexpr MRPad mr_pad(int q)
+{
+    return q == 5   ? MRPad{7, 12, 1, 1}
+           : q & 1  ? MRPad{1, 0, 1, 1}
+           : q == 4 ? MRPad{1, 4, 8, 1}
+           : q == 6 ? MRPad{1, 2, 8, 1}
+           : q == 8 ? MRPad{1, 8, 8, 1}
+                    : MRPad{1, 2, 2, 1};
+}
 // phase-cache entries per pair beyond 5 r (evaluating passes)
 __host__ __device__ constexpr int mr_pc_extra(int q)
 {
@@ -155,6 +165,10 @@ struct TileMR {
     using TL = Tile<2, Q, P, K>;
     using T2 = Tile2<Q, P, K, LB>;
     static constexpr int MID = T2::MID, END = T2::END;
+    // lane order of spread and gather: over the nodes first for even q, whose weights of a pair
+    // (q^2 complex numbers) start in the same bank for every pair or every second one; over the
+    // pairs first for odd q
+    static constexpr bool NF = Q % 2 == 0;
 
     // geometry of one merge block of a row level (in S during the phase stage): the parent
     // target box (level l) and the parent source box (level l+1)
@@ -540,10 +554,12 @@ struct TileMR {
     // has per <= NT items per right-hand side, NT / per of them run side by side, and the item
     // decoding and the pointers are computed once per level instead of once per item.
     //
-    // Lanes run over the pairs first: with q = 5 and the paddings of mr_pad every access of spread
-    // then takes the fewest wavefronts its bytes allow, those of gather 1.4 times that at most
+    // Lanes run over the pairs first at odd q: with q = 5 and the paddings of mr_pad every access of
+    // spread then takes the fewest wavefronts its bytes allow, those of gather 1.4 times that at most
     // (counted over the access patterns for 16 pairs; lanes over nodes first took 2.2 and 1.7
-    // times, and shared-memory wavefronts are what these stages are bound by).
+    // times, and shared-memory wavefronts are what these stages are bound by).  At even q pairs first
+    // would put all lanes of a load of W into one bank (q = 4: 9280 wavefronts against 3264 with
+    // lanes over nodes first).
     //
     // spread (column level; adjoint of a row level): out_j(t) = fB(j, t) sum_c sum_u M_c[t][u]
     // fA(j, c, u) in_c(u) for the four outputs j of a block, one dimension per stage.  A stage-A
@@ -556,14 +572,15 @@ struct TileMR {
         constexpr int QA = SP ? 2 : Q;
         // stage A: items (rb, block and j_1, c_1, u_1): modulate the inputs, contract dimension 0
         const int perA = x.npr * QA, rA = NT / perA, a0 = (int)threadIdx.x % perA, rbA = (int)threadIdx.x / perA;
-        const int tp = a0 >> x.lgp, chi = (a0 >> (x.lgp - 1)) & 1, pa = (a0 << 1) & (x.npr - 1), tq = SP ? (tp ? END : MID) : tp;
+        const int tp = NF ? a0 % QA : a0 >> x.lgp, chi = NF ? (a0 / QA) & 1 : (a0 >> (x.lgp - 1)) & 1;
+        const int pa = NF ? (a0 / (2 * QA)) << 1 : (a0 << 1) & (x.npr - 1), tq = SP ? (tp ? END : MID) : tp;
         const int SH = x.npr * RR + 1;   // scratch of the outputs with j_0 = 1
         const C *winA = W + (((pa >> (D * k)) << (D * k)) + block_base((pa >> D) & (nblk - 1), i) + (chi << (D * i + 1))) * RR + Q * tq;
         const C *phA = fA(pa, chi) + tq * Q;
         C *soA = S + ((pa + chi) * Q + tq) * Q;
         // stage B: items (rb, j, t_0): contract dimension 1 and the child bit c_1
         const int perB = x.npr * Q, rB = NT / perB, b0 = (int)threadIdx.x % perB, rbB = (int)threadIdx.x / perB;
-        const int tl = b0 >> x.lgp, pj = b0 & (x.npr - 1);
+        const int tl = NF ? b0 % Q : b0 >> x.lgp, pj = NF ? b0 / Q : b0 & (x.npr - 1);
         const C *siB = S + (pj & 1) * SH + (pj >> 1) * 2 * RR + tl;
         C *woB = W + (((pj >> (D * k)) << (D * k)) + block_base((pj >> D) & (nblk - 1), i) + ((pj & (NC - 1)) << (D * i))) * RR + tl;
         const C *phB = fB(pj) + tl;
@@ -628,7 +645,7 @@ struct TileMR {
         constexpr int SU = 2 * Q + PAD.rs, QB = SP ? 2 : Q;
         // stage A: items (rb, c, t_1): modulate input c, contract dimension 0 for both bits j_0
         const int perA = x.npr * Q, rA = NT / perA, a0 = (int)threadIdx.x % perA, rbA = (int)threadIdx.x / perA;
-        const int th = a0 >> x.lgp, pin = a0 & (x.npr - 1);
+        const int th = NF ? a0 % Q : a0 >> x.lgp, pin = NF ? a0 / Q : a0 & (x.npr - 1);
         const C *winA = W + (((pin >> (D * k)) << (D * k)) + block_base((pin >> D) & (nblk - 1), i) + ((pin & (NC - 1)) << (D * i))) * RR + th * Q;
         const C *phA = fA(pin) + th * Q;
         C *soA = S + (pin * Q + th) * SU;
@@ -636,7 +653,7 @@ struct TileMR {
         // is M_0 with both indices reversed: j_1 = 1 runs dimension 1 backwards, so the
         // coefficients are compile-time operands
         const int perB = x.npr * QB, rB = NT / perB, b0 = (int)threadIdx.x % perB, rbB = (int)threadIdx.x / perB;
-        const int sp = b0 >> x.lgp, s0 = SP ? (sp ? END : MID) : sp, pj = b0 & (x.npr - 1), al = pj & (NC - 1), j0 = al & 1, j1 = al >> 1;
+        const int sp = NF ? b0 % QB : b0 >> x.lgp, s0 = SP ? (sp ? END : MID) : sp, pj = NF ? b0 / QB : b0 & (x.npr - 1), al = pj & (NC - 1), j0 = al & 1, j1 = al >> 1;
         const int rev = j1 ? -SU : SU, wst = j1 ? -Q : Q, first = j1 && !SP ? Q - 1 : 0;
         const C *siB = S + (pj - al) * Q * SU + j0 * Q + s0 + (j1 ? (Q - 1) * SU : 0);
         C *woB = W + (((pj >> (D * k)) << (D * k)) + block_base((pj >> D) & (nblk - 1), i) + (al << (D * i))) * RR + s0 + first * Q;
