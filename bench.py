@@ -44,7 +44,7 @@ FP32_LANES_PER_SM = 128
 TRAFFIC = {"genradon2d": {"src_sha256": "dc76e76eb7bedb887e3406a09fcc93cc26f2fb4562519df8098120ea50debe0d",
                           "schedule": ["col2", "col3", "row2", "row3"],
                           "bytes": [161666560, 1272867328, 369475328, 215727104]}}
-TRAFFIC_SRC = ("bf_device.cuh", "bf_inst.cuh")   # the pass kernels and their launch configuration
+TRAFFIC_SRC = ("bf_device.cuh", "bf_tile2.cuh", "bf_host.h", "bf_inst.cuh")   # the pass kernels and their launch configuration
 
 
 def measured_hbm_gbs():

@@ -803,6 +803,11 @@ struct Cfg {
     static constexpr int MINB_TAB = D == 2 ? per_sm(640) + 1 : MINB;
 };
 
+// launch bounds for the registers of minb CTAs of nt threads per SM; at d = 2 as one CTA with the
+// threads of all of them, which is the same budget and lets a small grid launch such CTAs
+constexpr int cta_most(int nt, int minb, int d) { return d == 2 ? nt * minb : nt; }
+constexpr int cta_least(int minb, int d) { return d == 2 ? 1 : minb; }
+
 template <int D, int Q, class P, int K>
 struct Tile {
     using R = typename P::R;
@@ -2292,7 +2297,8 @@ template <int Q, class P, int K, bool LB> struct TileOf<2, Q, P, K, LB> { using 
 // accordingly): measured 7% faster with the polynomial sincos, 19% with the SFU one; the row
 // pass would spill.  At d = 3 the shared memory holds two CTAs per SM either way.
 template <int D, int Q, class P, int K, bool LB, int PM = PM_COMPUTE>
-__global__ void __launch_bounds__(Cfg<D, Q, P>::NT, PM == PM_TABLE ? Cfg<D, Q, P>::MINB_TAB : Cfg<D, Q, P>::MINB_COL)
+__global__ void __launch_bounds__(cta_most(Cfg<D, Q, P>::NT, PM == PM_TABLE ? Cfg<D, Q, P>::MINB_TAB : Cfg<D, Q, P>::MINB_COL, D),
+                                  cta_least(PM == PM_TABLE ? Cfg<D, Q, P>::MINB_TAB : Cfg<D, Q, P>::MINB_COL, D))
     k_col_pass(const KArgs<P> a)
 {
     static_assert(PM == PM_COMPUTE || !P::is_f64, "phase tables: mixed precisions");
@@ -2312,7 +2318,8 @@ __global__ void __launch_bounds__(Cfg<D, Q, P>::NT, PM == PM_TABLE ? Cfg<D, Q, P
 
 // k row merges + optional final evaluation (l0 + k = L)
 template <int D, int Q, class P, int K, bool LB, int PM = PM_COMPUTE>
-__global__ void __launch_bounds__(Cfg<D, Q, P>::NT, Cfg<D, Q, P>::MINB_ROW) k_row_pass(const KArgs<P> a)
+__global__ void __launch_bounds__(cta_most(Cfg<D, Q, P>::NT, Cfg<D, Q, P>::MINB_ROW, D), cta_least(Cfg<D, Q, P>::MINB_ROW, D))
+    k_row_pass(const KArgs<P> a)
 {
     static_assert(PM == PM_COMPUTE || !P::is_f64, "phase tables: mixed precisions");
     using TL = typename TileOf<D, Q, P, K, LB>::type;
@@ -2331,7 +2338,8 @@ __global__ void __launch_bounds__(Cfg<D, Q, P>::NT, Cfg<D, Q, P>::MINB_ROW) k_ro
 // adjoint of a column pass: optional switch^H at level l0 + k, k column levels in
 // reverse, optional init^H (writes the source values)
 template <int D, int Q, class P, int K, bool LB>
-__global__ void __launch_bounds__(Cfg<D, Q, P>::NT, Cfg<D, Q, P>::MINB) k_col_pass_adj(const KArgs<P> a)
+__global__ void __launch_bounds__(cta_most(Cfg<D, Q, P>::NT, Cfg<D, Q, P>::MINB, D), cta_least(Cfg<D, Q, P>::MINB, D))
+    k_col_pass_adj(const KArgs<P> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TileOf<D, Q, P, K, LB>::type::col_pass_adj(a, smem_raw);
@@ -2339,7 +2347,8 @@ __global__ void __launch_bounds__(Cfg<D, Q, P>::NT, Cfg<D, Q, P>::MINB) k_col_pa
 
 // adjoint of a row pass: optional final^H (reads the target values), k row levels in reverse
 template <int D, int Q, class P, int K, bool LB>
-__global__ void __launch_bounds__(Cfg<D, Q, P>::NT, Cfg<D, Q, P>::MINB) k_row_pass_adj(const KArgs<P> a)
+__global__ void __launch_bounds__(cta_most(Cfg<D, Q, P>::NT, Cfg<D, Q, P>::MINB, D), cta_least(Cfg<D, Q, P>::MINB, D))
+    k_row_pass_adj(const KArgs<P> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     TileOf<D, Q, P, K, LB>::type::row_pass_adj(a, smem_raw);

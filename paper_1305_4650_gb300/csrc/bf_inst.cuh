@@ -30,13 +30,17 @@ inline cudaError_t prepare(K kern, size_t smem, size_t *granted)
     return cudaSuccess;
 }
 
-// threads of a single-RHS pass: q per pair at d = 2 (at least four pairs), the compiled number at d = 3
+// threads of a single-RHS pass: q per pair at d = 2 (at least four pairs), the compiled number at
+// d = 3.  A grid of at most one CTA per SM leaves the SMs to single CTAs: at d = 2 each then gets the
+// threads of the `per_sm` CTAs that the registers are cut for, so that stages of more than q items
+// per pair (the switch, the first column stage, the first and last step) take fewer rounds.
+constexpr unsigned SMS = 152;
 template <int D, int Q, class P>
-unsigned tile_threads(int T, int k)
+unsigned tile_threads(int T, int k, unsigned ctas, int per_sm)
 {
     if constexpr (D == 3) return bfk::Cfg<D, Q, P>::NT;
     const int np = T << (D * k);
-    return (unsigned)((np < 4 ? 4 : np) * Q);
+    return (unsigned)((np < 4 ? 4 : np) * Q) * (ctas <= SMS ? (unsigned)per_sm : 1u);
 }
 
 template <int D, int Q, class P, int K, bool LB, int PM = bfk::PM_COMPUTE>
@@ -46,7 +50,8 @@ cudaError_t launch_col(const void *kargs, unsigned gx, unsigned gy, size_t smem,
     cudaError_t e = prepare(bfk::k_col_pass<D, Q, P, K, LB, PM>, smem, granted);
     if (e != cudaSuccess) return e;
     const bfk::KArgs<P> &a = *static_cast<const bfk::KArgs<P> *>(kargs);
-    bfk::k_col_pass<D, Q, P, K, LB, PM><<<dim3(gx, gy), tile_threads<D, Q, P>(a.T, a.k), smem, s>>>(a);
+    const unsigned nt = tile_threads<D, Q, P>(a.T, a.k, gx * gy, PM == bfk::PM_TABLE ? bfk::Cfg<D, Q, P>::MINB_TAB : bfk::Cfg<D, Q, P>::MINB_COL);
+    bfk::k_col_pass<D, Q, P, K, LB, PM><<<dim3(gx, gy), nt, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -57,7 +62,8 @@ cudaError_t launch_row(const void *kargs, unsigned gx, unsigned gy, size_t smem,
     cudaError_t e = prepare(bfk::k_row_pass<D, Q, P, K, LB, PM>, smem, granted);
     if (e != cudaSuccess) return e;
     const bfk::KArgs<P> &a = *static_cast<const bfk::KArgs<P> *>(kargs);
-    bfk::k_row_pass<D, Q, P, K, LB, PM><<<dim3(gx, gy), tile_threads<D, Q, P>(a.T, a.k), smem, s>>>(a);
+    const unsigned nt = tile_threads<D, Q, P>(a.T, a.k, gx * gy, bfk::Cfg<D, Q, P>::MINB_ROW);
+    bfk::k_row_pass<D, Q, P, K, LB, PM><<<dim3(gx, gy), nt, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -68,7 +74,8 @@ cudaError_t launch_col_adj(const void *kargs, unsigned gx, unsigned gy, size_t s
     cudaError_t e = prepare(bfk::k_col_pass_adj<D, Q, P, K, LB>, smem, granted);
     if (e != cudaSuccess) return e;
     const bfk::KArgs<P> &a = *static_cast<const bfk::KArgs<P> *>(kargs);
-    bfk::k_col_pass_adj<D, Q, P, K, LB><<<dim3(gx, gy), tile_threads<D, Q, P>(a.T, a.k), smem, s>>>(a);
+    const unsigned nt = tile_threads<D, Q, P>(a.T, a.k, gx * gy, bfk::Cfg<D, Q, P>::MINB);
+    bfk::k_col_pass_adj<D, Q, P, K, LB><<<dim3(gx, gy), nt, smem, s>>>(a);
     return cudaGetLastError();
 }
 
@@ -79,7 +86,8 @@ cudaError_t launch_row_adj(const void *kargs, unsigned gx, unsigned gy, size_t s
     cudaError_t e = prepare(bfk::k_row_pass_adj<D, Q, P, K, LB>, smem, granted);
     if (e != cudaSuccess) return e;
     const bfk::KArgs<P> &a = *static_cast<const bfk::KArgs<P> *>(kargs);
-    bfk::k_row_pass_adj<D, Q, P, K, LB><<<dim3(gx, gy), tile_threads<D, Q, P>(a.T, a.k), smem, s>>>(a);
+    const unsigned nt = tile_threads<D, Q, P>(a.T, a.k, gx * gy, bfk::Cfg<D, Q, P>::MINB);
+    bfk::k_row_pass_adj<D, Q, P, K, LB><<<dim3(gx, gy), nt, smem, s>>>(a);
     return cudaGetLastError();
 }
 
