@@ -37,13 +37,11 @@ FP32_LANES_PER_SM = 128
 
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) per launch of each pass of the default
 # workload, from one ncu capture of `python bench.py --steps 1 --warmup 1 --no-cpu-baseline --no-accuracy
-# --fp64-steps 0 --no-autotune --no-tables --no-batched` (the dominant pass writes 0.85 GB more than its
-# weights: register spills of its switch at three CTAs per SM reach DRAM).  They describe the kernels as
-# built from sources with the recorded hash and the recorded pass schedule; otherwise the figure is
+# --fp64-steps 0 --no-autotune --no-tables --no-batched`.  They describe the kernels as built from sources with the recorded hash and the recorded pass schedule; otherwise the figure is
 # dropped (traffic: null) until captured again.
-TRAFFIC = {"genradon2d": {"src_sha256": "dc76e76eb7bedb887e3406a09fcc93cc26f2fb4562519df8098120ea50debe0d",
+TRAFFIC = {"genradon2d": {"src_sha256": "00764ea7840952519b62d7bbfd2537b3adc4fa300fed5c36c8a98ec233cb1638",
                           "schedule": ["col2", "col3", "row2", "row3"],
-                          "bytes": [161666560, 1272867328, 369475328, 215727104]}}
+                          "bytes": [157255936, 368046336, 369234176, 215354368]}}
 TRAFFIC_SRC = ("bf_device.cuh", "bf_tile2.cuh", "bf_host.h", "bf_inst.cuh")   # the pass kernels and their launch configuration
 
 
