@@ -73,6 +73,14 @@ struct Tile2 {
     static constexpr int PROW = NCMP * QE;                     // numbers of one row: [component][QE]
     static constexpr int PSTR = 6 * PROW;                      // numbers of one pair: [coordinate][child 0, child 1, output]
 
+    // bytes of n arrays of r complex numbers per pair (W, the stage scratch), rounded up to the 16 bytes
+    // that the geometry behind them is aligned to: one pair of odd q (a sharded apply of four
+    // points) ends at 8 mod 16
+    static __host__ __device__ constexpr size_t arrays(int np, int n)
+    {
+        return ((size_t)np * n * RR * sizeof(C) + 15) & ~(size_t)15;
+    }
+
     // geometry of one output pair of a column level
     struct __align__(16) Geo {
         typename PH::T tA;   // features of the target box centre
@@ -865,14 +873,14 @@ struct Tile2 {
     static __host__ __device__ size_t row_adj_smem(int np, int T, int k)
     {
         const size_t boxes = (size_t)T * ((((size_t)1 << (D * k)) - 1) / 3);   // levels 0 .. k-1 of the tiles
-        return (size_t)np * (3 + NC) * RR * sizeof(C) + (size_t)k * (size_t)(np >> D) * sizeof(GeoR) + boxes * RR * sizeof(typename PH::T);
+        return arrays(np, 3 + NC) + (size_t)k * (size_t)(np >> D) * sizeof(GeoR) + boxes * RR * sizeof(typename PH::T);
     }
 
     static __device__ __forceinline__ void col_pass_adj(const KArgs<P> &a, unsigned char *smem)
     {
         const int np = npr(a), rhs = blockIdx.y;
         C *Wt = reinterpret_cast<C *>(smem), *S = Wt + np * RR;
-        Geo *G = reinterpret_cast<Geo *>(S + 2 * np * RR);
+        Geo *G = reinterpret_cast<Geo *>(smem + arrays(np, 3));
         R *PT = reinterpret_cast<R *>(reinterpret_cast<int4 *>(G + 2 * np) + np);
         const bool skip0 = LB && (a.corner & CORNER_SRC) && (a.flags & F_INIT), sp1 = LB && (a.corner & CORNER_SRC);
         const int i0 = skip0 ? 1 : 0;
@@ -933,7 +941,7 @@ struct Tile2 {
     {
         const int np = npr(a), rhs = blockIdx.y, nb = np >> D;
         C *Wt = reinterpret_cast<C *>(smem), *S = Wt + np * RR, *X = S + 2 * np * RR;
-        GeoR *G = reinterpret_cast<GeoR *>(X + NC * np * RR);
+        GeoR *G = reinterpret_cast<GeoR *>(smem + arrays(np, 3 + NC));
         typename PH::T *TC = reinterpret_cast<typename PH::T *>(G + a.k * nb);
         auto tc = [&](int i) { return TC + a.T * (((1 << (D * i)) - 1) / 3) * RR; };   // nodes of level l0 + i
         const bool skip = LB && (a.corner & CORNER_TGT) && (a.flags & F_FINAL);
@@ -994,12 +1002,12 @@ struct Tile2 {
     // geometry and the node features (two levels)
     static __host__ __device__ size_t col_smem(int np, bool tab)
     {
-        return (size_t)np * (3 * RR * sizeof(C) + (tab ? 0 : PSTR * sizeof(R)) + 2 * sizeof(Geo) + sizeof(int4));
+        return arrays(np, 3) + (size_t)np * ((tab ? 0 : PSTR * sizeof(R)) + 2 * sizeof(Geo) + sizeof(int4));
     }
     static __host__ __device__ size_t row_smem(int np, int T, int k, bool tab)
     {
         const size_t big = k > 0 ? (size_t)T << (D * (k - 1)) : 0, small = k > 1 ? (size_t)T << (D * (k - 2)) : 0;
-        return (size_t)np * 3 * RR * sizeof(C) + (tab ? 0 : (big + small) * RR * sizeof(typename PH::T)) +
+        return arrays(np, 3) + (tab ? 0 : (big + small) * RR * sizeof(typename PH::T)) +
                2 * (size_t)(np >> D) * sizeof(GeoR);
     }
 
@@ -1008,7 +1016,7 @@ struct Tile2 {
     {
         const int np = npr(a), rhs = blockIdx.y;
         C *Wt = reinterpret_cast<C *>(smem), *S = Wt + np * RR;
-        Geo *G = reinterpret_cast<Geo *>(S + 2 * np * RR);
+        Geo *G = reinterpret_cast<Geo *>(smem + arrays(np, 3));
         int4 *GS = reinterpret_cast<int4 *>(G + 2 * np);
         R *PT = reinterpret_cast<R *>(GS + np);
         const int nlev = (int)level_floats(a);
@@ -1082,7 +1090,7 @@ struct Tile2 {
     {
         const int np = npr(a), rhs = blockIdx.y;
         C *Wt = reinterpret_cast<C *>(smem), *S = Wt + np * RR;
-        GeoR *G = reinterpret_cast<GeoR *>(S + 2 * np * RR);
+        GeoR *G = reinterpret_cast<GeoR *>(smem + arrays(np, 3));
         const int big = a.k > 0 ? a.T << (D * (a.k - 1)) : 0;
         typename PH::T *T0 = reinterpret_cast<typename PH::T *>(G + 2 * (np >> D)), *T1 = T0 + big * RR;
         // level i's nodes: the larger buffer for the last level, alternating before it
