@@ -387,6 +387,7 @@ struct TileMR {
             }
             float4 *w4 = reinterpret_cast<float4 *>(W);
             for (int j = threadIdx.x; j < (x.nr * WS * (int)sizeof(C)) / 16; j += NT) w4[j] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (sizeof(C) == 8 && (x.nr * WS & 1) && threadIdx.x == 0) W[x.nr * WS - 1] = czero<C>();   // one pair, odd q
             __syncthreads();
             for (int j = threadIdx.x; j < x.nr * x.npr * nnz; j += NT) {
                 const int z = j % nnz, pr = (j / nnz) & (x.npr - 1), rb = (j / nnz) >> x.lgp;

@@ -47,3 +47,15 @@ def check(bf, spec, nrhs, precision, sg):
 def test_one_right_hand_side(bf, L, q, m, sg, off, phase, precision):
     base = wl.genradon2d(L, precision)
     check(bf, base.with_(q=q, m=m, phase=phase, tgt_off=off, src_off=off), 1, precision, sg)
+
+
+@pytest.mark.parametrize("nrhs", [2, 3, 17])
+@pytest.mark.parametrize("off,node_kind", [(0.0, 0), (0.5, 0), (0.25, 1)])
+@pytest.mark.parametrize("L,q,m,sg", [(1, 3, None, 2), (1, 5, None, 2), (1, 4, None, 2), (2, 5, 0, 2), (2, 3, None, 1)])
+def test_several_right_hand_sides(bf, L, q, m, sg, off, node_kind, nrhs):
+    """One pair of odd q and an odd number of right-hand sides: the weights of the first step are an
+    odd number of complex numbers, every one of them set."""
+    spec = wl.genradon2d(L).with_(q=q, m=m, phase="hypradon" if nrhs == 2 else "genradon", tgt_off=off, src_off=off, node_kind=node_kind)
+    if spec.phase == "hypradon":
+        spec = spec.with_(x_lo=(1.0, 0.0, 0.0), y_lo=(1.0, 0.0, 0.0), y_w=(1.0, 1.0, 1.0), scale=float(1 << L))
+    check(bf, spec, nrhs, "mixed", sg)
