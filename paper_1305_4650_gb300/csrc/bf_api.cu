@@ -41,6 +41,7 @@ struct bf_plan_s {
     void *ctab = nullptr;      // target features at box centres, levels 0..ctab_levels
     int ctab_levels = -1;
     int corner = 0;            // CORNER_* of the forward passes
+    bool wide = false;         // exact sums under the root (wide_root)
     void *gstage = nullptr, *fstage = nullptr;
     size_t csize = 8;          // bytes per complex number
     int64_t ws_bytes = 0;
@@ -85,10 +86,18 @@ struct bf_batch_s {
 };
 
 namespace bfl {
-const PassFns *get_fns(int d, int q, int prec, int kind, int nk)
+const PassFns *get_fns(int d, int q, int prec, int kind, int nk, bool wide)
 {
 #define BFL_PICK(dd, kn) \
     (prec == 0 ? fns_d##dd##_f64_##kn(q, nk) : prec == 1 ? fns_d##dd##_mix_##kn(q, nk) : fns_d##dd##_sfu_##kn(q, nk))
+#define BFL_PICKW(dd, kn) (prec == 1 ? fns_d##dd##_mixw_##kn(q, nk) : fns_d##dd##_sfuw_##kn(q, nk))
+    if (wide && prec != 0) {
+        if (d == 2 && kind == BF_PHASE_GENRADON) return BFL_PICKW(2, genradon);
+        if (d == 2 && kind == BF_PHASE_HYPRADON) return BFL_PICKW(2, hypradon);
+        if (d == 3 && kind == BF_PHASE_GENRADON) return BFL_PICKW(3, genradon);
+        return nullptr;
+    }
+#undef BFL_PICKW
     if (d == 2) {
         switch (kind) {
         case BF_PHASE_DOT: return BFL_PICK(2, dot);
@@ -970,7 +979,7 @@ void build_weight_maps(bf_plan p)
     p->tmaps = d;
 }
 
-bool supported_q(int d, int q) { return bfl::get_fns(d, q, 1, 0, 0) != nullptr && bfl::get_fns(d, q, 0, 0, 0) != nullptr; }
+bool supported_q(int d, int q) { return bfl::get_fns(d, q, 1, 0, 0, false) != nullptr && bfl::get_fns(d, q, 0, 0, 0, false) != nullptr; }
 
 }  // namespace
 
@@ -1206,7 +1215,8 @@ bf_status bf_plan_create(int d, int64_t N, int q, bf_phase_kind phase, const bf_
     p->prm = *prm;
     p->csize = p->prec == BF_PREC_FP64 ? 16 : 8;
     // BF16X3 and TF32X3 evaluate their phases as BF_PREC_MIXED does and run the same kernels but the switch
-    p->fns = bfl::get_fns(d, q, tc_prec(p->prec) ? (int)BF_PREC_MIXED : (int)p->prec, (int)phase, p->node_kind);
+    p->wide = bfl::wide_root(d, (int)phase, prm);
+    p->fns = bfl::get_fns(d, q, tc_prec(p->prec) ? (int)BF_PREC_MIXED : (int)p->prec, (int)phase, p->node_kind, p->wide);
     if (!p->fns) {   // this combination was not compiled into the library
         delete p;
         return BF_ERR_UNSUPPORTED;
@@ -1657,6 +1667,9 @@ bf_status bf_batch_create(const bf_plan *plans, const int *nrhs, int count, bf_b
     b->count = count;
     b->prec = p0->prec;
     b->fns = p0->fns;
+    // one kernel for all problems: the exact sums give plans on the common grid what they had
+    for (int i = 0; i < count; ++i)
+        if (plans[i]->wide) b->fns = plans[i]->fns;
     bf_status st = b->prec == BF_PREC_MIXED_SFU ? batch_build<bfk::PMIXF>(b, plans, nrhs, count)
                                                 : batch_build<bfk::PMIX>(b, plans, nrhs, count);
     if (st != BF_OK) {
@@ -1787,7 +1800,7 @@ bf_status bf_selfcheck_phase(bf_plan p, int n, double *max_err_cycles)
     bfk::KArgs<bfk::PF64> ad;
     fill_args<bfk::PMIX>(p, am);
     fill_args<bfk::PF64>(p, ad);
-    cudaError_t e = bfl::selfcheck_phase(&am, &ad, p->d, p->L, p->q, p->kind, n, max_err_cycles);
+    cudaError_t e = bfl::selfcheck_phase(&am, &ad, p->wide, p->d, p->L, p->q, p->kind, n, max_err_cycles);
     if (e != cudaSuccess) return cuda_fail(p, e);
     return BF_OK;
 }
@@ -1798,7 +1811,7 @@ bf_status bf_measure_phase_rate(bf_plan p, int paired, double *gphases_per_s)
         return BF_ERR_INVALID_ARG;
     bfk::KArgs<bfk::PMIX> am;
     fill_args<bfk::PMIX>(p, am);
-    cudaError_t e = bfl::phase_rate(&am, p->prec == BF_PREC_MIXED_SFU, p->L, p->q, p->kind, paired, gphases_per_s);
+    cudaError_t e = bfl::phase_rate(&am, p->prec == BF_PREC_MIXED_SFU, p->wide, p->L, p->q, p->kind, paired, gphases_per_s);
     if (e != cudaSuccess) return cuda_fail(p, e);
     return BF_OK;
 }

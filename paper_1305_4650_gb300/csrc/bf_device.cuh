@@ -164,8 +164,10 @@ struct MixSE { float4 a; };     // (f0.hi, f0.lo, f1.hi, f1.lo)
 struct MixSc { float c2hi, c2lo, sgn, mg; };   // 2|s|/3, sign(s), grid constant of the sqrt parts (Ph::quant)
 
 // complex64 weights, double-float phase; SFU = true takes sin/cos of the reduced phase
-// from the special-function unit (__sincosf) instead of the polynomial below
-template <bool SFU>
+// from the special-function unit (__sincosf) instead of the polynomial below.  WIDE = true: the
+// terms under a root are added with their rounding error kept (Ph::add), for plans whose roots
+// are too large, and too uneven, for the common grid of Ph::quant (bfl::wide_root)
+template <bool SFU, bool WIDE = false>
 struct PMIXT {
     using R = float;
     using C = float2;
@@ -177,6 +179,8 @@ struct PMIXT {
 };
 using PMIX = PMIXT<false>;
 using PMIXF = PMIXT<true>;
+using PMIXW = PMIXT<false, true>;    // the same layouts and arguments as PMIX and PMIXF
+using PMIXFW = PMIXT<true, true>;
 
 // sin and cos of 2 pi v in FP64, v not reduced: v = k/512 + r with |r| <= 1/1024, cos and sin of
 // 2 pi k/512 from a table (8 KB, read through L1) and of 2 pi r from two short polynomials
@@ -409,8 +413,8 @@ template <int Q> __device__ __forceinline__ int soff(int L, int l) { return ((2 
 
 template <class P, int D, int K> struct Ph;
 
-template <bool F, int D, int K>
-struct Ph<PMIXT<F>, D, K> {
+template <bool F, bool W, int D, int K>
+struct Ph<PMIXT<F, W>, D, K> {
     struct T { df x[D]; df A[D]; };
     struct S { df y[D]; df y2[D]; };
 
@@ -419,7 +423,7 @@ struct Ph<PMIXT<F>, D, K> {
 
     // target point from its per-dimension table entries.  GENRADON: A_k = (s a_k(x))^2, from
     // features that carry the factor sqrt(|s|/3); HYPRADON: A_0 = (s x_0)^2, A_1 = (s x_0 x_1)^2
-    static __device__ __forceinline__ T tgt(const KArgs<PMIXT<F>> &a, const MixTE *e)
+    static __device__ __forceinline__ T tgt(const KArgs<PMIXT<F, W>> &a, const MixTE *e)
     {
         T t;
 #pragma unroll
@@ -451,8 +455,11 @@ struct Ph<PMIXT<F>, D, K> {
     // (add), and fin() turns their sum into Phi minus an integer.  f: a linear phase mod 1.
     // h + l: a term of the sum of squares under the root, h a multiple of a power of two G
     // (quant) such that the sum of the parts' h, below 2^22 G, is exact: adding two terms takes
-    // two additions instead of an exact sum of double-floats.  Loops hoist the
-    // parts of the source coordinates that do not change.  g: at d = 2 the second linear part of
+    // two additions instead of an exact sum of double-floats.  The remainder l, at most G/2 of the
+    // plan, then holds the bits below G, so the sum is good to 2^-24 G and its root to that over
+    // twice the root; W: h and l are the term's double-float (sc.mg = 0) and the sum of the h is
+    // made exact by its rounding error, good to 2^-44 of the sum itself (six more additions).
+    // Loops hoist the parts of the source coordinates that do not change.  g: at d = 2 the second linear part of
     // a kind without a root, not added to the first (fin2), so that their sum is never rounded.
     static constexpr bool HAS_F = K != KIND_HYPRADON, HAS_Q = K == KIND_GENRADON || K == KIND_HYPRADON;
     static constexpr bool PAIR_F = !HAS_Q && D == 2;
@@ -470,14 +477,14 @@ struct Ph<PMIXT<F>, D, K> {
     }
     // h = p rounded to a multiple of G (sc.mg = 1.5 * 2^23 G, p < 2^22 G); the first part adds
     // a tiny number that keeps the root's argument positive
-    static __device__ __forceinline__ void quant(const KArgs<PMIXT<F>> &a, const df &p, bool first, Part &o)
+    static __device__ __forceinline__ void quant(const KArgs<PMIXT<F, W>> &a, const df &p, bool first, Part &o)
     {
         o.h = __fsub_rn(__fadd_rn(p.hi, a.sc.mg), a.sc.mg);
         o.l = __fadd_rn(__fsub_rn(p.hi, o.h), p.lo);
         o.l = __fadd_rn(o.l, first ? 1e-30f : 0.0f);
     }
     // the part of one source coordinate from the target's features x and A of that coordinate
-    static __device__ __forceinline__ Part part_of(const KArgs<PMIXT<F>> &a, const df &x, const df &A, const MixSE &e, bool first)
+    static __device__ __forceinline__ Part part_of(const KArgs<PMIXT<F, W>> &a, const df &x, const df &A, const MixSE &e, bool first)
     {
         Part p{0.0f, 0.0f, 0.0f, 0.0f};
         if constexpr (K == KIND_DOT || K == KIND_GENRADON) p.f = df_mul_frac(x, hi(e.a));
@@ -485,7 +492,7 @@ struct Ph<PMIXT<F>, D, K> {
         if constexpr (HAS_Q) quant(a, df_mul_u(A, lo(e.a)), first, p);
         return p;
     }
-    static __device__ __forceinline__ Part part(const KArgs<PMIXT<F>> &a, const T &t, const MixSE &e, int k)
+    static __device__ __forceinline__ Part part(const KArgs<PMIXT<F, W>> &a, const T &t, const MixSE &e, int k)
     {
         return part_of(a, t.x[k], t.A[k], e, k == 0);
     }
@@ -501,11 +508,12 @@ struct Ph<PMIXT<F>, D, K> {
         if constexpr (HAS_Q) {
             p.h = __fadd_rn(u.h, v.h);
             p.l = __fadd_rn(u.l, v.l);
+            if constexpr (W) p.l = __fadd_rn(p.l, two_sum(u.h, v.h).lo);
         }
         return p;
     }
     // sign of the root's term at a target
-    static __device__ __forceinline__ float sign(const KArgs<PMIXT<F>> &a, const T &t)
+    static __device__ __forceinline__ float sign(const KArgs<PMIXT<F, W>> &a, const T &t)
     {
         if constexpr (K == KIND_HYPRADON)
             return copysignf(1.0f, t.x[0].hi);
@@ -529,7 +537,7 @@ struct Ph<PMIXT<F>, D, K> {
     }
 
     // Phi(x, y) minus an integer, |result| < 3 (the sincos reduces it further)
-    static __device__ __forceinline__ float frac(const KArgs<PMIXT<F>> &a, const T &t, const S &s)
+    static __device__ __forceinline__ float frac(const KArgs<PMIXT<F, W>> &a, const T &t, const S &s)
     {
         Part p = part(a, t, MixSE{make_float4(s.y[0].hi, s.y[0].lo, s.y2[0].hi, s.y2[0].lo)}, 0);
 #pragma unroll

@@ -39,12 +39,46 @@ inline double phase_bound(int d, int kind, const bf_params *p)
     return lin + root;
 }
 
+// Lower bound over X x Y of the root part of |Phi| (0 for the kinds without a root).
+inline double root_floor(int d, int kind, const bf_params *p)
+{
+    double nx[3], ny[3], q2 = 0.0;   // distances of the intervals from 0
+    auto gap = [](double lo, double w) { return lo > 0.0 ? lo : (lo + w < 0.0 ? -(lo + w) : 0.0); };
+    for (int k = 0; k < d; ++k) {
+        nx[k] = gap(p->x_lo[k], p->x_w[k]);
+        ny[k] = gap(p->y_lo[k], p->y_w[k]);
+        q2 += ny[k] * ny[k];
+    }
+    const double s = std::fabs(p->phase_scale);
+    if (kind == BF_PHASE_GENRADON) return s * std::sqrt(q2) / 3.0;   // a_k(x) >= 1/3
+    if (kind == BF_PHASE_HYPRADON) return s * nx[0] * std::sqrt(ny[0] * ny[0] + ny[1] * ny[1] * nx[1] * nx[1]);
+    return 0.0;
+}
+
+// Whether the mixed precisions keep the rounding error of the sums under the root (PMIXW; the
+// kernels of get_fns(..., wide)).  With the common grid G of sqrt_grid, G < 2^-20 R^2 for
+// roots up to R, a sum is good to about 2^-23 G and a root x to 2^-44 R^2 / x; below
+// x = 2^-10.5 R, where the terms are smaller than G/2 and FP32 holds them relative to themselves,
+// the error falls again.  The grid serves plans where that is at most 6e-8 cycles (2^-24, the spacing of
+// the FP32 numbers below 1 that the reduced phase is made of): roots up to 724 cycles whatever the
+// domain, and any root of a domain away from the origin (hyperbolic Radon, tau in [1, 2): up to 4.5
+// times the smallest one).  NumPy restatement, worst error over all roots, grid and exact sums:
+// R = 724 3.8e-8 and 2.7e-8, 5.7e3 2.3e-7 and 2.9e-8, 3.3e4 1.2e-6 and 3.0e-8, 1.5e6 6.0e-5 and 4.2e-8.
+inline bool wide_root(int d, int kind, const bf_params *p)
+{
+    if (p->precision == BF_PREC_FP64 || (kind != BF_PHASE_GENRADON && kind != BF_PHASE_HYPRADON)) return false;
+    double lin, root;
+    phase_bounds(d, kind, p, &lin, &root);
+    const double x = std::fmax(root_floor(d, kind, p), std::exp2(-10.5) * root);
+    return std::exp2(-44.0) * root * root > 6e-8 * x;
+}
+
 // 1.5 * 2^23 G with G the smallest power of two for which every term of the sum of squares
 // under the root, and the sum, is at most 2^21 G: the terms rounded to multiples of G
-// (Ph::quant) then add without rounding, and differ by a multiple of G that FP32 holds from
-// the square of any integer next to the root.
+// (Ph::quant) then add without rounding.  0 for wide roots: the terms stay as they are.
 inline float sqrt_grid(int d, int kind, const bf_params *p)
 {
+    if (wide_root(d, kind, p)) return 0.0f;
     double lin, root;
     phase_bounds(d, kind, p, &lin, &root);
     int e = -60;

@@ -54,10 +54,11 @@ struct PassFns {
 };
 
 // (d, q, precision, phase kind, node kind) -> kernels, or null if that combination is not compiled.
-// precision: 0 FP64, 1 mixed, 2 mixed with SFU sincos; kind: bf_phase_kind
-const PassFns *get_fns(int d, int q, int prec, int kind, int node_kind);
+// precision: 0 FP64, 1 mixed, 2 mixed with SFU sincos; kind: bf_phase_kind; wide: exact sums under
+// the root (wide_root in bf_host.h; the kinds with one, mixed precisions)
+const PassFns *get_fns(int d, int q, int prec, int kind, int node_kind, bool wide);
 
-// one function per instantiation unit: bf_inst_d{d}_{f64|mix}_{kind}.cu
+// one function per instantiation unit: bf_inst_d{d}_{f64|mix|sfu|mixw|sfuw}_{kind}.cu
 #define BFL_DECLARE(d, pr, kn) const PassFns *fns_d##d##_##pr##_##kn(int q, int node_kind);
 BFL_DECLARE(2, f64, dot) BFL_DECLARE(2, f64, genradon) BFL_DECLARE(2, f64, hypradon) BFL_DECLARE(2, f64, separable)
 BFL_DECLARE(2, mix, dot) BFL_DECLARE(2, mix, genradon) BFL_DECLARE(2, mix, hypradon) BFL_DECLARE(2, mix, separable)
@@ -65,6 +66,8 @@ BFL_DECLARE(3, f64, dot) BFL_DECLARE(3, f64, genradon) BFL_DECLARE(3, f64, separ
 BFL_DECLARE(3, mix, dot) BFL_DECLARE(3, mix, genradon) BFL_DECLARE(3, mix, separable)
 BFL_DECLARE(2, sfu, dot) BFL_DECLARE(2, sfu, genradon) BFL_DECLARE(2, sfu, hypradon) BFL_DECLARE(2, sfu, separable)
 BFL_DECLARE(3, sfu, dot) BFL_DECLARE(3, sfu, genradon) BFL_DECLARE(3, sfu, separable)
+BFL_DECLARE(2, mixw, genradon) BFL_DECLARE(2, mixw, hypradon) BFL_DECLARE(3, mixw, genradon)
+BFL_DECLARE(2, sfuw, genradon) BFL_DECLARE(2, sfuw, hypradon) BFL_DECLARE(3, sfuw, genradon)
 #undef BFL_DECLARE
 
 
@@ -95,8 +98,8 @@ cudaError_t points_final(const PointsData &pd, int fp64, int r, const void *wl, 
 // device self-checks and the FMA rate probe (bf_selfcheck.cu)
 cudaError_t measure_fma(int fp64, double *tflops);
 cudaError_t selfcheck_sincos(int n, double *max_err);
-cudaError_t phase_rate(const void *kargs_mix, int sfu, int L, int q, int kind, int paired, double *gphases);
-cudaError_t selfcheck_phase(const void *kargs_mix, const void *kargs_f64, int d, int L, int q, int kind, int n,
+cudaError_t phase_rate(const void *kargs_mix, int sfu, int wide, int L, int q, int kind, int paired, double *gphases);
+cudaError_t selfcheck_phase(const void *kargs_mix, const void *kargs_f64, int wide, int d, int L, int q, int kind, int n,
                             double *max_err);
 cudaError_t selfcheck_umma(int fmt, int split, double *max_rel_err, int *timed_out);   // fmt 0 BF16, 1 TF32
 

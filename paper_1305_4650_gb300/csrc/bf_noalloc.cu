@@ -251,7 +251,7 @@ extern "C" bf_status bf_apply_noalloc(int d, int64_t N, int q, bf_phase_kind pha
     if (prec != BF_PREC_FP64) {   // |Phi| < 2^21 cycles for the mixed path's integer rounding
         if (bfl::phase_bound(d, (int)phase, prm) >= 2097152.0) return BF_ERR_UNSUPPORTED;
     }
-    const bfl::PassFns *fns = bfl::get_fns(d, q, prec, (int)phase, prm->node_kind);
+    const bfl::PassFns *fns = bfl::get_fns(d, q, prec, (int)phase, prm->node_kind, bfl::wide_root(d, (int)phase, prm));
     if (!fns) return BF_ERR_UNSUPPORTED;
 
     // scratch needed: 2d tables of nent entries (32 B target, 16 B source) + 2 weight buffers

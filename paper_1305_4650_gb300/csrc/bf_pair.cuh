@@ -124,9 +124,9 @@ __device__ __forceinline__ void quad_sincos2(float2 r, int q0, int q1, float2 &s
 // Ph<PMIXT> on two lanes: targets and sources are per lane (a shared one is duplicated)
 template <class P, int D, int K> struct Ph2;
 
-template <bool F, int D, int K>
-struct Ph2<PMIXT<F>, D, K> {
-    using PH = Ph<PMIXT<F>, D, K>;
+template <bool F, bool W, int D, int K>
+struct Ph2<PMIXT<F, W>, D, K> {
+    using PH = Ph<PMIXT<F, W>, D, K>;
     using V = float2;   // two lanes
     static __device__ __forceinline__ V dup(float a) { return dup2(a); }
     struct T { df2 x[D]; df2 A[D]; };
@@ -177,11 +177,11 @@ struct Ph2<PMIXT<F>, D, K> {
     }
 
     // contribution of source coordinate k: entries e0 (lane 0) and e1 (lane 1)
-    static __device__ __forceinline__ Part part(const KArgs<PMIXT<F>> &a, const T &t, const MixSE &e0, const MixSE &e1, int k)
+    static __device__ __forceinline__ Part part(const KArgs<PMIXT<F, W>> &a, const T &t, const MixSE &e0, const MixSE &e1, int k)
     {
         return part_of(a, t.x[k], t.A[k], e0, e1, k == 0);
     }
-    static __device__ __forceinline__ Part part_of(const KArgs<PMIXT<F>> &a, const df2 &x, const df2 &A, const MixSE &e0,
+    static __device__ __forceinline__ Part part_of(const KArgs<PMIXT<F, W>> &a, const df2 &x, const df2 &A, const MixSE &e0,
                                                    const MixSE &e1, bool first)
     {
         Part p{dup2(0.0f), dup2(0.0f), dup2(0.0f), dup2(0.0f)};
@@ -209,10 +209,11 @@ struct Ph2<PMIXT<F>, D, K> {
         if constexpr (PH::HAS_Q) {
             p.h = add2(u.h, v.h);
             p.l = add2(u.l, v.l);
+            if constexpr (W) p.l = add2(p.l, two_sum2(u.h, v.h).lo);
         }
         return p;
     }
-    static __device__ __forceinline__ float2 sign(const KArgs<PMIXT<F>> &a, const T &t)
+    static __device__ __forceinline__ float2 sign(const KArgs<PMIXT<F, W>> &a, const T &t)
     {
         if constexpr (K == KIND_HYPRADON)
             return make_float2(copysignf(1.0f, t.x[0].hi.x), copysignf(1.0f, t.x[0].hi.y));

@@ -42,17 +42,17 @@ __device__ __forceinline__ uint32_t hash32(uint32_t x)
     return x;
 }
 
-template <int D, int K>
-__global__ void k_check_phase(bfk::KArgs<bfk::PMIX> am, bfk::KArgs<bfk::PF64> ad, int L, int q, int n, double *out)
+template <int D, int K, class PM>
+__global__ void k_check_phase(bfk::KArgs<PM> am, bfk::KArgs<bfk::PF64> ad, int L, int q, int n, double *out)
 {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
         uint32_t h = hash32(0x9e3779b9u * (uint32_t)(i + 1));
         const int lt = (int)(h % (uint32_t)(L + 1));
         h = hash32(h);
         const int ls = (int)(h % (uint32_t)(L + 1));
-        bfk::PMIX::TE te[D];
+        typename PM::TE te[D];
         bfk::PF64::TE ted[D];
-        typename bfk::Ph<bfk::PMIX, D, K>::S sm;
+        typename bfk::Ph<PM, D, K>::S sm;
         typename bfk::Ph<bfk::PF64, D, K>::S sd;
         for (int k = 0; k < D; ++k) {
             h = hash32(h);
@@ -60,15 +60,15 @@ __global__ void k_check_phase(bfk::KArgs<bfk::PMIX> am, bfk::KArgs<bfk::PF64> ad
             h = hash32(h);
             const int bs = (int)(h % (1u << (L - ls))), js = (int)((h >> 20) % (uint32_t)(q + 2));
             te[k] = am.tt[k][((1LL << lt) - 1) * (q + 2) + (int64_t)bt * (q + 2) + jt];
-            const bfk::PMIX::SE se = am.st[k][((2LL << L) - (2LL << (L - ls))) * (q + 2) + (int64_t)bs * (q + 2) + js];
+            const typename PM::SE se = am.st[k][((2LL << L) - (2LL << (L - ls))) * (q + 2) + (int64_t)bs * (q + 2) + js];
             ted[k].a = make_double2((double)te[k].a.x + te[k].a.y, (double)te[k].a.z + te[k].a.w);
             ted[k].b = make_double2((double)te[k].b.x + te[k].b.y, 0.0);
-            bfk::Ph<bfk::PMIX, D, K>::src1(sm, k, se);
+            bfk::Ph<PM, D, K>::src1(sm, k, se);
             bfk::PF64::SE sed;
             sed.a = make_double2((double)se.a.x + se.a.y, (double)se.a.z + se.a.w);
             bfk::Ph<bfk::PF64, D, K>::src1(sd, k, sed);
         }
-        const float fm = bfk::Ph<bfk::PMIX, D, K>::frac(am, bfk::Ph<bfk::PMIX, D, K>::tgt(am, te), sm);
+        const float fm = bfk::Ph<PM, D, K>::frac(am, bfk::Ph<PM, D, K>::tgt(am, te), sm);
         const double fd = bfk::Ph<bfk::PF64, D, K>::frac(ad, bfk::Ph<bfk::PF64, D, K>::tgt(ad, ted), sd);
         double e = (double)fm - fd;
         e -= rint(e);
@@ -320,12 +320,14 @@ cudaError_t phase_rate_t(const void *kargs, int L, int q, int kind, int paired, 
 
 namespace bfl {
 
-cudaError_t phase_rate(const void *kargs, int sfu, int L, int q, int kind, int paired, double *gphases)
+cudaError_t phase_rate(const void *kargs, int sfu, int wide, int L, int q, int kind, int paired, double *gphases)
 {
+    if (wide)
+        return sfu ? phase_rate_t<bfk::PMIXFW>(kargs, L, q, kind, paired, gphases)
+                   : phase_rate_t<bfk::PMIXW>(kargs, L, q, kind, paired, gphases);
     return sfu ? phase_rate_t<bfk::PMIXF>(kargs, L, q, kind, paired, gphases)
                : phase_rate_t<bfk::PMIX>(kargs, L, q, kind, paired, gphases);
 }
-
 
 cudaError_t measure_fma(int fp64, double *tflops)
 {
@@ -375,7 +377,7 @@ cudaError_t selfcheck_sincos(int n, double *max_err)
     return e;
 }
 
-cudaError_t selfcheck_phase(const void *kargs_mix, const void *kargs_f64, int d, int L, int q, int kind, int n,
+cudaError_t selfcheck_phase(const void *kargs_mix, const void *kargs_f64, int wide, int d, int L, int q, int kind, int n,
                             double *max_err)
 {
     double *dd = nullptr;
@@ -383,16 +385,23 @@ cudaError_t selfcheck_phase(const void *kargs_mix, const void *kargs_f64, int d,
     if (e != cudaSuccess) return e;
     cudaMemset(dd, 0, sizeof(double));
     const auto &am = *static_cast<const bfk::KArgs<bfk::PMIX> *>(kargs_mix);
+    const auto &aw = *static_cast<const bfk::KArgs<bfk::PMIXW> *>(kargs_mix);
     const auto &ad = *static_cast<const bfk::KArgs<bfk::PF64> *>(kargs_f64);
+#define BF_CHECK(dd_, kn)                                                        \
+    do {                                                                         \
+        if (wide) k_check_phase<dd_, kn><<<512, 256>>>(aw, ad, L, q, n, dd);     \
+        else k_check_phase<dd_, kn><<<512, 256>>>(am, ad, L, q, n, dd);          \
+    } while (0)
     switch (d * 8 + kind) {
-    case 16 + bfk::KIND_DOT: k_check_phase<2, bfk::KIND_DOT><<<512, 256>>>(am, ad, L, q, n, dd); break;
-    case 16 + bfk::KIND_GENRADON: k_check_phase<2, bfk::KIND_GENRADON><<<512, 256>>>(am, ad, L, q, n, dd); break;
-    case 16 + bfk::KIND_HYPRADON: k_check_phase<2, bfk::KIND_HYPRADON><<<512, 256>>>(am, ad, L, q, n, dd); break;
-    case 16 + bfk::KIND_SEPARABLE: k_check_phase<2, bfk::KIND_SEPARABLE><<<512, 256>>>(am, ad, L, q, n, dd); break;
-    case 24 + bfk::KIND_DOT: k_check_phase<3, bfk::KIND_DOT><<<512, 256>>>(am, ad, L, q, n, dd); break;
-    case 24 + bfk::KIND_GENRADON: k_check_phase<3, bfk::KIND_GENRADON><<<512, 256>>>(am, ad, L, q, n, dd); break;
-    default: k_check_phase<3, bfk::KIND_SEPARABLE><<<512, 256>>>(am, ad, L, q, n, dd); break;
+    case 16 + bfk::KIND_DOT: BF_CHECK(2, bfk::KIND_DOT); break;
+    case 16 + bfk::KIND_GENRADON: BF_CHECK(2, bfk::KIND_GENRADON); break;
+    case 16 + bfk::KIND_HYPRADON: BF_CHECK(2, bfk::KIND_HYPRADON); break;
+    case 16 + bfk::KIND_SEPARABLE: BF_CHECK(2, bfk::KIND_SEPARABLE); break;
+    case 24 + bfk::KIND_DOT: BF_CHECK(3, bfk::KIND_DOT); break;
+    case 24 + bfk::KIND_GENRADON: BF_CHECK(3, bfk::KIND_GENRADON); break;
+    default: BF_CHECK(3, bfk::KIND_SEPARABLE); break;
     }
+#undef BF_CHECK
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpy(max_err, dd, sizeof(double), cudaMemcpyDeviceToHost);
     cudaFree(dd);
