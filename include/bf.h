@@ -307,11 +307,14 @@ bf_status bf_pass_info(bf_plan plan, int nrhs, int i, int *kind, int *l0, int *k
  * allocate and free a few bytes of device memory and synchronise).
  *   bf_selfcheck_sincos: largest |error| of the FP32 sin/cos of 2 pi f used by the
  *     mixed path, against CUDA's FP64 sincospi, over n evenly spaced f in [-1, 1).
+ *   bf_selfcheck_sqrt: how many of n FP64 square roots, as the FP64 path takes them, differ
+ *     from the correctly rounded ones (CUDA's), over n arguments in [1e-280, 1e280].
  *   bf_selfcheck_phase: largest |error|, in cycles and modulo 1, of the mixed
  *     path's double-float Phi against FP64 arithmetic on the same table features,
  *     over n pseudo-random (target node, source node) pairs of a BF_PREC_MIXED plan
  *     (BF_ERR_INVALID_ARG for an FP64 plan). */
 bf_status bf_selfcheck_sincos(int n, double *max_abs_err);
+bf_status bf_selfcheck_sqrt(int n, double *differing);
 /* Measured FMA rate of the current device in TFLOP/s (an FMA counts 2): fp64 = 0 for
  * FP32, 1 for FP64, 2 for FP32 in packed pairs (one instruction, two FMAs).  Independent
  * dependent-FMA chains on every SM, timed with events; the context for the FP32-issue

@@ -22,7 +22,7 @@ STATUS = {0: "BF_OK", 1: "BF_ERR_INVALID_ARG", 2: "BF_ERR_UNSUPPORTED", 3: "BF_E
 
 EXPORTS = ["bf_params_default", "bf_plan_create", "bf_apply", "bf_apply_adjoint", "bf_apply_host",
            "bf_apply_batched", "bf_destroy", "bf_status_string", "bf_last_cuda_error", "bf_plan_info",
-           "bf_apply_pass", "bf_pass_info", "bf_pass_count", "bf_selfcheck_sincos", "bf_selfcheck_phase", "bf_measure_fma_rate",
+           "bf_apply_pass", "bf_pass_info", "bf_pass_count", "bf_selfcheck_sincos", "bf_selfcheck_sqrt", "bf_selfcheck_phase", "bf_measure_fma_rate",
            "bf_measure_phase_rate", "bf_batch_create", "bf_batch_apply", "bf_batch_status",
            "bf_batch_selftest_timeout", "bf_batch_info", "bf_batch_wait_stats", "bf_batch_destroy", "bf_plan_autotune",
            "bf_plan_table_info", "bf_plan_create_points", "bf_plan_points_info", "bf_plan_tc_info"]
@@ -74,6 +74,7 @@ def load():
                                      ctypes.POINTER(i32)]
         lib.bf_pass_count.argtypes = [vp, i32, ctypes.POINTER(i32)]
         lib.bf_selfcheck_sincos.argtypes = [i32, ctypes.POINTER(ctypes.c_double)]
+        lib.bf_selfcheck_sqrt.argtypes = [i32, ctypes.POINTER(ctypes.c_double)]
         lib.bf_selfcheck_phase.argtypes = [vp, i32, ctypes.POINTER(ctypes.c_double)]
         lib.bf_measure_fma_rate.argtypes = [i32, ctypes.POINTER(ctypes.c_double)]
         lib.bf_measure_phase_rate.argtypes = [vp, i32, ctypes.POINTER(ctypes.c_double)]
@@ -332,6 +333,13 @@ def selfcheck_sincos(n: int = 1 << 22) -> float:
     e = ctypes.c_double()
     _check(load().bf_selfcheck_sincos(n, ctypes.byref(e)), "bf_selfcheck_sincos")
     return e.value
+
+
+def selfcheck_sqrt(n: int = 1 << 22) -> int:
+    """How many of n FP64 square roots of the FP64 path differ from the correctly rounded ones."""
+    e = ctypes.c_double()
+    _check(load().bf_selfcheck_sqrt(n, ctypes.byref(e)), "bf_selfcheck_sqrt")
+    return int(e.value)
 
 
 def selfcheck_umma(split: bool = False, fmt: str = "bf16") -> tuple[float, bool]:

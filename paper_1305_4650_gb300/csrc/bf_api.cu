@@ -1775,6 +1775,12 @@ bf_status bf_selfcheck_sincos(int n, double *max_abs_err)
     return e == cudaSuccess ? BF_OK : BF_ERR_CUDA;
 }
 
+bf_status bf_selfcheck_sqrt(int n, double *differing)
+{
+    if (n < 1 || !differing) return BF_ERR_INVALID_ARG;
+    return bfl::selfcheck_sqrt(n, differing) == cudaSuccess ? BF_OK : BF_ERR_CUDA;
+}
+
 bf_status bf_selfcheck_umma(int split, double *max_rel_err, int *timed_out)
 {
     if ((split != 0 && split != 1) || !max_rel_err || !timed_out) return BF_ERR_INVALID_ARG;

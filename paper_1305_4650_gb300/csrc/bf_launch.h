@@ -98,6 +98,7 @@ cudaError_t points_final(const PointsData &pd, int fp64, int r, const void *wl, 
 // device self-checks and the FMA rate probe (bf_selfcheck.cu)
 cudaError_t measure_fma(int fp64, double *tflops);
 cudaError_t selfcheck_sincos(int n, double *max_err);
+cudaError_t selfcheck_sqrt(int n, double *differing);
 cudaError_t phase_rate(const void *kargs_mix, int sfu, int wide, int L, int q, int kind, int paired, double *gphases);
 cudaError_t selfcheck_phase(const void *kargs_mix, const void *kargs_f64, int wide, int d, int L, int q, int kind, int n,
                             double *max_err);

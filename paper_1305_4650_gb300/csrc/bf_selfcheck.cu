@@ -32,6 +32,16 @@ __global__ void k_check_sincos(int n, double *out)
     }
 }
 
+// sqrt_newton against CUDA's correctly rounded root, q spread over [1e-280, 1e280]: how many differ
+__global__ void k_check_sqrt(int n, double *out)
+{
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const double m = 1.0 + 3.0 * fmod((double)i * 0.6180339887498949, 1.0);
+        const double q = ldexp(m, 2 * (i % 931 - 465));
+        if (bfk::sqrt_newton(q) != sqrt(q)) atomicAdd(out, 1.0);
+    }
+}
+
 __device__ __forceinline__ uint32_t hash32(uint32_t x)
 {
     x ^= x >> 16;
@@ -40,6 +50,26 @@ __device__ __forceinline__ uint32_t hash32(uint32_t x)
     x *= 0x846ca68bU;
     x ^= x >> 16;
     return x;
+}
+
+// Phi in FP64 from the features, with CUDA's square root (none of the kernels' phase code)
+template <int D, int K>
+__device__ double phase_ref(const double (&f0)[D], const double (&f1)[D], const double (&f2)[D], const double (&y)[D],
+                            const double (&y2)[D], double c2, double sgn)
+{
+    double p = 0.0, q = 0.0;
+    for (int k = 0; k < D; ++k) {
+        if (K == bfk::KIND_SEPARABLE) p += f0[k] + y[k];
+        else if (K != bfk::KIND_HYPRADON) p += f0[k] * y[k];
+        if (K == bfk::KIND_GENRADON) {
+            const double a = c2 + (D == 2 ? (k ? f2[0] * f2[1] : f1[0] * f1[1]) : f1[k] * f2[(k + 1) % D]);
+            q += a * a * y2[k];
+        }
+        if (K == bfk::KIND_HYPRADON) q += (k ? f1[1] : 1.0) * y2[k];
+    }
+    if (K == bfk::KIND_GENRADON) return p + sgn * sqrt(q);
+    if (K == bfk::KIND_HYPRADON) return f0[0] * sqrt(q);
+    return p;
 }
 
 template <int D, int K, class PM>
@@ -51,9 +81,8 @@ __global__ void k_check_phase(bfk::KArgs<PM> am, bfk::KArgs<bfk::PF64> ad, int L
         h = hash32(h);
         const int ls = (int)(h % (uint32_t)(L + 1));
         typename PM::TE te[D];
-        bfk::PF64::TE ted[D];
+        double f0[D], f1[D], f2[D], y[D], y2[D];
         typename bfk::Ph<PM, D, K>::S sm;
-        typename bfk::Ph<bfk::PF64, D, K>::S sd;
         for (int k = 0; k < D; ++k) {
             h = hash32(h);
             const int bt = (int)(h % (1u << lt)), jt = (int)((h >> 20) % (uint32_t)(q + 2));
@@ -61,15 +90,15 @@ __global__ void k_check_phase(bfk::KArgs<PM> am, bfk::KArgs<bfk::PF64> ad, int L
             const int bs = (int)(h % (1u << (L - ls))), js = (int)((h >> 20) % (uint32_t)(q + 2));
             te[k] = am.tt[k][((1LL << lt) - 1) * (q + 2) + (int64_t)bt * (q + 2) + jt];
             const typename PM::SE se = am.st[k][((2LL << L) - (2LL << (L - ls))) * (q + 2) + (int64_t)bs * (q + 2) + js];
-            ted[k].a = make_double2((double)te[k].a.x + te[k].a.y, (double)te[k].a.z + te[k].a.w);
-            ted[k].b = make_double2((double)te[k].b.x + te[k].b.y, 0.0);
+            f0[k] = (double)te[k].a.x + te[k].a.y;
+            f1[k] = (double)te[k].a.z + te[k].a.w;
+            f2[k] = (double)te[k].b.x + te[k].b.y;
             bfk::Ph<PM, D, K>::src1(sm, k, se);
-            bfk::PF64::SE sed;
-            sed.a = make_double2((double)se.a.x + se.a.y, (double)se.a.z + se.a.w);
-            bfk::Ph<bfk::PF64, D, K>::src1(sd, k, sed);
+            y[k] = (double)se.a.x + se.a.y;
+            y2[k] = (double)se.a.z + se.a.w;
         }
         const float fm = bfk::Ph<PM, D, K>::frac(am, bfk::Ph<PM, D, K>::tgt(am, te), sm);
-        const double fd = bfk::Ph<bfk::PF64, D, K>::frac(ad, bfk::Ph<bfk::PF64, D, K>::tgt(ad, ted), sd);
+        const double fd = phase_ref<D, K>(f0, f1, f2, y, y2, ad.sc.c2, ad.sc.sgn);
         double e = (double)fm - fd;
         e -= rint(e);
         atomic_max_nonneg(out, fabs(e));
@@ -373,6 +402,19 @@ cudaError_t selfcheck_sincos(int n, double *max_err)
     k_check_sincos<<<512, 256>>>(n, d);
     e = cudaGetLastError();
     if (e == cudaSuccess) e = cudaMemcpy(max_err, d, sizeof(double), cudaMemcpyDeviceToHost);
+    cudaFree(d);
+    return e;
+}
+
+cudaError_t selfcheck_sqrt(int n, double *differing)
+{
+    double *d = nullptr;
+    cudaError_t e = cudaMalloc(&d, sizeof(double));
+    if (e != cudaSuccess) return e;
+    cudaMemset(d, 0, sizeof(double));
+    k_check_sqrt<<<512, 256>>>(n, d);
+    e = cudaGetLastError();
+    if (e == cudaSuccess) e = cudaMemcpy(differing, d, sizeof(double), cudaMemcpyDeviceToHost);
     cudaFree(d);
     return e;
 }
