@@ -42,6 +42,7 @@ struct bf_plan_s {
     int ctab_levels = -1;
     int corner = 0;            // CORNER_* of the forward passes
     bool wide = false;         // exact sums under the root (wide_root)
+    float mg = 0.0f;           // grid constant of the terms under it (sqrt_grid)
     void *gstage = nullptr, *fstage = nullptr;
     size_t csize = 8;          // bytes per complex number
     int64_t ws_bytes = 0;
@@ -361,7 +362,7 @@ void fill_args(const bf_plan_s *p, bfk::KArgs<P> &a)
     } else {
         split(2.0 * std::fabs(s) / 3.0, a.sc.c2hi, a.sc.c2lo);
         a.sc.sgn = (float)sgn;
-        a.sc.mg = bfl::sqrt_grid(p->d, p->kind, &p->prm);
+        a.sc.mg = p->mg;
     }
     a.ctab = p->ctab;
     a.ctab_levels = p->ctab_levels;
@@ -1216,6 +1217,7 @@ bf_status bf_plan_create(int d, int64_t N, int q, bf_phase_kind phase, const bf_
     p->csize = p->prec == BF_PREC_FP64 ? 16 : 8;
     // BF16X3 and TF32X3 evaluate their phases as BF_PREC_MIXED does and run the same kernels but the switch
     p->wide = bfl::wide_root(d, (int)phase, prm);
+    p->mg = bfl::sqrt_grid(d, (int)phase, prm);
     p->fns = bfl::get_fns(d, q, tc_prec(p->prec) ? (int)BF_PREC_MIXED : (int)p->prec, (int)phase, p->node_kind, p->wide);
     if (!p->fns) {   // this combination was not compiled into the library
         delete p;

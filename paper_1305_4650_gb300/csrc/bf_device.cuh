@@ -812,6 +812,11 @@ struct Cfg {
     // 4 q complex numbers, 30 warps for q <= 4 and 20 beyond; FP64 needs few warps.
     static constexpr int MINB = SMALL ? 3 : per_sm(640);
     static constexpr int MINB_COL = D == 2 && !P::is_f64 ? per_sm(960) : MINB;
+    // (q = 4, additive phases: 64 registers suffice for a fourth CTA; Fourier N = 512 461 -> 450 us)
+    static constexpr int minb_col(int kind)
+    {
+        return D == 2 && !P::is_f64 && Q == 4 && (kind == KIND_DOT || kind == KIND_SEPARABLE) ? 4 : MINB_COL;
+    }
     static constexpr int MINB_ROW = D == 2 && !P::is_f64 && Q <= 4 ? per_sm(960) : MINB;
     // the column pass reading a phase table (d = 2: one more CTA per SM than evaluating)
     static constexpr int MINB_TAB = D == 2 ? per_sm(640) + 1 : MINB;
@@ -2311,8 +2316,8 @@ template <int Q, class P, int K, bool LB> struct TileOf<2, Q, P, K, LB> { using 
 // accordingly): measured 7% faster with the polynomial sincos, 19% with the SFU one; the row
 // pass would spill.  At d = 3 the shared memory holds two CTAs per SM either way.
 template <int D, int Q, class P, int K, bool LB, int PM = PM_COMPUTE>
-__global__ void __launch_bounds__(cta_most(Cfg<D, Q, P>::NT, PM == PM_TABLE ? Cfg<D, Q, P>::MINB_TAB : Cfg<D, Q, P>::MINB_COL, D),
-                                  cta_least(PM == PM_TABLE ? Cfg<D, Q, P>::MINB_TAB : Cfg<D, Q, P>::MINB_COL, D))
+__global__ void __launch_bounds__(cta_most(Cfg<D, Q, P>::NT, PM == PM_TABLE ? Cfg<D, Q, P>::MINB_TAB : Cfg<D, Q, P>::minb_col(K), D),
+                                  cta_least(PM == PM_TABLE ? Cfg<D, Q, P>::MINB_TAB : Cfg<D, Q, P>::minb_col(K), D))
     k_col_pass(const KArgs<P> a)
 {
     static_assert(PM == PM_COMPUTE || !P::is_f64, "phase tables: mixed precisions");

@@ -81,9 +81,10 @@ inline float sqrt_grid(int d, int kind, const bf_params *p)
     if (wide_root(d, kind, p)) return 0.0f;
     double lin, root;
     phase_bounds(d, kind, p, &lin, &root);
-    int e = -60;
-    while (std::ldexp(1.0, e + 21) < root * root) ++e;
-    return (float)std::ldexp(1.5, e + 23);
+    int e = 0;
+    const double m = std::frexp(root * root, &e);   // root^2 = m 2^e, m in [1/2, 1) (or 0)
+    e = (m == 0.5 ? e - 1 : e) - 21;
+    return (float)std::ldexp(1.5, (m > 0.0 && e > -60 ? e : -60) + 23);
 }
 
 // tiles of 2^{dk} pairs per CTA of a k-level pass, np_cta pairs per CTA

@@ -154,28 +154,44 @@ struct Tile2 {
         return f;
     }
 
+    // Thread index for the work that runs beside a stage (geometry, parts and node features of the
+    // next one): from the last thread down, after `used` items of other such work (4 per pair at
+    // most, two rounds of the threads), so that where a small grid's CTA has more threads than the
+    // stage has items, the two run on different warps instead of one after the other.
+    static __device__ __forceinline__ int side(int used = 0)
+    {
+        int t = (int)blockDim.x - 1 - (int)threadIdx.x - used;
+        if (used) {   // (0 at compile time where there is none)
+            t += t < 0 ? (int)blockDim.x : 0;
+            t += t < 0 ? (int)blockDim.x : 0;
+        }
+        return t;
+    }
+
     // ---- column levels
-    static __device__ __forceinline__ void geo_col(const KArgs<P> &a, Geo *G, int l, int i)
+    static __device__ __forceinline__ Geo pair_geo(const KArgs<P> &a, int l, int i, int j)
     {
         const int k = a.k, n = 1 << (D * k), nblk = n >> D, L = a.L;
-        for (int j = threadIdx.x; j < a.T * n; j += blockDim.x) {
-            const int alpha = j & (NC - 1), beta = (j >> D) & (nblk - 1), tau = j >> (D * k);
-            uint32_t Ap, Bstar, Apg, Bq;
-            int base;
-            TL::tile_of(a, tau, Ap, Bstar);
-            TL::block_geo(Ap, Bstar, beta, i, k, Apg, Bq, base);
-            const uint32_t Aa = (Apg << D) + alpha;
-            int ca[DMAX], cbq[DMAX];
-            morton_decode<D>(Aa, l + 1, ca);
-            morton_decode<D>(Bq, L - l - 1, cbq);
-            Geo &g = G[j];
-            g.cb[0] = cbq[0];
-            g.cb[1] = cbq[1];
-            g.base = tau * n + base;
-            const typename PH::T t = tcenter<P, D, Q, K>(a, l + 1, Aa, ca);
-            g.tA = t;
-            g.sg = PH::sign(a, t);
-        }
+        const int alpha = j & (NC - 1), beta = (j >> D) & (nblk - 1), tau = j >> (D * k);
+        uint32_t Ap, Bstar, Apg, Bq;
+        int base;
+        TL::tile_of(a, tau, Ap, Bstar);
+        TL::block_geo(Ap, Bstar, beta, i, k, Apg, Bq, base);
+        const uint32_t Aa = (Apg << D) + alpha;
+        int ca[DMAX], cbq[DMAX];
+        morton_decode<D>(Aa, l + 1, ca);
+        morton_decode<D>(Bq, L - l - 1, cbq);
+        Geo g;
+        g.cb[0] = cbq[0];
+        g.cb[1] = cbq[1];
+        g.base = tau * n + base;
+        g.tA = tcenter<P, D, Q, K>(a, l + 1, Aa, ca);
+        g.sg = PH::sign(a, g.tA);
+        return g;
+    }
+    static __device__ __forceinline__ void geo_col(const KArgs<P> &a, Geo *G, int l, int i, int used = 0)
+    {
+        for (int j = side(used); j < npr(a); j += blockDim.x) G[j] = pair_geo(a, l, i, j);
     }
     // the q parts of one row: target features x and A of the row's coordinate, source entries
     // e[0..q); sp: the two nodes MID and END only; REV: in reverse order
@@ -203,16 +219,28 @@ struct Tile2 {
     // parts of the children's nodes (rows 0, 1 of both coordinates) of every output pair
     static __device__ __forceinline__ void parts_in(const KArgs<P> &a, const Geo *G, R *PT, int l, bool sp)
     {
-        for (int it = threadIdx.x; it < npr(a) * 4; it += blockDim.x) {
+        for (int it = side(); it < npr(a) * 4; it += blockDim.x) {
             const int c = it & 1, dim = (it >> 1) & 1, j = it >> 2;
             part_row(a, G[j].tA.x[dim], G[j].tA.A[dim], dim == 0, a.st[dim] + soff<Q>(a.L, l) + (2 * G[j].cb[dim] + c) * (Q + 2),
                      PT + j * PSTR + (dim * 3 + c) * PROW, sp);
         }
     }
+    // the same for the first level of a pass, each item with its own geometry, which one item of a
+    // pair keeps: one barrier and one chain of loads less than the geometry first
+    static __device__ __forceinline__ void parts_first(const KArgs<P> &a, Geo *G, R *PT, int l, int i, bool sp)
+    {
+        for (int it = side(); it < npr(a) * 4; it += blockDim.x) {
+            const int c = it & 1, dim = (it >> 1) & 1, j = it >> 2;
+            const Geo g = pair_geo(a, l, i, j);
+            if ((it & 3) == 0) G[j] = g;
+            part_row(a, dim ? g.tA.x[1] : g.tA.x[0], dim ? g.tA.A[1] : g.tA.A[0], dim == 0,
+                     a.st[dim] + soff<Q>(a.L, l) + (2 * (dim ? g.cb[1] : g.cb[0]) + c) * (Q + 2), PT + j * PSTR + (dim * 3 + c) * PROW, sp);
+        }
+    }
     // parts of the output box's nodes (row 2)
     static __device__ __forceinline__ void parts_out(const KArgs<P> &a, const Geo *G, R *PT, int l)
     {
-        for (int it = threadIdx.x; it < npr(a) * 2; it += blockDim.x) {
+        for (int it = side(); it < npr(a) * 2; it += blockDim.x) {
             const int dim = it & 1, j = it >> 1;
             part_row(a, G[j].tA.x[dim], G[j].tA.A[dim], dim == 0, a.st[dim] + soff<Q>(a.L, l + 1) + G[j].cb[dim] * (Q + 2),
                      PT + j * PSTR + (dim * 3 + 2) * PROW);
@@ -379,7 +407,7 @@ struct Tile2 {
     static __device__ __forceinline__ void geo_switch(const KArgs<P> &a, int4 *GS, int l)
     {
         const int k = a.k, n = 1 << (D * k);
-        for (int j = threadIdx.x; j < a.T * n; j += blockDim.x) {
+        for (int j = side(); j < a.T * n; j += blockDim.x) {
             uint32_t Ap, Bstar;
             TL::tile_of(a, j >> (D * k), Ap, Bstar);
             int ca[DMAX], cb[DMAX];
@@ -447,7 +475,7 @@ struct Tile2 {
     static __device__ __forceinline__ void geo_row(const KArgs<P> &a, GeoR *G, int l, int i)
     {
         const int k = a.k, n = 1 << (D * k), nblk = n >> D, L = a.L, nb = 1 << (D * i);
-        for (int j = threadIdx.x; j < a.T * nblk; j += blockDim.x) {
+        for (int j = side(); j < a.T * nblk; j += blockDim.x) {
             const int beta = j & (nblk - 1), tau = j >> (D * (k - 1));
             uint32_t Ap, Bstar, Apg, Bq;
             int base, ca[DMAX], cb[DMAX];
@@ -459,10 +487,10 @@ struct Tile2 {
         }
     }
     // features of the nodes of the tiles' target boxes at level l = l0 + i (T 2^{Di} boxes x r)
-    static __device__ __forceinline__ void node_cache(const KArgs<P> &a, typename PH::T *TC, int l, int i)
+    static __device__ __forceinline__ void node_cache(const KArgs<P> &a, typename PH::T *TC, int l, int i, int used = 0)
     {
         const int nb = 1 << (D * i);
-        for (int j = threadIdx.x; j < a.T * nb * RR; j += blockDim.x) {
+        for (int j = side(used); j < a.T * nb * RR; j += blockDim.x) {
             const int t = j % RR, aloc = (j / RR) & (nb - 1), tau = (j / RR) >> (D * i);
             uint32_t Ap, Bstar;
             TL::tile_of(a, tau, Ap, Bstar);
@@ -708,7 +736,7 @@ struct Tile2 {
     }
     static __device__ __forceinline__ void parts_in_adj(const KArgs<P> &a, const Geo *G, R *PT, int l)
     {
-        for (int it = threadIdx.x; it < npr(a) * 4; it += blockDim.x) {
+        for (int it = side(); it < npr(a) * 4; it += blockDim.x) {
             const int c = it & 1, dim = (it >> 1) & 1, j = it >> 2;
             const typename P::SE *e = a.st[dim] + soff<Q>(a.L, l) + (2 * G[j].cb[dim] + c) * (Q + 2);
             R *o = PT + j * PSTR + (dim * 3 + c) * PROW;
@@ -907,7 +935,7 @@ struct Tile2 {
             else
                 col_adj_a<false>(a, Wt, S, Gi, PT, i);
             parts_in_adj(a, Gi, PT, l);
-            if (i > i0) geo_col(a, Gn, l - 1, i - 1);
+            if (i > i0) geo_col(a, Gn, l - 1, i - 1, 4 * np);
             __syncthreads();
             if (LB && sp)
                 col_adj_b<LB>(a, Wt, S, Gi, PT, i);
@@ -971,7 +999,7 @@ struct Tile2 {
         }
         for (int i = 0; i < k1; ++i) {
             geo_row(a, G + i * nb, a.l0 + i, i);
-            node_cache(a, tc(i), a.l0 + i, i);
+            node_cache(a, tc(i), a.l0 + i, i, np >> D);
         }
         __syncthreads();
         for (int i = k1 - 1; i >= 0; --i) {
@@ -1029,7 +1057,12 @@ struct Tile2 {
         if (PM != PM_COMPUTE && skip0) tb += nlev;
         if constexpr (PM == PM_TABLE)
             if (i0 < a.k) TL::prefetch_l2(tb, nlev);
-        if (i0 < a.k) geo_col(a, G + (i0 & 1) * np, a.l0 + i0, i0);
+        if (i0 < a.k) {
+            if constexpr (PM == PM_TABLE)
+                geo_col(a, G + (i0 & 1) * np, a.l0 + i0, i0);
+            else
+                parts_first(a, G + (i0 & 1) * np, PT, a.l0 + i0, i0, sp1 && a.l0 + i0 == 1);
+        }
         if (skip0)
             init_corner(a, Wt, rhs);
         else if (a.flags & F_INIT)
@@ -1038,10 +1071,6 @@ struct Tile2 {
             TL::load(a, Wt, rhs);
         if (i0 >= a.k && (a.flags & F_SWITCH)) geo_switch(a, GS, a.l0 + a.k);
         __syncthreads();
-        if (PM != PM_TABLE && i0 < a.k) {
-            parts_in(a, G + (i0 & 1) * np, PT, a.l0 + i0, sp1 && a.l0 + i0 == 1);
-            __syncthreads();
-        }
         for (int i = i0; i < a.k; ++i) {
             const int l = a.l0 + i;
             Geo *Gi = G + (i & 1) * np, *Gn = G + (~i & 1) * np;
@@ -1059,7 +1088,7 @@ struct Tile2 {
             else
                 col_a<PM, false>(a, Wt, S, Gi, PT, i, fa);
             if constexpr (PM != PM_TABLE) parts_out(a, Gi, PT, l);
-            if (i + 1 < a.k) geo_col(a, Gn, l + 1, i + 1);
+            if (i + 1 < a.k) geo_col(a, Gn, l + 1, i + 1, 2 * np);
             __syncthreads();
             if (LB && sp)
                 col_b<PM, LB>(a, Wt, S, Gi, PT, i, fb);
@@ -1105,7 +1134,7 @@ struct Tile2 {
         TL::load(a, Wt, rhs);
         if (k1 > 0) {
             geo_row(a, G, a.l0, 0);
-            if constexpr (PM != PM_TABLE) node_cache(a, tc(0), a.l0, 0);
+            if constexpr (PM != PM_TABLE) node_cache(a, tc(0), a.l0, 0, np >> D);
         }
         __syncthreads();
         for (int i = 0; i < k1; ++i) {
