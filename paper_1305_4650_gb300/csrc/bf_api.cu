@@ -15,6 +15,7 @@
 #include "bf_launch.h"
 #include "bf_mr.cuh"
 #include <algorithm>
+#include <atomic>
 
 namespace {
 
@@ -87,6 +88,17 @@ struct bf_batch_s {
 };
 
 namespace bfl {
+int sm_count()
+{
+    static std::atomic<int> known[64];
+    int dev = 0, n = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess) return 1;
+    if (dev >= 0 && dev < 64 && (n = known[dev].load(std::memory_order_relaxed)) > 0) return n;
+    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n < 1) return 1;
+    if (dev >= 0 && dev < 64) known[dev].store(n, std::memory_order_relaxed);
+    return n;
+}
+
 const PassFns *get_fns(int d, int q, int prec, int kind, int nk, bool wide)
 {
 #define BFL_PICK(dd, kn) \
@@ -427,9 +439,7 @@ bf_status run_forward_mr(bf_plan p, const void *g, void *f, int nrhs, cudaStream
         a.wmap = (ps.row == 2 && p->tmaps) ? static_cast<const char *>(p->tmaps) + (size_t)(i & 1) * sizeof(CUtensorMap)
                                            : nullptr;   // the map of a.win
         if (ps.row >= 2) {   // the switch (2) or a column level (3) on the tensor cores, persistent CTAs
-            int dev = 0, sms = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            const int sms = bfl::sm_count();
             const bool sw = ps.row == 2, t32 = p->prec == BF_PREC_TF32X3;
             const int per_sm = sw ? (t32 ? p->fns->switch_tc32_ctas_per_sm() : p->fns->switch_tc_ctas_per_sm())
                                   : p->fns->col_tc_ctas_per_sm();
@@ -448,9 +458,7 @@ bf_status run_forward_mr(bf_plan p, const void *g, void *f, int nrhs, cudaStream
         const size_t smem = p->ptab ? mr_smem_table(p, ps, nr, a.rc) : mr_smem(p, ps, nr, a.rc);
         int64_t grid = ctas;
         if (p->ptab) {   // as many CTAs as fit; each streams the table of several tile groups
-            int dev = 0, sms = 0;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+            const int sms = bfl::sm_count();
             const int per_sm = p->fns->mr_table_occupancy(ps.row, smem);
             if (per_sm < 1) return BF_ERR_UNSUPPORTED;
             if ((int64_t)sms * per_sm < grid) grid = (int64_t)sms * per_sm;
@@ -545,7 +553,7 @@ bool schedule_adjoint_mr(bf_plan p, int nrhs)
     int &rc = p->mra_rc;
     rc = 0;
     bool ok = false;
-    if (p->prec != BF_PREC_FP64 && p->npts >= 2 * ppr * 304) {
+    if (p->prec != BF_PREC_FP64 && p->npts >= 2 * ppr * 2 * bfl::sm_count()) {
         sc = schedule(p, kmax, 2 * ppr, true, p->corner);
         rc = chunk(2 * ppr);
         ok = fits(sc, rc, 112 * 1024);
@@ -1040,9 +1048,7 @@ bf_status batch_build(bf_batch b, const bf_plan *plans, const int *nrhs, int cou
     // a work unit runs `per` consecutive CTAs of a job: about 512 units per CTA slot over the
     // whole queue, so taking a unit (an atomic and a table search) costs a few percent at
     // most while the last units still balance
-    int dev = 0, sms = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    const int sms = bfl::sm_count();
     const size_t smem_total = smem;
     if (smem_total > 227 * 1024) return BF_ERR_UNSUPPORTED;
     const int per_sm = b->fns->batch_ctas_per_sm(smem_total);

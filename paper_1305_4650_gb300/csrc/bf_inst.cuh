@@ -38,13 +38,12 @@ inline cudaError_t prepare(K kern, size_t smem, size_t *granted)
 // items of the largest stage: idle warps only make the barriers slower.  With the side work and the
 // first level's parts beside its geometry: Fourier phase, offset 0.5, N = 64, q = 3 24.9 -> 20.8 us,
 // N = 32, q = 5 35.0 -> 31.0 us; hyperbolic Radon N = 64, q = 3 28.9 -> 24.8 us.
-constexpr unsigned SMS = 152;
 template <int D, int Q, class P>
-unsigned tile_threads(int T, int k, unsigned ctas, int per_sm, int stage)
+unsigned tile_threads(int T, int k, uint64_t ctas, int per_sm, int stage)
 {
     if constexpr (D == 3) return bfk::Cfg<D, Q, P>::NT;
     const int np = T << (D * k);
-    return (unsigned)((np < 4 ? 4 : np) * Q) * (ctas <= SMS ? (unsigned)(per_sm < stage ? per_sm : stage) : 1u);
+    return (unsigned)((np < 4 ? 4 : np) * Q) * (ctas <= (uint64_t)sm_count() ? (unsigned)(per_sm < stage ? per_sm : stage) : 1u);
 }
 
 template <int D, int Q, class P, int K, bool LB, int PM = bfk::PM_COMPUTE>
@@ -54,7 +53,7 @@ cudaError_t launch_col(const void *kargs, unsigned gx, unsigned gy, size_t smem,
     cudaError_t e = prepare(bfk::k_col_pass<D, Q, P, K, LB, PM>, smem, granted);
     if (e != cudaSuccess) return e;
     const bfk::KArgs<P> &a = *static_cast<const bfk::KArgs<P> *>(kargs);
-    const unsigned nt = tile_threads<D, Q, P>(a.T, a.k, gx * gy, PM == bfk::PM_TABLE ? bfk::Cfg<D, Q, P>::MINB_TAB : bfk::Cfg<D, Q, P>::minb_col(K),
+    const unsigned nt = tile_threads<D, Q, P>(a.T, a.k, (uint64_t)gx * gy, PM == bfk::PM_TABLE ? bfk::Cfg<D, Q, P>::MINB_TAB : bfk::Cfg<D, Q, P>::minb_col(K),
                                                 (a.flags & bfk::F_SWITCH) && K != bfk::KIND_DOT && K != bfk::KIND_SEPARABLE ? Q : 3);
     bfk::k_col_pass<D, Q, P, K, LB, PM><<<dim3(gx, gy), nt, smem, s>>>(a);
     return cudaGetLastError();
@@ -67,7 +66,7 @@ cudaError_t launch_row(const void *kargs, unsigned gx, unsigned gy, size_t smem,
     cudaError_t e = prepare(bfk::k_row_pass<D, Q, P, K, LB, PM>, smem, granted);
     if (e != cudaSuccess) return e;
     const bfk::KArgs<P> &a = *static_cast<const bfk::KArgs<P> *>(kargs);
-    const unsigned nt = tile_threads<D, Q, P>(a.T, a.k, gx * gy, bfk::Cfg<D, Q, P>::MINB_ROW, 2);
+    const unsigned nt = tile_threads<D, Q, P>(a.T, a.k, (uint64_t)gx * gy, bfk::Cfg<D, Q, P>::MINB_ROW, 2);
     bfk::k_row_pass<D, Q, P, K, LB, PM><<<dim3(gx, gy), nt, smem, s>>>(a);
     return cudaGetLastError();
 }
@@ -79,7 +78,7 @@ cudaError_t launch_col_adj(const void *kargs, unsigned gx, unsigned gy, size_t s
     cudaError_t e = prepare(bfk::k_col_pass_adj<D, Q, P, K, LB>, smem, granted);
     if (e != cudaSuccess) return e;
     const bfk::KArgs<P> &a = *static_cast<const bfk::KArgs<P> *>(kargs);
-    const unsigned nt = tile_threads<D, Q, P>(a.T, a.k, gx * gy, bfk::Cfg<D, Q, P>::MINB, Q);
+    const unsigned nt = tile_threads<D, Q, P>(a.T, a.k, (uint64_t)gx * gy, bfk::Cfg<D, Q, P>::MINB, Q);
     bfk::k_col_pass_adj<D, Q, P, K, LB><<<dim3(gx, gy), nt, smem, s>>>(a);
     return cudaGetLastError();
 }
@@ -91,7 +90,7 @@ cudaError_t launch_row_adj(const void *kargs, unsigned gx, unsigned gy, size_t s
     cudaError_t e = prepare(bfk::k_row_pass_adj<D, Q, P, K, LB>, smem, granted);
     if (e != cudaSuccess) return e;
     const bfk::KArgs<P> &a = *static_cast<const bfk::KArgs<P> *>(kargs);
-    const unsigned nt = tile_threads<D, Q, P>(a.T, a.k, gx * gy, bfk::Cfg<D, Q, P>::MINB, Q);
+    const unsigned nt = tile_threads<D, Q, P>(a.T, a.k, (uint64_t)gx * gy, bfk::Cfg<D, Q, P>::MINB, Q);
     bfk::k_row_pass_adj<D, Q, P, K, LB><<<dim3(gx, gy), nt, smem, s>>>(a);
     return cudaGetLastError();
 }

@@ -6,6 +6,10 @@
 
 namespace bfl {
 
+// SMs of the current device, asked once per device (1 if the device cannot be asked: the launch
+// that follows reports why)
+int sm_count();
+
 // kargs points to a bfk::KArgs<P> of the table's precision
 typedef cudaError_t (*pass_fn)(const void *kargs, unsigned grid_x, unsigned grid_y, size_t smem, cudaStream_t s);
 
