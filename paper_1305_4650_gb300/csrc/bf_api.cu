@@ -404,6 +404,19 @@ Pass shard_pass(const bf_plan_s *p, Pass ps, bool last, int sg, int *mode, int64
     return ps;
 }
 
+// Right-hand sides per CTA of a multi-RHS pass of `ctas` tile groups.  In FP64 an SM's one pipe works
+// through every right-hand side of its CTA, so a grid that leaves SMs idle is cut into as many blocks
+// of right-hand sides as they can take, although each evaluates the phases again: Fourier phase N = 16,
+// q = 8, 3 right-hand sides 632 -> 311 us.  The mixed passes keep them together: there the phases
+// and the chain of stages are most of the time.
+int rhs_block(const bf_plan_s *p, int nrhs, int64_t ctas)
+{
+    const int mx = p->fns->mr_max, nr = nrhs < mx ? nrhs : mx;
+    const int64_t blocks = (nrhs + mx - 1) / mx, fit = bfl::sm_count() / (ctas * blocks);
+    if (p->prec != BF_PREC_FP64) return mx;
+    return fit <= 1 ? nr : (int)((nr + (fit < nr ? fit : nr) - 1) / (fit < nr ? fit : nr));
+}
+
 // Run passes [first, last) of the forward schedule.  Pass i reads workspace
 // buffer i % 2 (or g when it initialises) and writes buffer (i + 1) % 2 (or f
 // when it evaluates the targets).
@@ -420,8 +433,7 @@ bf_status run_forward_mr(bf_plan p, const void *g, void *f, int nrhs, cudaStream
     a.f = static_cast<typename P::C *>(f);
     a.nrhs = nrhs;
     const int mx = p->fns->mr_max;
-    const int nr = nrhs < mx ? nrhs : mx;
-    a.rc = p->mr_rc < nr ? p->mr_rc : nr;
+    const int nr = nrhs < mx ? nrhs : mx, rc = p->mr_rc < nr ? p->mr_rc : nr;
     void *buf[2] = {p->w0, p->w1};
     const int mode = p->ptab ? bfk::PM_TABLE : bfk::PM_COMPUTE;
     for (int i = first; i < last; ++i) {
@@ -455,7 +467,10 @@ bf_status run_forward_mr(bf_plan p, const void *g, void *f, int nrhs, cudaStream
         a.ptab = p->ptab ? static_cast<typename P::C *>(p->ptab) + p->ptab_off[i] : nullptr;
         a.ptab_cta = p->ptab ? p->ptab_cta[i] : 0;
         a.ncta = (int)ctas;
-        const size_t smem = p->ptab ? mr_smem_table(p, ps, nr, a.rc) : mr_smem(p, ps, nr, a.rc);
+        a.nb = rhs_block(p, nrhs, ctas);
+        const int held = a.nb < nr ? a.nb : nr;   // of a CTA
+        a.rc = rc < held ? rc : held;
+        const size_t smem = p->ptab ? mr_smem_table(p, ps, held, a.rc) : mr_smem(p, ps, held, a.rc);
         int64_t grid = ctas;
         if (p->ptab) {   // as many CTAs as fit; each streams the table of several tile groups
             const int sms = bfl::sm_count();
@@ -464,7 +479,7 @@ bf_status run_forward_mr(bf_plan p, const void *g, void *f, int nrhs, cudaStream
             if ((int64_t)sms * per_sm < grid) grid = (int64_t)sms * per_sm;
         }
         cudaError_t e = (ps.row ? p->fns->row_mr : p->fns->col_mr)[mode](&a, (unsigned)grid,
-                                                                         (unsigned)((nrhs + mx - 1) / mx), smem, s);
+                                                                         (unsigned)((nrhs + a.nb - 1) / a.nb), smem, s);
         if (e != cudaSuccess) return cuda_fail(p, e);
     }
     return BF_OK;
@@ -576,13 +591,12 @@ bf_status run_adjoint_mr(bf_plan p, const void *f, void *g, int nrhs, cudaStream
         p->mra_nrhs = nrhs;
     }
     const std::vector<Pass> &sc = p->passes_mra;
-    const int mx = p->fns->mr_max, nr = nrhs < mx ? nrhs : mx, rc = p->mra_rc;
+    const int rc = p->mra_rc;
     bfk::KArgs<P> a;
     fill_args<P>(p, a);
     a.fadj = static_cast<const typename P::C *>(f);
     a.gadj = static_cast<typename P::C *>(g);
     a.nrhs = nrhs;
-    a.rc = rc;
     void *buf[2] = {p->w0, p->w1};
     for (int i = (int)sc.size() - 1; i >= 0; --i) {
         const Pass &ps = sc[i];
@@ -594,8 +608,11 @@ bf_status run_adjoint_mr(bf_plan p, const void *f, void *g, int nrhs, cudaStream
         a.wout = static_cast<typename P::C *>(buf[i & 1]);
         const int64_t ctas = (p->npts >> (p->d * ps.k)) / ps.T;
         a.ncta = (int)ctas;
-        cudaError_t e = (ps.row ? p->fns->row_mr_adj : p->fns->col_mr_adj)(&a, (unsigned)ctas, (unsigned)((nrhs + mx - 1) / mx),
-                                                                           mr_smem(p, ps, nr, rc), s);
+        a.nb = rhs_block(p, nrhs, ctas);
+        const int held = a.nb < nrhs ? a.nb : nrhs;   // of a CTA
+        a.rc = rc < held ? rc : held;
+        cudaError_t e = (ps.row ? p->fns->row_mr_adj : p->fns->col_mr_adj)(&a, (unsigned)ctas, (unsigned)((nrhs + a.nb - 1) / a.nb),
+                                                                           mr_smem(p, ps, held, a.rc), s);
         if (e != cudaSuccess) return cuda_fail(p, e);
     }
     return BF_OK;
@@ -855,7 +872,7 @@ bf_status build_phase_table(bf_plan p)
     cudaEventRecord(e0);
     bfk::KArgs<P> a;
     fill_args<P>(p, a);
-    a.nrhs = 1;
+    a.nrhs = a.nb = 1;
     a.rc = 1;
     for (size_t i = 0; i < p->passes_mr.size() && e == cudaSuccess; ++i) {
         const Pass &ps = p->passes_mr[i];
@@ -1244,7 +1261,7 @@ bf_status bf_plan_create(int d, int64_t N, int q, bf_phase_kind phase, const bf_
     const int kreq = prm->fuse_levels > 0 ? prm->fuse_levels : kfit;
     p->kc = p->kr = kreq < kfit ? kreq : kfit;
     p->corner = bfl::corner_of(d, q, p->m, prm, p->fns->lobatto, tc_prec(p->prec));
-    p->passes = schedule(p, p->kc, p->fns->np, true, p->corner);
+    p->passes = schedule(p, p->kc, bfl::single_pairs(p->fns, d, p->npts), true, p->corner);
     if (p->fns->col_mr[0]) {
         // 2 fused levels, as many pairs per CTA as one switch round covers (at least one tile);
         // scratch for enough right-hand sides to give every thread an item, fewer if the
@@ -1518,7 +1535,7 @@ bf_status bf_plan_autotune(bf_plan p, int nrhs, int reps, void *stream, double *
         st = time_it(best);
         for (int k = 1; k <= p->fns->kmax && st == BF_OK; ++k)
             for (int rem = 0; rem < 2 && st == BF_OK; ++rem) {
-                std::vector<Pass> cand = schedule(p, k, p->fns->np, rem != 0, p->corner);
+                std::vector<Pass> cand = schedule(p, k, bfl::single_pairs(p->fns, p->d, p->npts), rem != 0, p->corner);
                 bool fits = true;
                 for (const Pass &ps : cand)
                     if (fwd_smem(p, ps) > 227 * 1024) fits = false;

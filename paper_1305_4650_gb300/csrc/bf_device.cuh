@@ -316,6 +316,7 @@ struct KArgs {
     int T;                            // tiles per CTA (T * 2^{dk} pairs)
     int corner;                       // CORNER_*, LEAF_*: grid points on nodes, end levels shortened
     int nrhs;                         // right-hand sides of the launch (multi-RHS kernels)
+    int nb;                           // and of one CTA, at most MRMAX (FP64; else MRMAX)
     int rc;                           // right-hand sides per scratch chunk (multi-RHS kernels)
     const void *ctab;                 // target features at box centres, levels 0..ctab_levels (or null)
     int ctab_levels;

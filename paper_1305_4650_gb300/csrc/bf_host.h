@@ -5,6 +5,7 @@
 
 #include "../../include/bf.h"
 #include "bf_device.cuh"
+#include "bf_launch.h"
 
 namespace bfl {
 
@@ -93,6 +94,15 @@ inline int tiles_of(int64_t npts, int64_t np_cta, int d, int k)
     const int64_t np = npts < np_cta ? npts : np_cta;
     const int T = (int)(np >> (d * k));
     return T < 1 ? 1 : T;
+}
+
+// Pairs per CTA of the single-RHS forward passes.  FP64 at d = 2 puts two tiles in a CTA (whole
+// warps of its FP64 instructions: Fourier phase N = 256 6.10 ms, with one tile 7.12), one where
+// the grid of single tiles leaves SMs idle: hyperbolic Radon N = 32, q = 8 1.63 -> 0.87 ms.
+inline int64_t single_pairs(const PassFns *f, int d, int64_t npts)
+{
+    const int64_t tile = (int64_t)1 << (d * f->kmax);
+    return f->np > tile && npts / tile <= sm_count() ? tile : f->np;
 }
 
 // KArgs::corner of a plan: Lobatto nodes and grid points at the lower corners of their boxes.

@@ -1201,8 +1201,9 @@ struct TileMR {
     {
         Ctx x;
         x.tile0 = (int)shard_cta<D>(a, (uint32_t)cta) * a.T;
-        x.rhs0 = (int)blockIdx.y * MRMAX;
-        x.nr = min(MRMAX, a.nrhs - x.rhs0);
+        const int nb = P::is_f64 ? a.nb : MRMAX;   // (a compile-time number is worth 1% of the mixed passes)
+        x.rhs0 = (int)blockIdx.y * nb;
+        x.nr = min(nb, a.nrhs - x.rhs0);
         x.npr = a.T << (D * a.k);
         x.rc = a.rc;
         x.lgp = __ffs(x.npr) - 1;

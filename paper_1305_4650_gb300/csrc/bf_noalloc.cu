@@ -197,7 +197,7 @@ bf_status run(int d, int L, int q, int kind, const bf_params *prm, const void *g
     int np = 0;
     a.corner = bfl::corner_of(d, q, m, prm, fns->lobatto, false);
     bfl::each_pass(L, m, kmax, true, a.corner, [&](int row, int l0, int k, int fl) {
-        ps[np++] = NaPass{row, l0, k, fl, bfl::tiles_of(npts, fns->np, d, k)};
+        ps[np++] = NaPass{row, l0, k, fl, bfl::tiles_of(npts, bfl::single_pairs(fns, d, npts), d, k)};
     });
     void *buf[2] = {w0, w1};
     for (int i = 0; i < np; ++i) {

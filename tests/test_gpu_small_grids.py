@@ -56,3 +56,25 @@ def compare(bf, spec, nrhs, precision):
                                            (6, 5, "genradon", 0.5), (7, 4, "dot", 0.0), (7, 3, "genradon", 0.5)])
 def test_one_right_hand_side(bf, L, q, phase, off, precision):
     compare(bf, spec_of(L, q, phase, off), 1, precision)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+@pytest.mark.parametrize("L,q,phase,off,nrhs", [(5, 8, "hypradon", 0.0, 2), (5, 5, "genradon", 0.5, 2), (4, 8, "dot", 0.0, 3),
+                                                (4, 5, "hypradon", 0.0, 5), (3, 6, "genradon", 0.5, 17), (5, 3, "hypradon", 0.5, 16),
+                                                (2, 4, "dot", 0.5, 9), (1, 5, "genradon", 0.0, 33)])
+def test_several_right_hand_sides(bf, L, q, phase, off, nrhs, precision):
+    compare(bf, spec_of(L, q, phase, off), nrhs, precision)
+
+
+@pytest.mark.parametrize("precision", ["fp64", "mixed"])
+def test_blocks_of_right_hand_sides_do_not_change_a_result(bf, precision):
+    """N = 16 in FP64: 16 right-hand sides in blocks of two, five one by one."""
+    import torch
+    spec = spec_of(4, 5, "hypradon", 0.5)
+    _, _, v = inputs(spec, 16, precision)
+    plan = bf.Plan.from_spec(spec, max_nrhs=16, precision=precision)
+    x = torch.from_numpy(v).cuda()
+    f, g = plan.apply(x), plan.apply_adjoint(x)
+    assert torch.equal(plan.apply(x[3:8]), f[3:8])
+    assert torch.equal(plan.apply_adjoint(x[3:8]), g[3:8])
+    plan.close()

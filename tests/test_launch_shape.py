@@ -41,3 +41,29 @@ def test_threads_follow_the_number_of_sms(tmp_path):
     for line in run(tmp_path, SRC).splitlines():
         sms, one, more, huge, capped = (int(v) for v in line.split())
         assert (one, more, huge, capped) == (960, 320, 320, 640), line
+
+
+PAIRS = r"""
+#include <cstdio>
+#include "bf_host.h"
+static int g_sms;
+namespace bfl { int sm_count() { return g_sms; } }
+int main()
+{
+    bfl::PassFns two{}, one{};
+    two.kmax = 2; two.np = 32;    // FP64 at d = 2: two tiles of 16 pairs
+    one.kmax = 3; one.np = 64;    // one tile
+    for (int sms : {60, 152}) {
+        g_sms = sms;
+        for (int L = 1; L <= 8; ++L)
+            std::printf("%d %d %d %d\n", sms, L, (int)bfl::single_pairs(&two, 2, 1ll << (2 * L)), (int)bfl::single_pairs(&one, 2, 1ll << (2 * L)));
+    }
+}
+"""
+
+
+def test_fp64_blocks_hold_one_tile_where_sms_would_idle(tmp_path):
+    for line in run(tmp_path, PAIRS).splitlines():
+        sms, L, two, one = (int(v) for v in line.split())
+        assert one == 64
+        assert two == (16 if 4 ** L // 16 <= sms else 32), line
