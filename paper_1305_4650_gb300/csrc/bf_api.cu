@@ -582,6 +582,26 @@ bool schedule_adjoint_mr(bf_plan p, int nrhs)
     return ok;
 }
 
+// Whether several right-hand sides of a mixed-precision adjoint at d = 2 run the single-RHS passes,
+// one block of CTAs each, which fill the SMs at most once and at least half.  The multi-RHS passes share
+// the phases, but a grid of few CTAs more than the SMs takes two rounds or shares an SM with too
+// few threads to hide their chains of stages; and of an additive phase, cheap to evaluate, they share
+// little where they have no more CTAs per right-hand side (many nodes per box).  N = 64, 2
+// right-hand sides, offset 0.5, multi and single: hyperbolic Radon q = 3 31 and 29 us, q = 4 39 and 37,
+// q = 6 93 and 74, but q = 5, two CTAs of 400 threads, 54 and 56; Fourier N = 32, q = 8 51 and 49,
+// hyperbolic Radon 76 and 82.
+bool adjoint_by_one(const bf_plan_s *p, int nrhs)
+{
+    if (p->prec == BF_PREC_FP64 || p->passes_adj.empty()) return false;
+    const Pass &ps = p->passes_adj.front();
+    const int64_t sms = bfl::sm_count(), one = (p->npts >> (p->d * ps.k)) / ps.T;
+    const int64_t ppr = p->fns->mr_nthreads / p->r, pairs = ppr < 16 && p->prm.fuse_levels != 1 ? 16 : ppr;   // of a multi-RHS CTA
+    const int64_t many = p->npts / pairs, round = (many + sms - 1) / sms;
+    const int64_t threads = (round < p->fns->mr_per_sm ? round : p->fns->mr_per_sm) * p->fns->mr_nthreads;
+    const bool additive = p->kind == BF_PHASE_DOT || p->kind == BF_PHASE_SEPARABLE;
+    return one * nrhs <= sms && 2 * one * nrhs >= sms && ((round > 1 && threads < 640) || (additive && many <= one));
+}
+
 template <class P>
 bf_status run_adjoint_mr(bf_plan p, const void *f, void *g, int nrhs, cudaStream_t s)
 {
@@ -1618,7 +1638,7 @@ bf_status bf_apply_adjoint(bf_plan p, const void *f, void *g, int nrhs, void *st
     bool capturing = false;
     bf_status st = stream_guard(p, s, &capturing);
     if (st != BF_OK) return st;
-    if (p->d == 2 && (nrhs > 1 || p->prec == BF_PREC_FP64)) {
+    if (p->d == 2 && ((nrhs > 1 && !adjoint_by_one(p, nrhs)) || p->prec == BF_PREC_FP64)) {
         if (p->prec == BF_PREC_FP64) st = run_adjoint_mr<bfk::PF64>(p, f, g, nrhs, s);
         else if (p->prec == BF_PREC_MIXED_SFU) st = run_adjoint_mr<bfk::PMIXF>(p, f, g, nrhs, s);
         else st = run_adjoint_mr<bfk::PMIX>(p, f, g, nrhs, s);

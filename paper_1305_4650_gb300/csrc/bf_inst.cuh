@@ -300,7 +300,7 @@ const PassFns *fns_set()
                                   {launch_row_mr<Q, P, K, LB, bfk::PM_COMPUTE>, launch_row_mr<Q, P, K, LB, bfk::PM_BUILD>,
                                    launch_row_mr<Q, P, K, LB, bfk::PM_TABLE>},
                                   launch_mr_adj<Q, P, K, LB, false>, launch_mr_adj<Q, P, K, LB, true>,
-                                  bfk::MRMAX, bfk::CfgMR<Q>::NT,
+                                  bfk::MRMAX, bfk::CfgMR<Q>::NT, bfk::MinbMR<Q, P>::v,
                                   launch_batch<Q, P, K, LB>, batch_ctas_per_sm<Q, P, K, LB>, mr_table_occupancy<Q, P, K, LB>,
                                   launch_ctab<D, Q, P, K>, (int)sizeof(typename bfk::Ph<P, D, K>::T),
                                   {TAB ? launch_col<D, (TAB ? Q : 2), P, K, TAB && LB, bfk::PM_BUILD> : nullptr,
@@ -318,7 +318,7 @@ const PassFns *fns_set()
         // d = 3: single-RHS passes with a reduced-phase table; no multi-RHS kernels
         static const PassFns f = {launch_col<D, Q, P, K, LB>, launch_row<D, Q, P, K, LB>, launch_col_adj<D, Q, P, K, LB>,
                                   launch_row_adj<D, Q, P, K, LB>, CF::KMAX, CF::NP, CF::NT, LB ? 1 : 0, tile_smem<D, Q, P, K>, adj_smem<D, Q, P, K>, {nullptr, nullptr, nullptr},
-                                  {nullptr, nullptr, nullptr}, nullptr, nullptr, 0, 0, nullptr, nullptr, nullptr,
+                                  {nullptr, nullptr, nullptr}, nullptr, nullptr, 0, 0, 0, nullptr, nullptr, nullptr,
                                   launch_ctab<D, Q, P, K>, (int)sizeof(typename bfk::Ph<P, D, K>::T),
                                   {launch_col<D, Q, P, K, LB, bfk::PM_BUILD>, launch_col<D, Q, P, K, LB, bfk::PM_TABLE>},
                                   {launch_row<D, Q, P, K, LB, bfk::PM_BUILD>, launch_row<D, Q, P, K, LB, bfk::PM_TABLE>},
@@ -331,14 +331,14 @@ const PassFns *fns_set()
                                   {launch_col_mr<Q, P, K, LB, bfk::PM_COMPUTE>, nullptr, nullptr},
                                   {launch_row_mr<Q, P, K, LB, bfk::PM_COMPUTE>, nullptr, nullptr},
                                   launch_mr_adj<Q, P, K, LB, false>, launch_mr_adj<Q, P, K, LB, true>,
-                                  bfk::MRMAX, bfk::CfgMR<Q>::NT, nullptr, nullptr, nullptr,
+                                  bfk::MRMAX, bfk::CfgMR<Q>::NT, bfk::MinbMR<Q, P>::v, nullptr, nullptr, nullptr,
                                   launch_ctab<D, Q, P, K>, (int)sizeof(typename bfk::Ph<P, D, K>::T),
                                   {nullptr, nullptr}, {nullptr, nullptr}, nullptr, nullptr, 0, nullptr, nullptr, 0};
         return &f;
     } else {
         static const PassFns f = {launch_col<D, Q, P, K, LB>, launch_row<D, Q, P, K, LB>, launch_col_adj<D, Q, P, K, LB>,
                                   launch_row_adj<D, Q, P, K, LB>, CF::KMAX, CF::NP, CF::NT, LB ? 1 : 0, tile_smem<D, Q, P, K>, adj_smem<D, Q, P, K>, {nullptr, nullptr, nullptr},
-                                  {nullptr, nullptr, nullptr}, nullptr, nullptr, 0, 0, nullptr, nullptr, nullptr,
+                                  {nullptr, nullptr, nullptr}, nullptr, nullptr, 0, 0, 0, nullptr, nullptr, nullptr,
                                   launch_ctab<D, Q, P, K>, (int)sizeof(typename bfk::Ph<P, D, K>::T),
                                   {nullptr, nullptr}, {nullptr, nullptr}, nullptr, nullptr, 0, nullptr, nullptr, 0};
         return &f;

@@ -31,6 +31,7 @@ struct PassFns {
     pass_fn col_mr_adj, row_mr_adj;   // multi-RHS adjoint passes (d = 2)
     int mr_max;                  // right-hand sides one multi-RHS CTA holds
     int mr_nthreads;             // threads per multi-RHS CTA
+    int mr_per_sm;               // multi-RHS CTAs per SM that the registers are cut for
     // persistent batch kernel (bf_mr.cuh): bargs points to a bfk::BatchArgs<P>
     cudaError_t (*batch)(const void *bargs, unsigned grid, size_t smem, cudaStream_t s);
     int (*batch_ctas_per_sm)(size_t smem);

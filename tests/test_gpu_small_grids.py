@@ -78,3 +78,17 @@ def test_blocks_of_right_hand_sides_do_not_change_a_result(bf, precision):
     assert torch.equal(plan.apply(x[3:8]), f[3:8])
     assert torch.equal(plan.apply_adjoint(x[3:8]), g[3:8])
     plan.close()
+
+
+@pytest.mark.parametrize("L,q,phase", [(6, 3, "hypradon"), (6, 4, "genradon"), (6, 6, "hypradon"), (7, 2, "dot"), (5, 8, "dot")])
+def test_two_right_hand_sides_of_the_adjoint_run_as_one_each(bf, L, q, phase):
+    """Where the single-RHS passes fill the SMs once, two right-hand sides give the bits of one at a time."""
+    import torch
+    spec = spec_of(L, q, phase, 0.5)
+    _, _, v = inputs(spec, 2, "mixed")
+    plan = bf.Plan.from_spec(spec, max_nrhs=2)
+    x = torch.from_numpy(v).cuda()
+    both = plan.apply_adjoint(x)
+    assert all(torch.equal(both[j], plan.apply_adjoint(x[j:j + 1])[0]) for j in range(2))
+    plan.close()
+    compare(bf, spec, 2, "mixed")
