@@ -76,15 +76,6 @@ __device__ __forceinline__ df fast_two_sum(float a, float b)
     return {s, __fsub_rn(b, __fsub_rn(s, a))};
 }
 
-__device__ __forceinline__ df df_mul(df x, df y)
-{
-    float p = __fmul_rn(x.hi, y.hi);
-    float e = __fmaf_rn(x.hi, y.hi, -p);
-    e = __fmaf_rn(x.hi, y.lo, e);
-    e = __fmaf_rn(x.lo, y.hi, e);
-    return fast_two_sum(p, e);
-}
-
 __device__ __forceinline__ df df_add(df x, df y)
 {
     df s = two_sum(x.hi, y.hi);
@@ -118,9 +109,9 @@ __device__ __forceinline__ float rsqrt_approx(float x)
     return r;
 }
 
-// sg sqrt(h + l) minus its nearest integer, sg = +-1, for h + l > 0 given to about 2^-44
-// relative: one Newton step from the FP32 reciprocal root, added to the exact difference of
-// the FP32 root and its nearest integer, so only a number of at most 1/2 is rounded
+// sg sqrt(h + l) minus its nearest integer, sg = +-1, for h + l > 0 (the sum of Ph::add): one Newton
+// step from the FP32 reciprocal root, added to the exact difference of the FP32 root and its nearest
+// integer, so only a number of at most 1/2 is rounded
 __device__ __forceinline__ float sqrt_frac(float h, float l, float sg)
 {
     const float M = 12582912.0f;
@@ -283,6 +274,8 @@ __device__ __forceinline__ float2 cjmul(float2 a, float2 b)
     return make_float2(__fmaf_rn(a.x, b.x, a.y * b.y), __fmaf_rn(a.x, b.y, -(a.y * b.x)));
 }
 __device__ __forceinline__ double2 cjmul(double2 a, double2 b) { return make_double2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x); }
+__device__ __forceinline__ float2 madd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
+__device__ __forceinline__ double2 madd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ void cfma(float2 &acc, float m, float2 v) { acc.x = fmaf(m, v.x, acc.x); acc.y = fmaf(m, v.y, acc.y); }
 __device__ __forceinline__ void cfma(double2 &acc, double m, double2 v) { acc.x = fma(m, v.x, acc.x); acc.y = fma(m, v.y, acc.y); }
 // acc += m v with m given twice (m2 = (m, m)): one packed FMA on sm_100+, the same roundings as cfma
@@ -786,9 +779,10 @@ __global__ void k_center_table(const KArgs<P> a, typename Ph<P, D, K>::T *out, i
 // ------------------------------------------------------------ tile passes
 //
 // A CTA owns NP consecutive pairs of the pass's input level: T = NP / 2^{dk}
-// tiles of 2^{dk} pairs.  It runs NT = NP * q threads, and every stage below is
-// cut into a multiple of NT equal work items, so no thread idles at a barrier
-// while others finish a longer item.
+// tiles of 2^{dk} pairs.  It runs NT = NP * q threads (more where a small grid
+// leaves SMs idle, tile_threads), and most stages are cut into a multiple of
+// NP * q equal items; the shortened end levels and the work beside a stage
+// (parts, geometry) have fewer.
 
 constexpr int kmax_for(int D, int RR, int CS, int Q)
 {
@@ -828,6 +822,8 @@ struct Cfg {
 constexpr int cta_most(int nt, int minb, int d) { return d == 2 ? nt * minb : nt; }
 constexpr int cta_least(int minb, int d) { return d == 2 ? 1 : minb; }
 
+// The tile code of both dimensions (indexes, end steps, the factorised switch, the factors of ph and
+// ph2) and the levels of d = 3; those of d = 2 are Tile2 and TileMR.
 template <int D, int Q, class P, int K>
 struct Tile {
     using R = typename P::R;
@@ -844,8 +840,7 @@ struct Tile {
         int cbq[DMAX];       // coordinates of the parent source box
         int base;            // the merge block's first input slot in the tile
     };
-    static_assert(sizeof(Geo) % 16 == 0 && sizeof(Geo) == (sizeof(typename PH::T) + 16 + 15) / 16 * 16,
-                  "Geo size (the host reserves round16(tsize + 16) bytes per pair)");
+    static_assert(sizeof(Geo) % 16 == 0, "Geo records lie one behind the other on 16-byte boundaries");
 
     // ---- reduced-phase table of a single-RHS pass (mixed precisions).  The block of
     // one stage is [phase j of an item][item], so one phase index over a warp's items is one
@@ -986,9 +981,6 @@ struct Tile {
         e1.y = sn.y;
     }
 
-    static __device__ __forceinline__ float2 cadd(float2 x, float2 y) { return make_float2(x.x + y.x, x.y + y.y); }
-    static __device__ __forceinline__ double2 cadd(double2 x, double2 y) { return make_double2(x.x + y.x, x.y + y.y); }
-
     // (Ap, B*) of the CTA's tile tau: tile index = Ap * 2^{D(L-l0-k)} + B*
     static __device__ __forceinline__ void tile_of(const KArgs<P> &a, int tau, uint32_t &Ap, uint32_t &Bstar)
     {
@@ -1073,19 +1065,9 @@ struct Tile {
         Bq = (Bstar << (D * (k - i - 1))) + bp;
     }
 
-    // acc += M[h][t][u] v in the column levels and the first stage of the row levels.  d = 2:
-    // two scalar FMAs, the coefficient a kernel-parameter operand (a packed FMA needs the
-    // duplicated pair M2 in registers first; at N = 1024, q = 5 the column passes 1% and the
-    // row passes 1% faster); d = 3 and the row levels' second stage, whose coefficient index
-    // is not a compile-time constant, keep the packed form, which measured 0.5-2% faster
-    // there.  The same roundings either way.
-    static __device__ __forceinline__ void imac(C &acc, const KArgs<P> &a, int h, int t, int u, C v)
-    {
-        if constexpr (D == 2)
-            cfma(acc, a.M[h][t][u], v);
-        else
-            cfma2(acc, a.M2[h][t][u], v);
-    }
+    // acc += M[h][t][u] v in the column levels and the first stage of the row levels as one packed
+    // FMA (d = 3; 0.5-2% faster there than two scalar ones, with the same roundings)
+    static __device__ __forceinline__ void imac(C &acc, const KArgs<P> &a, int h, int t, int u, C v) { cfma2(acc, a.M2[h][t][u], v); }
 
     // ---- one column-form merge level (l -> l+1) on all tiles of the CTA
     template <int PM = PM_COMPUTE>
@@ -1279,7 +1261,7 @@ struct Tile {
                 for (int j = 0; j < D - 1; ++j) { tk[j] = tt % Q; tt /= Q; }
             }
             typename PH::Part pl = PH::part(a, tA, sget<P, Q>(a, 0, l + 1, cbq[0], tk[0]), 0);
-            if constexpr (D == 3) pl = PH::add(pl, PH::part(a, tA, sget<P, Q>(a, 1, l + 1, cbq[1], tk[1]), 1));
+            pl = PH::add(pl, PH::part(a, tA, sget<P, Q>(a, 1, l + 1, cbq[1], tk[1]), 1));
             C *wo = Wt + tau * n * RR + (base + (alpha << (D * i))) * RR + tl;
             if constexpr (!P::is_f64) {
                 // phases two at a time: lanes t_{d-1} and t_{d-1} + 1 (the last one alone for odd q)
@@ -1445,7 +1427,7 @@ struct Tile {
                     for (int u = 0; u < Q; ++u) {
                         const C v = in[off + u * pw[dim]];
                         if constexpr (ADJ)
-                            acc = cadd(acc, cjmul(e[u], v));
+                            acc = madd(acc, cjmul(e[u], v));
                         else
                             cmac(acc, e[u], v);
                     }
@@ -1577,7 +1559,7 @@ struct Tile {
                 const int base = ((beta >> (D * i)) << (D * (i + 1))) + (beta & ((1 << (D * i)) - 1));
                 C acc = X[it * NC];
 #pragma unroll
-                for (int c = 1; c < NC; ++c) acc = cadd(acc, X[it * NC + c]);
+                for (int c = 1; c < NC; ++c) acc = madd(acc, X[it * NC + c]);
                 Wt[(tau * n + base + (alpha << (D * i))) * RR + RR - 1] = acc;
             }
             __syncthreads();
@@ -1817,7 +1799,7 @@ struct Tile {
                 for (int j = 1; j < D; ++j) { tk[j] = tt % Q; tt /= Q; }
             }
             typename PH::Part hp = PH::part(a, tA, sget<P, Q>(a, 1, l + 1, cbq[1], tk[1]), 1);
-            if constexpr (D == 3) hp = PH::add(hp, PH::part(a, tA, sget<P, Q>(a, 2, l + 1, cbq[2], tk[2]), 2));
+            hp = PH::add(hp, PH::part(a, tA, sget<P, Q>(a, 2, l + 1, cbq[2], tk[2]), 2));
             const C *wi = Wt + tau * n * RR + (base + (alpha << (D * i))) * RR + th * Q;
             C z[2][Q];
 #pragma unroll
@@ -1918,7 +1900,7 @@ struct Tile {
 #pragma unroll
                             for (int t1 = 0; t1 < Q; ++t1) cfma2(v, a.M2[c1][t1][s1], w[t1 * Q + s2]);
                             const C e = expphase_part<P, D, K>(a, tA, PH::add(p2, PH::part(a, tA, sget<P, Q>(a, 1, l, cb[1], s1), 1)));
-                            acc[s1 + Q * s2] = cadd(acc[s1 + Q * s2], cjmul(e, v));
+                            acc[s1 + Q * s2] = madd(acc[s1 + Q * s2], cjmul(e, v));
                         }
                     }
                 }
@@ -2095,24 +2077,24 @@ struct Tile {
                     using PH2 = Ph2<P, D, K>;
                     const typename PH2::T tS2 = PH2::dup(tS);
                     typename PH2::Part hp = PH2::part(a, tS2, eh[1], eh[1], 1);
-                    if constexpr (D == 3) hp = PH2::add(hp, PH2::part(a, tS2, eh[2], eh[2], 2));
+                    hp = PH2::add(hp, PH2::part(a, tS2, eh[2], eh[2], 2));
 #pragma unroll
                     for (int t0 = 0; t0 + 1 < Q; t0 += 2) {
                         float2 E0, E1;
                         expphase_part2<P, D, K>(a, tS2, PH2::add(PH2::part(a, tS2, e0[t0], e0[t0 + 1], 0), hp), E0, E1);
-                        acc[t0] = cadd(acc[t0], cjmul(E0, vs));
-                        acc[t0 + 1] = cadd(acc[t0 + 1], cjmul(E1, vs));
+                        acc[t0] = madd(acc[t0], cjmul(E0, vs));
+                        acc[t0 + 1] = madd(acc[t0 + 1], cjmul(E1, vs));
                     }
                     if constexpr (Q & 1)
-                        acc[Q - 1] = cadd(acc[Q - 1], cjmul(expphase_part<P, D, K>(
+                        acc[Q - 1] = madd(acc[Q - 1], cjmul(expphase_part<P, D, K>(
                                                                 a, tS, PH::add(PH::part(a, tS, e0[Q - 1], 0), PH2::lane0(hp))),
                                                             vs));
                 } else {
                     typename PH::Part hp = PH::part(a, tS, eh[1], 1);
-                    if constexpr (D == 3) hp = PH::add(hp, PH::part(a, tS, eh[2], 2));
+                    hp = PH::add(hp, PH::part(a, tS, eh[2], 2));
 #pragma unroll
                     for (int t0 = 0; t0 < Q; ++t0)
-                        acc[t0] = cadd(acc[t0], cjmul(expphase_part<P, D, K>(a, tS, PH::add(PH::part(a, tS, e0[t0], 0), hp)), vs));
+                        acc[t0] = madd(acc[t0], cjmul(expphase_part<P, D, K>(a, tS, PH::add(PH::part(a, tS, e0[t0], 0), hp)), vs));
                 }
             }
             C *w = S + (tau * n + sl) * RR + th * Q;

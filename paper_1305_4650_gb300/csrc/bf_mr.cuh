@@ -14,7 +14,8 @@
 //   W  [nr][npr][r]       weights of every right-hand side (in place, as in Tile)
 //   S  [rc][2 npr r + ..] stage scratch (row scratch units padded, mr_pad)
 //   PC [5 r npr + ..]     phase cache of the current stage (strides padded, mr_pad)
-// Stage items and the order of every accumulation follow Tile<2,...>.
+// Stages and accumulations are those of Tile2 (bf_tile2.cuh), in another order where lanes run over
+// pairs or two outputs share an item.
 //
 // Phase tables (the precompute trade-off of Section 1.4).  A plan may keep every phase
 // factor of its apply in device memory: PM_BUILD runs the phase stages only and writes
@@ -116,7 +117,7 @@ struct MinbMR {
 // bytes), chosen per q by counting the wavefronts of every access pattern of the stages
 // (TileMR::spread, gather) for 16 pairs; the phase-table layout stays compact.  Wavefronts
 // without and with them: q = 3 1242 and 720, q = 4 5120 and 3264, q = 6 6360 and 4956,
-// q = 7 7770 and 4032, q = 8 33792 and 20736.
+// q = 8 33792 and 20736.
 struct MRPad {
     int ca;   // column modulation: per (pair, chi) block of 2 r factors
     int cb;   // column demodulation: per pair (r factors)
@@ -993,7 +994,7 @@ struct TileMR {
 #pragma unroll
                     for (int u = 0; u < Q; ++u) {
                         if constexpr (ADJ)
-                            acc = TL::cadd(acc, cjmul(e[u * Q + s], v[u]));
+                            acc = madd(acc, cjmul(e[u * Q + s], v[u]));
                         else
                             cmac(acc, e[s * Q + u], v[u]);
                     }
@@ -1146,7 +1147,7 @@ struct TileMR {
             } else {
                 const C *w = W + rb * WS + pr * RR;
                 for (int t = 0; t < RR; ++t)
-                    if (a.lsrc[t % Q] * a.lsrc[t / Q] != R(0)) acc = TL::cadd(acc, cjmul(PC[pr * RR + t], w[t]));
+                    if (a.lsrc[t % Q] * a.lsrc[t / Q] != R(0)) acc = madd(acc, cjmul(PC[pr * RR + t], w[t]));
             }
             a.gadj[(int64_t)(x.rhs0 + rb) * a.npts + ((int64_t)cb[0] << L) + cb[1]] = acc;
         }

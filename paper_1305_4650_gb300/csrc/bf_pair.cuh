@@ -52,12 +52,6 @@ __device__ __forceinline__ df2 df_mul_u2(const df2 &x, const df2 &y)
     return {p, e};
 }
 
-__device__ __forceinline__ df2 df_mul2(const df2 &x, const df2 &y)
-{
-    const df2 u = df_mul_u2(x, y);
-    return fast_two_sum2(u.hi, u.lo);
-}
-
 __device__ __forceinline__ df2 df_add2(const df2 &x, const df2 &y)
 {
     const df2 s = two_sum2(x.hi, y.hi);

@@ -40,9 +40,6 @@ __host__ __device__ constexpr int triv(int h, int u)
     return u == 0 ? 0 : (u == Q - 1 ? (Q - 1) / 2 : -1);
 }
 
-__device__ __forceinline__ float2 madd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ double2 madd(double2 a, double2 b) { return make_double2(a.x + b.x, a.y + b.y); }
-
 // acc += M[h][t][u] v with compile-time h, t, u: two scalar FMAs whose coefficient is a
 // kernel-parameter operand (a packed FMA needs the coefficient pair in registers first and
 // measured 1% slower), nothing or an addition for the unit columns
@@ -118,11 +115,6 @@ struct Tile2 {
     static __device__ __forceinline__ void store2(R *p, Part2 o)
     {
         PH::each(o, [&](V &v, int c) { *reinterpret_cast<V *>(p + c * QE) = v; });
-    }
-    static __device__ __forceinline__ Part2 swap(Part2 p)
-    {
-        PH::each(p, [&](V &v, int) { const R x = v.x; v.x = v.y; v.y = x; });
-        return p;
     }
     static __device__ __forceinline__ Part lane(Part2 p, int j)
     {
@@ -514,7 +506,7 @@ struct Tile2 {
             P1 = PH2::part(a, t2, s1[0], s1[1], 1);   // lanes c_1 = 0, 1
         }
         TL::template ph2<PM>(sg, PH2::add(P0, P1), ft.at(j0, it), ft.at(j0 + 3, it), E[0], E[3]);
-        TL::template ph2<PM>(sg, PH2::add(P0, swap(P1)), ft.at(j0 + 2, it), ft.at(j0 + 1, it), E[2], E[1]);
+        TL::template ph2<PM>(sg, PH2::add(P0, PH2::swap(P1)), ft.at(j0 + 2, it), ft.at(j0 + 1, it), E[2], E[1]);
     }
     // pre-modulation, in place: items (block, t), the block's four inputs at node t of the parent
     // box (conjugate factors; ADJ: the factors themselves)
