@@ -638,7 +638,12 @@ bf_status run_adjoint_mr(bf_plan p, const void *f, void *g, int nrhs, cudaStream
     return BF_OK;
 }
 
-// the multi-RHS schedule serves nrhs >= 2 where it is compiled (d = 2)
+// The multi-RHS schedule serves two and more right-hand sides where it is compiled (d = 2): an apply
+// then gives the bits of the persistent batch, which has no other kernels.  Time of the single-RHS
+// passes over that of the multi-RHS ones, offset 0.5, N = 64 to 256: mixed, three right-hand sides,
+// q = 5 1.35 to 1.44 (generalized Radon), 1.30 to 1.39 (hyperbolic), 1.09 to 1.12 (Fourier), q = 3 0.80
+// to 1.16; two, q = 5 0.99 to 1.06, 0.94 to 1.03 and 0.80 to 0.84, so there the line costs up to a
+// fifth; FP64 1.04 to 1.9 from two on.
 bool use_mr(const bf_plan_s *p, int nrhs)
 {
     return (nrhs >= 2 || p->ptab) && !p->passes_mr.empty() && !p->points;
