@@ -39,10 +39,10 @@ FP32_LANES_PER_SM = 128
 # workload, from one ncu capture of `python bench.py --steps 1 --warmup 1 --no-cpu-baseline --no-accuracy
 # --fp64-steps 0 --no-autotune --no-tables --no-batched`.  They describe the kernels as built from sources with the recorded hash and the recorded pass schedule; otherwise the figure is
 # dropped (traffic: null) until captured again.
-TRAFFIC = {"genradon2d": {"src_sha256": "00764ea7840952519b62d7bbfd2537b3adc4fa300fed5c36c8a98ec233cb1638",
+TRAFFIC = {"genradon2d": {"src_sha256": "ba7275b5bd8a363209d02743a1496760d6fe99629de7a6fe5c33491a09039c1c",
                           "schedule": ["col2", "col3", "row2", "row3"],
-                          "bytes": [157255936, 368046336, 369234176, 215354368]}}
-TRAFFIC_SRC = ("bf_device.cuh", "bf_tile2.cuh", "bf_host.h", "bf_inst.cuh")   # the pass kernels and their launch configuration
+                          "bytes": [158853376, 369362432, 369629952, 215116032]}}
+TRAFFIC_SRC = ("bf_device.cuh", "bf_pair.cuh", "bf_tile2.cuh", "bf_host.h", "bf_inst.cuh")   # the pass kernels and their launch configuration
 
 
 def measured_hbm_gbs():
@@ -245,6 +245,29 @@ def work_ops(spec, w):
     return w["phases"] * phase_ops(spec.phase, spec.d, spec.q) + 2 * w["macs"] + 4 * w["cmuls"] + 4 * w["cmacs"]
 
 
+LEFT_OPS = {"genradon": 37, "hypradon": 33, "dot": 20, "separable": 20}   # of a factor with shared parts (mixed)
+
+
+def left_ops(spec, nrhs=1):
+    """Operations of one mixed-precision apply that the kernels still do, where pass_work counts the method's:
+    parts of the phases shared by a pair, no multiply-adds for the unit columns of odd q, and the
+    shortened end levels of corner grids (Lobatto nodes, offset 0; odd q at d = 2, any q at d = 3)."""
+    d, q, L = spec.d, spec.q, spec.L
+    n, r = 2.0 ** (L * d), q ** d
+    lobatto = spec.node_kind == 0
+    per_level = (2 ** d + 1) * r
+    macs = (2 ** (d + 1) - 2) * q ** (d + 1) * (0.6 if d == 2 and q % 2 and lobatto else 1.0)
+    factors, mac = L * per_level, L * macs
+    if lobatto and spec.tgt_off == 0.0 and spec.src_off == 0.0:
+        if d == 2 and q % 2 and L >= 4:        # two levels free, two from four nodes of a child
+            factors, mac = (L - 4) * per_level + 2 * (2 ** d * 4 + r), (L - 4) * macs + 2 * 0.35 * macs
+        elif d == 3 and L >= 2:                # one node per leaf
+            factors, mac = (L - 2) * per_level + 2 * (2 ** d + r), (L - 2) * macs + macs * q / r
+    split = spec.phase in ("dot", "separable")
+    sw_factors, sw_macs = (d * q * q, d * q ** (d + 1)) if split else (r * r, r * r)
+    return n * (factors + sw_factors) * LEFT_OPS[spec.phase] + nrhs * n * (2 * mac + 4 * factors + 4 * sw_macs)
+
+
 # ---------------------------------------------------------------- our arm
 
 def run_ours(args, rank, world, local_rank):
@@ -342,6 +365,9 @@ def run_ours(args, rank, world, local_rank):
                 "pass_ms": [round(t, 4) for t in tpass]}
     all_ops = sum(work_ops(spec, pass_work(spec, p, nrhs)) for p in passes)
     roofline["apply_frac"] = round(all_ops / (ms * 1e-3) / 1e12 / peak, 4)
+    roofline["counts"] = ("frac, apply_frac: the method's operations, every level in general form and parts of the phases "
+                          "per factor; apply_frac_left: those that the kernels still do")
+    roofline["apply_frac_left"] = round(left_ops(spec, nrhs) / (ms * 1e-3) / 1e12 / peak, 4) if prec != "fp64" else None
     roofline["measured_fma_tflops"] = {"fp32": round(bf.measure_fma_rate(False), 1),
                                        "fp32_packed_pairs": round(bf.measure_fma_rate(packed=True), 1),
                                        "fp64": round(fma64, 3)}
@@ -528,8 +554,8 @@ def run_ours(args, rank, world, local_rank):
             "config": {"workload": spec.name, "d": spec.d, "N": spec.N, "q": spec.q, "r": spec.r,
                        "phase": spec.phase, "precision": prec, "nrhs": nrhs, "switch_level": spec.switch_level,
                        "arithmetic": {"fp64": "complex128 weights, FP64 phase and sincos",
-                                      "mixed": "complex64 weights, FP32 interpolation; Phi in double-float FP32 (>= 44 "
-                                               "bits) reduced mod 1, polynomial FP32 sincos",
+                                      "mixed": "complex64 weights, FP32 interpolation; Phi in double-float FP32 reduced "
+                                               "mod 1 (error below 3e-7 cycles), polynomial FP32 sincos",
                                       "mixed_sfu": "as mixed, sin/cos from the special-function unit",
                                       "bf16x3": "as mixed; with several RHS the switch on the tensor cores, BF16x3 "
                                                 "products with FP32 accumulation",
