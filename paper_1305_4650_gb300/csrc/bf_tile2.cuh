@@ -19,8 +19,8 @@
 //    level 1 has four non-zero nodes per input, and the transposed statements hold for the
 //    last two levels: the target values are sums of weights of level L - 1 at four nodes.
 //
-// Measured (generalized Radon, q = 5, one right-hand side): N = 1024 5.28 -> 3.75 ms, N = 128
-// 100 -> 63 us; hyperbolic Radon N = 512 with 16 right-hand sides (TileMR, the same three
+// Measured (generalized Radon, q = 5, one right-hand side): N = 1024 5.28 -> 3.69 ms, N = 128
+// 100 -> 60 us; hyperbolic Radon N = 512 with 16 right-hand sides (TileMR, the same three
 // points) 8.24 -> 6.10 ms; the largest share is point 3, which leaves 8 of 10 levels at
 // N = 1024, two of them with a third of the factors.
 //
